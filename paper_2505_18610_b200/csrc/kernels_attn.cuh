@@ -3,7 +3,7 @@
 //
 // Work decomposition.  Every (batch, kv_head) slice is two runs of 16-token tiles: the INT16 run
 // (sink tiles + window ring) and the body run at the block's current width.  A tile of the body
-// weighs one unit, an INT16 tile `w16` units (their byte ratio), and every slice starts with a few
+// weighs one unit, an INT16 tile int16_units() of them (their byte ratio), and every slice starts with a few
 // empty units that stand for the fixed cost of a segment.  All units of all slices form one
 // line that is cut into equal contiguous pieces, one per CTA of a persistent grid (one CTA of 16
 // warps per SM), so every CTA streams the same number of bytes whatever the shape.  The part of a
@@ -13,6 +13,12 @@
 // own running (max, sum, accumulator), the warps are merged in shared memory and the segment
 // publishes one partial (m, l, o[128]) per head.  The CTA that publishes the
 // last partial of a slice (atomic ticket, nobody waits) merges the slice and writes the output.
+//
+// A segment's fixed part is a chain of latencies, and a short context is nothing else: which block and slice
+// (the host says which block a CTA starts in, divisions are 32-bit or double products), query, fragments, ...,
+// warp merge, publish, combine.  Written as few dependent steps as possible it costs about 5 us of the 10.5 us a
+// one-block launch over a 4K context takes (15.6 us before, with 64-bit divisions, a fence in every thread,
+// bank conflicts in the merge and one memory round trip per pass of the combine).
 //
 // Two contraction paths share this decomposition.  The 4- and 2-bit body, which holds most bytes of a
 // cache in its steady state, runs on tcgen05.mma with its code operands in tensor memory
@@ -61,15 +67,16 @@ struct AttnParams {
   int kv_heads, group, q_heads, n_slices;
   int n_tokens, n_sink_eff, win_start, cur_bits;
   int n_body, body_tiles, aux_tiles, sink_tiles;
-  int w16;                    // units of one INT16 tile
   int units_lead;             // empty units at the start of every slice: the fixed cost of one more segment
-  long long units_aux, units_slice, units_total, units_per_cta;  // units_aux includes units_lead
+  int units_aux, units_slice, units_total;  // units of the lead and the INT16 tiles, of a slice, of the block
   // Where this block's units sit on the line that is cut into CTA pieces.  A launch for one block has
   // origin 0 and weight 1; the all-blocks launch strings the blocks together, each unit weighing
   // `unit_weight` fine units (blocks of different widths cost different time per tile).
   long long line_origin;      // fine units before this block's first unit
   int unit_weight;            // fine units per unit
   int cta_origin;             // first CTA that touches this block (partials are numbered from it)
+  long long per_cta;          // fine units of a CTA's piece, and its reciprocal
+  double inv_per_cta;
   float qk_scale;             // sm_scale * log2(e)
 };
 
@@ -125,6 +132,7 @@ __device__ __forceinline__ float ex2(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+__device__ __forceinline__ float exp2i(int e) { return __int_as_float((e + 127) << 23); }  // 2^e, -126 <= e <= 127
 __device__ __forceinline__ uint32_t pack_half2(float lo, float hi) {
   const __half2 h = __floats2half2_rn(lo, hi);
   return *reinterpret_cast<const uint32_t *>(&h);
@@ -211,13 +219,17 @@ __device__ __forceinline__ void qk_phase(const uint8_t *tile0, const QFrag &qa, 
   constexpr int CHUNKS = BITS / 2;
   // ---- scores: S = Q'' K^T, heads on M (hi rows 0-7, lo rows 8-15), tokens on N ----
   if constexpr (BITS == 16) {
+    // every K chunk is asked for before the first MMA: one round trip to memory instead of two
     const uint8_t *kp = tile0 + lane * 16;
+    uint4 kc[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) kc[q] = __ldcg(reinterpret_cast<const uint4 *>(kp + q * 512));
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       uint32_t kw[16];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const uint4 a = __ldcg(reinterpret_cast<const uint4 *>(kp + (4 * r + q) * 512));
+        const uint4 a = kc[4 * r + q];
         kw[4 * q] = a.x; kw[4 * q + 1] = a.y; kw[4 * q + 2] = a.z; kw[4 * q + 3] = a.w;
       }
       float lo[4] = {0.f, 0.f, 0.f, 0.f}, hi[4] = {0.f, 0.f, 0.f, 0.f};
@@ -425,51 +437,59 @@ __device__ __forceinline__ void process_tiles(const uint8_t *tile0, uint32_t mas
 
 // ---- where the partials of a slice live ------------------------------------------------------
 // Slice s covers units [s U, (s+1) U); the segment of CTA c in it publishes partial number (c - cta_origin) + s.
-// A unit belongs to the CTA whose piece holds the unit's first fine unit (units_per_cta counts fine units).
-__device__ __forceinline__ int unit_owner(const AttnParams &p, long long unit) {
-  return (int)((p.line_origin + unit * p.unit_weight) / p.units_per_cta);
+// A unit belongs to the CTA whose piece holds the unit's first fine unit (per_cta counts fine units).  Fine units
+// are 64-bit numbers below 2^53: their quotients are taken as a double product (off by one at most) and put
+// right, a handful of instructions where a 64-bit division is a call of a hundred.
+__device__ __forceinline__ long long floor_div(long long x, long long d, double inv_d) {
+  long long q = (long long)((double)x * inv_d);
+  const long long r = x - q * d;
+  if (r < 0) --q;
+  else if (r >= d) ++q;
+  return q;
+}
+__device__ __forceinline__ int unit_owner(const AttnParams &p, int unit) {
+  return (int)floor_div(p.line_origin + (long long)unit * p.unit_weight, p.per_cta, p.inv_per_cta);
 }
 __device__ __forceinline__ void slice_ctas(const AttnParams &p, int slice, int &c_first, int &c_last) {
-  const long long lo = (long long)slice * p.units_slice;
+  const int lo = slice * p.units_slice;
   c_first = unit_owner(p, lo + p.units_lead);  // a CTA that only touches the lead units has no segment
   c_last = unit_owner(p, lo + p.units_slice - 1);
 }
 
-// Log-sum-exp merge of the partials of one slice (all published).  Warp w merges head w;
-// a lane owns 4 channels, and the weights of up to 32 partials at a time (one per lane).
-__device__ __forceinline__ void combine_slice(const AttnParams &p, int slice) {
+// Log-sum-exp merge of the n_parts partials of one slice (all published), the first one at `base`.  Warp w
+// merges head w; a lane owns 4 channels.  Partials are taken eight at a time with all their loads in flight
+// together, so up to eight cost one round trip to L2.
+__device__ __forceinline__ void combine_slice(const AttnParams &p, int slice, const float *base, int n_parts) {
+  constexpr int kAtOnce = 8;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int b = slice / p.kv_heads, hkv = slice % p.kv_heads;
-  int cf, cl;
-  slice_ctas(p, slice, cf, cl);
-  const int n_parts = cl - cf + 1;
-  const float *base = p.partials + (size_t)(cf - p.cta_origin + slice) * kMaxGroup * kPartialStride;
+  const int b = slice / p.kv_heads, hkv = slice - b * p.kv_heads;
   for (int h = warp; h < p.group; h += kAttnWarps) {
     const float *ph = base + (size_t)h * kPartialStride;
-    float M = kNegBig;
-    for (int c = lane; c < n_parts; c += 32) M = fmaxf(M, __ldcg(ph + (size_t)c * kMaxGroup * kPartialStride));
-#pragma unroll
-    for (int o = 16; o; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+    float M = kNegBig, den = 0.f;
     float4 num = make_float4(0.f, 0.f, 0.f, 0.f);
-    float den = 0.f;
-    for (int c0 = 0; c0 < n_parts; c0 += 32) {
-      float w = 0.f;
-      if (c0 + lane < n_parts) {
-        const float2 ml = __ldcg(reinterpret_cast<const float2 *>(ph + (size_t)(c0 + lane) * kMaxGroup * kPartialStride));
-        w = ex2(ml.x - M);
-        den = fmaf(w, ml.y, den);
+    for (int c0 = 0; c0 < n_parts; c0 += kAtOnce) {
+      float2 ml[kAtOnce];
+      float4 o4[kAtOnce];
+#pragma unroll
+      for (int j = 0; j < kAtOnce; ++j) {
+        const float *pc = ph + (size_t)min(c0 + j, n_parts - 1) * (kMaxGroup * kPartialStride);
+        ml[j] = __ldcg(reinterpret_cast<const float2 *>(pc));
+        o4[j] = __ldcg(reinterpret_cast<const float4 *>(pc + 4) + lane);
       }
-      const int nb = min(32, n_parts - c0);
-#pragma unroll 8
-      for (int j = 0; j < nb; ++j) {
-        const float wj = __shfl_sync(0xffffffffu, w, j);
-        const float4 o4 = __ldcg(reinterpret_cast<const float4 *>(ph + (size_t)(c0 + j) * kMaxGroup * kPartialStride + 4) + lane);
-        num.x = fmaf(wj, o4.x, num.x); num.y = fmaf(wj, o4.y, num.y);
-        num.z = fmaf(wj, o4.z, num.z); num.w = fmaf(wj, o4.w, num.w);
+      float m_new = M;
+#pragma unroll
+      for (int j = 0; j < kAtOnce; ++j) m_new = fmaxf(m_new, ml[j].x);
+      const float f = ex2(M - m_new);
+      den *= f; num.x *= f; num.y *= f; num.z *= f; num.w *= f;
+      M = m_new;
+#pragma unroll
+      for (int j = 0; j < kAtOnce; ++j) {
+        const float w = c0 + j < n_parts ? ex2(ml[j].x - M) : 0.f;
+        den = fmaf(w, ml[j].y, den);
+        num.x = fmaf(w, o4[j].x, num.x); num.y = fmaf(w, o4[j].y, num.y);
+        num.z = fmaf(w, o4[j].z, num.z); num.w = fmaf(w, o4[j].w, num.w);
       }
     }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) den += __shfl_xor_sync(0xffffffffu, den, o);
     const float inv = 1.0f / den;
     float4 *dst = reinterpret_cast<float4 *>(p.out + ((size_t)b * p.q_heads + hkv * p.group + h) * kHeadDim) + lane;
     *dst = make_float4(num.x * inv, num.y * inv, num.z * inv, num.w * inv);
@@ -485,7 +505,7 @@ __device__ __forceinline__ uint4 q_fragment(const float (*s_q)[kHeadDim], int e_
 #pragma unroll
   for (int beta = 0; beta < 2; ++beta) {
     const int W = 2 * s + beta;
-    const float scl = ldexpf(1.0f, F::EQ - F::pos(W % F::N) - e_g);
+    const float scl = exp2i(F::EQ - F::pos(W % F::N) - e_g);
     const int c0 = 16 * s + 8 * beta + 2 * tig;
     const float x0 = s_q[g][c0] * scl, x1 = s_q[g][c0 + 1] * scl;
     const __half h0 = __float2half_rn(x0), h1 = __float2half_rn(x1);
@@ -497,10 +517,13 @@ __device__ __forceinline__ uint4 q_fragment(const float (*s_q)[kHeadDim], int e_
   return make_uint4(r[0], r[1], r[2], r[3]);
 }
 
-// Fills the CTA's copy of the fragments at width BITS (all threads; a barrier must follow).
+// Fills the CTA's copy of the fragments at width BITS, by the threads first_thread .. first_thread + 255 (a barrier
+// must follow).
 template <int BITS>
-__device__ __forceinline__ void fill_q_fragments(uint4 *s_frag, const float (*s_q)[kHeadDim], const float *s_stat) {
-  for (int i = threadIdx.x; i < 256; i += kAttnThreads) {  // entry (k-step i / 32, lane i % 32)
+__device__ __forceinline__ void fill_q_fragments(uint4 *s_frag, const float (*s_q)[kHeadDim], const float *s_stat,
+                                                 int first_thread = 0) {
+  const int i = (int)threadIdx.x - first_thread;  // entry (k-step i / 32, lane i % 32)
+  if (i >= 0 && i < 256) {
     const int l = i & 31, g = l >> 2;
     s_frag[i] = q_fragment<BITS>(s_q, (int)s_stat[g], g, l & 3, i >> 5);
   }
@@ -509,21 +532,27 @@ __device__ __forceinline__ void fill_q_fragments(uint4 *s_frag, const float (*s_
 // ---- pieces of a segment that both contraction paths share --------------------------------------
 
 // Q'' = Q * lambda * sm_scale * log2(e)  (Eq. 9: the equalization scale migrates into Q), per-head
-// exponent of max |q''| and sum of q''.  Ends with a CTA-wide barrier.
+// exponent of max |q''| and sum of q''.  Warp h takes head h, four channels per lane.  Ends with a CTA-wide barrier.
 __device__ __forceinline__ void build_query(const AttnParams &p, int b, int hkv, float (*s_q)[kHeadDim], float *s_stat) {
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  for (int i = tid; i < kMaxGroup * kHeadDim; i += kAttnThreads) {
-    const int h = i >> 7, ch = i & 127;
-    float v = 0.f;
-    if (h < p.group) {
-      const uint16_t raw = p.Q[((size_t)b * p.q_heads + hkv * p.group + h) * kHeadDim + ch];
-      v = __fmul_rn(__fmul_rn(__uint_as_float((uint32_t)raw << 16), p.lambda[hkv * kHeadDim + ch]), p.qk_scale);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (warp < kMaxGroup) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (warp < p.group) {
+      const uint16_t *src = p.Q + ((size_t)b * p.q_heads + hkv * p.group + warp) * kHeadDim + 4 * lane;
+      uint2 raw;
+      if ((reinterpret_cast<uintptr_t>(p.Q) & 7) == 0) {
+        raw = *reinterpret_cast<const uint2 *>(src);
+      } else {  // a caller's query tensor may sit at any bf16 address
+        raw.x = src[0] | ((uint32_t)src[1] << 16);
+        raw.y = src[2] | ((uint32_t)src[3] << 16);
+      }
+      const float4 lam = *reinterpret_cast<const float4 *>(p.lambda + hkv * kHeadDim + 4 * lane);
+      v.x = __fmul_rn(__fmul_rn(__uint_as_float(raw.x << 16), lam.x), p.qk_scale);
+      v.y = __fmul_rn(__fmul_rn(__uint_as_float(raw.x & 0xFFFF0000u), lam.y), p.qk_scale);
+      v.z = __fmul_rn(__fmul_rn(__uint_as_float(raw.y << 16), lam.z), p.qk_scale);
+      v.w = __fmul_rn(__fmul_rn(__uint_as_float(raw.y & 0xFFFF0000u), lam.w), p.qk_scale);
     }
-    s_q[h][ch] = v;
-  }
-  __syncthreads();
-  if (warp < kMaxGroup) {  // per-head max |q''| and sum q''
-    const float4 v = *reinterpret_cast<const float4 *>(&s_q[warp][lane * 4]);
+    *reinterpret_cast<float4 *>(&s_q[warp][4 * lane]) = v;
     float mx = fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
     float sm = (v.x + v.y) + (v.z + v.w);
 #pragma unroll
@@ -532,8 +561,8 @@ __device__ __forceinline__ void build_query(const AttnParams &p, int b, int hkv,
       sm += __shfl_xor_sync(0xffffffffu, sm, o);
     }
     if (lane == 0) {
-      int e = 0;
-      if (mx > 0.f) frexpf(mx, &e);  // mx = f * 2^e, f in [0.5, 1)
+      // mx = f * 2^e, f in [0.5, 1); the bounds keep every power of two built from e a normal number
+      const int e = mx > 0.f ? max(-100, min(110, (int)(__float_as_uint(mx) >> 23) - 126)) : 0;
       s_stat[warp] = (float)e;
       s_stat[8 + warp] = sm;
     }
@@ -543,13 +572,8 @@ __device__ __forceinline__ void build_query(const AttnParams &p, int b, int hkv,
 
 // unit of the V accumulators: a power of two >= every INT16 V scale of this slice
 __device__ __forceinline__ float slice_sigma16(const AttnParams &p, int slice) {
-  const float s16 = __uint_as_float(__ldcg(p.vmax_bits + slice));
-  if (s16 > 0.f) {
-    int e;
-    frexpf(s16, &e);
-    return ldexpf(1.0f, e);
-  }
-  return 1.0f;
+  const unsigned s16 = __ldcg(p.vmax_bits + slice);  // a non-negative float's bit pattern
+  return s16 ? exp2i(max(-126, (int)(s16 >> 23) - 126)) : 1.0f;
 }
 
 // The INT16 tiles [a_lo, a_hi) of a slice (sink tiles, then the window ring), drawn from the shared
@@ -562,12 +586,12 @@ __device__ __forceinline__ void run_int16_tiles(const AttnParams &p, const uint8
   if (it >= a_hi) return;
   QFrag qa;
   qa.mine = s_frag + lane;
-  const float mu = ldexpf(1.0f, 24 - F16::EQ + e_g);
-  const float inv_sigma_e = ldexpf(1.0f, F16::EP) / sigma16;
+  const float mu = exp2i(24 - F16::EQ + e_g);
+  const float inv_sigma_e = exp2i(F16::EP) / sigma16;
   const int n_win = p.n_tokens - p.win_start;
   const int first_slot = n_win > 0 ? (p.win_start - p.geom.n_sink) % p.geom.ring_tokens : 0;
   do {
-    uint32_t mask = 0;
+    uint32_t mask;
     const uint8_t *tile;
     if (it < p.sink_tiles) {
       const int live = max(0, min(16, p.n_sink_eff - 16 * it));
@@ -576,18 +600,24 @@ __device__ __forceinline__ void run_int16_tiles(const AttnParams &p, const uint8
     } else {
       const int rt = it - p.sink_tiles;
       tile = slice_base + p.geom.ring_off + (size_t)rt * tile_bytes(16);
-      if (n_win > 0) {
-        for (int r = 0; r < 16; ++r) {
-          int d = rt * 16 + r - first_slot;
-          if (d < 0) d += p.geom.ring_tokens;
-          if (d < n_win) mask |= 1u << r;
-        }
-      }
+      int d = rt * 16 + (lane & 15) - first_slot;  // lane r looks at row r of the tile
+      if (d < 0) d += p.geom.ring_tokens;
+      mask = __ballot_sync(0xffffffffu, d < n_win) & 0xFFFFu;
     }
     if (mask == 0xFFFFu) process_tiles<16, 1, false>(tile, mask, st, qa, mu, sumq, inv_sigma_e, lane);
     else if (mask) process_tiles<16, 1, true>(tile, mask, st, qa, mu, sumq, inv_sigma_e, lane);
     it = a_lo + claim_next(s_ctr, lane);
   } while (it < a_hi);
+}
+
+// Sums of a warp's state over the quad of a head: every lane of the quad gets them.
+__device__ __forceinline__ void quad_sums(const WarpState &st, float &l_sum, float &zs_sum) {
+  l_sum = st.l.x + st.l.y;
+  zs_sum = st.zs.x + st.zs.y;
+  l_sum += __shfl_xor_sync(0xffffffffu, l_sum, 1);
+  l_sum += __shfl_xor_sync(0xffffffffu, l_sum, 2);
+  zs_sum += __shfl_xor_sync(0xffffffffu, zs_sum, 1);
+  zs_sum += __shfl_xor_sync(0xffffffffu, zs_sum, 2);
 }
 
 // A warp's running state -> its partial (m, l, o[128]) per head in real units, slot `slot`.
@@ -596,11 +626,8 @@ template <class FactorOf>
 __device__ __forceinline__ void store_warp_partial(const WarpState &st, FactorOf f_of, float (*s_o)[kMaxGroup][kHeadDim],
                                                    float *s_m, float *s_l, int slot, int lane) {
   const int g = lane >> 2, tig = lane & 3;
-  float l_sum = st.l.x + st.l.y, zs_sum = st.zs.x + st.zs.y;
-  l_sum += __shfl_xor_sync(0xffffffffu, l_sum, 1);
-  l_sum += __shfl_xor_sync(0xffffffffu, l_sum, 2);
-  zs_sum += __shfl_xor_sync(0xffffffffu, zs_sum, 1);
-  zs_sum += __shfl_xor_sync(0xffffffffu, zs_sum, 2);
+  float l_sum, zs_sum;
+  quad_sums(st, l_sum, zs_sum);
   if (tig == 0) {
     s_m[slot * 8 + g] = st.m;
     s_l[slot * 8 + g] = l_sum;
@@ -619,13 +646,40 @@ __device__ __forceinline__ void store_warp_partial(const WarpState &st, FactorOf
   }
 }
 
-// Merges the segment's n_parts partials (all written, a CTA-wide barrier passed), publishes the segment's
-// partial, and lets the CTA that publishes the slice's last partial merge the slice (nobody waits).
+// Where this CTA's partial of a slice goes.
+__device__ __forceinline__ float *partial_slot(const AttnParams &p, int slice) {
+  return p.partials + (size_t)((int)blockIdx.x - p.cta_origin + slice) * kMaxGroup * kPartialStride;
+}
+
+// The segment's partial is written (by all threads): count it, and let the CTA that publishes the slice's last
+// partial merge the slice (nobody waits).  One thread's fence after the CTA-wide barrier covers the whole CTA's
+// stores (barrier and fence order them cumulatively); a fence in every thread costs a microsecond.
+__device__ __forceinline__ void publish_partial(const AttnParams &p, int slice, int *s_ctr) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const unsigned t = atomicAdd(p.tickets + slice, 1u);
+    int cf, cl;
+    slice_ctas(p, slice, cf, cl);
+    s_ctr[2] = (t + 1u == (unsigned)(cl - cf + 1)) ? 1 : 0;
+    s_ctr[3] = cl - cf + 1;
+    s_ctr[4] = cf;
+    __threadfence();
+  }
+  __syncthreads();
+  if (s_ctr[2]) {
+    combine_slice(p, slice, p.partials + (size_t)(s_ctr[4] - p.cta_origin + slice) * kMaxGroup * kPartialStride, s_ctr[3]);
+    if (threadIdx.x == 0) p.tickets[slice] = 0u;  // ready for the next launch (stream order)
+  }
+  __syncthreads();  // the segment's shared memory may be reused
+}
+
+// Merges the segment's n_parts partials (all written, a CTA-wide barrier passed) and publishes the result.
 __device__ __forceinline__ void publish_segment(const AttnParams &p, int slice, int n_parts,
                                                 const float (*s_o)[kMaxGroup][kHeadDim], const float *s_m, const float *s_l,
                                                 int *s_ctr) {
   const int tid = threadIdx.x;
-  float *part = p.partials + (size_t)((int)blockIdx.x - p.cta_origin + slice) * kMaxGroup * kPartialStride;
+  float *part = partial_slot(p, slice);
   for (int i = tid; i < p.group * kHeadDim; i += kAttnThreads) {
     const int h = i >> 7, ch = i & 127;
     float M = kNegBig;
@@ -642,35 +696,87 @@ __device__ __forceinline__ void publish_segment(const AttnParams &p, int slice, 
       __stcg(part + h * kPartialStride + 1, l);
     }
   }
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) {
-    int cf, cl;
-    slice_ctas(p, slice, cf, cl);
-    const unsigned t = atomicAdd(p.tickets + slice, 1u);
-    s_ctr[2] = (t + 1u == (unsigned)(cl - cf + 1)) ? 1 : 0;
-  }
-  __syncthreads();
-  if (s_ctr[2]) {
-    __threadfence();
-    combine_slice(p, slice);
-    if (tid == 0) p.tickets[slice] = 0u;  // ready for the next launch (stream order)
-  }
-  __syncthreads();  // the segment's shared memory may be reused
+  publish_partial(p, slice, s_ctr);
 }
 
-// Ranges of a segment [u_lo, u_hi) (units relative to the slice): INT16 tiles [a_lo, a_hi) (a tile belongs to
-// the segment that holds its first unit) and body tiles [t_lo, t_hi).
-__device__ __forceinline__ void segment_ranges(const AttnParams &p, long long u_lo, long long u_hi, int &a_lo, int &a_hi,
-                                               int &t_lo, int &t_hi) {
+// A segment on the warp-level MMA path ends here: the warps' states become one partial per head.  The warps first
+// exchange their references, so each scales its own accumulators to the segment's common one on the way to
+// shared memory and the merge is a plain sum of 16 numbers per output.  Head rows are padded to kMergeRow floats:
+// the four heads a store instruction touches then fall into different banks (unpadded, the 32 stores of a
+// warp each took four passes and the merge 3 of a short segment's 9 us).
+constexpr int kMergeRow = kHeadDim + 8;
+constexpr int kMergeBytes = kAttnWarps * kMaxGroup * kMergeRow * 4;
+template <class FactorOf>
+__device__ __forceinline__ void merge_warps(const AttnParams &p, int slice, const WarpState &st, FactorOf f_of,
+                                            float (*s_o)[kMaxGroup][kMergeRow], float *s_ml, int *s_ctr) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, tig = lane & 3;
+  float l_sum, zs_sum;
+  quad_sums(st, l_sum, zs_sum);
+  if (tig == 0) {  // [head][warp], sums behind the references
+    s_ml[g * kAttnWarps + warp] = st.m;
+    s_ml[(kMaxGroup + g) * kAttnWarps + warp] = l_sum;
+  }
+  __syncthreads();  // also: every warp is done with its stages, which s_o shares memory with
+  float M = kNegBig;
+#pragma unroll
+  for (int w = 0; w < kAttnWarps; w += 4) {
+    const float4 m4 = *reinterpret_cast<const float4 *>(s_ml + g * kAttnWarps + w);
+    M = fmaxf(M, fmaxf(fmaxf(m4.x, m4.y), fmaxf(m4.z, m4.w)));
+  }
+  const float f_mine = ex2(st.m - M);
+  const float z_mine = zs_sum * f_mine;
+  const float f0 = __shfl_sync(0xffffffffu, f_mine, (2 * tig) * 4), f1 = __shfl_sync(0xffffffffu, f_mine, (2 * tig + 1) * 4);
+  const float zs0 = __shfl_sync(0xffffffffu, z_mine, (2 * tig) * 4), zs1 = __shfl_sync(0xffffffffu, z_mine, (2 * tig + 1) * 4);
+#pragma unroll
+  for (int mt = 0; mt < 8; ++mt) {
+#pragma unroll
+    for (int rr = 0; rr < 2; ++rr) {
+      const float f = f_of(2 * mt + rr);
+      const int ch = 16 * mt + 8 * rr + g;
+      s_o[warp][2 * tig][ch] = fmaf(st.acc[mt][2 * rr], f * f0, zs0);
+      s_o[warp][2 * tig + 1][ch] = fmaf(st.acc[mt][2 * rr + 1], f * f1, zs1);
+    }
+  }
+  float *part = partial_slot(p, slice);
+  if (warp < p.group) {  // warp h: the reference and the denominator of head h
+    float m = kNegBig, l = 0.f;
+    if (lane < kAttnWarps) {
+      m = s_ml[warp * kAttnWarps + lane];
+      l = s_ml[(kMaxGroup + warp) * kAttnWarps + lane];
+    }
+    float mm = m;
+#pragma unroll
+    for (int o = 8; o; o >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, o));
+    l *= ex2(m - mm);
+#pragma unroll
+    for (int o = 8; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    if (lane == 0) __stcg(reinterpret_cast<float2 *>(part + warp * kPartialStride), make_float2(mm, l));
+  }
+  __syncthreads();
+  for (int i = tid; i < p.group * (kHeadDim / 2); i += kAttnThreads) {
+    const int h = i >> 6, c2 = i & 63;
+    float2 o = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int w = 0; w < kAttnWarps; ++w) o = __fadd2_rn(o, *reinterpret_cast<const float2 *>(&s_o[w][h][2 * c2]));
+    __stcg(reinterpret_cast<float2 *>(part + h * kPartialStride + 4) + c2, o);
+  }
+  publish_partial(p, slice, s_ctr);
+}
+
+// Ranges of a segment [u_lo, u_hi) (units relative to the slice) of a block at width BITS: INT16 tiles [a_lo, a_hi) (a
+// tile belongs to the segment that holds its first unit) and body tiles [t_lo, t_hi).
+template <int BITS> __host__ __device__ constexpr int int16_tile_units() { return (tile_bytes(16) + tile_bytes(BITS) - 1) / tile_bytes(BITS); }
+template <int BITS>
+__device__ __forceinline__ void segment_ranges(const AttnParams &p, int u_lo, int u_hi, int &a_lo, int &a_hi, int &t_lo, int &t_hi) {
+  constexpr int W16 = int16_tile_units<BITS>();
   a_lo = a_hi = t_lo = t_hi = 0;
   if (u_lo < p.units_aux) {
-    a_lo = (int)((max(u_lo - p.units_lead, 0ll) + p.w16 - 1) / p.w16);
-    a_hi = (int)((min(u_hi, p.units_aux) - p.units_lead + p.w16 - 1) / p.w16);
+    a_lo = (max(u_lo - p.units_lead, 0) + W16 - 1) / W16;
+    a_hi = (min(u_hi, p.units_aux) - p.units_lead + W16 - 1) / W16;
   }
   if (u_hi > p.units_aux) {
-    t_lo = (int)(max(u_lo, p.units_aux) - p.units_aux);
-    t_hi = (int)(u_hi - p.units_aux);
+    t_lo = max(u_lo, p.units_aux) - p.units_aux;
+    t_hi = u_hi - p.units_aux;
   }
 }
 
@@ -681,19 +787,19 @@ __device__ __forceinline__ void segment_ranges(const AttnParams &p, long long u_
 // whatever share of the issue slots each of them gets.  `ring` is the CTA's dynamic shared memory: the
 // per-warp cp.async stages while tiles stream, then the warps' outputs.
 template <int BITS>
-__device__ __forceinline__ void run_segment(const AttnParams &p, int slice, long long u_lo, long long u_hi,
+__device__ __forceinline__ void run_segment(const AttnParams &p, int slice, int u_lo, int u_hi,
                                             float (*s_q)[kHeadDim], float *s_stat, int *s_ctr, uint4 *s_frag,
                                             uint8_t *ring) {
   using F = Fmt<BITS>;
   using F16 = Fmt<16>;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2;
-  const int b = slice / p.kv_heads, hkv = slice % p.kv_heads;
+  const int b = slice / p.kv_heads, hkv = slice - b * p.kv_heads;
 
   // (the previous segment ended with a CTA-wide barrier after its last use of s_q / s_stat / s_ctr / ring)
   if (tid == 0) s_ctr[0] = s_ctr[1] = 0;
   __syncthreads();
   int a_lo, a_hi, t_lo, t_hi;
-  segment_ranges(p, u_lo, u_hi, a_lo, a_hi, t_lo, t_hi);
+  segment_ranges<BITS>(p, u_lo, u_hi, a_lo, a_hi, t_lo, t_hi);
   const uint8_t *slice_base = p.geom.base + (size_t)slice * p.geom.slice_stride;
 
   // ---- body stream set-up: claim the first steps and start their copies before anything else ----
@@ -741,8 +847,8 @@ __device__ __forceinline__ void run_segment(const AttnParams &p, int slice, long
   build_query(p, b, hkv, s_q, s_stat);
   const int e_g = (int)s_stat[g];
   const float sumq = s_stat[8 + g];
-  fill_q_fragments<16>(s_frag, s_q, s_stat);
-  if constexpr (BITS != 16) fill_q_fragments<BITS>(s_frag + 256, s_q, s_stat);
+  fill_q_fragments<16>(s_frag, s_q, s_stat);  // half of the threads each
+  if constexpr (BITS != 16) fill_q_fragments<BITS>(s_frag + 256, s_q, s_stat, 256);
   __syncthreads();
   const float sigma16 = slice_sigma16(p, slice);
 
@@ -760,7 +866,7 @@ __device__ __forceinline__ void run_segment(const AttnParams &p, int slice, long
       for (int mt = 0; mt < 8; ++mt) {
 #pragma unroll
         for (int rr = 0; rr < 2; ++rr) {
-          const float f = ldexpf(1.0f, F::EP - F16::EP + F::pos((2 * mt + rr) % F::N) - F::SIGMA_LOG2);
+          const float f = exp2i(F::EP - F16::EP + F::pos((2 * mt + rr) % F::N) - F::SIGMA_LOG2);
           st.acc[mt][2 * rr] *= f;
           st.acc[mt][2 * rr + 1] *= f;
         }
@@ -769,12 +875,12 @@ __device__ __forceinline__ void run_segment(const AttnParams &p, int slice, long
   }
 
   // ---- body tiles ----
-  const float sigma_u = sigma16 * ldexpf(1.0f, F::SIGMA_LOG2);
+  const float sigma_u = sigma16 * exp2i(F::SIGMA_LOG2);
   if (n_steps > 0) {
     QFrag qa;
     qa.mine = (BITS != 16 ? s_frag + 256 : s_frag) + lane;
-    const float mu = ldexpf(1.0f, 24 - F::EQ + e_g);
-    const float inv_sigma_e = ldexpf(1.0f, F::EP) / sigma_u;
+    const float mu = exp2i(24 - F::EQ + e_g);
+    const float inv_sigma_e = exp2i(F::EP) / sigma_u;
     const uint32_t tail_mask = (p.n_body & 15) ? (1u << (p.n_body & 15)) - 1u : 0xFFFFu;
     const int tail_tile = tail_mask != 0xFFFFu ? p.body_tiles - 1 : -1;  // the one tile with dead rows
     if constexpr (F::SLOTS == 0) {
@@ -817,13 +923,9 @@ __device__ __forceinline__ void run_segment(const AttnParams &p, int slice, long
   }
   if constexpr (F::SLOTS > 0) cp_async_wait<0>();
 
-  // ---- warp epilogue: quad sums, real units, to shared memory (the ring is free now) ----
-  __syncthreads();  // every warp is done with its stages
-  float(*s_o)[kMaxGroup][kHeadDim] = reinterpret_cast<float(*)[kMaxGroup][kHeadDim]>(ring);
-  float *s_m = s_stat + 16, *s_l = s_stat + 16 + kParts * kMaxGroup;
-  store_warp_partial(st, [&](int J) { return ldexpf(sigma_u, 24 - F::EP - F::pos(J % F::N)); }, s_o, s_m, s_l, warp, lane);
-  __syncthreads();
-  publish_segment(p, slice, kAttnWarps, s_o, s_m, s_l, s_ctr);
+  // ---- the warps' states become the segment's partial, in real units (the ring's memory is reused) ----
+  merge_warps(p, slice, st, [&](int J) { return sigma_u * exp2i(24 - F::EP - F::pos(J % F::N)); },
+              reinterpret_cast<float(*)[kMaxGroup][kMergeRow]>(ring), s_stat + 16, s_ctr);
 }
 
 }  // namespace pmkvq
@@ -841,16 +943,16 @@ constexpr int kSmemTcTotal = kSmemParts + kParts * kMaxGroup * kHeadDim * 4;
 // every warp parks its partial in shared memory; the body then runs through the tensor-memory pipeline
 // and leaves one more partial.
 template <int BITS>
-__device__ __forceinline__ void run_segment_tc(const AttnParams &p, int slice, long long u_lo, long long u_hi,
+__device__ __forceinline__ void run_segment_tc(const AttnParams &p, int slice, int u_lo, int u_hi,
                                                float (*s_q)[kHeadDim], float *s_stat, int *s_ctr, uint4 *s_frag,
                                                TcCtx &tc) {
   using F16 = Fmt<16>;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2;
-  const int b = slice / p.kv_heads, hkv = slice % p.kv_heads;
+  const int b = slice / p.kv_heads, hkv = slice - b * p.kv_heads;
   if (tid == 0) s_ctr[0] = s_ctr[1] = 0;
   __syncthreads();
   int a_lo, a_hi, t_lo, t_hi;
-  segment_ranges(p, u_lo, u_hi, a_lo, a_hi, t_lo, t_hi);
+  segment_ranges<BITS>(p, u_lo, u_hi, a_lo, a_hi, t_lo, t_hi);
   const uint8_t *slice_base = p.geom.base + (size_t)slice * p.geom.slice_stride;
 
   build_query(p, b, hkv, s_q, s_stat);
@@ -870,7 +972,7 @@ __device__ __forceinline__ void run_segment_tc(const AttnParams &p, int slice, l
 #pragma unroll
     for (int mt = 0; mt < 8; ++mt) st.acc[mt][0] = st.acc[mt][1] = st.acc[mt][2] = st.acc[mt][3] = 0.f;
     if (a_hi > a_lo) run_int16_tiles(p, slice_base, a_lo, a_hi, st, s_frag, s_ctr, (int)s_stat[g], s_stat[8 + g], sigma16, lane);
-    store_warp_partial(st, [&](int J) { return ldexpf(sigma16, 24 - F16::EP - F16::pos(J % F16::N)); }, s_o, s_m, s_l, warp, lane);
+    store_warp_partial(st, [&](int J) { return sigma16 * exp2i(24 - F16::EP - F16::pos(J % F16::N)); }, s_o, s_m, s_l, warp, lane);
   }
   if (t_hi > t_lo) {
     tc_body<BITS>(p, tc, slice_base + p.geom.body_off, t_lo, t_hi, s_stat, sigma16, s_m, s_l, kAttnWarps);
@@ -888,7 +990,7 @@ __device__ __forceinline__ void run_segment_tc(const AttnParams &p, int slice, l
 // at least the warps' outputs they are reused for.
 template <int BITS>
 constexpr int attn_ring_bytes() {
-  constexpr int out_bytes = kAttnWarps * kMaxGroup * kHeadDim * 4;
+  constexpr int out_bytes = kMergeBytes;
   constexpr int ring = kAttnWarps * Fmt<BITS>::SLOTS * Fmt<BITS>::NT * tile_bytes(BITS);
   return ring > out_bytes ? ring : out_bytes;
 }
@@ -947,25 +1049,24 @@ __device__ __forceinline__ void tc_teardown(TcCtx &tc) {
 template <int BODY_BITS, bool ROWS>
 __global__ void __launch_bounds__(kAttnThreads, 1) decode_attn_splitk_kernel(const AttnParams p, unsigned *error_word) {
   __shared__ __align__(16) float s_q[kMaxGroup][kHeadDim];
-  __shared__ float s_stat[16 + 2 * kParts * kMaxGroup];  // head stats, per-partial (m, l)
-  __shared__ int s_ctr[4];                                // work counters (INT16 tiles, body tiles), combine flag
+  __shared__ __align__(16) float s_stat[16 + 2 * kParts * kMaxGroup];  // head stats, per-partial (m, l)
+  __shared__ int s_ctr[5];                                // work counters (INT16 tiles, body tiles), combine flag and range
   __shared__ uint4 s_frag[512];                           // query fragments at INT16 and at the body width
   __shared__ TcShared s_tc;
   extern __shared__ __align__(128) uint8_t ring[];
   TcCtx tc;
   constexpr bool tensor_path = BODY_BITS <= 4 && ROWS;
   if constexpr (tensor_path) tc_setup(&s_tc, tc, ring, error_word);
-  const long long u_begin = (long long)blockIdx.x * p.units_per_cta;
-  const long long u_end = min(u_begin + p.units_per_cta, p.units_total);
-  for (long long u = u_begin; u < u_end;) {
-    const int slice = (int)(u / p.units_slice);
-    const long long base = (long long)slice * p.units_slice;
-    const long long hi = min(u_end - base, p.units_slice);
+  const int per = (int)p.per_cta;
+  const int u_begin = (int)blockIdx.x * per;
+  const int u_end = min(u_begin + per, p.units_total);
+  int slice = u_begin / p.units_slice;
+  for (int base = slice * p.units_slice; base < u_end; base += p.units_slice, ++slice) {
+    const int lo = max(u_begin - base, 0), hi = min(u_end - base, p.units_slice);
     if (hi > p.units_lead) {
-      if constexpr (tensor_path) run_segment_tc<BODY_BITS>(p, slice, u - base, hi, s_q, s_stat, s_ctr, s_frag, tc);
-      else run_segment<BODY_BITS>(p, slice, u - base, hi, s_q, s_stat, s_ctr, s_frag, ring);
+      if constexpr (tensor_path) run_segment_tc<BODY_BITS>(p, slice, lo, hi, s_q, s_stat, s_ctr, s_frag, tc);
+      else run_segment<BODY_BITS>(p, slice, lo, hi, s_q, s_stat, s_ctr, s_frag, ring);
     }
-    u = base + hi;
   }
   if constexpr (tensor_path) tc_teardown(tc);
 }
@@ -978,6 +1079,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) decode_attn_splitk_kernel(con
 // count and width; geometry comes from the table the cache keeps in device memory.
 // ---------------------------------------------------------------------------------------------
 constexpr int kMaxFusedLayers = 128;
+constexpr int kMaxAttnCtas = 1024;  // upper bound on the attention grid (sizes the partials workspace)
 struct FusedParams {
   const LayerGeom *geoms;     // [layers]
   const uint16_t *Q;          // bf16 [layers][batch][q_heads][128]
@@ -989,14 +1091,27 @@ struct FusedParams {
   unsigned *error_word;       // bits set by a wait that ran out
   size_t partial_stride;
   int layers, kv_heads, group, q_heads, n_slices, batch;
-  int n_sink, window, evict_chunk, sink_tiles, ring_tiles;
-  int rows;                   // 1: tensor-memory path (row tiles at 4 and 2 bit)
+  int n_sink, sink_tiles, aux_tiles;
   float qk_scale;
   long long per_cta, total;              // fine units
+  double inv_per_cta;
   long long start[kMaxFusedLayers + 1];  // fine units before each block
-  int n_tokens[kMaxFusedLayers];
-  unsigned char bits[kMaxFusedLayers], lead[kMaxFusedLayers], weight[kMaxFusedLayers];
+  int n_tokens[kMaxFusedLayers], n_body[kMaxFusedLayers];
+  short cta_origin[kMaxFusedLayers];     // first CTA whose piece reaches into the block
+  unsigned char bits[kMaxFusedLayers];
+  unsigned char first_layer[kMaxAttnCtas];  // block that holds the first fine unit of each CTA's piece
 };
+static_assert(kMaxFusedLayers <= 256 && sizeof(FusedParams) <= 4096, "block numbers are bytes; kernel parameters fit one 4 KB bank");
+
+// What a tile of each width weighs, in fine units, and the lead of a slice in tiles (see segment_cost_tiles).
+// Time per 16-token tile at each width, in fiftieths of a 2-bit tile's (measured: 52.6 / 55.4 / 84.1 us per
+// block of 130 560 tiles at 2 / 4 / 8 bit, about 160 us at 16 bit).
+__host__ __device__ constexpr int tile_weight(int bits) { return bits == 16 ? 152 : bits == 8 ? 80 : bits == 4 ? 53 : 50; }
+// Fixed cost of one more segment (set-up, warp merge, publish, its share of the slice combine), in
+// body tiles of each width: about 12 us at the measured per-SM tile rates.
+__host__ __device__ constexpr int segment_cost_tiles(int bits) { return bits == 16 ? 48 : bits == 8 ? 96 : bits == 4 ? 176 : 160; }
+__host__ __device__ constexpr int int16_units(int bits) { return (tile_bytes(16) + tile_bytes(bits) - 1) / tile_bytes(bits); }
+__device__ __forceinline__ double inv_tile_weight(int bits) { return bits == 16 ? 1.0 / tile_weight(16) : bits == 8 ? 1.0 / tile_weight(8) : bits == 4 ? 1.0 / tile_weight(4) : 1.0 / tile_weight(2); }
 
 __device__ __forceinline__ void fused_layer_params(const FusedParams &fp, int l, AttnParams &p) {
   const int n = fp.n_tokens[l], bits = fp.bits[l];
@@ -1010,30 +1125,29 @@ __device__ __forceinline__ void fused_layer_params(const FusedParams &fp, int l,
   p.kv_heads = fp.kv_heads; p.group = fp.group; p.q_heads = fp.q_heads; p.n_slices = fp.n_slices;
   p.n_tokens = n;
   p.n_sink_eff = min(n, fp.n_sink);
-  const int excess = n - fp.n_sink - fp.window;
-  p.n_body = excess <= 0 ? 0 : excess / fp.evict_chunk * fp.evict_chunk;
+  p.n_body = fp.n_body[l];
   p.win_start = p.n_sink_eff + p.n_body;
   p.cur_bits = bits;
   p.body_tiles = (p.n_body + 15) / 16;
   p.sink_tiles = fp.sink_tiles;
-  p.aux_tiles = fp.sink_tiles + fp.ring_tiles;
-  p.w16 = (tile_bytes(16) + tile_bytes(bits) - 1) / tile_bytes(bits);
-  p.units_lead = fp.lead[l];
-  p.units_aux = p.units_lead + (long long)p.aux_tiles * p.w16;
+  p.aux_tiles = fp.aux_tiles;
+  p.units_lead = segment_cost_tiles(bits);
+  p.units_aux = p.units_lead + p.aux_tiles * int16_units(bits);
   p.units_slice = p.units_aux + p.body_tiles;
   p.units_total = p.units_slice * fp.n_slices;
-  p.units_per_cta = fp.per_cta;
   p.line_origin = fp.start[l];
-  p.unit_weight = fp.weight[l];
-  p.cta_origin = (int)(fp.start[l] / fp.per_cta);
+  p.unit_weight = tile_weight(bits);
+  p.cta_origin = fp.cta_origin[l];
+  p.per_cta = fp.per_cta;
+  p.inv_per_cta = fp.inv_per_cta;
   p.qk_scale = fp.qk_scale;
 }
 
 template <bool ROWS>
 __global__ void __launch_bounds__(kAttnThreads, 1) decode_attn_fused_kernel(const __grid_constant__ FusedParams fp) {
   __shared__ __align__(16) float s_q[kMaxGroup][kHeadDim];
-  __shared__ float s_stat[16 + 2 * kParts * kMaxGroup];
-  __shared__ int s_ctr[4];
+  __shared__ __align__(16) float s_stat[16 + 2 * kParts * kMaxGroup];
+  __shared__ int s_ctr[5];
   __shared__ uint4 s_frag[512];
   __shared__ TcShared s_tc;
   extern __shared__ __align__(128) uint8_t ring[];
@@ -1042,37 +1156,31 @@ __global__ void __launch_bounds__(kAttnThreads, 1) decode_attn_fused_kernel(cons
   if constexpr (tensor_path) tc_setup(&s_tc, tc, ring, fp.error_word);
   const long long f_begin = (long long)blockIdx.x * fp.per_cta;
   const long long f_end = min(f_begin + fp.per_cta, fp.total);
-  int l = 0;
-  for (long long f = f_begin; f < f_end;) {
-    while (l + 1 < fp.layers && fp.start[l + 1] <= f) ++l;  // the block this fine unit belongs to
+  for (int l = fp.first_layer[blockIdx.x]; l < fp.layers && fp.start[l] < f_end; ++l) {
     AttnParams p;
     fused_layer_params(fp, l, p);
-    const long long f_hi = min(f_end, fp.start[l + 1]);
-    // units of this block whose first fine unit lies in [f, f_hi)
+    // units of this block whose first fine unit lies in the piece
     const int w = p.unit_weight;
-    long long u = (f - p.line_origin + w - 1) / w;
-    const long long u_end = (f_hi - p.line_origin + w - 1) / w;
-    while (u < u_end) {
-      const int slice = (int)(u / p.units_slice);
-      const long long base = (long long)slice * p.units_slice;
-      const long long hi = min(u_end - base, p.units_slice);
-      if (hi > p.units_lead) {
-        switch (p.cur_bits) {
-          case 16: run_segment<16>(p, slice, u - base, hi, s_q, s_stat, s_ctr, s_frag, ring); break;
-          case 8: run_segment<8>(p, slice, u - base, hi, s_q, s_stat, s_ctr, s_frag, ring); break;
-          case 4:
-            if constexpr (tensor_path) run_segment_tc<4>(p, slice, u - base, hi, s_q, s_stat, s_ctr, s_frag, tc);
-            else run_segment<4>(p, slice, u - base, hi, s_q, s_stat, s_ctr, s_frag, ring);
-            break;
-          default:
-            if constexpr (tensor_path) run_segment_tc<2>(p, slice, u - base, hi, s_q, s_stat, s_ctr, s_frag, tc);
-            else run_segment<2>(p, slice, u - base, hi, s_q, s_stat, s_ctr, s_frag, ring);
-            break;
-        }
+    const double inv_w = inv_tile_weight(p.cur_bits);
+    const int u_begin = (int)floor_div(max(f_begin - p.line_origin, 0ll) + w - 1, w, inv_w);
+    const int u_end = (int)floor_div(min(f_end, fp.start[l + 1]) - p.line_origin + w - 1, w, inv_w);
+    int slice = u_begin / p.units_slice;
+    for (int base = slice * p.units_slice; base < u_end; base += p.units_slice, ++slice) {
+      const int lo = max(u_begin - base, 0), hi = min(u_end - base, p.units_slice);
+      if (hi <= p.units_lead) continue;
+      switch (p.cur_bits) {
+        case 16: run_segment<16>(p, slice, lo, hi, s_q, s_stat, s_ctr, s_frag, ring); break;
+        case 8: run_segment<8>(p, slice, lo, hi, s_q, s_stat, s_ctr, s_frag, ring); break;
+        case 4:
+          if constexpr (tensor_path) run_segment_tc<4>(p, slice, lo, hi, s_q, s_stat, s_ctr, s_frag, tc);
+          else run_segment<4>(p, slice, lo, hi, s_q, s_stat, s_ctr, s_frag, ring);
+          break;
+        default:
+          if constexpr (tensor_path) run_segment_tc<2>(p, slice, lo, hi, s_q, s_stat, s_ctr, s_frag, tc);
+          else run_segment<2>(p, slice, lo, hi, s_q, s_stat, s_ctr, s_frag, ring);
+          break;
       }
-      u = base + hi;
     }
-    f = f_hi;
   }
   if constexpr (tensor_path) tc_teardown(tc);
 }

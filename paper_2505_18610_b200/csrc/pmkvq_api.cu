@@ -22,10 +22,7 @@ using namespace pmkvq;
 namespace {
 
 constexpr size_t kAlign = 256;
-constexpr int kMaxCtas = 1024;      // upper bound on the attention grid (sizes the partials workspace)
-// Fixed cost of one more segment (set-up, warp merge, publish, its share of the slice combine), in
-// body tiles of each width: about 12 us at the measured per-SM tile rates.
-inline int segment_cost_tiles(int bits) { return bits == 16 ? 48 : bits == 8 ? 96 : bits == 4 ? 176 : 160; }
+constexpr int kMaxCtas = kMaxAttnCtas;
 constexpr int kMinUnitsPerCta = 32;  // do not cut the work finer than two tiles per warp
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -449,21 +446,22 @@ static pmkvq_status attn_params(pmkvq_cache *k, int32_t layer, const void *d_Q, 
   p.sink_tiles = k->sink_tiles;
   p.aux_tiles = k->sink_tiles + k->ring_tiles;
   p.n_slices = k->n_slices;
-  // one line of work units over all slices: a body tile is one unit, an INT16 tile their byte ratio
-  p.w16 = (tile_bytes(16) + tile_bytes(l.cur_bits) - 1) / tile_bytes(l.cur_bits);
-  // every slice starts with empty units that stand for the fixed cost of a segment
+  // one line of work units over all slices: a body tile is one unit, an INT16 tile their byte ratio; every
+  // slice starts with empty units that stand for the fixed cost of a segment
   p.units_lead = segment_cost_tiles(l.cur_bits);
-  p.units_aux = p.units_lead + (long long)p.aux_tiles * p.w16;
+  p.units_aux = p.units_lead + p.aux_tiles * int16_units(l.cur_bits);
   p.units_slice = p.units_aux + p.body_tiles;
-  p.units_total = p.units_slice * k->n_slices;
+  const long long total = (long long)p.units_slice * k->n_slices;
+  if (total > (1ll << 30)) return PMKVQ_ERR_STATE;  // a block of more than a terabyte
+  p.units_total = (int)total;
   const int width_idx = l.cur_bits == 16 ? 0 : l.cur_bits == 8 ? 1 : l.cur_bits == 4 ? 2 : 3;
   const int want = k->user_ctas > 0 ? k->user_ctas : k->resident_ctas[width_idx];
-  const long long per = std::max<long long>((p.units_total + want - 1) / want, k->user_ctas > 0 ? 1 : kMinUnitsPerCta);
-  p.units_per_cta = per;
+  p.per_cta = std::max<long long>((total + want - 1) / want, k->user_ctas > 0 ? 1 : kMinUnitsPerCta);
+  p.inv_per_cta = 1.0 / (double)p.per_cta;
   p.line_origin = 0;
   p.unit_weight = 1;
   p.cta_origin = 0;
-  n_ctas = (unsigned)((p.units_total + per - 1) / per);
+  n_ctas = (unsigned)((total + p.per_cta - 1) / p.per_cta);
   p.qk_scale = k->sm_scale * 1.4426950408889634f;
   return PMKVQ_OK;
 }
@@ -498,10 +496,6 @@ static pmkvq_status attention_on_arena(pmkvq_cache *k, int32_t layer, const void
   return e == cudaSuccess ? PMKVQ_OK : PMKVQ_ERR_CUDA;
 }
 
-// Time per 16-token tile at each width, in fiftieths of a 2-bit tile's (measured: 52.6 / 55.4 / 84.1 us per
-// block of 130 560 tiles at 2 / 4 / 8 bit, about 160 us at 16 bit).
-inline int tile_weight(int bits) { return bits == 16 ? 152 : bits == 8 ? 80 : bits == 4 ? 53 : 50; }
-
 static pmkvq_status attention_all_blocks(pmkvq_cache *k, const void *d_Q, float *d_out, cudaStream_t st) {
   static_assert(kMaxFusedLayers >= kMaxStepLayers, "the step's argument tables share one size");
   FusedParams fp;
@@ -516,23 +510,20 @@ static pmkvq_status attention_all_blocks(pmkvq_cache *k, const void *d_Q, float 
   fp.partial_stride = k->partial_bytes / sizeof(float);
   fp.layers = k->layers; fp.kv_heads = k->kv_heads; fp.group = k->group; fp.q_heads = k->q_heads;
   fp.n_slices = k->n_slices; fp.batch = k->batch;
-  fp.n_sink = k->n_sink; fp.window = k->window; fp.evict_chunk = k->evict_chunk;
-  fp.sink_tiles = k->sink_tiles; fp.ring_tiles = k->ring_tiles;
-  fp.rows = k->rows;
+  fp.n_sink = k->n_sink;
+  fp.sink_tiles = k->sink_tiles; fp.aux_tiles = k->sink_tiles + k->ring_tiles;
   fp.qk_scale = k->sm_scale * 1.4426950408889634f;
   long long total = 0;
   for (int l = 0; l < k->layers; ++l) {
     const Layer &L = k->L[l];
     if (L.n_tokens <= 0) return PMKVQ_ERR_INVALID_ARG;
     const int bits = L.cur_bits;
-    const int w16 = (tile_bytes(16) + tile_bytes(bits) - 1) / tile_bytes(bits);
-    const long long body_tiles = (k->body_at(L.n_tokens) + 15) / 16;
-    const long long units_slice = segment_cost_tiles(bits) + (long long)(k->sink_tiles + k->ring_tiles) * w16 + body_tiles;
     fp.start[l] = total;
     fp.n_tokens[l] = L.n_tokens;
+    fp.n_body[l] = k->body_at(L.n_tokens);
     fp.bits[l] = (unsigned char)bits;
-    fp.lead[l] = (unsigned char)segment_cost_tiles(bits);
-    fp.weight[l] = (unsigned char)tile_weight(bits);
+    const long long units_slice = segment_cost_tiles(bits) + (long long)fp.aux_tiles * int16_units(bits) + (fp.n_body[l] + 15) / 16;
+    if (units_slice * k->n_slices > (1ll << 30)) return PMKVQ_ERR_STATE;  // a block of more than a terabyte
     total += units_slice * k->n_slices * tile_weight(bits);
   }
   fp.start[k->layers] = total;
@@ -543,7 +534,14 @@ static pmkvq_status attention_all_blocks(pmkvq_cache *k, const void *d_Q, float 
   // partial, which is what the slice's ticket count expects.
   fp.per_cta = std::max<long long>((total + want - 1) / want,
                                    k->user_ctas > 0 ? (long long)tile_weight(16) : 50ll * kMinUnitsPerCta);
+  fp.inv_per_cta = 1.0 / (double)fp.per_cta;
   const unsigned n_ctas = (unsigned)((total + fp.per_cta - 1) / fp.per_cta);
+  for (int l = 0; l < k->layers; ++l) fp.cta_origin[l] = (short)(fp.start[l] / fp.per_cta);
+  int l0 = 0;
+  for (unsigned c = 0; c < n_ctas; ++c) {
+    while (fp.start[l0 + 1] <= (long long)c * fp.per_cta) ++l0;
+    fp.first_layer[c] = (unsigned char)l0;
+  }
   if (k->rows) decode_attn_fused_kernel<true><<<n_ctas, kAttnThreads, attn_fused_smem_bytes<true>(), st>>>(fp);
   else decode_attn_fused_kernel<false><<<n_ctas, kAttnThreads, attn_fused_smem_bytes<false>(), st>>>(fp);
   k->launches += 1;
