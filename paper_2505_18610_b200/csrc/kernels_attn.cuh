@@ -51,6 +51,7 @@ namespace pmkvq {
 constexpr int kMaxGroup = 8;         // query heads per KV head handled by one MMA row block
 constexpr int kPartialStride = 132;  // floats per (segment, head): m, l, 2 pad, o[128]
 constexpr float kNegBig = -1.0e30f;
+constexpr int kNoTiles = 0x7fffffff;  // AttnParams::clean_tiles once the wait is over
 constexpr float kMaxAhead = 3.0f;    // a score may exceed the reference by this much (log2 units)
 constexpr int kAttnWarps = 16;       // one CTA per SM; these warps share the CTA's INT16 / 8- / 16-bit tiles dynamically
 constexpr int kAttnThreads = 32 * kAttnWarps;
@@ -78,6 +79,7 @@ struct AttnParams {
   long long per_cta;          // fine units of a CTA's piece, and its reciprocal
   double inv_per_cta;
   float qk_scale;             // sm_scale * log2(e)
+  int clean_tiles;            // body tiles below this one may be read before pdl_wait()
 };
 
 __device__ __forceinline__ void mma_f16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
@@ -839,7 +841,10 @@ __device__ __forceinline__ void run_segment(const AttnParams &p, int slice, int 
 #pragma unroll
     for (int i = 0; i < S - 1; ++i) {
       pending[i] = n_steps > 0 ? claim(1) : 0;
-      if (pending[i] < n_steps) issue(pending[i], i);
+      if (pending[i] < n_steps) {
+        if (step_tile(pending[i], NT - 1) >= p.clean_tiles) pdl_wait();
+        issue(pending[i], i);
+      }
       cp_async_commit();
     }
   }
@@ -850,6 +855,7 @@ __device__ __forceinline__ void run_segment(const AttnParams &p, int slice, int 
   fill_q_fragments<16>(s_frag, s_q, s_stat);  // half of the threads each
   if constexpr (BITS != 16) fill_q_fragments<BITS>(s_frag + 256, s_q, s_stat, 256);
   __syncthreads();
+  pdl_wait();  // from here on the segment reads what the append in front of this launch may have written
   const float sigma16 = slice_sigma16(p, slice);
 
   WarpState st;
@@ -1056,6 +1062,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) decode_attn_splitk_kernel(con
   extern __shared__ __align__(128) uint8_t ring[];
   TcCtx tc;
   constexpr bool tensor_path = BODY_BITS <= 4 && ROWS;
+  pdl_launch_next();
+  pdl_wait();
   if constexpr (tensor_path) tc_setup(&s_tc, tc, ring, error_word);
   const int per = (int)p.per_cta;
   const int u_begin = (int)blockIdx.x * per;
@@ -1091,7 +1099,10 @@ struct FusedParams {
   unsigned *error_word;       // bits set by a wait that ran out
   size_t partial_stride;
   int layers, kv_heads, group, q_heads, n_slices, batch;
-  int n_sink, sink_tiles, aux_tiles;
+  int n_sink, sink_tiles, aux_tiles, evict_chunk;
+  // 1: this launch sits right behind append_step_kernel in its stream.  That kernel lets us start only once everything
+  // before it is complete, so the queries and the tiles it cannot touch may be read while it still runs.
+  int behind_append;
   float qk_scale;
   long long per_cta, total;              // fine units
   double inv_per_cta;
@@ -1140,6 +1151,7 @@ __device__ __forceinline__ void fused_layer_params(const FusedParams &fp, int l,
   p.cta_origin = fp.cta_origin[l];
   p.per_cta = fp.per_cta;
   p.inv_per_cta = fp.inv_per_cta;
+  p.clean_tiles = fp.behind_append ? max(0, p.n_body - fp.evict_chunk) >> 4 : kNoTiles;
   p.qk_scale = fp.qk_scale;
 }
 
@@ -1153,6 +1165,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) decode_attn_fused_kernel(cons
   extern __shared__ __align__(128) uint8_t ring[];
   TcCtx tc;
   constexpr bool tensor_path = ROWS;  // the cache was created for the tensor-memory path
+  pdl_launch_next();
+  if (!fp.behind_append || tensor_path) pdl_wait();
   if constexpr (tensor_path) tc_setup(&s_tc, tc, ring, fp.error_word);
   const long long f_begin = (long long)blockIdx.x * fp.per_cta;
   const long long f_end = min(f_begin + fp.per_cta, fp.total);

@@ -10,6 +10,13 @@
 
 namespace pmkvq {
 
+// Programmatic dependent launch.  The kernels of the decode path are launched with the attribute that lets a
+// grid start while its predecessor in the stream drains; every thread waits here before it touches memory, until
+// the predecessor is complete and its writes are visible, so only launch latency and start-up overlap.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+// allows the next grid to be launched once every CTA of this one has come here (or left)
+__device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+
 // Where one block's slices live inside the arena.
 struct LayerGeom {
   uint8_t *base;        // first slice of this block
@@ -76,6 +83,20 @@ __device__ __forceinline__ float chain_zero(float z16, float s16, int bits, int 
   return z;
 }
 
+// The whole chain 16 -> BITS of Eq. 3 on one INT16 code at once: each step rounds X / (2^b + 1) to nearest, the divisors
+// are odd (no ties), and nested roundings of this kind collapse to one, X_b = round(X_16 / D) with D = 257, 4369, 21845 at
+// 8, 4, 2 bit.  As fp32: X_16 and 2^23 are exact and X_16 / D is never closer than 1 / (2 D) to a half-integer, far more
+// than the rounding of 1 / D, so one fused multiply-add with 2^23 leaves the code in the low mantissa bits (equal to
+// the chain on all 65 536 codes and all widths).
+template <int BITS> __host__ __device__ constexpr float inv_chain_divisor() { return 1.0f / (float)(65535 / ((1 << BITS) - 1)); }
+template <int BITS>
+__device__ __forceinline__ uint32_t chain_code(uint32_t c16, int variant) {
+  if constexpr (BITS == 16) return c16;
+  if (variant != kShiftEquivalent) return c16 >> (16 - BITS);
+  const float x = __int_as_float(0x4B000000 | (int)c16) - 8388608.0f;
+  return __float_as_uint(__fmaf_rn(x, inv_chain_divisor<BITS>(), 8388608.0f)) & ((1u << BITS) - 1u);
+}
+
 // Write one token's 128 codes (given as INT16 codes in shared memory) into a tile at `bits`,
 // applying the Eq. 3 chain; one warp, every half-word of the token is written by one lane.
 template <int BITS>
@@ -100,7 +121,7 @@ __device__ __forceinline__ void store_token_w(uint8_t *part, int row, const uint
     uint32_t val = 0;
     for (int j = 0; j < n; ++j) {
       const int ch = chan_step * (w * n + j) + chan0;
-      val |= shift_chain(codes16[ch], bits, variant) << (j * bits);
+      val |= chain_code<bits>(codes16[ch], variant) << (j * bits);
     }
     int byte_off, bit_off;
     lane_slot(bits, owner, r, w * n, h, byte_off, bit_off);
@@ -116,7 +137,7 @@ __device__ __forceinline__ void store_key_row(uint8_t *k_part, int row, const ui
     uint32_t val = 0;
 #pragma unroll
     for (int i = 0; i < per_word; ++i)
-      val |= shift_chain(codes16[per_word * lane + i], BITS, variant) << (16 * (i & 1) + BITS * (i >> 1));
+      val |= chain_code<BITS>(codes16[per_word * lane + i], variant) << (16 * (i & 1) + BITS * (i >> 1));
     *reinterpret_cast<uint32_t *>(k_part + row * 16 * BITS + 4 * lane) = val;
   }
 }
@@ -133,7 +154,7 @@ __device__ __forceinline__ void insert_value_row(uint8_t *v_part, int row, const
     const int ch = lane + 32 * j;
     uint16_t *hw = reinterpret_cast<uint16_t *>(v_part + ch * 2 * BITS + bo);
     const uint32_t v = *hw;
-    *hw = (uint16_t)((v & ~(mask << sh)) | (shift_chain(codes16[ch], BITS, variant) << sh));
+    *hw = (uint16_t)((v & ~(mask << sh)) | (chain_code<BITS>(codes16[ch], variant) << sh));
   }
 }
 
@@ -284,6 +305,8 @@ __global__ void __launch_bounds__(128) append_kernel(const uint16_t *__restrict_
                                                      int n_old, int win_start, int cur_bits, int i0) {
   // new tokens i0 .. i0 + n_new - 1 of the K / V arrays, one by one
   __shared__ uint16_t s_codes[4][kHeadDim];
+  pdl_launch_next();
+  pdl_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long wid = (long long)blockIdx.x * 4 + warp;
   if (wid >= (long long)n_new * n_slices * 2) return;
@@ -300,8 +323,9 @@ __global__ void __launch_bounds__(128) append_kernel(const uint16_t *__restrict_
 // loads of one warp cover whole 4 KB of input; the sectors they share are served by L1.
 
 // Eq. 1-2 at 16 bit on N values of one token that a lane holds, given the token's min and max; the
-// values are replaced by their codes at `BITS` (Eq. 3 chain).  Returns the INT16 scale.
-template <int BITS, int N>
+// values are replaced by their codes at `BITS` (Eq. 3 chain).  Returns the INT16 scale.  With CLEAN = false only the low
+// BITS (at 16 bit: 16) bits of a result are the code and bits 16 .. 23 are zero; what sits above may be anything.
+template <int BITS, int N, bool CLEAN>
 __device__ __forceinline__ float quantize_owned(float (&x)[N], float mn, float mx, int variant) {
   const float scale = __fdiv_rn(__fsub_rn(mx, mn), 65535.0f);
   if (scale >= 0x1p-60f && scale <= 0x1p60f) {  // one scale per token: the branch is uniform in the warp
@@ -322,16 +346,22 @@ __device__ __forceinline__ float quantize_owned(float (&x)[N], float mn, float m
       if constexpr (BITS == 16) {  // the code is the low half of the sum's bit pattern; the packing keeps only that
         x[i] = c.x;
         x[i + 1] = c.y;
+      } else if (variant == kShiftEquivalent) {  // chain_code on both
+        const float2 c16 = __fadd2_rn(c, make_float2(-8388608.0f, -8388608.0f));
+        constexpr float inv = inv_chain_divisor<BITS>();
+        const float2 cb = __ffma2_rn(c16, make_float2(inv, inv), make_float2(8388608.0f, 8388608.0f));
+        x[i] = CLEAN ? __uint_as_float(__float_as_uint(cb.x) & 0xFFu) : cb.x;
+        x[i + 1] = CLEAN ? __uint_as_float(__float_as_uint(cb.y) & 0xFFu) : cb.y;
       } else {
-        x[i] = __uint_as_float(shift_chain((uint32_t)(__float_as_int(c.x) - 0x4B000000), BITS, variant));
-        x[i + 1] = __uint_as_float(shift_chain((uint32_t)(__float_as_int(c.y) - 0x4B000000), BITS, variant));
+        x[i] = __uint_as_float((uint32_t)(__float_as_int(c.x) - 0x4B000000) >> (16 - BITS));
+        x[i + 1] = __uint_as_float((uint32_t)(__float_as_int(c.y) - 0x4B000000) >> (16 - BITS));
       }
     }
   } else {  // constant tokens (0 / 0 converts to code 0) and scales far outside any real tensor's range
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       const int c = min(max(__float2int_rn(__fdiv_rn(__fsub_rn(x[i], mn), scale)), 0), 65535);
-      x[i] = __uint_as_float(shift_chain((uint32_t)c, BITS, variant));
+      x[i] = __uint_as_float(chain_code<BITS>((uint32_t)c, variant));
     }
   }
   return scale;
@@ -352,10 +382,11 @@ __device__ __forceinline__ void pack_words(const float *lo, const float *hi, int
       uint32_t a = 0, b = 0;
 #pragma unroll
       for (int j = 0; j < n; ++j) {
-        a |= __float_as_uint(lo[(w * n + j) * step]) << (j * BITS);
-        b |= __float_as_uint(hi[(w * n + j) * step]) << (j * BITS);
+        // a sum: what sits above bit 23 of a pattern only moves further up
+        a += __float_as_uint(lo[(w * n + j) * step]) << (j * BITS);
+        b += __float_as_uint(hi[(w * n + j) * step]) << (j * BITS);
       }
-      words[w] = a | (b << 16);
+      words[w] = __byte_perm(a, b, 0x5410);
     }
   }
 }
@@ -416,7 +447,7 @@ __device__ __forceinline__ void append_tile_half(const uint16_t *__restrict__ sr
         mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
         mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
       }
-      const float s16 = quantize_owned<BITS>(x, mn, mx, variant);
+      const float s16 = quantize_owned<BITS, 32, false>(x, mn, mx, variant);
       pack_words<BITS>(x, x + 1, 2, words);  // halves of a word: channels h = 0, 1 of the token
       store_words<BITS>(dst_tile, r, lane, words);
       // metadata record g / 2 holds tokens {2t, 2t+1, 8+2t, 9+2t} at entries {0, 1, 2, 3}
@@ -448,7 +479,7 @@ __device__ __forceinline__ void append_tile_half(const uint16_t *__restrict__ sr
           mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
           mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         }
-        S[h] = quantize_owned<BITS>(x[h], mn, mx, variant);
+        S[h] = quantize_owned<BITS, 16, false>(x[h], mn, mx, variant);
         Z[h] = mn;
         smax = fmaxf(smax, S[h]);
       }
@@ -509,7 +540,7 @@ __device__ __forceinline__ void append_tile_half_row(const uint16_t *__restrict_
       mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
       mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     }
-    const float s16 = quantize_owned<BITS>(x, mn, mx, variant);
+    const float s16 = quantize_owned<BITS, 32, true>(x, mn, mx, variant);
     if (!is_value) {
       uint32_t words[words_per_lane];
 #pragma unroll
@@ -564,14 +595,12 @@ __device__ __forceinline__ void append_tile_half_row(const uint16_t *__restrict_
   }
 }
 
-__global__ void __launch_bounds__(128, 8) append_tiles_kernel(const uint16_t *__restrict__ K, const uint16_t *__restrict__ V,
-                                                           const float *__restrict__ inv_lambda, unsigned *vmax_bits,
-                                                           LayerGeom geom, int n_slices, int kv_heads, int n_old,
-                                                           int tile_lo, int n_tiles, int bits) {
-  __shared__ __align__(16) uint8_t s_scratch[4][kTileTokens * kStageRowBytes];  // the warp's staged input rows, or its code bytes (row tiles)
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long wid = (long long)blockIdx.x * 4 + warp;
-  if (wid >= (long long)n_tiles * n_slices * 2) return;
+// One warp: half (K or V) of body tile `tile` of a slice, all 16 tokens new.  `wid` counts halves, slices, tiles.
+template <bool ROWS>
+__device__ __forceinline__ void append_tile_one(long long wid, uint8_t *stage, int lane, const uint16_t *__restrict__ K,
+                                                const uint16_t *__restrict__ V, const float *__restrict__ inv_lambda,
+                                                unsigned *vmax_bits, const LayerGeom &geom, int n_slices, int kv_heads,
+                                                int n_old, int tile_lo, int bits) {
   const int is_value = (int)(wid & 1);
   const int slice = (int)((wid >> 1) % n_slices);
   const int tile = tile_lo + (int)((wid >> 1) / n_slices);
@@ -581,17 +610,31 @@ __global__ void __launch_bounds__(128, 8) append_tiles_kernel(const uint16_t *__
   const float *il = inv_lambda + (size_t)(slice % kv_heads) * kHeadDim;
   uint8_t *dst_tile = geom.base + (size_t)slice * geom.slice_stride + geom.body_off + body_tile_offset(tile, bits, geom.stream_stride);
   switch (bits) {
-    case 16: append_tile_half<16>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, geom.shift_variant, s_scratch[warp]); break;
-    case 8: append_tile_half<8>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, geom.shift_variant, s_scratch[warp]); break;
+    case 16: append_tile_half<16>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, geom.shift_variant, stage); break;
+    case 8: append_tile_half<8>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, geom.shift_variant, stage); break;
     case 4:
-      if (geom.rows) append_tile_half_row<4>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, geom.shift_variant, s_scratch[warp]);
-      else append_tile_half<4>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, geom.shift_variant, s_scratch[warp]);
+      if constexpr (ROWS) append_tile_half_row<4>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, geom.shift_variant, stage);
+      else append_tile_half<4>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, geom.shift_variant, stage);
       break;
     default:
-      if (geom.rows) append_tile_half_row<2>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, geom.shift_variant, s_scratch[warp]);
-      else append_tile_half<2>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, geom.shift_variant, s_scratch[warp]);
+      if constexpr (ROWS) append_tile_half_row<2>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, geom.shift_variant, stage);
+      else append_tile_half<2>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, geom.shift_variant, stage);
       break;
   }
+}
+
+// the same as a kernel of its own (row-tile caches)
+__global__ void __launch_bounds__(128, 8) append_tiles_kernel(const uint16_t *__restrict__ K, const uint16_t *__restrict__ V,
+                                                           const float *__restrict__ inv_lambda, unsigned *vmax_bits,
+                                                           LayerGeom geom, int n_slices, int kv_heads, int n_old,
+                                                           int tile_lo, int n_tiles, int bits) {
+  __shared__ __align__(16) uint8_t s_scratch[4][kTileTokens * kStageRowBytes];  // the warp's staged input rows, or its code bytes
+  pdl_launch_next();
+  pdl_wait();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const long long wid = (long long)blockIdx.x * 4 + warp;
+  if (wid >= (long long)n_tiles * n_slices * 2) return;
+  append_tile_one<true>(wid, s_scratch[warp], lane, K, V, inv_lambda, vmax_bits, geom, n_slices, kv_heads, n_old, tile_lo, bits);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -633,10 +676,63 @@ __device__ __forceinline__ void evict_one(long long wid, uint16_t *codes, int la
 __global__ void __launch_bounds__(128) evict_kernel(LayerGeom geom, int n_slices, int first_token, int n_evict,
                                                     int cur_bits) {
   __shared__ uint16_t s_codes[4][kHeadDim];
+  pdl_launch_next();
+  pdl_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long wid = (long long)blockIdx.x * 4 + warp;
   if (wid >= (long long)n_evict * n_slices * 2) return;
   evict_one(wid, s_codes[warp], lane, geom, n_slices, first_token, n_evict, cur_bits);
+}
+
+// A bulk append to a cache of lane-owned tiles in one launch: whole body tiles, then the new tokens around them (sink,
+// window, ragged ends) one by one, then the evictions.  The one hazard is the ring: a new window token may land
+// in the slot of a token that leaves it.  The warp of the new token then moves the old one out first, and the old
+// token's own warp leaves.  (As three to four launches a short prompt's append cost 16.8 us per block, nearly all of
+// it launches of a few microseconds.)
+struct BulkParams {
+  int n_old, n_after, win_start;       // tokens before and after, first token of the window afterwards
+  int tile_lo, n_tiles;                // body tiles written whole
+  int head_first, head_cnt;            // new tokens (absolute) before the whole tiles ...
+  int tail_first, tail_cnt;            // ... and behind them
+  int ev_first, n_evict;               // tokens that leave the window
+};
+__global__ void __launch_bounds__(128, 8) append_bulk_kernel(const uint16_t *__restrict__ K, const uint16_t *__restrict__ V,
+                                                             const float *__restrict__ inv_lambda, unsigned *vmax_bits,
+                                                             const LayerGeom geom, int n_slices, int kv_heads, int cur_bits,
+                                                             const BulkParams bp) {
+  __shared__ __align__(16) uint8_t s_scratch[4][kTileTokens * kStageRowBytes];
+  pdl_launch_next();
+  pdl_wait();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  long long wid = (long long)blockIdx.x * 4 + warp;
+  const long long per = 2ll * n_slices;
+  if (wid < per * bp.n_tiles) {
+    append_tile_one<false>(wid, s_scratch[warp], lane, K, V, inv_lambda, vmax_bits, geom, n_slices, kv_heads, bp.n_old, bp.tile_lo, cur_bits);
+    return;
+  }
+  wid -= per * bp.n_tiles;
+  uint16_t *codes = reinterpret_cast<uint16_t *>(s_scratch[warp]);
+  const int ring = geom.ring_tokens;
+  if (wid < per * (bp.head_cnt + bp.tail_cnt)) {
+    const int k = (int)(wid / per);
+    const long long in_token = wid - k * per;  // slice and half
+    const int t = k < bp.head_cnt ? bp.head_first + k : bp.tail_first + (k - bp.head_cnt);
+    if (bp.n_evict > 0 && t >= bp.win_start && t >= geom.n_sink) {
+      const int old = t - ((t - bp.n_old) / ring + 1) * ring;  // the last token before this append in the same slot
+      if (old >= bp.ev_first && old < bp.ev_first + bp.n_evict)
+        evict_one(in_token, codes, lane, geom, n_slices, old, 1, cur_bits);
+    }
+    append_one(in_token, codes, lane, K, V, inv_lambda, vmax_bits, geom, n_slices, kv_heads, bp.n_old, bp.win_start, cur_bits, t - bp.n_old, 1);
+    return;
+  }
+  wid -= per * (bp.head_cnt + bp.tail_cnt);
+  if (wid < per * bp.n_evict) {
+    const int k = (int)(wid / per), t = bp.ev_first + k;
+    const int first = max(bp.n_old, bp.win_start);         // new window tokens: first .. n_after - 1
+    const int taker = t + (first - t + ring - 1) / ring * ring;  // the first of them (or later) that lands in t's slot
+    if (taker < bp.n_after) return;
+    evict_one(wid - k * per, codes, lane, geom, n_slices, t, 1, cur_bits);
+  }
 }
 
 // One decode step's cache update in a single launch: the tokens that leave the window (warps
@@ -650,6 +746,8 @@ __global__ void __launch_bounds__(128) append_decode_kernel(const uint16_t *__re
                                                             LayerGeom geom, int n_slices, int kv_heads, int n_old,
                                                             int win_start, int cur_bits, int first_evicted, int n_evict) {
   __shared__ uint16_t s_codes[4][kHeadDim];
+  pdl_launch_next();
+  pdl_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long wid = (long long)blockIdx.x * 4 + warp;
   const long long n_ev = (long long)n_evict * n_slices * 2;
@@ -679,6 +777,8 @@ __global__ void __launch_bounds__(128) append_step_kernel(const uint16_t *__rest
                                                           int layers, int n_slices, int kv_heads, int n_sink, int window,
                                                           int evict_chunk) {
   __shared__ uint16_t s_codes[4][kHeadDim];
+  pdl_wait();
+  pdl_launch_next();  // behind the wait: what the next grid reads before its own wait is complete then
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long per_layer = 2ll * (evict_chunk + 1) * n_slices;
   const long long gw = (long long)blockIdx.x * 4 + warp;
@@ -1062,6 +1162,8 @@ __global__ void __launch_bounds__(reduce_warps<B>() * 32, reduce_min_ctas<B>()) 
   uint8_t *base = geom.base + (size_t)blockIdx.y * geom.slice_stride + geom.body_off + (size_t)stream * geom.stream_stride;
   const int cnt = (n_tiles - stream + kStreams - 1) / kStreams;  // tiles of this stream
   uint8_t *scratch = s_scratch[B == 4 ? warp : 0];
+  pdl_launch_next();
+  pdl_wait();
   if (cnt <= 0) return;
   reduce_one_tile<B>(geom, base + (size_t)warp * tile_bytes(2 * B), base + (size_t)warp * tile_bytes(B), lane, warp < cnt, true, scratch);
   for (int lo = kReduceWarps; lo < cnt;) {

@@ -166,12 +166,29 @@ size_t plan(pmkvq_cache &k, const pmkvq_config *c) {
   return off;
 }
 
+// Launches with programmatic stream serialization: the grid may start while its predecessor in the stream drains
+// (its threads wait with pdl_wait before they touch memory).
+template <class... Params, class... Args>
+cudaError_t launch(uint64_t &launches, void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, Args... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  ++launches;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+inline unsigned four_warp_ctas(long long warps) { return (unsigned)((warps + 3) / 4); }
+
 template <int B>
 cudaError_t launch_reduce(const LayerGeom &g, int n_slices, int n_tiles, cudaStream_t st, uint64_t &launches) {
   // one CTA per (stream, slice): the streams compact in place independently of one another
-  reduce_stream_kernel<B><<<dim3(kStreams, (unsigned)n_slices), reduce_warps<B>() * 32, 0, st>>>(g, n_tiles);
-  ++launches;
-  return cudaGetLastError();
+  return launch(launches, reduce_stream_kernel<B>, dim3(kStreams, (unsigned)n_slices), reduce_warps<B>() * 32, 0, st, g, n_tiles);
 }
 
 template <int BITS, bool ROWS>
@@ -377,46 +394,47 @@ pmkvq_status pmkvq_append(pmkvq_cache *k, int32_t layer, const void *d_K, const 
   // With window = 0 and chunked eviction the new token enters the body together with the chunk's other
   // tokens, possibly in one tile: they then go through separate launches (see append_decode_kernel).
   const bool shares_tile = k->window == 0 && k->evict_chunk > 1;
+  const uint16_t *K = static_cast<const uint16_t *>(d_K), *V = static_cast<const uint16_t *>(d_V);
+  // new tokens that fill whole body tiles are written tile-wise, the rest (sink, ring, ragged ends) one by one
+  const int j_lo = std::max(n_old, k->n_sink) - k->n_sink, j_hi = std::max(new_win_start, k->n_sink) - k->n_sink;
+  const int tile_lo = (j_lo + 15) / 16, tile_hi = std::max(j_hi / 16, tile_lo);
+  int skip_lo = n_old, skip_hi = n_old;  // absolute token range written tile-wise
+  if (tile_hi > tile_lo) {
+    skip_lo = k->n_sink + 16 * tile_lo;
+    skip_hi = k->n_sink + 16 * tile_hi;
+  }
+  cudaError_t e = cudaSuccess;
   if (n_new == 1 && !shares_tile) {
     // decode step: evictions and the new token in one launch (their ring slots cannot coincide)
-    const long long warps = 2ll * (n_evict + 1) * k->n_slices;
-    append_decode_kernel<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(
-        static_cast<const uint16_t *>(d_K), static_cast<const uint16_t *>(d_V), inv_lam, vmax, g, k->n_slices, k->kv_heads,
-        n_old, new_win_start, l.cur_bits, ev_first, n_evict);
-    ++k->launches;
+    e = launch(k->launches, append_decode_kernel, four_warp_ctas(2ll * (n_evict + 1) * k->n_slices), 128, 0, st, K, V, inv_lam, vmax, g,
+               k->n_slices, k->kv_heads, n_old, new_win_start, l.cur_bits, ev_first, n_evict);
+  } else if (!k->rows) {
+    BulkParams bp;
+    bp.n_old = n_old; bp.n_after = n_after; bp.win_start = new_win_start;
+    bp.tile_lo = tile_lo; bp.n_tiles = tile_hi - tile_lo;
+    bp.head_first = n_old; bp.head_cnt = skip_lo - n_old;
+    bp.tail_first = skip_hi; bp.tail_cnt = n_after - skip_hi;
+    bp.ev_first = ev_first; bp.n_evict = n_evict;
+    const long long warps = 2ll * k->n_slices * ((long long)bp.n_tiles + bp.head_cnt + bp.tail_cnt + n_evict);
+    e = launch(k->launches, append_bulk_kernel, four_warp_ctas(warps), 128, 0, st, K, V, inv_lam, vmax, g, k->n_slices, k->kv_heads,
+               l.cur_bits, bp);
   } else {
-    if (n_evict > 0) {
-      const long long warps = 2ll * n_evict * k->n_slices;
-      evict_kernel<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(g, k->n_slices, ev_first, n_evict, l.cur_bits);
-      ++k->launches;
-    }
-    // new tokens that fill whole body tiles are written tile-wise, the rest (sink, ring, ragged ends) one by one
-    const int j_lo = std::max(n_old, k->n_sink) - k->n_sink, j_hi = std::max(new_win_start, k->n_sink) - k->n_sink;
-    const int tile_lo = (j_lo + 15) / 16, tile_hi = j_hi / 16;
-    int skip_lo = n_old, skip_hi = n_old;  // absolute token range written tile-wise
-    if (tile_hi > tile_lo) {
-      skip_lo = k->n_sink + 16 * tile_lo;
-      skip_hi = k->n_sink + 16 * tile_hi;
-      const long long tw = 2ll * (tile_hi - tile_lo) * k->n_slices;
-      append_tiles_kernel<<<(unsigned)((tw + 3) / 4), 128, 0, st>>>(static_cast<const uint16_t *>(d_K),
-                                                                   static_cast<const uint16_t *>(d_V), inv_lam, vmax, g,
-                                                                   k->n_slices, k->kv_heads, n_old, tile_lo,
-                                                                   tile_hi - tile_lo, l.cur_bits);
-      ++k->launches;
-    }
+    // row tiles: Values are inserted by read-modify-write of half-words that the tokens of a tile share, so the
+    // evictions, the whole tiles and the single tokens are launches of their own
+    if (n_evict > 0)
+      e = launch(k->launches, evict_kernel, four_warp_ctas(2ll * n_evict * k->n_slices), 128, 0, st, g, k->n_slices, ev_first, n_evict, l.cur_bits);
+    if (e == cudaSuccess && tile_hi > tile_lo)
+      e = launch(k->launches, append_tiles_kernel, four_warp_ctas(2ll * (tile_hi - tile_lo) * k->n_slices), 128, 0, st, K, V, inv_lam, vmax, g,
+                 k->n_slices, k->kv_heads, n_old, tile_lo, tile_hi - tile_lo, l.cur_bits);
     const int ranges[2][2] = {{n_old, skip_lo}, {skip_hi, n_after}};  // what is left, one token per warp
     for (int r = 0; r < 2; ++r) {
       const int cnt = ranges[r][1] - ranges[r][0];
-      if (cnt <= 0) continue;
-      const long long warps = 2ll * cnt * k->n_slices;
-      append_kernel<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(static_cast<const uint16_t *>(d_K),
-                                                                static_cast<const uint16_t *>(d_V), inv_lam, vmax, g, cnt,
-                                                                k->n_slices, k->kv_heads, n_old, new_win_start, l.cur_bits,
-                                                                ranges[r][0] - n_old);
-      ++k->launches;
+      if (cnt <= 0 || e != cudaSuccess) continue;
+      e = launch(k->launches, append_kernel, four_warp_ctas(2ll * cnt * k->n_slices), 128, 0, st, K, V, inv_lam, vmax, g, cnt, k->n_slices,
+                 k->kv_heads, n_old, new_win_start, l.cur_bits, ranges[r][0] - n_old);
     }
   }
-  if (cudaGetLastError() != cudaSuccess) return PMKVQ_ERR_CUDA;
+  if (e != cudaSuccess) return PMKVQ_ERR_CUDA;
   l.n_tokens = n_after;
   return PMKVQ_OK;
 }
@@ -461,26 +479,26 @@ static pmkvq_status attn_params(pmkvq_cache *k, int32_t layer, const void *d_Q, 
   p.line_origin = 0;
   p.unit_weight = 1;
   p.cta_origin = 0;
+  p.clean_tiles = kNoTiles;
   n_ctas = (unsigned)((total + p.per_cta - 1) / p.per_cta);
   p.qk_scale = k->sm_scale * 1.4426950408889634f;
   return PMKVQ_OK;
 }
 
 template <int BITS>
-static cudaError_t attn_launch_width(const AttnParams &p, unsigned n_ctas, cudaStream_t st, unsigned *error_word) {
+static cudaError_t attn_launch_width(pmkvq_cache *k, const AttnParams &p, unsigned n_ctas, cudaStream_t st, unsigned *error_word) {
   if (p.geom.rows)
-    decode_attn_splitk_kernel<BITS, true><<<n_ctas, kAttnThreads, attn_smem_bytes<BITS, true>(), st>>>(p, error_word);
-  else
-    decode_attn_splitk_kernel<BITS, false><<<n_ctas, kAttnThreads, attn_smem_bytes<BITS, false>(), st>>>(p, error_word);
-  return cudaGetLastError();
+    return launch(k->launches, decode_attn_splitk_kernel<BITS, true>, n_ctas, kAttnThreads, attn_smem_bytes<BITS, true>(), st, p, error_word);
+  return launch(k->launches, decode_attn_splitk_kernel<BITS, false>, n_ctas, kAttnThreads, attn_smem_bytes<BITS, false>(), st, p, error_word);
 }
 
-static cudaError_t attn_launch(const AttnParams &p, unsigned n_ctas, cudaStream_t st, unsigned *error_word) {
+static cudaError_t attn_launch(pmkvq_cache *k, const AttnParams &p, unsigned n_ctas, cudaStream_t st) {
+  unsigned *error_word = reinterpret_cast<unsigned *>(k->arena + k->off_error);
   switch (p.cur_bits) {
-    case 16: return attn_launch_width<16>(p, n_ctas, st, error_word);
-    case 8: return attn_launch_width<8>(p, n_ctas, st, error_word);
-    case 4: return attn_launch_width<4>(p, n_ctas, st, error_word);
-    default: return attn_launch_width<2>(p, n_ctas, st, error_word);
+    case 16: return attn_launch_width<16>(k, p, n_ctas, st, error_word);
+    case 8: return attn_launch_width<8>(k, p, n_ctas, st, error_word);
+    case 4: return attn_launch_width<4>(k, p, n_ctas, st, error_word);
+    default: return attn_launch_width<2>(k, p, n_ctas, st, error_word);
   }
 }
 
@@ -491,12 +509,11 @@ static pmkvq_status attention_on_arena(pmkvq_cache *k, int32_t layer, const void
   if (s != PMKVQ_OK) return s;
   p.partials = reinterpret_cast<float *>(k->arena + k->off_partials + (size_t)layer * k->partial_bytes);
   p.tickets = reinterpret_cast<unsigned *>(k->arena + k->off_tickets) + (size_t)layer * k->n_slices;
-  const cudaError_t e = attn_launch(p, n_ctas, st, reinterpret_cast<unsigned *>(k->arena + k->off_error));
-  k->launches += 1;
+  const cudaError_t e = attn_launch(k, p, n_ctas, st);
   return e == cudaSuccess ? PMKVQ_OK : PMKVQ_ERR_CUDA;
 }
 
-static pmkvq_status attention_all_blocks(pmkvq_cache *k, const void *d_Q, float *d_out, cudaStream_t st) {
+static pmkvq_status attention_all_blocks(pmkvq_cache *k, const void *d_Q, float *d_out, cudaStream_t st, bool behind_append) {
   static_assert(kMaxFusedLayers >= kMaxStepLayers, "the step's argument tables share one size");
   FusedParams fp;
   fp.geoms = reinterpret_cast<const LayerGeom *>(k->arena + k->off_geoms);
@@ -510,7 +527,8 @@ static pmkvq_status attention_all_blocks(pmkvq_cache *k, const void *d_Q, float 
   fp.partial_stride = k->partial_bytes / sizeof(float);
   fp.layers = k->layers; fp.kv_heads = k->kv_heads; fp.group = k->group; fp.q_heads = k->q_heads;
   fp.n_slices = k->n_slices; fp.batch = k->batch;
-  fp.n_sink = k->n_sink;
+  fp.n_sink = k->n_sink; fp.evict_chunk = k->evict_chunk;
+  fp.behind_append = behind_append ? 1 : 0;
   fp.sink_tiles = k->sink_tiles; fp.aux_tiles = k->sink_tiles + k->ring_tiles;
   fp.qk_scale = k->sm_scale * 1.4426950408889634f;
   long long total = 0;
@@ -542,10 +560,10 @@ static pmkvq_status attention_all_blocks(pmkvq_cache *k, const void *d_Q, float 
     while (fp.start[l0 + 1] <= (long long)c * fp.per_cta) ++l0;
     fp.first_layer[c] = (unsigned char)l0;
   }
-  if (k->rows) decode_attn_fused_kernel<true><<<n_ctas, kAttnThreads, attn_fused_smem_bytes<true>(), st>>>(fp);
-  else decode_attn_fused_kernel<false><<<n_ctas, kAttnThreads, attn_fused_smem_bytes<false>(), st>>>(fp);
-  k->launches += 1;
-  return cudaGetLastError() == cudaSuccess ? PMKVQ_OK : PMKVQ_ERR_CUDA;
+  const cudaError_t e =
+      k->rows ? launch(k->launches, decode_attn_fused_kernel<true>, n_ctas, kAttnThreads, attn_fused_smem_bytes<true>(), st, fp)
+              : launch(k->launches, decode_attn_fused_kernel<false>, n_ctas, kAttnThreads, attn_fused_smem_bytes<false>(), st, fp);
+  return e == cudaSuccess ? PMKVQ_OK : PMKVQ_ERR_CUDA;
 }
 
 extern "C" {
@@ -570,8 +588,7 @@ pmkvq_status pmkvq_decode_attention_static(pmkvq_cache *k, int32_t layer, const 
   p.partials = reinterpret_cast<float *>(scratch + kStaticTicketBytes);
   // the array keeps whatever the previous call left: the tickets must start at zero
   if (cudaMemsetAsync(p.tickets, 0, (size_t)k->n_slices * sizeof(unsigned), st) != cudaSuccess) return PMKVQ_ERR_CUDA;
-  const cudaError_t e = attn_launch(p, n_ctas, st, reinterpret_cast<unsigned *>(k->arena + k->off_error));
-  k->launches += 1;
+  const cudaError_t e = attn_launch(k, p, n_ctas, st);
   return e == cudaSuccess ? PMKVQ_OK : PMKVQ_ERR_CUDA;
 }
 
@@ -615,22 +632,21 @@ pmkvq_status pmkvq_decode_step(pmkvq_cache *k, const void *d_K, const void *d_V,
     sp.cur_bits[layer] = (unsigned char)k->L[layer].cur_bits;
   }
   const long long warps = 2ll * (k->evict_chunk + 1) * k->n_slices * k->layers;
-  append_step_kernel<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(
-      static_cast<const uint16_t *>(d_K), static_cast<const uint16_t *>(d_V),
+  const cudaError_t e = launch(
+      k->launches, append_step_kernel, four_warp_ctas(warps), 128, 0, st, static_cast<const uint16_t *>(d_K), static_cast<const uint16_t *>(d_V),
       reinterpret_cast<const float *>(k->arena + k->off_inv_lambda), reinterpret_cast<unsigned *>(k->arena + k->off_vmax),
-      reinterpret_cast<const LayerGeom *>(k->arena + k->off_geoms), sp, k->layers, k->n_slices, k->kv_heads, k->n_sink,
-      k->window, k->evict_chunk);
-  ++k->launches;
-  if (cudaGetLastError() != cudaSuccess) return PMKVQ_ERR_CUDA;
+      reinterpret_cast<const LayerGeom *>(k->arena + k->off_geoms), sp, k->layers, k->n_slices, k->kv_heads, k->n_sink, k->window,
+      k->evict_chunk);
+  if (e != cudaSuccess) return PMKVQ_ERR_CUDA;
   for (int layer = 0; layer < k->layers; ++layer) k->L[layer].n_tokens += 1;
   // 3. attention of all blocks in one launch: their tiles form one line of work cut into one piece per CTA
-  return attention_all_blocks(k, d_Q, d_out, st);
+  return attention_all_blocks(k, d_Q, d_out, st, true);
 }
 
 pmkvq_status pmkvq_decode_attention_all(pmkvq_cache *k, const void *d_Q, float *d_out, void *stream) {
   if (!k || !d_Q || !d_out) return PMKVQ_ERR_INVALID_ARG;
   if (k->layers > kMaxFusedLayers) return PMKVQ_ERR_INVALID_ARG;
-  return attention_all_blocks(k, d_Q, d_out, static_cast<cudaStream_t>(stream));
+  return attention_all_blocks(k, d_Q, d_out, static_cast<cudaStream_t>(stream), false);
 }
 
 pmkvq_status pmkvq_device_status(pmkvq_cache *k, uint32_t *h_wait_bits) {

@@ -1,0 +1,66 @@
+"""Bulk appends at the sizes where the one-launch kernel can go wrong: runs around a tile, around the ring and around
+several rings (a new window token then lands in the slot of a token that leaves the window in the same launch), ragged
+starts, every body width, evictions one by one and in groups; and decode steps enqueued back to back, whose attention
+launch may start while the append in front of it still runs."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2505_18610_b200 import synth
+from tests.helpers import Mirror, make_inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("bits", [2, 4, 8, 16])
+@pytest.mark.parametrize("window,evict_chunk,n_sink,sizes", [
+    (32, 1, 1, (1, 2, 15, 16, 17, 31, 47, 48, 49, 64, 97, 200)),
+    (32, 8, 5, (3, 33, 16, 40, 2, 130, 63)),
+    (0, 1, 0, (5, 16, 27, 2, 32)),
+    (128, 16, 1, (100, 45, 143, 144, 145, 161, 7)),
+])
+def test_append_runs_around_tile_and_ring_edges(bits, window, evict_chunk, n_sink, sizes):
+    total = sum(sizes)
+    k, v = make_inputs(7, 0, total, 2, 2)
+    lam = synth.make_lambda(k[:64]).numpy()[None]
+    # a cache whose budget asks for `bits` from the first token on
+    m = Mirror(1, 4, 2, 2, total, [bits], lam=lam, window=window, evict_chunk=evict_chunk, n_sink=n_sink)
+    m.cache.restore_layer_state(0, 0, bits)
+    m.oracles[0].p.cur_bits = bits
+    done = 0
+    for n in sizes:
+        m.append(0, k[done:done + n], v[done:done + n])
+        done += n
+        m.check_state(0)
+
+
+@pytest.mark.parametrize("evict_chunk", [1, 16])
+@pytest.mark.parametrize("context,batch", [(20, 1), (300, 2), (2100, 3)])
+def test_back_to_back_decode_steps_equal_separate_calls(context, batch, evict_chunk):
+    layers, kvh, hq, steps = 3, 2, 8, 24
+    mk = lambda: Mirror(layers, hq, kvh, batch, context + steps, [4, 2, 16], window=64, evict_chunk=evict_chunk)  # noqa: E731
+    a, b = mk(), mk()
+    for l in range(layers):
+        k, v = make_inputs(3, l, context, batch, kvh)
+        for m in (a, b):
+            m.cache.append(l, k.cuda().contiguous(), v.cuda().contiguous())
+    kv = [make_inputs(4, l, steps, batch, kvh, pos0=context) for l in range(layers)]
+    K = torch.stack([x[0] for x in kv], 1).cuda().contiguous()
+    V = torch.stack([x[1] for x in kv], 1).cuda().contiguous()
+    Q = torch.randn(steps, layers, batch, hq, 128, generator=torch.Generator().manual_seed(5)).bfloat16().cuda()
+    together = [a.cache.decode_step(K[s], V[s], Q[s]) for s in range(steps)]      # nothing waits in between
+    torch.cuda.synchronize()
+    for s in range(steps):
+        for l in range(layers):
+            b.cache.append(l, K[s, l], V[s, l])
+            torch.cuda.synchronize()
+            want = b.cache.decode_attention(l, Q[s, l])
+            torch.cuda.synchronize()
+            got = together[s][l]
+            # two partitions of one sum at the kernels' precision (the bound of the split-invariance test)
+            assert float((got - want).abs().max()) <= 1e-3
+    for l in range(layers):
+        for s in range(batch * kvh):
+            for is_v in (False, True):
+                for x, y in zip(a.cache.export_slice(l, s // kvh, s % kvh, is_v), b.cache.export_slice(l, s // kvh, s % kvh, is_v)):
+                    assert np.array_equal(x, y)
