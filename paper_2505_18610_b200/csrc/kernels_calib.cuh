@@ -14,44 +14,105 @@
 
 namespace pmkvq {
 
-// amax_bits [kv_heads][128] must be zero before the launch.  Grid: one CTA per chunk of tokens;
-// thread t owns channel pair (t % 64, t % 64 + 64) of vector (t / 64 + 2 j) of the token.
-__global__ void __launch_bounds__(128) calib_absmax_kernel(const uint16_t *__restrict__ K, unsigned *amax_bits,
-                                                           int n_tokens, int n_vec /* sequences x kv_heads */,
-                                                           int kv_heads, int tokens_per_cta, double pos_scale,
-                                                           double theta) {
-  __shared__ float s_cos[64], s_sin[64];
-  __shared__ unsigned s_max[8][kHeadDim];  // per kv head (at most 8 per pass), per channel
-  const int tid = threadIdx.x, pair = tid & 63, sub = tid >> 6;
+// Rotation frequencies theta^(-2 pair / 128) in fp64, computed on the host once per call.
+struct RopeFreqs { double f[64]; };
+
+// amax_bits [kv_heads][128] must be zero before the launch.  The Keys are read once, and that is what bounds the kernel
+// (see launch_absmax for the measurement).  Grid: chunks of tokens x chunks of sequences.  A CTA first makes the
+// (cos, sin) table of its tokens (fp64 angles, one per thread at a time); then two warps take a token.  Eight lanes share
+// a vector, every lane eight channels i .. i + 7 and their rotation partners i + 64 .. (two 16-byte loads), so a lane's cos
+// and sin stay in registers for a whole token and its running maxima, for one fixed KV head, for the whole CTA;
+// they meet in shared memory once at the end.
+constexpr int kAbsmaxThreads = 256;
+constexpr int kAbsmaxTokens = 4;      // tokens in flight per CTA: two warps each
+constexpr int kAbsmaxMaxTokens = 16;  // tokens of a CTA
+__global__ void __launch_bounds__(kAbsmaxThreads, 3) calib_absmax_kernel(const uint16_t *__restrict__ K, unsigned *amax_bits,
+                                                                         int n_tokens, int n_seq, int kv_heads,
+                                                                         int tokens_per_cta, int seqs_per_cta,
+                                                                         double pos_scale, const RopeFreqs freqs) {
+  __shared__ __align__(16) float2 s_cs[kAbsmaxMaxTokens][64];
+  __shared__ unsigned s_max[8][kHeadDim];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int t0 = blockIdx.x * tokens_per_cta, t1 = min(n_tokens, t0 + tokens_per_cta);
-  const double inv_freq = pow(theta, -2.0 * pair / (double)kHeadDim);
+  const int s0 = blockIdx.y * seqs_per_cta, s1 = min(n_seq, s0 + seqs_per_cta);
+  for (int i = tid; i < (t1 - t0) * 64; i += kAbsmaxThreads) {
+    double sn, cs;
+    sincos((double)(t0 + (i >> 6)) * pos_scale * freqs.f[i & 63], &sn, &cs);
+    s_cs[i >> 6][i & 63] = make_float2((float)cs, (float)sn);
+  }
+  const int slot = (warp & 1) * 4 + (lane >> 3);  // vector slot of this quarter warp, 0 .. 7
+  const int c0 = (lane & 7) * 8;                  // its lane's channels c0 .. c0 + 7 and c0 + 64 ..
+  const bool aligned = (reinterpret_cast<uintptr_t>(K) & 15) == 0;
   for (int h0 = 0; h0 < kv_heads; h0 += 8) {
-    for (int i = tid; i < 8 * kHeadDim; i += 128) (&s_max[0][0])[i] = 0u;
+    // the eight slots are dealt out over this group's heads: slot -> (head, first sequence)
+    const int nh = min(8, kv_heads - h0), reps = 8 / nh, head = slot % nh;
+    for (int i = tid; i < 8 * kHeadDim; i += kAbsmaxThreads) (&s_max[0][0])[i] = 0u;
     __syncthreads();
-    for (int t = t0; t < t1; ++t) {
-      if (tid < 64) {
-        double s, c;
-        sincos((double)t * pos_scale * inv_freq, &s, &c);
-        s_cos[pair] = (float)c;
-        s_sin[pair] = (float)s;
+    float2 m1[4], m2[4];  // maxima of channels c0 + 2 j, + 1 and of their partners
+#pragma unroll
+    for (int j = 0; j < 4; ++j) m1[j] = m2[j] = make_float2(0.f, 0.f);
+    if (slot < reps * nh) {
+      for (int t = t0 + (warp >> 1); t < t1; t += kAbsmaxTokens) {
+        float2 cs[4], sn[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float4 v = *reinterpret_cast<const float4 *>(&s_cs[t - t0][c0 + 2 * j]);
+          cs[j] = make_float2(v.x, v.z);
+          sn[j] = make_float2(v.y, v.w);
+        }
+        const uint16_t *src = K + (((size_t)t * n_seq + s0 + slot / nh) * kv_heads + h0 + head) * kHeadDim + c0;
+        const size_t step = (size_t)reps * kv_heads * kHeadDim;
+        auto rotate = [&](const uint32_t (&a)[4], const uint32_t (&b)[4]) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float2 x1 = make_float2(__uint_as_float(a[j] << 16), __uint_as_float(a[j] & 0xFFFF0000u));
+            const float2 x2 = make_float2(__uint_as_float(b[j] << 16), __uint_as_float(b[j] & 0xFFFF0000u));
+            const float2 xs = __fmul2_rn(x2, sn[j]);
+            const float2 y1 = __fadd2_rn(__fmul2_rn(x1, cs[j]), make_float2(-xs.x, -xs.y));  // Eq. 11 with the scaled position
+            const float2 y2 = __fadd2_rn(__fmul2_rn(x1, sn[j]), __fmul2_rn(x2, cs[j]));
+            m1[j].x = fmaxf(m1[j].x, fabsf(y1.x)); m1[j].y = fmaxf(m1[j].y, fabsf(y1.y));
+            m2[j].x = fmaxf(m2[j].x, fabsf(y2.x)); m2[j].y = fmaxf(m2[j].y, fabsf(y2.y));
+          }
+        };
+        int s = s0 + slot / nh;
+        if (aligned) {
+          for (; s + 3 * reps < s1; s += 4 * reps, src += 4 * step) {  // four vectors in flight per lane
+            uint4 a[4], b[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              a[u] = __ldcs(reinterpret_cast<const uint4 *>(src + u * step));
+              b[u] = __ldcs(reinterpret_cast<const uint4 *>(src + u * step + 64));
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const uint32_t aw[4] = {a[u].x, a[u].y, a[u].z, a[u].w}, bw[4] = {b[u].x, b[u].y, b[u].z, b[u].w};
+              rotate(aw, bw);
+            }
+          }
+        }
+        for (; s < s1; s += reps, src += step) {  // the rest, or Keys at an address no 16-byte load can take
+          uint32_t aw[4], bw[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            aw[j] = src[2 * j] | ((uint32_t)src[2 * j + 1] << 16);
+            bw[j] = src[64 + 2 * j] | ((uint32_t)src[64 + 2 * j + 1] << 16);
+          }
+          rotate(aw, bw);
+        }
       }
-      __syncthreads();
-      const float c = s_cos[pair], s = s_sin[pair];
-      for (int v = sub; v < n_vec; v += 2) {
-        const int head = v % kv_heads;
-        if (head < h0 || head >= h0 + 8) continue;
-        const uint16_t *src = K + ((size_t)t * n_vec + v) * kHeadDim;
-        const float x1 = __uint_as_float((uint32_t)src[pair] << 16), x2 = __uint_as_float((uint32_t)src[pair + 64] << 16);
-        const float y1 = __fsub_rn(__fmul_rn(x1, c), __fmul_rn(x2, s));  // Eq. 11 with the scaled position
-        const float y2 = __fadd_rn(__fmul_rn(x1, s), __fmul_rn(x2, c));
-        atomicMax(&s_max[head - h0][pair], __float_as_uint(fabsf(y1)));
-        atomicMax(&s_max[head - h0][pair + 64], __float_as_uint(fabsf(y2)));
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        atomicMax(&s_max[head][c0 + 2 * j], __float_as_uint(m1[j].x));
+        atomicMax(&s_max[head][c0 + 2 * j + 1], __float_as_uint(m1[j].y));
+        atomicMax(&s_max[head][c0 + 2 * j + 64], __float_as_uint(m2[j].x));
+        atomicMax(&s_max[head][c0 + 2 * j + 65], __float_as_uint(m2[j].y));
       }
-      __syncthreads();
     }
-    for (int i = tid; i < 8 * kHeadDim; i += 128) {
-      const int head = h0 + i / kHeadDim;
-      if (head < kv_heads && (&s_max[0][0])[i]) atomicMax(amax_bits + (size_t)head * kHeadDim + (i % kHeadDim), (&s_max[0][0])[i]);
+    __syncthreads();
+    for (int i = tid; i < nh * kHeadDim; i += kAbsmaxThreads) {
+      unsigned *dst = amax_bits + (size_t)h0 * kHeadDim + i;
+      const unsigned v = (&s_max[0][0])[i];
+      if (v > __ldcg(dst)) atomicMax(dst, v);  // most CTAs find a larger maximum there already
     }
     __syncthreads();
   }

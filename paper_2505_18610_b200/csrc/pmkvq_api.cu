@@ -793,6 +793,28 @@ pmkvq_status pmkvq_set_attention_ctas(pmkvq_cache *k, int32_t n_ctas) {
   return PMKVQ_OK;
 }
 
+// |K_rot| maxima into d_amax_bits (zeroed here).  Enough CTAs to fill the GPU several times over, each with at least
+// a thousand vectors behind its table of angles.
+static cudaError_t launch_absmax(const uint16_t *K, unsigned *d_amax_bits, int n_tokens, int n_seq, int kv_heads, double pos_scale,
+                                 double theta, cudaStream_t st) {
+  cudaError_t e = cudaMemsetAsync(d_amax_bits, 0, (size_t)kv_heads * kHeadDim * sizeof(unsigned), st);
+  if (e != cudaSuccess) return e;
+  RopeFreqs freqs;
+  for (int i = 0; i < 64; ++i) freqs.f[i] = std::pow(theta, -2.0 * i / (double)kHeadDim);
+  int tokens = kAbsmaxTokens;
+  while (tokens < kAbsmaxMaxTokens && n_tokens > tokens * 148 * 8 && (long long)n_seq * kv_heads < 256) tokens += kAbsmaxTokens;
+  const int tc = (n_tokens + tokens - 1) / tokens;
+  // split the sequences while that leaves a CTA 1024 vectors
+  auto parts = [&](int seqs) { return (n_seq + seqs - 1) / seqs; };
+  int seqs = n_seq;
+  while (seqs > 1 && (long long)tokens * ((seqs + 1) / 2) * kv_heads >= 1024 && (long long)tc * parts(seqs) < 148 * 16 &&
+         parts((seqs + 1) / 2) <= 65535)
+    seqs = (seqs + 1) / 2;
+  calib_absmax_kernel<<<dim3((unsigned)tc, (unsigned)parts(seqs)), kAbsmaxThreads, 0, st>>>(K, d_amax_bits, n_tokens, n_seq, kv_heads, tokens,
+                                                                                          seqs, pos_scale, freqs);
+  return cudaGetLastError();
+}
+
 pmkvq_status pmkvq_calibrate_lambda(const void *d_K, int32_t n_tokens, int32_t n_seq, int32_t kv_heads, double pos_scale,
                                     double theta, float alpha, float floor_value, float *d_lambda, void *stream) {
   if (!d_K || !d_lambda || n_tokens <= 0 || n_seq <= 0 || kv_heads <= 0 || !(pos_scale > 0.0) || !(theta > 1.0) ||
@@ -801,11 +823,9 @@ pmkvq_status pmkvq_calibrate_lambda(const void *d_K, int32_t n_tokens, int32_t n
   if ((int64_t)n_seq * kv_heads > (1 << 20)) return PMKVQ_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int n = kv_heads * kHeadDim;
-  if (cudaMemsetAsync(d_lambda, 0, (size_t)n * sizeof(float), st) != cudaSuccess) return PMKVQ_ERR_CUDA;
-  const int tokens_per_cta = std::max(1, (n_tokens + 148 * 8 - 1) / (148 * 8));
-  const unsigned grid = (unsigned)((n_tokens + tokens_per_cta - 1) / tokens_per_cta);
-  calib_absmax_kernel<<<grid, 128, 0, st>>>(static_cast<const uint16_t *>(d_K), reinterpret_cast<unsigned *>(d_lambda),
-                                            n_tokens, n_seq * kv_heads, kv_heads, tokens_per_cta, pos_scale, theta);
+  if (launch_absmax(static_cast<const uint16_t *>(d_K), reinterpret_cast<unsigned *>(d_lambda), n_tokens, n_seq, kv_heads, pos_scale, theta,
+                    st) != cudaSuccess)
+    return PMKVQ_ERR_CUDA;
   calib_finish_kernel<<<(n + 255) / 256, 256, 0, st>>>(d_lambda, n, floor_value, alpha);
   return cudaGetLastError() == cudaSuccess ? PMKVQ_OK : PMKVQ_ERR_CUDA;
 }
@@ -860,15 +880,13 @@ pmkvq_status pmkvq_alpha_grid_search(const void *d_K, const void *d_Q, const voi
   float *d_alphas = reinterpret_cast<float *>(ws + w.alphas);
   float *d_k = reinterpret_cast<float *>(ws + w.k_pass), *d_v_raw = reinterpret_cast<float *>(ws + w.v_raw);
   float *d_v_hat = reinterpret_cast<float *>(ws + w.v_hat), *d_o_ref = reinterpret_cast<float *>(ws + w.o_ref);
-  if (cudaMemsetAsync(d_amax, 0, (size_t)kv_heads * kHeadDim * sizeof(float), st) != cudaSuccess ||
-      cudaMemsetAsync(d_loss, 0, kMaxAlphas * sizeof(double), st) != cudaSuccess ||
+  if (cudaMemsetAsync(d_loss, 0, kMaxAlphas * sizeof(double), st) != cudaSuccess ||
       cudaMemcpyAsync(d_alphas, h_alphas, (size_t)n_alphas * sizeof(float), cudaMemcpyHostToDevice, st) != cudaSuccess)
     return PMKVQ_ERR_CUDA;
   const uint16_t *K = static_cast<const uint16_t *>(d_K), *Q = static_cast<const uint16_t *>(d_Q),
                  *V = static_cast<const uint16_t *>(d_V);
-  const int tokens_per_cta = std::max(1, (n_tokens + 148 * 8 - 1) / (148 * 8));
-  calib_absmax_kernel<<<(unsigned)((n_tokens + tokens_per_cta - 1) / tokens_per_cta), 128, 0, st>>>(
-      K, reinterpret_cast<unsigned *>(d_amax), n_tokens, n_seq * kv_heads, kv_heads, tokens_per_cta, pos_scale, theta);
+  if (launch_absmax(K, reinterpret_cast<unsigned *>(d_amax), n_tokens, n_seq, kv_heads, pos_scale, theta, st) != cudaSuccess)
+    return PMKVQ_ERR_CUDA;
   rope_table_kernel<<<(unsigned)((n_tokens * 64 + 255) / 256), 256, 0, st>>>(d_table, n_tokens, pos_scale, theta);
   if (cudaFuncSetAttribute(alpha_grid_attn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGridSmemBytes) != cudaSuccess)
     return PMKVQ_ERR_CUDA;

@@ -1,0 +1,26 @@
+"""Abs-max calibration at the edges of its work split: fewer and more tokens than a CTA takes, sequence counts around the
+unrolled and the split loop, head counts that do and do not divide the eight vector slots of a CTA, more than eight
+heads, and Keys at an address that allows no 16-byte load."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import pmkvq_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n_tokens,n_seq,kv_heads,offset", [
+    (1, 1, 1, 0), (3, 5, 3, 0), (4, 31, 1, 0), (5, 33, 1, 1), (17, 4, 8, 0), (17, 3, 8, 4), (9, 7, 5, 0), (33, 2, 11, 0),
+    (70, 65, 8, 0), (6, 257, 4, 0), (10000, 1, 2, 0)])
+def test_absmax_work_split_edges(n_tokens, n_seq, kv_heads, offset):
+    from paper_2505_18610_b200 import binding as B
+    n = n_tokens * n_seq * kv_heads * 128
+    flat = torch.randn(n, generator=torch.Generator().manual_seed(n)).to(torch.bfloat16)
+    buf = torch.zeros(n + 8, dtype=torch.bfloat16, device="cuda")
+    buf[offset:offset + n] = flat.cuda()
+    k = buf[offset:offset + n].view(n_tokens, n_seq, kv_heads, 128)
+    want = O.calibrate_lambda(flat.float().numpy().reshape(n_tokens, n_seq, kv_heads, 128), pos_scale=2.0, alpha=1.0)
+    got = B.calibrate_lambda(k, pos_scale=2.0, alpha=1.0).cpu().numpy()
+    # fp32 rotation from correctly rounded angles: two products and a sum, each within half an ulp, and the power
+    assert np.allclose(got, want, rtol=2e-6, atol=0)
