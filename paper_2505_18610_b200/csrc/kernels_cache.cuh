@@ -404,20 +404,47 @@ __device__ __forceinline__ void store_words(uint8_t *part, int r, int lane, cons
   }
 }
 
+// The same when only some rows of the tile are written: the lower and the upper halves of the words belong to tokens
+// that are kept or not.
+template <int BITS>
+__device__ __forceinline__ void store_word_halves(uint8_t *part, int r, int lane, const uint32_t *words, bool lo, bool hi) {
+#pragma unroll
+  for (int w = 0; w < BITS; ++w) {
+    const int lw = r * BITS + w;
+    uint16_t *dst = reinterpret_cast<uint16_t *>(part + ((lw >> 2) * 32 + lane) * 16 + (lw & 3) * 4);
+    if (lo) dst[0] = (uint16_t)words[w];
+    if (hi) dst[1] = (uint16_t)(words[w] >> 16);
+  }
+}
+constexpr uint32_t kAllRows = 0xFFFFu;
+
 constexpr int kStageRowBytes = 272;  // a staged bf16 row of 128 channels plus 16 bytes: the owner-mapped reads below hit 32 different banks
+// Rows [row_lo, row_hi) of the tile are new tokens and may be loaded; the rows of `keep` are written, the tile's others left
+// alone.
 template <int BITS>
 __device__ __forceinline__ void append_tile_half(const uint16_t *__restrict__ src, size_t row_stride,
                                                  const float *__restrict__ il, uint8_t *dst_tile, int is_value,
-                                                 unsigned *vmax_slot, int lane, int variant, uint8_t *stage) {
+                                                 unsigned *vmax_slot, int lane, int variant, uint8_t *stage, int row_lo = 0,
+                                                 int row_hi = kTileTokens, uint32_t keep = kAllRows) {
   const int g = lane >> 2, tig = lane & 3;
   uint32_t words[BITS];
   // the tile's 16 rows of 256 bytes come in with eight coalesced 16-byte loads per lane, all in flight at once
   {
+    const bool aligned = (reinterpret_cast<uintptr_t>(src) & 15) == 0;
     uint4 v[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
       const int id = lane + 32 * c;
-      v[c] = *reinterpret_cast<const uint4 *>(src + (size_t)(id >> 4) * row_stride + (id & 15) * 8);
+      // a row that may not be loaded stands in as a copy of one that may (zeros would send the whole warp through
+      // the quantizer's rare branch)
+      const int row = max(row_lo, min(id >> 4, row_hi - 1));
+      const uint16_t *from = src + (ptrdiff_t)row * (ptrdiff_t)row_stride + (id & 15) * 8;
+      if (aligned) {
+        v[c] = *reinterpret_cast<const uint4 *>(from);
+      } else {  // inputs on an 8-byte boundary
+        const uint2 a = *reinterpret_cast<const uint2 *>(from), b = *reinterpret_cast<const uint2 *>(from + 4);
+        v[c] = make_uint4(a.x, a.y, b.x, b.y);
+      }
     }
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
@@ -449,9 +476,11 @@ __device__ __forceinline__ void append_tile_half(const uint16_t *__restrict__ sr
       }
       const float s16 = quantize_owned<BITS, 32, false>(x, mn, mx, variant);
       pack_words<BITS>(x, x + 1, 2, words);  // halves of a word: channels h = 0, 1 of the token
-      store_words<BITS>(dst_tile, r, lane, words);
+      const bool kept = (keep >> (g + 8 * r)) & 1u;
+      if (keep == kAllRows) store_words<BITS>(dst_tile, r, lane, words);
+      else store_word_halves<BITS>(dst_tile, r, lane, words, kept, kept);
       // metadata record g / 2 holds tokens {2t, 2t+1, 8+2t, 9+2t} at entries {0, 1, 2, 3}
-      if (tig == 0) {
+      if (tig == 0 && kept) {
         float *rec = reinterpret_cast<float *>(dst_tile + meta_offset(BITS) + (g >> 1) * 64) + 2 * r + (g & 1);
         rec[0] = chain_scale(s16, BITS, variant);
         rec[4] = chain_zero(mn, s16, BITS, variant);
@@ -484,12 +513,17 @@ __device__ __forceinline__ void append_tile_half(const uint16_t *__restrict__ sr
         smax = fmaxf(smax, S[h]);
       }
       pack_words<BITS>(x[0], x[1], 1, words);  // halves of a word: tokens h = 0, 1 of one channel
-      store_words<BITS>(dst_tile + v_part_offset(BITS), r, lane, words);
+      const bool kept0 = (keep >> (2 * tig + 8 * r)) & 1u, kept1 = (keep >> (2 * tig + 8 * r + 1)) & 1u;
+      if (keep == kAllRows) store_words<BITS>(dst_tile + v_part_offset(BITS), r, lane, words);
+      else store_word_halves<BITS>(dst_tile + v_part_offset(BITS), r, lane, words, kept0, kept1);
       if (g == 0) {  // record tig: S_V at bytes 32.., Z_V at 48.., entries 2 r + h
         float *rec = reinterpret_cast<float *>(dst_tile + meta_offset(BITS) + tig * 64 + 32) + 2 * r;
-        *reinterpret_cast<float2 *>(rec) = make_float2(chain_scale(S[0], BITS, variant), chain_scale(S[1], BITS, variant));
-        *reinterpret_cast<float2 *>(rec + 4) =
-            make_float2(chain_zero(Z[0], S[0], BITS, variant), chain_zero(Z[1], S[1], BITS, variant));
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          if (h == 0 ? kept0 : kept1) {
+            rec[h] = chain_scale(S[h], BITS, variant);
+            rec[4 + h] = chain_zero(Z[h], S[h], BITS, variant);
+          }
       }
     }
     smax = fmaxf(smax, __shfl_xor_sync(0xffffffffu, smax, 1));  // the four tig groups hold different tokens
@@ -595,30 +629,25 @@ __device__ __forceinline__ void append_tile_half_row(const uint16_t *__restrict_
   }
 }
 
-// One warp: half (K or V) of body tile `tile` of a slice, all 16 tokens new.  `wid` counts halves, slices, tiles.
+// One warp: half (K or V) of one tile of a slice; row 0 is number i0 of the new tokens (see append_tile_half for the rows).
 template <bool ROWS>
-__device__ __forceinline__ void append_tile_one(long long wid, uint8_t *stage, int lane, const uint16_t *__restrict__ K,
-                                                const uint16_t *__restrict__ V, const float *__restrict__ inv_lambda,
-                                                unsigned *vmax_bits, const LayerGeom &geom, int n_slices, int kv_heads,
-                                                int n_old, int tile_lo, int bits) {
-  const int is_value = (int)(wid & 1);
-  const int slice = (int)((wid >> 1) % n_slices);
-  const int tile = tile_lo + (int)((wid >> 1) / n_slices);
-  const int i0 = geom.n_sink + tile * kTileTokens - n_old;  // index of the tile's first token among the new ones
+__device__ __forceinline__ void append_tile_one(int is_value, int slice, int i0, uint8_t *dst_tile, int bits, uint8_t *stage, int lane,
+                                                const uint16_t *__restrict__ K, const uint16_t *__restrict__ V,
+                                                const float *__restrict__ inv_lambda, unsigned *vmax_bits, int n_slices, int kv_heads,
+                                                int variant, int row_lo = 0, int row_hi = kTileTokens, uint32_t keep = kAllRows) {
   const size_t row_stride = (size_t)n_slices * kHeadDim;
-  const uint16_t *src = (is_value ? V : K) + ((size_t)i0 * n_slices + slice) * kHeadDim;
+  const uint16_t *src = (is_value ? V : K) + ((ptrdiff_t)i0 * n_slices + slice) * kHeadDim;
   const float *il = inv_lambda + (size_t)(slice % kv_heads) * kHeadDim;
-  uint8_t *dst_tile = geom.base + (size_t)slice * geom.slice_stride + geom.body_off + body_tile_offset(tile, bits, geom.stream_stride);
   switch (bits) {
-    case 16: append_tile_half<16>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, geom.shift_variant, stage); break;
-    case 8: append_tile_half<8>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, geom.shift_variant, stage); break;
+    case 16: append_tile_half<16>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, variant, stage, row_lo, row_hi, keep); break;
+    case 8: append_tile_half<8>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, variant, stage, row_lo, row_hi, keep); break;
     case 4:
-      if constexpr (ROWS) append_tile_half_row<4>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, geom.shift_variant, stage);
-      else append_tile_half<4>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, geom.shift_variant, stage);
+      if constexpr (ROWS) append_tile_half_row<4>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, variant, stage);
+      else append_tile_half<4>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, variant, stage, row_lo, row_hi, keep);
       break;
     default:
-      if constexpr (ROWS) append_tile_half_row<2>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, geom.shift_variant, stage);
-      else append_tile_half<2>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, geom.shift_variant, stage);
+      if constexpr (ROWS) append_tile_half_row<2>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, variant, stage);
+      else append_tile_half<2>(src, row_stride, il, dst_tile, is_value, vmax_bits + slice, lane, variant, stage, row_lo, row_hi, keep);
       break;
   }
 }
@@ -634,7 +663,10 @@ __global__ void __launch_bounds__(128, 8) append_tiles_kernel(const uint16_t *__
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long wid = (long long)blockIdx.x * 4 + warp;
   if (wid >= (long long)n_tiles * n_slices * 2) return;
-  append_tile_one<true>(wid, s_scratch[warp], lane, K, V, inv_lambda, vmax_bits, geom, n_slices, kv_heads, n_old, tile_lo, bits);
+  const int slice = (int)((wid >> 1) % n_slices), tile = tile_lo + (int)((wid >> 1) / n_slices);
+  append_tile_one<true>((int)(wid & 1), slice, geom.n_sink + tile * kTileTokens - n_old,
+                        geom.base + (size_t)slice * geom.slice_stride + geom.body_off + body_tile_offset(tile, bits, geom.stream_stride), bits,
+                        s_scratch[warp], lane, K, V, inv_lambda, vmax_bits, n_slices, kv_heads, geom.shift_variant);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -684,17 +716,76 @@ __global__ void __launch_bounds__(128) evict_kernel(LayerGeom geom, int n_slices
   evict_one(wid, s_codes[warp], lane, geom, n_slices, first_token, n_evict, cur_bits);
 }
 
-// A bulk append to a cache of lane-owned tiles in one launch: whole body tiles, then the new tokens around them (sink,
-// window, ragged ends) one by one, then the evictions.  The one hazard is the ring: a new window token may land
-// in the slot of a token that leaves it.  The warp of the new token then moves the old one out first, and the old
-// token's own warp leaves.  (As three to four launches a short prompt's append cost 16.8 us per block, nearly all of
-// it launches of a few microseconds.)
+// Half (K or V) of the rows `keep` of a ring tile -> the same tokens' rows of their body tile at BITS, lane-owned on both sides: a lane's sixteen INT16
+// words per token half become BITS words, nothing crosses lanes.  (Token by token a tile is sixteen warps that each
+// gather 2-byte codes through shared memory.)
+template <int BITS>
+__device__ __forceinline__ void evict_tile_half(const uint8_t *src_tile, uint8_t *dst_tile, int is_value, int lane, int variant,
+                                                uint32_t keep) {
+  constexpr int n = 16 / BITS;
+  const uint8_t *src = src_tile + (is_value ? v_part_offset(16) : 0);
+  uint8_t *dst = dst_tile + (is_value ? v_part_offset(BITS) : 0);
+  uint4 in[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) in[q] = *reinterpret_cast<const uint4 *>(src + (q * 32 + lane) * 16);
+  const float *smeta = reinterpret_cast<const float *>(src_tile + meta_offset(16));
+  float s16 = 0.f, z16 = 0.f;
+  const int kind = is_value ? 2 : 0, row = lane & 15;
+  if (lane < 16) {
+    s16 = smeta[meta_slot(16, false, kind, row) >> 2];
+    z16 = smeta[meta_slot(16, false, kind + 1, row) >> 2];
+  }
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    uint32_t words[BITS];
+#pragma unroll
+    for (int w = 0; w < BITS; ++w) {
+      uint32_t a = 0, b = 0;
+#pragma unroll
+      for (int j = 0; j < n; ++j) {
+        const int i = w * n + j;
+        const uint4 &c4 = in[4 * r + (i >> 2)];
+        const uint32_t x = (i & 3) == 0 ? c4.x : (i & 3) == 1 ? c4.y : (i & 3) == 2 ? c4.z : c4.w;
+        a |= chain_code<BITS>(x & 0xFFFFu, variant) << (j * BITS);
+        b |= chain_code<BITS>(x >> 16, variant) << (j * BITS);
+      }
+      words[w] = __byte_perm(a, b, 0x5410);
+    }
+    if (keep == kAllRows) {
+      store_words<BITS>(dst, r, lane, words);
+    } else {
+      const int g = lane >> 2, tig = lane & 3, row0 = is_value ? 2 * tig + 8 * r : g + 8 * r, row1 = is_value ? row0 + 1 : row0;
+      store_word_halves<BITS>(dst, r, lane, words, (keep >> row0) & 1u, (keep >> row1) & 1u);
+    }
+  }
+  if (lane < 16 && ((keep >> row) & 1u)) store_meta(dst_tile, BITS, row, is_value, s16, z16, variant, false);
+}
+__device__ __forceinline__ void evict_tile_one(int is_value, int slice, int group, const LayerGeom &geom, int bits, int lane,
+                                               uint32_t keep = kAllRows) {
+  uint8_t *slice_base = geom.base + (size_t)slice * geom.slice_stride;
+  const uint8_t *src = slice_base + geom.ring_off + (size_t)(group % (geom.ring_tokens >> 4)) * tile_bytes(16);
+  uint8_t *dst = slice_base + geom.body_off + body_tile_offset(group, bits, geom.stream_stride);
+  switch (bits) {
+    case 16: evict_tile_half<16>(src, dst, is_value, lane, geom.shift_variant, keep); break;
+    case 8: evict_tile_half<8>(src, dst, is_value, lane, geom.shift_variant, keep); break;
+    case 4: evict_tile_half<4>(src, dst, is_value, lane, geom.shift_variant, keep); break;
+    default: evict_tile_half<2>(src, dst, is_value, lane, geom.shift_variant, keep); break;
+  }
+}
+
+// A bulk append to a cache of lane-owned tiles in one launch.  Tokens behind the sink go in groups of 16: group m is body tile m
+// and, while it is in the window, ring tile m mod ring_tiles, row for row.  An item is one group: new rows of it to the
+// body, new rows of it to the window ring, or rows of it that leave the window (a group may be several items); a warp takes
+// half (K or V) of an item of one slice.  Only sink tokens go one by one.  The one hazard is the ring: new window tokens may
+// land in slots of tokens that leave it.  The warp that writes a slot then moves its old contents out first, and the
+// leaving rows' own item leaves them out.
+// (Before, the window and the ragged ends went token by token, 16 times the warps, in three to four launches: 16.8 us per block
+// for a 2537-token prompt, 35 us for a chunk of 2048 tokens x 32 slices.)
 struct BulkParams {
-  int n_old, n_after, win_start;       // tokens before and after, first token of the window afterwards
-  int tile_lo, n_tiles;                // body tiles written whole
-  int head_first, head_cnt;            // new tokens (absolute) before the whole tiles ...
-  int tail_first, tail_cnt;            // ... and behind them
-  int ev_first, n_evict;               // tokens that leave the window
+  int n_old, n_after, win_start;  // tokens before and after, first token of the window afterwards
+  int ev_first, ev_end;           // tokens that leave the window
+  int ring_lo, body_lo, evict_lo; // first group of each kind, and the items of this and the kinds before it (ring items
+  int ring_end, body_end, evict_end, sink_end;  // take longest and go first)
 };
 __global__ void __launch_bounds__(128, 8) append_bulk_kernel(const uint16_t *__restrict__ K, const uint16_t *__restrict__ V,
                                                              const float *__restrict__ inv_lambda, unsigned *vmax_bits,
@@ -704,34 +795,41 @@ __global__ void __launch_bounds__(128, 8) append_bulk_kernel(const uint16_t *__r
   pdl_launch_next();
   pdl_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  long long wid = (long long)blockIdx.x * 4 + warp;
-  const long long per = 2ll * n_slices;
-  if (wid < per * bp.n_tiles) {
-    append_tile_one<false>(wid, s_scratch[warp], lane, K, V, inv_lambda, vmax_bits, geom, n_slices, kv_heads, bp.n_old, bp.tile_lo, cur_bits);
-    return;
-  }
-  wid -= per * bp.n_tiles;
-  uint16_t *codes = reinterpret_cast<uint16_t *>(s_scratch[warp]);
-  const int ring = geom.ring_tokens;
-  if (wid < per * (bp.head_cnt + bp.tail_cnt)) {
-    const int k = (int)(wid / per);
-    const long long in_token = wid - k * per;  // slice and half
-    const int t = k < bp.head_cnt ? bp.head_first + k : bp.tail_first + (k - bp.head_cnt);
-    if (bp.n_evict > 0 && t >= bp.win_start && t >= geom.n_sink) {
-      const int old = t - ((t - bp.n_old) / ring + 1) * ring;  // the last token before this append in the same slot
-      if (old >= bp.ev_first && old < bp.ev_first + bp.n_evict)
-        evict_one(in_token, codes, lane, geom, n_slices, old, 1, cur_bits);
+  const long long wid = (long long)blockIdx.x * 4 + warp, per = 2ll * n_slices;
+  if (wid >= per * bp.sink_end) return;
+  const int item = (int)(wid / per);
+  const int in_item = (int)(wid - item * per), is_value = in_item & 1, slice = in_item >> 1;
+  const int ring = geom.ring_tokens, ring_tiles = ring >> 4, first_new = max(bp.n_old, bp.win_start);  // first new window token
+  const int row = lane & 15;
+  if (item < bp.body_end) {
+    const bool to_ring = item < bp.ring_end;
+    const int group = to_ring ? bp.ring_lo + item : bp.body_lo + item - bp.ring_end;
+    const int t0 = geom.n_sink + group * kTileTokens, i0 = t0 - bp.n_old, t = t0 + row;
+    const bool mine = to_ring ? t >= first_new && t < bp.n_after : t >= bp.n_old && t < bp.win_start;
+    const uint32_t keep = __ballot_sync(0xffffffffu, mine) & kAllRows;
+    uint8_t *dst = geom.base + (size_t)slice * geom.slice_stride;
+    int bits = 16;
+    if (to_ring) {
+      dst += geom.ring_off + (size_t)(group % ring_tiles) * tile_bytes(16);
+      // the last group before this append in the same ring tile: its rows that leave the window and are overwritten here
+      const int old = group - (max(i0, 0) / ring + 1) * ring_tiles, t_old = geom.n_sink + old * kTileTokens + row;
+      const uint32_t out = __ballot_sync(0xffffffffu, mine && t_old >= bp.ev_first && t_old < bp.ev_end) & kAllRows;
+      if (out) evict_tile_one(is_value, slice, old, geom, cur_bits, lane, out);
+      __syncwarp();
+    } else {
+      bits = cur_bits;
+      dst += geom.body_off + body_tile_offset(group, bits, geom.stream_stride);
     }
-    append_one(in_token, codes, lane, K, V, inv_lambda, vmax_bits, geom, n_slices, kv_heads, bp.n_old, bp.win_start, cur_bits, t - bp.n_old, 1);
-    return;
-  }
-  wid -= per * (bp.head_cnt + bp.tail_cnt);
-  if (wid < per * bp.n_evict) {
-    const int k = (int)(wid / per), t = bp.ev_first + k;
-    const int first = max(bp.n_old, bp.win_start);         // new window tokens: first .. n_after - 1
-    const int taker = t + (first - t + ring - 1) / ring * ring;  // the first of them (or later) that lands in t's slot
-    if (taker < bp.n_after) return;
-    evict_one(wid - k * per, codes, lane, geom, n_slices, t, 1, cur_bits);
+    append_tile_one<false>(is_value, slice, i0, dst, bits, s_scratch[warp], lane, K, V, inv_lambda, vmax_bits, n_slices, kv_heads,
+                           geom.shift_variant, max(0, -i0), min(kTileTokens, bp.n_after - t0), keep);
+  } else if (item < bp.evict_end) {
+    const int group = bp.evict_lo + item - bp.body_end, t = geom.n_sink + group * kTileTokens + row;
+    const int taker = t + max(1, (first_new - t + ring - 1) / ring) * ring;  // the new window token that lands in t's slot, if any
+    const uint32_t out = __ballot_sync(0xffffffffu, t >= bp.ev_first && t < bp.ev_end && taker >= bp.n_after) & kAllRows;
+    if (out) evict_tile_one(is_value, slice, group, geom, cur_bits, lane, out);
+  } else {
+    append_one(in_item, reinterpret_cast<uint16_t *>(s_scratch[warp]), lane, K, V, inv_lambda, vmax_bits, geom, n_slices, kv_heads, bp.n_old,
+               bp.win_start, cur_bits, item - bp.evict_end, 1);
   }
 }
 
@@ -771,6 +869,10 @@ struct StepParams {
   unsigned char cur_bits[kMaxStepLayers];  // body width of each block
 };
 
+// Whole 16-token groups leave the window at once when evict_chunk is a multiple of 16 (the first evicted token is then the
+// first of a group): TILES moves them as tiles, 16 times fewer warps.
+__host__ __device__ constexpr int step_evict_items(int evict_chunk, bool tiles) { return tiles ? evict_chunk / kTileTokens : evict_chunk; }
+template <bool TILES>
 __global__ void __launch_bounds__(128) append_step_kernel(const uint16_t *__restrict__ K, const uint16_t *__restrict__ V,
                                                           const float *__restrict__ inv_lambda, unsigned *vmax_bits,
                                                           const LayerGeom *__restrict__ geoms, const StepParams sp,
@@ -780,7 +882,8 @@ __global__ void __launch_bounds__(128) append_step_kernel(const uint16_t *__rest
   pdl_wait();
   pdl_launch_next();  // behind the wait: what the next grid reads before its own wait is complete then
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long per_layer = 2ll * (evict_chunk + 1) * n_slices;
+  const int ev_items = step_evict_items(evict_chunk, TILES);
+  const long long per_layer = 2ll * (ev_items + 1) * n_slices;
   const long long gw = (long long)blockIdx.x * 4 + warp;
   const int layer = (int)(gw / per_layer);
   if (layer >= layers) return;
@@ -793,9 +896,12 @@ __global__ void __launch_bounds__(128) append_step_kernel(const uint16_t *__rest
   };
   const int old_ws = min(n_old, n_sink) + body_at(n_old), new_ws = min(n_after, n_sink) + body_at(n_after);
   const int ev_first = max(old_ws, n_sink), n_evict = max(0, min(new_ws, n_old) - ev_first);
-  const long long ev_room = 2ll * evict_chunk * n_slices;
+  const long long ev_room = 2ll * ev_items * n_slices;
   if (w < ev_room) {
-    if (w < 2ll * n_evict * n_slices) evict_one(w, s_codes[warp], lane, geom, n_slices, ev_first, n_evict, cur_bits);
+    if constexpr (TILES) {
+      if (n_evict > 0)
+        evict_tile_one((int)(w & 1), (int)((w >> 1) % n_slices), ((ev_first - n_sink) >> 4) + (int)((w >> 1) / n_slices), geom, cur_bits, lane);
+    } else if (w < 2ll * n_evict * n_slices) evict_one(w, s_codes[warp], lane, geom, n_slices, ev_first, n_evict, cur_bits);
   } else {
     const size_t in_off = (size_t)layer * n_slices * kHeadDim;
     append_one(w - ev_room, s_codes[warp], lane, K + in_off, V + in_off, inv_lambda + (size_t)layer * kv_heads * kHeadDim,

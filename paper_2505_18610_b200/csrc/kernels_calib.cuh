@@ -26,6 +26,7 @@ struct RopeFreqs { double f[64]; };
 constexpr int kAbsmaxThreads = 256;
 constexpr int kAbsmaxTokens = 4;      // tokens in flight per CTA: two warps each
 constexpr int kAbsmaxMaxTokens = 16;  // tokens of a CTA
+constexpr int kAbsmaxPrefetch = 32768;  // bytes per token asked for (to L2) while the CTA makes its table: 118 -> 108 us, 64 KB 127
 __global__ void __launch_bounds__(kAbsmaxThreads, 3) calib_absmax_kernel(const uint16_t *__restrict__ K, unsigned *amax_bits,
                                                                          int n_tokens, int n_seq, int kv_heads,
                                                                          int tokens_per_cta, int seqs_per_cta,
@@ -35,6 +36,16 @@ __global__ void __launch_bounds__(kAbsmaxThreads, 3) calib_absmax_kernel(const u
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int t0 = blockIdx.x * tokens_per_cta, t1 = min(n_tokens, t0 + tokens_per_cta);
   const int s0 = blockIdx.y * seqs_per_cta, s1 = min(n_seq, s0 + seqs_per_cta);
+  const bool aligned = (reinterpret_cast<uintptr_t>(K) & 15) == 0;
+  pdl_launch_next();
+  pdl_wait();
+  if (tid < t1 - t0 && aligned) {
+    const size_t row = (size_t)kv_heads * kHeadDim * sizeof(uint16_t);
+    const uint32_t bytes = (uint32_t)min((size_t)kAbsmaxPrefetch, (size_t)(s1 - s0) * row);
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(reinterpret_cast<const uint8_t *>(K) + ((size_t)(t0 + tid) * n_seq + s0) * row),
+                 "r"(bytes)
+                 : "memory");
+  }
   for (int i = tid; i < (t1 - t0) * 64; i += kAbsmaxThreads) {
     double sn, cs;
     sincos((double)(t0 + (i >> 6)) * pos_scale * freqs.f[i & 63], &sn, &cs);
@@ -42,7 +53,6 @@ __global__ void __launch_bounds__(kAbsmaxThreads, 3) calib_absmax_kernel(const u
   }
   const int slot = (warp & 1) * 4 + (lane >> 3);  // vector slot of this quarter warp, 0 .. 7
   const int c0 = (lane & 7) * 8;                  // its lane's channels c0 .. c0 + 7 and c0 + 64 ..
-  const bool aligned = (reinterpret_cast<uintptr_t>(K) & 15) == 0;
   for (int h0 = 0; h0 < kv_heads; h0 += 8) {
     // the eight slots are dealt out over this group's heads: slot -> (head, first sequence)
     const int nh = min(8, kv_heads - h0), reps = 8 / nh, head = slot % nh;
@@ -120,6 +130,7 @@ __global__ void __launch_bounds__(kAbsmaxThreads, 3) calib_absmax_kernel(const u
 
 // In place: bit pattern of amax -> lambda = max(amax, floor)^alpha (Eq. 10).
 __global__ void calib_finish_kernel(float *lambda, int n, float floor_value, float alpha) {
+  pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) lambda[i] = powf(fmaxf(lambda[i], floor_value), alpha);
 }

@@ -18,6 +18,8 @@ pytestmark = pytest.mark.gpu
     (32, 8, 5, (3, 33, 16, 40, 2, 130, 63)),
     (0, 1, 0, (5, 16, 27, 2, 32)),
     (128, 16, 1, (100, 45, 143, 144, 145, 161, 7)),
+    (200, 1, 17, (217, 1, 16, 208, 15, 33, 400, 31)),
+    (64, 16, 0, (64, 16, 80, 5, 96, 11, 64, 160, 48)),
 ])
 def test_append_runs_around_tile_and_ring_edges(bits, window, evict_chunk, n_sink, sizes):
     total = sum(sizes)
@@ -32,6 +34,19 @@ def test_append_runs_around_tile_and_ring_edges(bits, window, evict_chunk, n_sin
         m.append(0, k[done:done + n], v[done:done + n])
         done += n
         m.check_state(0)
+
+
+def test_append_of_inputs_no_16_byte_load_can_take():
+    k, v = make_inputs(9, 0, 300, 1, 2)
+    m = Mirror(1, 2, 2, 1, 300, [4], window=32)
+    dev = []
+    for x in (k, v):
+        buf = torch.empty(x.numel() + 4, dtype=torch.bfloat16, device="cuda")
+        buf[4:] = x.cuda().view(-1)                 # 8 bytes behind a 256-byte boundary
+        dev.append(buf[4:].view(x.shape))
+    m.cache.append(0, dev[0], dev[1])
+    m.oracles[0].append_bulk(k.float().numpy().reshape(300, 2, 128), v.float().numpy().reshape(300, 2, 128))
+    m.check_state(0)
 
 
 @pytest.mark.parametrize("evict_chunk", [1, 16])
