@@ -153,42 +153,20 @@ __global__ void rope_table_kernel(float2 *table, int n_tokens, double pos_scale,
   table[i] = make_float2((float)c, (float)s);
 }
 
-constexpr int kGridQueries = 64;            // queries of one CTA: four warps of 16
-constexpr int kGridKeys = 32;               // keys per shared-memory tile
 constexpr int kMaxAlphas = 64;
 __device__ __forceinline__ float ex2_fast(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-// A tile in shared memory: four planes (K hi, K lo, V hi, V lo) of kGridKeys rows of 128 fp16; a row takes 272
-// bytes so that the eight 16-byte rows of an 8 x 8 ldmatrix tile fall into different banks.
-constexpr int kGridRowBytes = 2 * kHeadDim + 16;
-constexpr int kGridPlaneBytes = kGridKeys * kGridRowBytes;
-constexpr int kGridStageBytes = 4 * kGridPlaneBytes;
-constexpr int kGridSmemBytes = 2 * kGridStageBytes;  // two stages
-
 // x = hi + lo with both parts fp16: 22 significant bits (an absolute 2^-25 below 1/8), which three tensor-core
-// products hi*hi + hi*lo + lo*hi carry into the fp32 accumulator.
-__device__ __forceinline__ void split_half(float x, __half &hi, __half &lo) {
-  hi = __float2half_rn(x);
-  lo = __float2half_rn(x - __half2float(hi));
-}
+// products hi*hi + lo*hi + hi*lo carry into the fp32 accumulator.
 __device__ __forceinline__ void split_half2(float x, float y, uint32_t &hi, uint32_t &lo) {
-  __half hx, lx, hy, ly;
-  split_half(x, hx, lx);
-  split_half(y, hy, ly);
-  const __half2 h = __halves2half2(hx, hy), l = __halves2half2(lx, ly);
+  const __half2 h = __floats2half2_rn(x, y);
+  const float2 back = __half22float2(h), rest = __fadd2_rn(make_float2(x, y), make_float2(-back.x, -back.y));
+  const __half2 l = __floats2half2_rn(rest.x, rest.y);
   hi = *reinterpret_cast<const uint32_t *>(&h);
   lo = *reinterpret_cast<const uint32_t *>(&l);
-}
-__device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t (&r)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-__device__ __forceinline__ void ldsm_x4_trans(uint32_t addr, uint32_t (&r)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
 }
 
 // One token's 4 channels per lane (channels 4 lane .. 4 lane + 3): rotate by the token's angles.  The
@@ -205,9 +183,10 @@ __device__ __forceinline__ void rotate_token(float (&x)[4], const float2 *__rest
   }
 }
 
-// Eq. 1-2 at 16 bit on one token's 128 channels spread over a warp, the Eq. 3 chain to `bits`, and back
-// to real values: x <- S_b * code_b + Z.
-__device__ __forceinline__ void quantize_dequantize_token(float (&x)[4], int bits) {
+// Eq. 1-2 at 16 bit on one token's 128 channels spread over a warp and the Eq. 3 chain to `bits`: x becomes the code minus
+// half the largest code (exact in fp32, and in one fp16 up to 8 bit), so that the dequantized value is scale * x + zero
+// with the middle of the token's range as `zero`.
+__device__ __forceinline__ void quantize_token_centred(float (&x)[4], int bits, float &scale, float &zero) {
   float mn = fminf(fminf(x[0], x[1]), fminf(x[2], x[3]));
   float mx = fmaxf(fmaxf(x[0], x[1]), fmaxf(x[2], x[3]));
 #pragma unroll
@@ -216,16 +195,17 @@ __device__ __forceinline__ void quantize_dequantize_token(float (&x)[4], int bit
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   }
   const float s16 = __fdiv_rn(__fsub_rn(mx, mn), 65535.0f);
-  float sb = s16;
-  for (int w = 8; w >= bits; w >>= 1) sb = __fmul_rn(sb, (float)((1 << w) + 1));
   const bool plain = s16 >= 0x1p-60f && s16 <= 0x1p60f;  // else: constant token (0 / 0 converts to code 0) or absurd range
   const float y = plain ? __frcp_rn(s16) : 0.f;
+  const float half = 0.5f * (float)((1 << bits) - 1);
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
     const float d = __fsub_rn(x[e], mn);
     const int c = plain ? code_of_quotient(quotient_rn(d, s16, y)) : min(max(__float2int_rn(__fdiv_rn(d, s16)), 0), 65535);
-    x[e] = fmaf((float)shift_chain((uint32_t)c, bits), sb, mn);
+    x[e] = (float)shift_chain((uint32_t)c, bits) - half;
   }
+  scale = chain_scale(s16, bits);
+  zero = fmaf(scale, half, mn);
 }
 
 __device__ __forceinline__ void load_bf16x4(const uint16_t *src, float (&x)[4]) {
@@ -236,257 +216,510 @@ __device__ __forceinline__ void load_bf16x4(const uint16_t *src, float (&x)[4]) 
   x[3] = __uint_as_float(raw.y & 0xFFFF0000u);
 }
 
-// Four values of vector `vec` (channels 4 lane ..) as fp16 hi and lo parts: the hi plane [n_vectors][128] fp16
-// is followed by the lo plane, together the 4 bytes per element of the fp32 buffer they replace.
-__device__ __forceinline__ void store_split4(float *out, long long n_vectors, long long vec, int lane, const float (&x)[4]) {
-  uint2 hi, lo;
-  split_half2(x[0], x[1], hi.x, lo.x);
-  split_half2(x[2], x[3], hi.y, lo.y);
-  __half *planes = reinterpret_cast<__half *>(out);
-  *reinterpret_cast<uint2 *>(planes + vec * kHeadDim + 4 * lane) = hi;
-  *reinterpret_cast<uint2 *>(planes + (n_vectors + vec) * kHeadDim + 4 * lane) = lo;
-}
+// ---- tensors of a pass as the attention kernel reads them ----------------------------------------------------
+// Slice s = (sequence, KV head), s = seq * kv_heads + head, is cut into tiles of 64 tokens (the last one shorter).  A tile of
+// r tokens is PLANES planes of r * 256 bytes, each [16 groups of 8 channels][r tokens][8 channels] fp16: one bulk copy (or one
+// per channel group, for the short tile) puts it into shared memory in the core-matrix order of the MMAs, as the K-major
+// operand of the scores and as the MN-major operand of the outputs alike.  One plane holds centred codes, two planes hold
+// fp16 hi and lo parts of a value.  Per token a scale and a zero-point (not for plain values): [slice][n4] fp32 each, n4 = tokens
+// rounded up to 4, the padding zero.
+constexpr int kGridTile = 64;
+constexpr int kGridMaxBatch = 4;  // alphas whose Keys sit in the workspace side by side (codes up to 8 bit)
+__host__ __device__ constexpr int grid_n4(int n_tokens) { return (n_tokens + 3) & ~3; }
 
-// One pass's Keys and Values as the attention kernel reads them: [n_tokens][n_seq][kv_heads][128] as fp16 hi and
-// lo planes (see store_split4).
-// One warp per (token, sequence, KV head) vector, lane l on channels 4 l .. 4 l + 3.
-//   alpha_index < 0  (the unquantized operator): k_out = rotated Keys, v_out = Values
-//   alpha_index >= 0: k_out = dequantized Q_bits(rotated Keys * Lambda^-1), lambda = max(amax, floor)^alpha;
-//                     v_out (if not null) = dequantized Q_bits(Values), which no alpha changes
-__global__ void __launch_bounds__(128) alpha_grid_prep_kernel(const uint16_t *__restrict__ K, const uint16_t *__restrict__ V,
-                                                              const float *__restrict__ amax, const float2 *__restrict__ table,
-                                                              const float *__restrict__ alphas, int alpha_index,
-                                                              long long n_vectors, int vec_per_token, int kv_heads, int bits,
-                                                              float floor_value, float *__restrict__ k_out,
-                                                              float *__restrict__ v_out) {
-  const int lane = threadIdx.x & 31;
-  const long long vec = (long long)blockIdx.x * 4 + (threadIdx.x >> 5);
-  if (vec >= n_vectors) return;
-  const int t = (int)(vec / vec_per_token), kv_head = (int)(vec % kv_heads);
-  float xk[4];
-  load_bf16x4(K + vec * kHeadDim + 4 * lane, xk);
-  rotate_token(xk, table + (size_t)t * 64, lane);
-  if (alpha_index >= 0) {
-    const float alpha = alphas[alpha_index];
-    const float4 am = *reinterpret_cast<const float4 *>(amax + (size_t)kv_head * kHeadDim + 4 * lane);
-    xk[0] = __fmul_rn(xk[0], __fdiv_rn(1.0f, powf(fmaxf(am.x, floor_value), alpha)));
-    xk[1] = __fmul_rn(xk[1], __fdiv_rn(1.0f, powf(fmaxf(am.y, floor_value), alpha)));
-    xk[2] = __fmul_rn(xk[2], __fdiv_rn(1.0f, powf(fmaxf(am.z, floor_value), alpha)));
-    xk[3] = __fmul_rn(xk[3], __fdiv_rn(1.0f, powf(fmaxf(am.w, floor_value), alpha)));
-    quantize_dequantize_token(xk, bits);
-  }
-  store_split4(k_out, n_vectors, vec, lane, xk);
-  if (v_out) {
-    float xv[4];
-    load_bf16x4(V + vec * kHeadDim + 4 * lane, xv);
-    if (alpha_index >= 0) quantize_dequantize_token(xv, bits);
-    store_split4(v_out, n_vectors, vec, lane, xv);
-  }
-}
-
-// One pass of causal self-attention on the tensor cores at fp32-like precision.  Grid: (query blocks, query
-// heads, sequences); a CTA takes 64 queries, a warp 16 of them against all their keys.
-// Q: bf16 [n_tokens][n_seq][kv_heads * group][128] before RoPE (rotated here, and scaled by lambda(alpha)
-// when alpha_index >= 0, Eq. 9); k_in, v_in: this pass's tensors from alpha_grid_prep_kernel (fp16 hi and lo
-// planes).  alpha_index < 0: the outputs go to o_ref [n_tokens][n_seq][q_heads][128]; otherwise the squared
-// differences to o_ref are added to loss_sums[alpha_index] (fp64).
-// Every operand of the two contractions is a sum of two fp16 numbers (queries and probabilities split in
-// registers, keys and values by the prep kernel), and a product takes three mma.sync.m16n8k16 (hi hi, hi lo,
-// lo hi; the lo lo term is below 2^-22 of the product): the loss is a small difference of two attention
-// outputs, so plain fp16 or bf16 operands would drown it.  Key / Value tiles of 32 tokens arrive through a
-// two-stage cp.async ring; ldmatrix (transposed for the Values) builds the B fragments.
-__global__ void __launch_bounds__(128, 2) alpha_grid_attn_kernel(const uint16_t *__restrict__ Q, const float *__restrict__ k_in,
-                                                                 const float *__restrict__ v_in, const float *__restrict__ amax,
-                                                                 const float2 *__restrict__ table,
-                                                                 const float *__restrict__ alphas, int alpha_index, int n_tokens,
-                                                                 int n_seq, int kv_heads, int group, float floor_value,
-                                                                 float *__restrict__ o_ref, double *loss_sums) {
-  extern __shared__ __align__(16) uint8_t s_tiles[];  // [stage][K hi | K lo | V hi | V lo][32 keys][272 bytes]
-  __shared__ float s_lam[kHeadDim];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, tig = lane & 3;
-  const int qb = (int)gridDim.x - 1 - (int)blockIdx.x;  // long rows first
-  const int q_head = blockIdx.y, seq = blockIdx.z, kv_head = q_head / group, q_heads = kv_heads * group;
-  const int q0 = qb * kGridQueries + 16 * warp;                   // first of the warp's queries
-  const int q_last = min(n_tokens, (qb + 1) * kGridQueries) - 1;  // last live query of the CTA
-  const size_t kv_row = (size_t)n_seq * kv_heads * kHeadDim;      // halfs from one token to the next
-  const size_t plane = (size_t)n_tokens * kv_row;                 // halfs from the hi plane to the lo plane
-  const __half *kv_base[4];
-  kv_base[0] = reinterpret_cast<const __half *>(k_in) + ((size_t)seq * kv_heads + kv_head) * kHeadDim;
-  kv_base[1] = kv_base[0] + plane;
-  kv_base[2] = reinterpret_cast<const __half *>(v_in) + ((size_t)seq * kv_heads + kv_head) * kHeadDim;
-  kv_base[3] = kv_base[2] + plane;
-  const float scale_log2 = 1.4426950408889634f * rsqrtf((float)kHeadDim);
-  const uint32_t ring = (uint32_t)__cvta_generic_to_shared(s_tiles);
-
-  // tile j -> stage j & 1: thread i copies 16-byte pieces i, i + 128, ... of the 4 x 32 rows of 256 bytes
-  auto issue = [&](int j) {
-    const uint32_t dst = ring + (uint32_t)((j & 1) * kGridStageBytes);
+struct GridPrep {
+  const uint16_t *src;     // K or V, bf16 [n_tokens][n_seq][kv_heads][128]
+  const float *amax;       // [kv_heads][128]
+  const float2 *table;     // [n_tokens][64]
+  const float *alphas;     // those of this batch
+  uint8_t *out[kGridMaxBatch];
+  float *scale[kGridMaxBatch], *zero[kGridMaxBatch];
+  unsigned *vmax;          // per slice, the largest scale (Values)
+  int n_out;               // buffers to fill (alphas of the batch; 1 for Values and for plain Keys)
+  int is_key, quantize;    // rotate (and, quantized, equalize); quantize or keep plain
+  int n_tokens, n_seq, kv_heads, bits;
+  float floor_value;
+};
+// One CTA per (slice, tile): the tile's vectors are read (and rotated) once, a warp on eight of them, and every alpha's
+// version leaves through shared memory as whole 16-byte pieces.
+constexpr int kPrepChunkStride = kGridTile * 16 + 16;  // padded: the 16 channel groups a warp writes fall into different banks
+template <int PLANES>
+__global__ void __launch_bounds__(256) alpha_grid_prep_kernel(const GridPrep p) {
+  __shared__ __align__(16) uint8_t s_tile[PLANES][16 * kPrepChunkStride];
+  __shared__ float s_scale[kGridTile], s_zero[kGridTile];
+  __shared__ __align__(16) float s_inv[kHeadDim];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int n_tiles = (p.n_tokens + kGridTile - 1) / kGridTile;
+  const int tile = (int)(blockIdx.x % (unsigned)n_tiles), slice = (int)(blockIdx.x / (unsigned)n_tiles), n_slices = p.n_seq * p.kv_heads;
+  const int t0 = tile * kGridTile, rows = min(kGridTile, p.n_tokens - t0), n4 = grid_n4(p.n_tokens);
+  float x0[8][4];
 #pragma unroll
-    for (int c = 0; c < 16; ++c) {
-      const int piece = tid + 128 * c, pl = piece >> 9, row = (piece >> 4) & 31, col = piece & 15;
-      const int t = min(j * kGridKeys + row, n_tokens - 1);  // rows behind the last token are masked below
-      cp_async16(dst + (uint32_t)(pl * kGridPlaneBytes + row * kGridRowBytes + col * 16), kv_base[pl] + (size_t)t * kv_row + col * 8);
+  for (int i = 0; i < 8; ++i) {
+    const int t = t0 + min(warp + 8 * i, rows - 1);
+    load_bf16x4(p.src + ((size_t)t * n_slices + slice) * kHeadDim + 4 * lane, x0[i]);
+  }
+  if (p.is_key) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) rotate_token(x0[i], p.table + (size_t)(t0 + min(warp + 8 * i, rows - 1)) * 64, lane);
+  }
+  for (int a = 0; a < p.n_out; ++a) {
+    if (p.is_key && p.quantize && tid < kHeadDim)
+      s_inv[tid] = __fdiv_rn(1.0f, powf(fmaxf(p.amax[(size_t)(slice % p.kv_heads) * kHeadDim + tid], p.floor_value), p.alphas[a]));
+    __syncthreads();
+    float smax = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int row = warp + 8 * i;
+      float x[4] = {x0[i][0], x0[i][1], x0[i][2], x0[i][3]};
+      if (p.quantize) {
+        if (p.is_key) {
+          const float4 il = *reinterpret_cast<const float4 *>(s_inv + 4 * lane);
+          x[0] = __fmul_rn(x[0], il.x); x[1] = __fmul_rn(x[1], il.y); x[2] = __fmul_rn(x[2], il.z); x[3] = __fmul_rn(x[3], il.w);
+        }
+        float scale, zero;
+        quantize_token_centred(x, p.bits, scale, zero);
+        smax = fmaxf(smax, scale);
+        if (lane == 0) { s_scale[row] = row < rows ? scale : 0.f; s_zero[row] = row < rows ? zero : 0.f; }
+      }
+      uint2 hi, lo;
+      split_half2(x[0], x[1], hi.x, lo.x);
+      split_half2(x[2], x[3], hi.y, lo.y);
+      const int at = (lane >> 1) * kPrepChunkStride + row * 16 + (lane & 1) * 8;
+      *reinterpret_cast<uint2 *>(&s_tile[0][at]) = hi;
+      if constexpr (PLANES == 2) *reinterpret_cast<uint2 *>(&s_tile[1][at]) = lo;
     }
-  };
-  const int n_tiles = q_last / kGridKeys + 1;
-  issue(0);
-  cp_async_commit();
+    if (p.vmax && lane == 0) atomicMax(p.vmax + slice, __float_as_uint(smax));  // scale >= 0: uint order = float order
+    __syncthreads();
+    uint8_t *dst = p.out[a] + ((size_t)slice * p.n_tokens + t0) * (size_t)(256 * PLANES);
+#pragma unroll
+    for (int pl = 0; pl < PLANES; ++pl)
+      for (int i = tid; i < 16 * rows; i += 256) {
+        const int g = i / rows, r = i - g * rows;
+        *reinterpret_cast<uint4 *>(dst + ((size_t)pl * 16 * rows + i) * 16) = *reinterpret_cast<const uint4 *>(&s_tile[pl][g * kPrepChunkStride + r * 16]);
+      }
+    if (p.quantize && tid < grid_n4(rows)) {
+      p.scale[a][(size_t)slice * n4 + t0 + tid] = s_scale[tid];
+      p.zero[a][(size_t)slice * n4 + t0 + tid] = s_zero[tid];
+    }
+    __syncthreads();
+  }
+}
 
-  s_lam[tid] = alpha_index >= 0 ? powf(fmaxf(amax[(size_t)kv_head * kHeadDim + tid], floor_value), alphas[alpha_index]) : 1.0f;
+// ---- causal self-attention of the passes ------------------------------------------------------------------------
+// Grid: (sequences x query heads, alphas of the batch, query blocks from the longest to the shortest); a CTA takes 256
+// queries, two tiles of 128, against their Keys in tiles of 64.  Both contractions run on tcgen05.mma (fp16 in, fp32
+// accumulators in tensor memory): S[query, key] = Q K^T with both operands in shared memory, O[query, channel] += P V with P
+// in tensor memory, where it overwrites the scores it came from.  Warps:
+//   0-3, 4-7   one warpgroup per query tile, thread = query: builds the tile's Q operand (rotated, equalized, scaled by a power of
+//              two, split), then per key tile reads its 64 scores, takes probabilities against a running reference that
+//              only moves when a score exceeds it by more than 8 (log2 units; the thread then rescales its own row of O),
+//              and writes the weights back;
+//   8          issues all MMAs: scores of tile j + 1, then outputs of tile j, for one query tile after the other, so the softmax
+//              of one tile runs under the MMAs of the other three;
+//   9          the bulk copies of K, V, scales and zero-points, as far ahead as the rings have room.
+// Arithmetic.  The loss is a small difference of two attention outputs, so plain fp16 operands would drown it.  Queries and weights
+// are sums of two fp16 numbers (22 bits).  A quantized Key or Value is scale * code + zero per token, and the centred code
+// is one exact fp16 up to 8 bit, so q . k = scale_K (q . c) + zero_K sum(q) and sum p v = sum (p scale_V) c + sum p zero_V take
+// two products where values split in two (the unquantized pass, 16-bit codes) take three.  Scale and zero-point work is fp32.
+constexpr int kGridThreads = 320;
+constexpr int kGridQTile = 128, kGridQueries = 256;
+constexpr int kGridKSlots = 2, kGridVSlots = 3, kGridMetaSlots = 4;
+constexpr int kGridPlaneBytes = kGridTile * 256;   // one plane of a tile
+constexpr int kGridQBytes = kGridQTile * 256;      // one part (hi or lo) of a query tile's operand
+constexpr int kGridSmemQ = 0, kGridSmemK = kGridSmemQ + 4 * kGridQBytes, kGridSmemV = kGridSmemK + kGridKSlots * kGridPlaneBytes,
+              kGridSmemMeta = kGridSmemV + kGridVSlots * kGridPlaneBytes, kGridMetaBytes = 4 * kGridTile * 4,
+              kGridSmemBytes = kGridSmemMeta + kGridMetaSlots * kGridMetaBytes;
+constexpr int kGridTmemS = 0, kGridTmemO = 256;    // scores / weights [query tile][buffer] 64 columns each, outputs 128 columns each
+constexpr int kGridUnitLog2 = 6;                   // weights stay below 2^(6 + 8): fp16 with room
+constexpr float kGridMaxAhead = 8.0f;
+
+struct GridAttn {
+  const uint16_t *Q;       // bf16 [n_tokens][n_seq][kv_heads * group][128] before RoPE
+  const uint8_t *k[kGridMaxBatch], *v;
+  const float *k_scale[kGridMaxBatch], *k_zero[kGridMaxBatch], *v_scale, *v_zero;
+  const unsigned *vmax;    // per slice
+  const float *amax;
+  const float2 *table;
+  const float *alphas;     // those of this batch
+  float *o_ref;            // the unquantized outputs, [sequence x head][tile of 128 queries][32 groups of 4 channels][rows][4] fp32
+  double *loss_sums;       // those of this batch
+  unsigned *error_word;
+  int n_tokens, n_seq, kv_heads, group;
+  float floor_value;
+};
+
+struct GridShared {
+  unsigned long long k_full[kGridKSlots], k_free[kGridKSlots], v_full[kGridVSlots], v_free[kGridVSlots], m_full[kGridMetaSlots];
+  unsigned long long q_full[2], s_full[2][2], p_full[2][2], o_done[2];
+  uint32_t tmem_base;
+  int abort;
+  float lam[kHeadDim];
+};
+
+__device__ __forceinline__ void grid_wait(GridShared &sh, const unsigned long long *bar, uint32_t parity, unsigned *error_word) {
+  const uint32_t addr = tc05::smem_u32(bar);
+  if (tc05::mbar_test_wait(addr, parity & 1u)) return;
+  if (*reinterpret_cast<volatile int *>(&sh.abort)) return;
+  if (!tc05::mbar_wait(addr, parity & 1u)) {
+    sh.abort = 1;
+    atomicOr(error_word, 1u);
+  }
+}
+
+// PLANES: planes of K and V.  SCALED: quantized tensors with scales and zero-points, whose outputs are compared with o_ref;
+// otherwise the unquantized operator, whose outputs are kept there.
+template <int PLANES, bool SCALED>
+__global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const __grid_constant__ GridAttn p) {
+  extern __shared__ __align__(128) uint8_t smem[];
+  __shared__ GridShared sh;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int q_heads = p.kv_heads * p.group;
+  const int seq = (int)blockIdx.x / q_heads, q_head = (int)blockIdx.x - seq * q_heads, kv_head = q_head / p.group;
+  const int slice = seq * p.kv_heads + kv_head, batch = blockIdx.y;
+  const int q_block = ((int)gridDim.z - 1 - (int)blockIdx.z) * kGridQueries;  // long rows first
+  const int n = p.n_tokens, n4 = grid_n4(n);
+  int nt[2];  // key tiles of the two query tiles
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int first = q_block + q * kGridQTile;
+    nt[q] = first < n ? (min(n, first + kGridQTile) - 1) / kGridTile + 1 : 0;
+  }
+  const int n_kt = max(nt[0], nt[1]);
+  const bool ragged = n_kt * kGridTile > n;  // the last tile is the slice's short one
+
+  if (tid == 0) {
+    for (int i = 0; i < kGridKSlots; ++i) { tc05::mbar_init(tc05::smem_u32(&sh.k_full[i]), 1); tc05::mbar_init(tc05::smem_u32(&sh.k_free[i]), 1); }
+    for (int i = 0; i < kGridVSlots; ++i) { tc05::mbar_init(tc05::smem_u32(&sh.v_full[i]), 1); tc05::mbar_init(tc05::smem_u32(&sh.v_free[i]), 1); }
+    for (int i = 0; i < kGridMetaSlots; ++i) tc05::mbar_init(tc05::smem_u32(&sh.m_full[i]), 1);
+    for (int q = 0; q < 2; ++q) {
+      for (int b = 0; b < 2; ++b) { tc05::mbar_init(tc05::smem_u32(&sh.s_full[q][b]), 1); tc05::mbar_init(tc05::smem_u32(&sh.p_full[q][b]), 4); }
+      tc05::mbar_init(tc05::smem_u32(&sh.q_full[q]), 4);
+      tc05::mbar_init(tc05::smem_u32(&sh.o_done[q]), 1);
+    }
+    sh.abort = 0;
+    tc05::mbar_init_fence();
+  }
+  if (warp == 8) tc05::tmem_alloc(tc05::smem_u32(&sh.tmem_base), 512);
+  if (SCALED && tid < kHeadDim) sh.lam[tid] = powf(fmaxf(p.amax[(size_t)kv_head * kHeadDim + tid], p.floor_value), p.alphas[batch]);
+  if (ragged) {  // rows behind the last token stay as they are in the operands: they must be finite
+    for (int i = kGridSmemK + 16 * tid; i < kGridSmemBytes; i += 16 * kGridThreads) *reinterpret_cast<uint4 *>(smem + i) = make_uint4(0u, 0u, 0u, 0u);
+    tc05::fence_async_smem();
+  }
+  tc05::fence_before_sync();
   __syncthreads();
+  tc05::fence_after_sync();
+  const uint32_t tmem = sh.tmem_base;
+  const uint32_t s_base = tc05::smem_u32(smem);
+  auto wait = [&](const unsigned long long *bar, int phase) { grid_wait(sh, bar, (uint32_t)phase, p.error_word); };
 
-  // ---- the warp's queries as A fragments: rotated, equalized, pre-scaled, split; qh / ql[k-step][register] ----
-  // register 0: row g, channels 16 ks + 2 tig, + 1; 1: row g + 8; 2: row g, channels + 8; 3: row g + 8, channels + 8
-  uint32_t qh[8][4], ql[8][4];
+  if (warp == 9) {
+    // ---- copies ----
+    const uint8_t *k_src = p.k[batch] + (size_t)slice * n * (256 * PLANES), *v_src = p.v + (size_t)slice * n * (256 * PLANES);
+    auto tile_copy = [&](uint32_t dst, const uint8_t *src, int rows, const unsigned long long *bar) {
+      if (lane == 0) {
+        const uint32_t b = tc05::smem_u32(bar);
+        tc05::mbar_arrive_expect_tx(b, (uint32_t)rows * 256u);
+        if (rows == kGridTile) {
+          tc05::bulk_g2s(dst, src, kGridPlaneBytes, b);
+        } else {
+          for (int g = 0; g < 16; ++g) tc05::bulk_g2s(dst + g * (kGridTile * 16), src + (size_t)g * rows * 16, (uint32_t)rows * 16u, b);
+        }
+      }
+      __syncwarp();
+    };
+    for (int j = 0; j < n_kt; ++j) {
+      const int rows = min(kGridTile, n - j * kGridTile);
+      for (int pl = 0; pl < PLANES; ++pl) {
+        const int a = j * PLANES + pl, slot = a % kGridKSlots;
+        if (a >= kGridKSlots) wait(&sh.k_free[slot], a / kGridKSlots - 1);
+        tile_copy(s_base + kGridSmemK + slot * kGridPlaneBytes, k_src + ((size_t)j * kGridTile * PLANES + (size_t)pl * rows) * 256, rows, &sh.k_full[slot]);
+      }
+      if constexpr (SCALED) {
+        // slot j mod 4 was last read for tile j - 4, whose weights were all written before the scores of tile j - 2 that freed
+        // this tile's K slot could be issued
+        if (lane == 0) {
+          const uint32_t b = tc05::smem_u32(&sh.m_full[j % kGridMetaSlots]), bytes = (uint32_t)grid_n4(rows) * 4u;
+          const uint32_t dst = s_base + kGridSmemMeta + (j % kGridMetaSlots) * kGridMetaBytes;
+          const size_t at = (size_t)slice * n4 + (size_t)j * kGridTile;
+          tc05::mbar_arrive_expect_tx(b, 4u * bytes);
+          tc05::bulk_g2s(dst, p.k_scale[batch] + at, bytes, b);
+          tc05::bulk_g2s(dst + kGridTile * 4, p.k_zero[batch] + at, bytes, b);
+          tc05::bulk_g2s(dst + 2 * kGridTile * 4, p.v_scale + at, bytes, b);
+          tc05::bulk_g2s(dst + 3 * kGridTile * 4, p.v_zero + at, bytes, b);
+        }
+        __syncwarp();
+      }
+      for (int pl = 0; pl < PLANES; ++pl) {
+        const int a = j * PLANES + pl, slot = a % kGridVSlots;
+        if (a >= kGridVSlots) wait(&sh.v_free[slot], a / kGridVSlots - 1);
+        tile_copy(s_base + kGridSmemV + slot * kGridPlaneBytes, v_src + ((size_t)j * kGridTile * PLANES + (size_t)pl * rows) * 256, rows, &sh.v_full[slot]);
+      }
+    }
+  } else if (warp == 8) {
+    // ---- MMAs ----
+    constexpr uint32_t idesc_s = tc05::idesc_f16(128, kGridTile, 0), idesc_o = tc05::idesc_f16(128, kHeadDim, 1);
+    auto scores = [&](int q, int j) {
+      if (j >= nt[q]) return;
 #pragma unroll
-  for (int rr = 0; rr < 2; ++rr) {
-    const int qi = min(q0 + g + 8 * rr, n_tokens - 1);  // a dead row repeats the last query; its output is dropped
-    const uint16_t *src = Q + (((size_t)qi * n_seq + seq) * q_heads + q_head) * kHeadDim;
-    const float2 *tab = table + (size_t)qi * 64;
+      for (int pl = 0; pl < PLANES; ++pl) wait(&sh.k_full[(j * PLANES + pl) % kGridKSlots], (j * PLANES + pl) / kGridKSlots);
+      if (j >= 2) wait(&sh.o_done[q], j - 2);  // the output MMAs that read this buffer's weights are complete
+      if (j == 0) wait(&sh.q_full[q], 0);
+      __syncwarp();
+      tc05::fence_after_sync();
+      const uint32_t d = tmem + kGridTmemS + 64 * (2 * q + (j & 1));
+      const uint64_t qh = tc05::smem_desc(s_base + kGridSmemQ + 2 * q * kGridQBytes, kGridQTile * 16, 128);
+      const uint64_t ql = tc05::smem_desc(s_base + kGridSmemQ + (2 * q + 1) * kGridQBytes, kGridQTile * 16, 128);
 #pragma unroll
-    for (int ks = 0; ks < 4; ++ks)
+      for (int pl = 0; pl < PLANES; ++pl) {
+        const uint64_t kd = tc05::smem_desc(s_base + kGridSmemK + ((j * PLANES + pl) % kGridKSlots) * kGridPlaneBytes, kGridTile * 16, 128);
+        // 16 channels per MMA: two channel groups
 #pragma unroll
-      for (int c8 = 0; c8 < 2; ++c8) {
-        const int ch = 16 * ks + 8 * c8 + 2 * tig;  // channels ch, ch + 1 and their rotation partners + 64
-        const uint32_t r1 = *reinterpret_cast<const uint32_t *>(src + ch), r2 = *reinterpret_cast<const uint32_t *>(src + ch + 64);
-        float y1[2], y2[2];
+        for (int ks = 0; ks < 8; ++ks) tc05::mma_f16_ss_elect(d, qh + ks * (2 * kGridQTile), kd + ks * (2 * kGridTile), idesc_s, pl > 0 || ks > 0 ? 1u : 0u);
+        if (pl == 0) {
+#pragma unroll
+          for (int ks = 0; ks < 8; ++ks) tc05::mma_f16_ss_elect(d, ql + ks * (2 * kGridQTile), kd + ks * (2 * kGridTile), idesc_s, 1u);
+        }
+      }
+      tc05::mma_commit_elect(tc05::smem_u32(&sh.s_full[q][j & 1]));
+    };
+    auto outputs = [&](int q, int j) {
+      if (j >= nt[q]) return;
+#pragma unroll
+      for (int pl = 0; pl < PLANES; ++pl) wait(&sh.v_full[(j * PLANES + pl) % kGridVSlots], (j * PLANES + pl) / kGridVSlots);
+      wait(&sh.p_full[q][j & 1], j >> 1);
+      __syncwarp();
+      tc05::fence_after_sync();
+      const uint32_t d = tmem + kGridTmemO + 128 * q, w_hi = tmem + kGridTmemS + 64 * (2 * q + (j & 1)), w_lo = w_hi + 32;
+#pragma unroll
+      for (int pl = 0; pl < PLANES; ++pl) {
+        const uint64_t vd = tc05::smem_desc(s_base + kGridSmemV + ((j * PLANES + pl) % kGridVSlots) * kGridPlaneBytes, 128, kGridTile * 16);
+        // 16 keys per MMA: two rows of core matrices
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks) tc05::mma_f16_ts_elect(d, w_hi + 8 * ks, vd + ks * 16, idesc_o, j > 0 || pl > 0 || ks > 0 ? 1u : 0u);
+        if (pl == 0) {
+#pragma unroll
+          for (int ks = 0; ks < 4; ++ks) tc05::mma_f16_ts_elect(d, w_lo + 8 * ks, vd + ks * 16, idesc_o, 1u);
+        }
+      }
+      tc05::mma_commit_elect(tc05::smem_u32(&sh.o_done[q]));
+    };
+    // a slot is given back only if a later tile will use it: no arrival may be on its way when the CTA ends
+    auto free_k = [&](int j) {
+      for (int a = j * PLANES; a < (j + 1) * PLANES; ++a)
+        if (a + kGridKSlots < n_kt * PLANES) tc05::mma_commit_elect(tc05::smem_u32(&sh.k_free[a % kGridKSlots]));
+    };
+    auto free_v = [&](int j) {
+      for (int a = j * PLANES; a < (j + 1) * PLANES; ++a)
+        if (a + kGridVSlots < n_kt * PLANES) tc05::mma_commit_elect(tc05::smem_u32(&sh.v_free[a % kGridVSlots]));
+    };
+    scores(0, 0);
+    scores(1, 0);
+    free_k(0);
+    for (int j = 0; j < n_kt; ++j) {
+      scores(0, j + 1);
+      outputs(0, j);
+      scores(1, j + 1);
+      if (j + 1 < n_kt) free_k(j + 1);
+      outputs(1, j);
+      free_v(j);
+    }
+  } else if (nt[warp >> 2] > 0) {
+    // ---- a query tile ----
+    const int q = warp >> 2, row = tid & 127;
+    const int first_q = q_block + q * kGridQTile;
+    const int qi = min(first_q + row, n - 1);  // a dead row repeats the last query; its output is dropped
+    const bool alive = first_q + row < n;
+    const uint32_t t_lane = (uint32_t)((warp & 3) * 32) << 16;
+    const float scale_log2 = 1.4426950408889634f * rsqrtf((float)kHeadDim);
+    float sum_q = 0.f, f = 1.f;  // sum of the operand's elements; scores are f times the dot products
+    {
+      const uint16_t *src = p.Q + (((size_t)qi * p.n_seq + seq) * q_heads + q_head) * kHeadDim;
+      const float2 *tab = p.table + (size_t)qi * 64;
+      auto rotated = [&](int c, float (&y1)[2], float (&y2)[2]) {  // channels c, c + 1 and their partners
+        const uint32_t r1 = *reinterpret_cast<const uint32_t *>(src + c), r2 = *reinterpret_cast<const uint32_t *>(src + c + 64);
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-          const float x1 = __uint_as_float(e ? (r1 & 0xFFFF0000u) : (r1 << 16));
-          const float x2 = __uint_as_float(e ? (r2 & 0xFFFF0000u) : (r2 << 16));
-          const float2 cs = tab[ch + e];
-          y1[e] = __fsub_rn(__fmul_rn(x1, cs.x), __fmul_rn(x2, cs.y)) * s_lam[ch + e] * scale_log2;
-          y2[e] = __fadd_rn(__fmul_rn(x1, cs.y), __fmul_rn(x2, cs.x)) * s_lam[ch + e + 64] * scale_log2;
+          const float x1 = __uint_as_float(e ? (r1 & 0xFFFF0000u) : (r1 << 16)), x2 = __uint_as_float(e ? (r2 & 0xFFFF0000u) : (r2 << 16));
+          const float2 cs = tab[c + e];
+          const float l1 = SCALED ? sh.lam[c + e] : 1.0f, l2 = SCALED ? sh.lam[c + e + 64] : 1.0f;
+          y1[e] = __fsub_rn(__fmul_rn(x1, cs.x), __fmul_rn(x2, cs.y)) * l1 * scale_log2;
+          y2[e] = __fadd_rn(__fmul_rn(x1, cs.y), __fmul_rn(x2, cs.x)) * l2 * scale_log2;
         }
-        split_half2(y1[0], y1[1], qh[ks][2 * c8 + rr], ql[ks][2 * c8 + rr]);
-        split_half2(y2[0], y2[1], qh[ks + 4][2 * c8 + rr], ql[ks + 4][2 * c8 + rr]);
+      };
+      float mx = 0.f;
+#pragma unroll 8
+      for (int c = 0; c < 64; c += 2) {
+        float y1[2], y2[2];
+        rotated(c, y1, y2);
+        mx = fmaxf(fmaxf(fmaxf(mx, fabsf(y1[0])), fmaxf(fabsf(y1[1]), fabsf(y2[0]))), fabsf(y2[1]));
       }
-  }
-
-  float acc[16][4];          // O[16 queries][128]: n-block nb holds channels 8 nb + 2 tig, + 1 of rows g (0, 1) and g + 8 (2, 3)
-  float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};  // rows g, g + 8 (l: this thread's columns only)
+      const int shift = mx > 0.f ? max(-100, min(100, 136 - (int)(__float_as_uint(mx) >> 23))) : 0;  // largest element to [2^9, 2^10)
+      const float up = exp2i(shift);
+      f = exp2i(-shift);
+      uint8_t *q_op = smem + kGridSmemQ + 2 * q * kGridQBytes + row * 16;
+#pragma unroll 2
+      for (int g = 0; g < 8; ++g) {  // channel group g and its partner g + 8
+        uint32_t h1[4], l1[4], h2[4], l2[4];
 #pragma unroll
-  for (int nb = 0; nb < 16; ++nb) acc[nb][0] = acc[nb][1] = acc[nb][2] = acc[nb][3] = 0.f;
-  // ldmatrix row addresses of this lane inside a plane: lane = 8 mat + row
-  const int lm_row = lane & 7, lm_mat = lane >> 3;
-  const uint32_t k_lane_off = (uint32_t)((((lm_mat >> 1) * 8 + lm_row) * kGridRowBytes) + (lm_mat & 1) * 16);  // keys of two n-blocks, channels k0 / k0 + 8
-  const uint32_t v_lane_off = (uint32_t)((((lm_mat & 1) * 8 + lm_row) * kGridRowBytes) + (lm_mat >> 1) * 16);  // keys k0 / k0 + 8, channels of two n-blocks
-
-  for (int j = 0; j < n_tiles; ++j) {
-    __syncthreads();  // everyone is done with the stage that tile j + 1 will overwrite
-    if (j + 1 < n_tiles) issue(j + 1);
-    cp_async_commit();
-    cp_async_wait<1>();  // tile j has landed (this thread's pieces)
-    __syncthreads();     // ... and everyone else's
-    const int k0 = j * kGridKeys;
-    if (k0 > q0 + 15) continue;  // every key of the tile lies behind every query of this warp (the barriers above still run)
-    const uint32_t st = ring + (uint32_t)((j & 1) * kGridStageBytes);
-    // ---- S[16 queries][32 keys] = Q K^T ----
-    float sc[4][4];
-#pragma unroll
-    for (int nb = 0; nb < 4; ++nb) sc[nb][0] = sc[nb][1] = sc[nb][2] = sc[nb][3] = 0.f;
-#pragma unroll
-    for (int ks = 0; ks < 8; ++ks) {
-#pragma unroll
-      for (int np = 0; np < 2; ++np) {  // n-blocks 2 np, 2 np + 1
-        uint32_t bh[4], bl[4];
-        const uint32_t a = st + k_lane_off + (uint32_t)(np * 16 * kGridRowBytes + ks * 32);
-        ldsm_x4(a, bh);
-        ldsm_x4(a + kGridPlaneBytes, bl);
-        mma_f16(sc[2 * np], qh[ks], bh[0], bh[1]);
-        mma_f16(sc[2 * np], qh[ks], bl[0], bl[1]);
-        mma_f16(sc[2 * np], ql[ks], bh[0], bh[1]);
-        mma_f16(sc[2 * np + 1], qh[ks], bh[2], bh[3]);
-        mma_f16(sc[2 * np + 1], qh[ks], bl[2], bl[3]);
-        mma_f16(sc[2 * np + 1], ql[ks], bh[2], bh[3]);
+        for (int c = 0; c < 4; ++c) {
+          float y1[2], y2[2];
+          rotated(8 * g + 2 * c, y1, y2);
+          y1[0] *= up; y1[1] *= up; y2[0] *= up; y2[1] *= up;
+          sum_q += (y1[0] + y1[1]) + (y2[0] + y2[1]);
+          split_half2(y1[0], y1[1], h1[c], l1[c]);
+          split_half2(y2[0], y2[1], h2[c], l2[c]);
+        }
+        *reinterpret_cast<uint4 *>(q_op + g * (kGridQTile * 16)) = make_uint4(h1[0], h1[1], h1[2], h1[3]);
+        *reinterpret_cast<uint4 *>(q_op + kGridQBytes + g * (kGridQTile * 16)) = make_uint4(l1[0], l1[1], l1[2], l1[3]);
+        *reinterpret_cast<uint4 *>(q_op + (g + 8) * (kGridQTile * 16)) = make_uint4(h2[0], h2[1], h2[2], h2[3]);
+        *reinterpret_cast<uint4 *>(q_op + kGridQBytes + (g + 8) * (kGridQTile * 16)) = make_uint4(l2[0], l2[1], l2[2], l2[3]);
       }
+      tc05::fence_async_smem();
+      warp_arrive(&sh.q_full[q], lane);
     }
-    // ---- causal mask, running maximum, probabilities ----
-    const bool diagonal = k0 + kGridKeys - 1 > q0;  // some key of the tile may lie behind some query of the warp
+    // Probabilities are taken times 2^bias: with the weights' unit folded in, numerator and denominator share the factor.
+    float bias = (float)kGridUnitLog2;
+    if constexpr (SCALED) {
+      const unsigned vm = __ldg(p.vmax + slice);
+      if (vm) bias -= (float)max((int)(vm >> 23) - 126, -60);
+    }
+    float m = -INFINITY;      // reference; arguments of the exponential are f * t - m_b
+    float m_b = 0.f;          // m - bias
+    float2 l2 = make_float2(0.f, 0.f), z2 = make_float2(0.f, 0.f);
+    const uint32_t t_o = tmem + kGridTmemO + 128 * q + t_lane;
+    for (int j = 0; j < nt[q]; ++j) {
+      const uint32_t t_s = tmem + kGridTmemS + 64 * (2 * q + (j & 1)) + t_lane;
+      const float *meta = reinterpret_cast<const float *>(smem + kGridSmemMeta + (j % kGridMetaSlots) * kGridMetaBytes);
+      wait(&sh.s_full[q][j & 1], j >> 1);
+      if constexpr (SCALED) wait(&sh.m_full[j % kGridMetaSlots], j / kGridMetaSlots);
+      __syncwarp();
+      tc05::fence_after_sync();
+      float t[64];
+      {
+        uint32_t raw[64];
+        tc05::tmem_ld32(t_s, raw);
+        tc05::tmem_ld32(t_s + 32, raw + 32);
+        tc05::wait_ld();
+        const float2 sq2 = make_float2(sum_q, sum_q);
 #pragma unroll
-    for (int rr = 0; rr < 2; ++rr) {
-      const int qi = q0 + g + 8 * rr;
+        for (int k = 0; k < 64; k += 4) {
+          float2 d0 = make_float2(__uint_as_float(raw[k]), __uint_as_float(raw[k + 1]));
+          float2 d1 = make_float2(__uint_as_float(raw[k + 2]), __uint_as_float(raw[k + 3]));
+          if constexpr (SCALED) {
+            const float4 sk = *reinterpret_cast<const float4 *>(meta + k), zk = *reinterpret_cast<const float4 *>(meta + kGridTile + k);
+            d0 = __ffma2_rn(make_float2(sk.x, sk.y), d0, __fmul2_rn(make_float2(zk.x, zk.y), sq2));
+            d1 = __ffma2_rn(make_float2(sk.z, sk.w), d1, __fmul2_rn(make_float2(zk.z, zk.w), sq2));
+          }
+          t[k] = d0.x; t[k + 1] = d0.y; t[k + 2] = d1.x; t[k + 3] = d1.y;
+        }
+      }
+      if (j * kGridTile + kGridTile - 1 > first_q) {  // some key of the tile may lie behind some query of the tile
+#pragma unroll
+        for (int k = 0; k < 64; ++k)
+          if (j * kGridTile + k > qi) t[k] = -INFINITY;
+      }
       float mx = -INFINITY;
 #pragma unroll
-      for (int nb = 0; nb < 4; ++nb)
+      for (int k = 0; k < 64; k += 2) mx = fmaxf(mx, fmaxf(t[k], t[k + 1]));
+      mx *= f;
+      if (__any_sync(0xffffffffu, mx > m + kGridMaxAhead)) {
+        // key 0 is live for every query and sits in the first tile, so m is finite from the first tile on
+        const float m_new = fmaxf(m, mx);
+        const float corr = ex2_fast(m - m_new);  // 0 on the first tile
+        m = m_new;
+        m_b = m - bias;
+        l2 = __fmul2_rn(l2, make_float2(corr, corr));
+        z2 = __fmul2_rn(z2, make_float2(corr, corr));
+        if (j > 0) {  // this thread's row of the outputs, once all output MMAs issued so far are complete
+          wait(&sh.o_done[q], j - 1);
+          __syncwarp();
+          tc05::fence_after_sync();
+#pragma unroll 1
+          for (int c = 0; c < 128; c += 32) {
+            uint32_t o[32];
+            tc05::tmem_ld32(t_o + c, o);
+            tc05::wait_ld();
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          if (diagonal && k0 + 8 * nb + 2 * tig + e > qi) sc[nb][2 * rr + e] = -INFINITY;
-          mx = fmaxf(mx, sc[nb][2 * rr + e]);
-        }
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-      // key 0 is live for every query and sits in the first tile, so m is finite from the first tile on
-      const float m_new = fmaxf(m[rr], mx);
-      const float corr = ex2_fast(m[rr] - m_new);  // 0 on the first tile
-      m[rr] = m_new;
-      l[rr] *= corr;
-#pragma unroll
-      for (int nb = 0; nb < 16; ++nb) { acc[nb][2 * rr] *= corr; acc[nb][2 * rr + 1] *= corr; }
-#pragma unroll
-      for (int nb = 0; nb < 4; ++nb)
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const float pe = ex2_fast(sc[nb][2 * rr + e] - m_new);
-          sc[nb][2 * rr + e] = pe;
-          l[rr] += pe;
-        }
-    }
-    // ---- O += P V: the probability fragments of two key n-blocks are the A fragment of one k-step ----
-#pragma unroll
-    for (int ks = 0; ks < 2; ++ks) {
-      uint32_t ph[4], pl[4];
-      split_half2(sc[2 * ks][0], sc[2 * ks][1], ph[0], pl[0]);
-      split_half2(sc[2 * ks][2], sc[2 * ks][3], ph[1], pl[1]);
-      split_half2(sc[2 * ks + 1][0], sc[2 * ks + 1][1], ph[2], pl[2]);
-      split_half2(sc[2 * ks + 1][2], sc[2 * ks + 1][3], ph[3], pl[3]);
-#pragma unroll
-      for (int np = 0; np < 8; ++np) {  // channel n-blocks 2 np, 2 np + 1
-        uint32_t bh[4], bl[4];
-        const uint32_t a = st + 2 * kGridPlaneBytes + v_lane_off + (uint32_t)(ks * 16 * kGridRowBytes + np * 32);
-        ldsm_x4_trans(a, bh);
-        ldsm_x4_trans(a + kGridPlaneBytes, bl);
-        mma_f16(acc[2 * np], ph, bh[0], bh[1]);
-        mma_f16(acc[2 * np], ph, bl[0], bl[1]);
-        mma_f16(acc[2 * np], pl, bh[0], bh[1]);
-        mma_f16(acc[2 * np + 1], ph, bh[2], bh[3]);
-        mma_f16(acc[2 * np + 1], ph, bl[2], bl[3]);
-        mma_f16(acc[2 * np + 1], pl, bh[2], bh[3]);
-      }
-    }
-  }
-  cp_async_wait<0>();
-
-  // ---- the pass's output: keep it (the unquantized pass) or compare with the kept one ----
-  float err = 0.f;
-#pragma unroll
-  for (int rr = 0; rr < 2; ++rr) {
-    float ls = l[rr];
-    ls += __shfl_xor_sync(0xffffffffu, ls, 1);
-    ls += __shfl_xor_sync(0xffffffffu, ls, 2);
-    const int qi = q0 + g + 8 * rr;
-    if (qi < n_tokens) {
-      const float inv_l = __fdiv_rn(1.0f, ls);
-      float *kept = o_ref + (((size_t)qi * n_seq + seq) * q_heads + q_head) * kHeadDim + 2 * tig;
-#pragma unroll
-      for (int nb = 0; nb < 16; ++nb) {
-        float2 o = make_float2(acc[nb][2 * rr] * inv_l, acc[nb][2 * rr + 1] * inv_l);
-        if (alpha_index < 0) {
-          *reinterpret_cast<float2 *>(kept + 8 * nb) = o;
-        } else {
-          const float2 r = *reinterpret_cast<const float2 *>(kept + 8 * nb);
-          o.x -= r.x; o.y -= r.y;
-          err = fmaf(o.x, o.x, err); err = fmaf(o.y, o.y, err);
+            for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * corr);
+            tc05::tmem_st32(t_o + c, o);
+          }
+          tc05::wait_st();
         }
       }
+      uint32_t hi[32], lo[32];
+      const float2 f2 = make_float2(f, f), nm2 = make_float2(-m_b, -m_b);
+#pragma unroll
+      for (int k = 0; k < 64; k += 4) {
+        float4 sv = make_float4(0.f, 0.f, 0.f, 0.f), zv = sv;
+        if constexpr (SCALED) {
+          sv = *reinterpret_cast<const float4 *>(meta + 2 * kGridTile + k);
+          zv = *reinterpret_cast<const float4 *>(meta + 3 * kGridTile + k);
+        }
+#pragma unroll
+        for (int e = 0; e < 4; e += 2) {
+          const float2 arg = __ffma2_rn(f2, make_float2(t[k + e], t[k + e + 1]), nm2);
+          const float2 pr = make_float2(ex2_fast(arg.x), ex2_fast(arg.y));
+          l2 = __fadd2_rn(l2, pr);
+          float2 w = pr;
+          if constexpr (SCALED) {
+            z2 = __ffma2_rn(pr, e ? make_float2(zv.z, zv.w) : make_float2(zv.x, zv.y), z2);
+            w = __fmul2_rn(pr, e ? make_float2(sv.z, sv.w) : make_float2(sv.x, sv.y));
+          }
+          split_half2(w.x, w.y, hi[(k + e) / 2], lo[(k + e) / 2]);
+        }
+      }
+      tc05::tmem_st32(t_s, hi);
+      tc05::tmem_st32(t_s + 32, lo);
+      tc05::wait_st();
+      tc05::fence_before_sync();
+      warp_arrive(&sh.p_full[q][j & 1], lane);
+    }
+    // ---- the pass's output: keep it (the unquantized pass) or compare with the kept one ----
+    if (nt[q] > 1) wait(&sh.o_done[q], nt[q] - 2);  // a parity wait must not run two phases ahead
+    wait(&sh.o_done[q], nt[q] - 1);
+    __syncwarp();
+    tc05::fence_after_sync();
+    const int rows = min(kGridQTile, n - first_q);
+    float4 *kept = reinterpret_cast<float4 *>(p.o_ref) + (((size_t)seq * q_heads + q_head) * n + first_q) * (kHeadDim / 4) + row;
+    const float inv_l = __fdiv_rn(1.0f, l2.x + l2.y), zs = z2.x + z2.y;
+    float err = 0.f;
+#pragma unroll 1
+    for (int c = 0; c < 128; c += 32) {
+      uint32_t o[32];
+      tc05::tmem_ld32(t_o + c, o);
+      tc05::wait_ld();
+      if (alive) {
+#pragma unroll
+        for (int i = 0; i < 32; i += 4) {
+          float4 *at = kept + (size_t)((c + i) >> 2) * rows;
+          float4 v = make_float4((__uint_as_float(o[i]) + zs) * inv_l, (__uint_as_float(o[i + 1]) + zs) * inv_l,
+                                 (__uint_as_float(o[i + 2]) + zs) * inv_l, (__uint_as_float(o[i + 3]) + zs) * inv_l);
+          if constexpr (SCALED) {
+            const float4 r = *at;
+            v.x -= r.x; v.y -= r.y; v.z -= r.z; v.w -= r.w;
+            err = fmaf(v.x, v.x, err); err = fmaf(v.y, v.y, err); err = fmaf(v.z, v.z, err); err = fmaf(v.w, v.w, err);
+          } else {
+            *at = v;
+          }
+        }
+      }
+    }
+    if constexpr (SCALED) {
+      double e = (double)err;
+#pragma unroll
+      for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+      if (lane == 0) atomicAdd(p.loss_sums + batch, e);
     }
   }
-  if (alpha_index >= 0) {
-    double e = (double)err;
-#pragma unroll
-    for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-    if (lane == 0) atomicAdd(loss_sums + alpha_index, e);
+  tc05::fence_before_sync();
+  __syncthreads();
+  if (*reinterpret_cast<volatile int *>(&sh.abort)) {
+    // a wait gave up: copies and MMAs may still be in flight; give them about a millisecond (a bounded delay)
+    const long long c0 = clock64();
+    while (clock64() - c0 < 2000000ll) {}
+    __syncthreads();
   }
+  if (warp == 8) tc05::tmem_dealloc(tmem, 512);
 }
 
 }  // namespace pmkvq

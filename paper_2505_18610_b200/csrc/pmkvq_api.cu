@@ -847,10 +847,13 @@ pmkvq_status pmkvq_calibrate_lambda(const void *d_K, int32_t n_tokens, int32_t n
 
 static size_t grid_ws_round(size_t b) { return (b + 255) / 256 * 256; }
 
-// workspace of the alpha grid search: abs-max, rotation table, loss sums, alphas, then fp32 copies of this
-// pass's Keys, of the Values (as given and quantized) and the unquantized operator's output
+// Workspace of the alpha grid search: abs-max, rotation table, loss sums, alphas, the error word, three regions of 4 bytes
+// per Key element and the unquantized operator's output.  The unquantized pass keeps its Keys in region 0 and its Values
+// in region 1 (two fp16 planes each).  The quantized passes keep Values in region 2 and scales, zero-points and the slices'
+// largest Value scales in the upper half of region 1; their Keys take region 0 (16 bit), or, as one plane per alpha (codes
+// up to 8 bit), both halves of region 0, the upper half of region 2 and the lower half of region 1.
 struct GridWorkspace {
-  size_t amax, table, loss, alphas, k_pass, v_raw, v_hat, o_ref, total;
+  size_t amax, table, loss, alphas, error, region[3], o_ref, total;
 };
 static GridWorkspace grid_workspace(int64_t n_tokens, int64_t n_seq, int64_t kv_heads, int64_t group) {
   GridWorkspace w;
@@ -860,9 +863,8 @@ static GridWorkspace grid_workspace(int64_t n_tokens, int64_t n_seq, int64_t kv_
   w.table = off; off += grid_ws_round((size_t)n_tokens * 64 * sizeof(float2));
   w.loss = off; off += grid_ws_round(kMaxAlphas * sizeof(double));
   w.alphas = off; off += grid_ws_round(kMaxAlphas * sizeof(float));
-  w.k_pass = off; off += grid_ws_round(kv);
-  w.v_raw = off; off += grid_ws_round(kv);
-  w.v_hat = off; off += grid_ws_round(kv);
+  w.error = off; off += 256;
+  for (int r = 0; r < 3; ++r) { w.region[r] = off; off += grid_ws_round(kv); }
   w.o_ref = off; off += grid_ws_round(kv * (size_t)group);
   w.total = off;
   return w;
@@ -893,9 +895,10 @@ pmkvq_status pmkvq_alpha_grid_search(const void *d_K, const void *d_Q, const voi
   float2 *d_table = reinterpret_cast<float2 *>(ws + w.table);
   double *d_loss = reinterpret_cast<double *>(ws + w.loss);
   float *d_alphas = reinterpret_cast<float *>(ws + w.alphas);
-  float *d_k = reinterpret_cast<float *>(ws + w.k_pass), *d_v_raw = reinterpret_cast<float *>(ws + w.v_raw);
-  float *d_v_hat = reinterpret_cast<float *>(ws + w.v_hat), *d_o_ref = reinterpret_cast<float *>(ws + w.o_ref);
+  unsigned *d_error = reinterpret_cast<unsigned *>(ws + w.error);
+  float *d_o_ref = reinterpret_cast<float *>(ws + w.o_ref);
   if (cudaMemsetAsync(d_loss, 0, kMaxAlphas * sizeof(double), st) != cudaSuccess ||
+      cudaMemsetAsync(d_error, 0, sizeof(unsigned), st) != cudaSuccess ||
       cudaMemcpyAsync(d_alphas, h_alphas, (size_t)n_alphas * sizeof(float), cudaMemcpyHostToDevice, st) != cudaSuccess)
     return PMKVQ_ERR_CUDA;
   const uint16_t *K = static_cast<const uint16_t *>(d_K), *Q = static_cast<const uint16_t *>(d_Q),
@@ -903,25 +906,67 @@ pmkvq_status pmkvq_alpha_grid_search(const void *d_K, const void *d_Q, const voi
   if (launch_absmax(K, reinterpret_cast<unsigned *>(d_amax), n_tokens, n_seq, kv_heads, pos_scale, theta, st) != cudaSuccess)
     return PMKVQ_ERR_CUDA;
   rope_table_kernel<<<(unsigned)((n_tokens * 64 + 255) / 256), 256, 0, st>>>(d_table, n_tokens, pos_scale, theta);
-  if (cudaFuncSetAttribute(alpha_grid_attn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGridSmemBytes) != cudaSuccess)
-    return PMKVQ_ERR_CUDA;
-  const long long n_vectors = (long long)n_tokens * n_seq * kv_heads;
-  const unsigned prep_grid = (unsigned)((n_vectors + 3) / 4);
-  const dim3 grid((unsigned)((n_tokens + kGridQueries - 1) / kGridQueries), (unsigned)(kv_heads * group), (unsigned)n_seq);
-  // pass -1: the unquantized operator; passes 0 .. n_alphas - 1: Eq. 9 at each alpha
-  for (int pass = -1; pass < n_alphas; ++pass) {
-    float *v_out = pass == -1 ? d_v_raw : pass == 0 ? d_v_hat : nullptr;
-    alpha_grid_prep_kernel<<<prep_grid, 128, 0, st>>>(K, V, d_amax, d_table, d_alphas, pass, n_vectors, n_seq * kv_heads,
-                                                      kv_heads, bits, floor_value, d_k, v_out);
-    alpha_grid_attn_kernel<<<grid, 128, kGridSmemBytes, st>>>(Q, d_k, pass == -1 ? d_v_raw : d_v_hat, d_amax, d_table,
-                                                              d_alphas, pass, n_tokens, n_seq, kv_heads, group, floor_value,
-                                                              d_o_ref, d_loss);
+  const size_t slices = (size_t)n_seq * kv_heads, half = (size_t)n_tokens * slices * 256;  // half a region: one fp16 plane of all vectors
+  const size_t meta_bytes = slices * (size_t)grid_n4(n_tokens) * sizeof(float);
+  const int n_tiles = (n_tokens + kGridTile - 1) / kGridTile;
+  const int planes = bits <= 8 ? 1 : 2, per_batch = planes == 1 ? kGridMaxBatch : 1;
+  uint8_t *meta = ws + w.region[1] + half;
+  auto meta_array = [&](int i) { return reinterpret_cast<float *>(meta + (size_t)i * meta_bytes); };
+  unsigned *d_vmax = reinterpret_cast<unsigned *>(meta + (2 * kGridMaxBatch + 2) * meta_bytes);
+
+  GridPrep prep{};
+  prep.amax = d_amax; prep.table = d_table; prep.n_tokens = n_tokens; prep.n_seq = n_seq; prep.kv_heads = kv_heads;
+  prep.bits = bits; prep.floor_value = floor_value;
+  GridAttn attn{};
+  attn.Q = Q; attn.amax = d_amax; attn.table = d_table; attn.o_ref = d_o_ref; attn.error_word = d_error;
+  attn.n_tokens = n_tokens; attn.n_seq = n_seq; attn.kv_heads = kv_heads; attn.group = group; attn.floor_value = floor_value;
+  auto run_prep = [&](int pl) {
+    const unsigned grid = (unsigned)(slices * (size_t)n_tiles);
+    if (pl == 1) alpha_grid_prep_kernel<1><<<grid, 256, 0, st>>>(prep);
+    else alpha_grid_prep_kernel<2><<<grid, 256, 0, st>>>(prep);
+  };
+  auto run_attn = [&](auto kernel, int n_pass) {
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGridSmemBytes) != cudaSuccess) return;
+    const dim3 grid((unsigned)(n_seq * kv_heads * group), (unsigned)n_pass, (unsigned)((n_tokens + kGridQueries - 1) / kGridQueries));
+    kernel<<<grid, kGridThreads, kGridSmemBytes, st>>>(attn);
+  };
+  // the unquantized operator
+  prep.n_out = 1;
+  prep.src = K; prep.is_key = 1; prep.out[0] = ws + w.region[0];
+  run_prep(2);
+  prep.src = V; prep.is_key = 0; prep.out[0] = ws + w.region[1];
+  run_prep(2);
+  attn.k[0] = ws + w.region[0]; attn.v = ws + w.region[1];
+  run_attn(alpha_grid_attn_kernel<2, false>, 1);
+  // Eq. 9 at each alpha: the Values once, the Keys of up to four alphas at a time
+  if (cudaMemsetAsync(d_vmax, 0, slices * sizeof(unsigned), st) != cudaSuccess) return PMKVQ_ERR_CUDA;
+  prep.quantize = 1;
+  prep.out[0] = ws + w.region[2]; prep.scale[0] = meta_array(0); prep.zero[0] = meta_array(1); prep.vmax = d_vmax;
+  run_prep(planes);
+  attn.v = prep.out[0]; attn.v_scale = prep.scale[0]; attn.v_zero = prep.zero[0]; attn.vmax = d_vmax;
+  prep.src = K; prep.is_key = 1; prep.vmax = nullptr;
+  uint8_t *const buffers[kGridMaxBatch] = {ws + w.region[0], ws + w.region[0] + half, ws + w.region[2] + half, ws + w.region[1]};
+  for (int i = 0; i < kGridMaxBatch; ++i) {
+    attn.k[i] = prep.out[i] = buffers[i];
+    attn.k_scale[i] = prep.scale[i] = meta_array(2 + 2 * i);
+    attn.k_zero[i] = prep.zero[i] = meta_array(3 + 2 * i);
+  }
+  for (int first = 0; first < n_alphas; first += per_batch) {
+    prep.n_out = std::min(per_batch, n_alphas - first);
+    prep.alphas = attn.alphas = d_alphas + first;
+    attn.loss_sums = d_loss + first;
+    run_prep(planes);
+    if (planes == 1) run_attn(alpha_grid_attn_kernel<1, true>, prep.n_out);
+    else run_attn(alpha_grid_attn_kernel<2, true>, prep.n_out);
   }
   if (cudaGetLastError() != cudaSuccess) return PMKVQ_ERR_CUDA;
+  unsigned error = 0;
+  if (cudaMemcpyAsync(&error, d_error, sizeof(error), cudaMemcpyDeviceToHost, st) != cudaSuccess) return PMKVQ_ERR_CUDA;
   double sums[kMaxAlphas];
   if (cudaMemcpyAsync(sums, d_loss, (size_t)n_alphas * sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess)
     return PMKVQ_ERR_CUDA;
+  if (error) return PMKVQ_ERR_DEVICE_WAIT;
   const double count = (double)n_tokens * n_seq * kv_heads * group * kHeadDim;
   int best = 0;
   for (int i = 0; i < n_alphas; ++i) {
