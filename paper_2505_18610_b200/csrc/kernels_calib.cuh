@@ -533,46 +533,64 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
     const float scale_log2 = 1.4426950408889634f * rsqrtf((float)kHeadDim);
     float sum_q = 0.f, f = 1.f;  // sum of the operand's elements; scores are f times the dot products
     {
-      const uint16_t *src = p.Q + (((size_t)qi * p.n_seq + seq) * q_heads + q_head) * kHeadDim;
-      const float2 *tab = p.table + (size_t)qi * 64;
-      auto rotated = [&](int c, float (&y1)[2], float (&y2)[2]) {  // channels c, c + 1 and their partners
-        const uint32_t r1 = *reinterpret_cast<const uint32_t *>(src + c), r2 = *reinterpret_cast<const uint32_t *>(src + c + 64);
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const float x1 = __uint_as_float(e ? (r1 & 0xFFFF0000u) : (r1 << 16)), x2 = __uint_as_float(e ? (r2 & 0xFFFF0000u) : (r2 << 16));
-          const float2 cs = tab[c + e];
-          const float l1 = SCALED ? sh.lam[c + e] : 1.0f, l2 = SCALED ? sh.lam[c + e + 64] : 1.0f;
-          y1[e] = __fsub_rn(__fmul_rn(x1, cs.x), __fmul_rn(x2, cs.y)) * l1 * scale_log2;
-          y2[e] = __fadd_rn(__fmul_rn(x1, cs.y), __fmul_rn(x2, cs.x)) * l2 * scale_log2;
-        }
-      };
-      float mx = 0.f;
-#pragma unroll 8
-      for (int c = 0; c < 64; c += 2) {
-        float y1[2], y2[2];
-        rotated(c, y1, y2);
-        mx = fmaxf(fmaxf(fmaxf(mx, fabsf(y1[0])), fmaxf(fabsf(y1[1]), fabsf(y2[0]))), fabsf(y2[1]));
-      }
-      const int shift = mx > 0.f ? max(-100, min(100, 136 - (int)(__float_as_uint(mx) >> 23))) : 0;  // largest element to [2^9, 2^10)
-      const float up = exp2i(shift);
-      f = exp2i(-shift);
-      uint8_t *q_op = smem + kGridSmemQ + 2 * q * kGridQBytes + row * 16;
+      // Four rows at a time: eight lanes share a row, each with the channels of group cg and of its partner group cg + 8 (a row of
+      // 256 bytes is then read in whole lines; thread = row would touch 32 lines per load and took 60 000 cycles here).
+      const int cg = lane & 7;
+      const bool aligned = (reinterpret_cast<uintptr_t>(p.Q) & 15) == 0;
+      uint8_t *q_op = smem + kGridSmemQ + 2 * q * kGridQBytes + cg * (kGridQTile * 16);
 #pragma unroll 2
-      for (int g = 0; g < 8; ++g) {  // channel group g and its partner g + 8
-        uint32_t h1[4], l1[4], h2[4], l2[4];
+      for (int it = 0; it < 8; ++it) {
+        const int r = (warp & 3) * 32 + 4 * it + (lane >> 3), t = min(first_q + r, n - 1);
+        const uint16_t *src = p.Q + (((size_t)t * p.n_seq + seq) * q_heads + q_head) * kHeadDim + 8 * cg;
+        const float4 *tab = reinterpret_cast<const float4 *>(p.table + (size_t)t * 64 + 8 * cg);
+        uint32_t r1[4], r2[4];
+        if (aligned) {
+          const uint4 u1 = *reinterpret_cast<const uint4 *>(src), u2 = *reinterpret_cast<const uint4 *>(src + 64);
+          r1[0] = u1.x; r1[1] = u1.y; r1[2] = u1.z; r1[3] = u1.w;
+          r2[0] = u2.x; r2[1] = u2.y; r2[2] = u2.z; r2[3] = u2.w;
+        } else {
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            r1[c] = src[2 * c] | ((uint32_t)src[2 * c + 1] << 16);
+            r2[c] = src[64 + 2 * c] | ((uint32_t)src[64 + 2 * c + 1] << 16);
+          }
+        }
+        float y1[8], y2[8];
+        float mx = 0.f, sum = 0.f;
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-          float y1[2], y2[2];
-          rotated(8 * g + 2 * c, y1, y2);
-          y1[0] *= up; y1[1] *= up; y2[0] *= up; y2[1] *= up;
-          sum_q += (y1[0] + y1[1]) + (y2[0] + y2[1]);
-          split_half2(y1[0], y1[1], h1[c], l1[c]);
-          split_half2(y2[0], y2[1], h2[c], l2[c]);
+          const float4 cs = tab[c];  // (cos, sin) of channels 2 c, 2 c + 1 of the group
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const float x1 = __uint_as_float(e ? (r1[c] & 0xFFFF0000u) : (r1[c] << 16)), x2 = __uint_as_float(e ? (r2[c] & 0xFFFF0000u) : (r2[c] << 16));
+            const float co = e ? cs.z : cs.x, si = e ? cs.w : cs.y;
+            const float l1 = SCALED ? sh.lam[8 * cg + 2 * c + e] : 1.0f, l2 = SCALED ? sh.lam[8 * cg + 2 * c + e + 64] : 1.0f;
+            const float a1 = __fsub_rn(__fmul_rn(x1, co), __fmul_rn(x2, si)) * l1 * scale_log2;
+            const float a2 = __fadd_rn(__fmul_rn(x1, si), __fmul_rn(x2, co)) * l2 * scale_log2;
+            y1[2 * c + e] = a1; y2[2 * c + e] = a2;
+            mx = fmaxf(mx, fmaxf(fabsf(a1), fabsf(a2)));
+          }
         }
-        *reinterpret_cast<uint4 *>(q_op + g * (kGridQTile * 16)) = make_uint4(h1[0], h1[1], h1[2], h1[3]);
-        *reinterpret_cast<uint4 *>(q_op + kGridQBytes + g * (kGridQTile * 16)) = make_uint4(l1[0], l1[1], l1[2], l1[3]);
-        *reinterpret_cast<uint4 *>(q_op + (g + 8) * (kGridQTile * 16)) = make_uint4(h2[0], h2[1], h2[2], h2[3]);
-        *reinterpret_cast<uint4 *>(q_op + kGridQBytes + (g + 8) * (kGridQTile * 16)) = make_uint4(l2[0], l2[1], l2[2], l2[3]);
+#pragma unroll
+        for (int o = 1; o <= 4; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        const int shift = mx > 0.f ? max(-100, min(100, 136 - (int)(__float_as_uint(mx) >> 23))) : 0;  // largest element to [2^9, 2^10)
+        const float up = exp2i(shift);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) { y1[i] *= up; y2[i] *= up; sum += y1[i] + y2[i]; }
+#pragma unroll
+        for (int o = 1; o <= 4; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        uint32_t h[4], l[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) split_half2(y1[2 * c], y1[2 * c + 1], h[c], l[c]);
+        *reinterpret_cast<uint4 *>(q_op + r * 16) = make_uint4(h[0], h[1], h[2], h[3]);
+        *reinterpret_cast<uint4 *>(q_op + kGridQBytes + r * 16) = make_uint4(l[0], l[1], l[2], l[3]);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) split_half2(y2[2 * c], y2[2 * c + 1], h[c], l[c]);
+        *reinterpret_cast<uint4 *>(q_op + 8 * (kGridQTile * 16) + r * 16) = make_uint4(h[0], h[1], h[2], h[3]);
+        *reinterpret_cast<uint4 *>(q_op + kGridQBytes + 8 * (kGridQTile * 16) + r * 16) = make_uint4(l[0], l[1], l[2], l[3]);
+        // row L of the warp is lane L's from here on
+        const float s_row = __shfl_sync(0xffffffffu, sum, (lane & 3) * 8), f_row = __shfl_sync(0xffffffffu, exp2i(-shift), (lane & 3) * 8);
+        if ((lane >> 2) == it) { sum_q = s_row; f = f_row; }
       }
       tc05::fence_async_smem();
       warp_arrive(&sh.q_full[q], lane);
