@@ -314,14 +314,15 @@ __global__ void __launch_bounds__(256) alpha_grid_prep_kernel(const GridPrep p) 
 //              two, split), then per key tile reads its 64 scores, takes probabilities against a running reference that
 //              only moves when a score exceeds it by more than 8 (log2 units; the thread then rescales its own row of O),
 //              and writes the weights back;
-//   8          issues all MMAs: scores of tile j + 1, then outputs of tile j, for one query tile after the other, so the softmax
-//              of one tile runs under the MMAs of the other three;
-//   9          the bulk copies of K, V, scales and zero-points, as far ahead as the rings have room.
+//   8, 9       one per query tile, issue its MMAs: scores of key tile j + 1, then outputs of key tile j, so the softmax of one tile
+//              runs under the MMAs of the others.  (A satisfied barrier wait costs a warp about 150 cycles and a batch of MMAs waits
+//              for two or three: one warp for both tiles took 4500 cycles per key tile, the MMAs take 2600.)
+//   10         the bulk copies of K, V, scales and zero-points, as far ahead as the rings have room.
 // Arithmetic.  The loss is a small difference of two attention outputs, so plain fp16 operands would drown it.  Queries and weights
 // are sums of two fp16 numbers (22 bits).  A quantized Key or Value is scale * code + zero per token, and the centred code
 // is one exact fp16 up to 8 bit, so q . k = scale_K (q . c) + zero_K sum(q) and sum p v = sum (p scale_V) c + sum p zero_V take
 // two products where values split in two (the unquantized pass, 16-bit codes) take three.  Scale and zero-point work is fp32.
-constexpr int kGridThreads = 320;
+constexpr int kGridThreads = 352;
 constexpr int kGridQTile = 128, kGridQueries = 256;
 constexpr int kGridKSlots = 2, kGridVSlots = 3, kGridMetaSlots = 4;
 constexpr int kGridPlaneBytes = kGridTile * 256;   // one plane of a tile
@@ -388,8 +389,9 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
   const bool ragged = n_kt * kGridTile > n;  // the last tile is the slice's short one
 
   if (tid == 0) {
-    for (int i = 0; i < kGridKSlots; ++i) { tc05::mbar_init(tc05::smem_u32(&sh.k_full[i]), 1); tc05::mbar_init(tc05::smem_u32(&sh.k_free[i]), 1); }
-    for (int i = 0; i < kGridVSlots; ++i) { tc05::mbar_init(tc05::smem_u32(&sh.v_full[i]), 1); tc05::mbar_init(tc05::smem_u32(&sh.v_free[i]), 1); }
+    const uint32_t users = nt[1] > 0 ? 2 : 1;  // query tiles whose MMAs read a slot
+    for (int i = 0; i < kGridKSlots; ++i) { tc05::mbar_init(tc05::smem_u32(&sh.k_full[i]), 1); tc05::mbar_init(tc05::smem_u32(&sh.k_free[i]), users); }
+    for (int i = 0; i < kGridVSlots; ++i) { tc05::mbar_init(tc05::smem_u32(&sh.v_full[i]), 1); tc05::mbar_init(tc05::smem_u32(&sh.v_free[i]), users); }
     for (int i = 0; i < kGridMetaSlots; ++i) tc05::mbar_init(tc05::smem_u32(&sh.m_full[i]), 1);
     for (int q = 0; q < 2; ++q) {
       for (int b = 0; b < 2; ++b) { tc05::mbar_init(tc05::smem_u32(&sh.s_full[q][b]), 1); tc05::mbar_init(tc05::smem_u32(&sh.p_full[q][b]), 4); }
@@ -412,7 +414,7 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
   const uint32_t s_base = tc05::smem_u32(smem);
   auto wait = [&](const unsigned long long *bar, int phase) { grid_wait(sh, bar, (uint32_t)phase, p.error_word); };
 
-  if (warp == 9) {
+  if (warp == 10) {
     // ---- copies ----
     const uint8_t *k_src = p.k[batch] + (size_t)slice * n * (256 * PLANES), *v_src = p.v + (size_t)slice * n * (256 * PLANES);
     auto tile_copy = [&](uint32_t dst, const uint8_t *src, int rows, const unsigned long long *bar) {
@@ -436,7 +438,7 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
       }
       if constexpr (SCALED) {
         // slot j mod 4 was last read for tile j - 4, whose weights were all written before the scores of tile j - 2 that freed
-        // this tile's K slot could be issued
+        // this tile's K slot could be issued (a query tile without a tile j - 2 has no tile j - 4 to be read late either)
         if (lane == 0) {
           const uint32_t b = tc05::smem_u32(&sh.m_full[j % kGridMetaSlots]), bytes = (uint32_t)grid_n4(rows) * 4u;
           const uint32_t dst = s_base + kGridSmemMeta + (j % kGridMetaSlots) * kGridMetaBytes;
@@ -455,11 +457,13 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
         tile_copy(s_base + kGridSmemV + slot * kGridPlaneBytes, v_src + ((size_t)j * kGridTile * PLANES + (size_t)pl * rows) * 256, rows, &sh.v_full[slot]);
       }
     }
-  } else if (warp == 8) {
-    // ---- MMAs ----
+  } else if (warp >= 8) {
+    // ---- MMAs of query tile q ----
+    const int q = warp - 8, n_mine = nt[q];
     constexpr uint32_t idesc_s = tc05::idesc_f16(128, kGridTile, 0), idesc_o = tc05::idesc_f16(128, kHeadDim, 1);
-    auto scores = [&](int q, int j) {
-      if (j >= nt[q]) return;
+    const uint64_t qh = tc05::smem_desc(s_base + kGridSmemQ + 2 * q * kGridQBytes, kGridQTile * 16, 128);
+    const uint64_t ql = tc05::smem_desc(s_base + kGridSmemQ + (2 * q + 1) * kGridQBytes, kGridQTile * 16, 128);
+    auto scores = [&](int j) {
 #pragma unroll
       for (int pl = 0; pl < PLANES; ++pl) wait(&sh.k_full[(j * PLANES + pl) % kGridKSlots], (j * PLANES + pl) / kGridKSlots);
       if (j >= 2) wait(&sh.o_done[q], j - 2);  // the output MMAs that read this buffer's weights are complete
@@ -467,8 +471,6 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
       __syncwarp();
       tc05::fence_after_sync();
       const uint32_t d = tmem + kGridTmemS + 64 * (2 * q + (j & 1));
-      const uint64_t qh = tc05::smem_desc(s_base + kGridSmemQ + 2 * q * kGridQBytes, kGridQTile * 16, 128);
-      const uint64_t ql = tc05::smem_desc(s_base + kGridSmemQ + (2 * q + 1) * kGridQBytes, kGridQTile * 16, 128);
 #pragma unroll
       for (int pl = 0; pl < PLANES; ++pl) {
         const uint64_t kd = tc05::smem_desc(s_base + kGridSmemK + ((j * PLANES + pl) % kGridKSlots) * kGridPlaneBytes, kGridTile * 16, 128);
@@ -481,9 +483,14 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
         }
       }
       tc05::mma_commit_elect(tc05::smem_u32(&sh.s_full[q][j & 1]));
+      // a slot is given back only if a later tile will use it: no arrival may be on its way when the CTA ends
+#pragma unroll
+      for (int pl = 0; pl < PLANES; ++pl) {
+        const int a = j * PLANES + pl;
+        if (a + kGridKSlots < n_kt * PLANES) tc05::mma_commit_elect(tc05::smem_u32(&sh.k_free[a % kGridKSlots]));
+      }
     };
-    auto outputs = [&](int q, int j) {
-      if (j >= nt[q]) return;
+    auto outputs = [&](int j) {
 #pragma unroll
       for (int pl = 0; pl < PLANES; ++pl) wait(&sh.v_full[(j * PLANES + pl) % kGridVSlots], (j * PLANES + pl) / kGridVSlots);
       wait(&sh.p_full[q][j & 1], j >> 1);
@@ -502,26 +509,29 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
         }
       }
       tc05::mma_commit_elect(tc05::smem_u32(&sh.o_done[q]));
-    };
-    // a slot is given back only if a later tile will use it: no arrival may be on its way when the CTA ends
-    auto free_k = [&](int j) {
-      for (int a = j * PLANES; a < (j + 1) * PLANES; ++a)
-        if (a + kGridKSlots < n_kt * PLANES) tc05::mma_commit_elect(tc05::smem_u32(&sh.k_free[a % kGridKSlots]));
-    };
-    auto free_v = [&](int j) {
-      for (int a = j * PLANES; a < (j + 1) * PLANES; ++a)
+#pragma unroll
+      for (int pl = 0; pl < PLANES; ++pl) {
+        const int a = j * PLANES + pl;
         if (a + kGridVSlots < n_kt * PLANES) tc05::mma_commit_elect(tc05::smem_u32(&sh.v_free[a % kGridVSlots]));
+      }
     };
-    scores(0, 0);
-    scores(1, 0);
-    free_k(0);
-    for (int j = 0; j < n_kt; ++j) {
-      scores(0, j + 1);
-      outputs(0, j);
-      scores(1, j + 1);
-      if (j + 1 < n_kt) free_k(j + 1);
-      outputs(1, j);
-      free_v(j);
+    if (n_mine > 0) scores(0);
+    for (int j = 0; j < n_mine; ++j) {
+      if (j + 1 < n_mine) scores(j + 1);
+      outputs(j);
+    }
+    // The key tiles that only the second query tile uses: nothing of this warp reads them.  It gives a slot back once the tile is
+    // there (the slot's earlier uses are then all over, so no arrival is counted for the wrong use).
+    for (int a = n_mine * PLANES; n_mine > 0 && a < n_kt * PLANES; ++a) {
+      if (a + kGridKSlots < n_kt * PLANES) {
+        wait(&sh.k_full[a % kGridKSlots], a / kGridKSlots);
+        if (lane == 0) tc05::mbar_arrive(tc05::smem_u32(&sh.k_free[a % kGridKSlots]));
+      }
+      if (a + kGridVSlots < n_kt * PLANES) {
+        wait(&sh.v_full[a % kGridVSlots], a / kGridVSlots);
+        if (lane == 0) tc05::mbar_arrive(tc05::smem_u32(&sh.v_free[a % kGridVSlots]));
+      }
+      __syncwarp();
     }
   } else if (nt[warp >> 2] > 0) {
     // ---- a query tile ----
