@@ -143,14 +143,18 @@ __global__ void calib_finish_kernel(float *lambda, int n, float floor_value, flo
 // interpolated RoPE of Eq. 12 from a (cos, sin) table.
 // ---------------------------------------------------------------------------------------------
 
-// table[t][pair] = (cos, sin) of pos_scale * t * theta^(-2 pair / 128), rounded from fp64.
-__global__ void rope_table_kernel(float2 *table, int n_tokens, double pos_scale, double theta) {
+// cos and sin of pos_scale * t * theta^(-2 pair / 128), rounded from fp64: table[t][pair / 2] = (cos of the even pair, cos of the
+// odd one, sin of the even pair, sin of the odd one), so that packed fp32 instructions find adjacent channels in adjacent
+// registers.
+__global__ void rope_table_kernel(float *table, int n_tokens, double pos_scale, double theta) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n_tokens * 64) return;
   const int t = i >> 6, pair = i & 63;
   double s, c;
   sincos((double)t * pos_scale * pow(theta, -2.0 * pair / (double)kHeadDim), &s, &c);
-  table[i] = make_float2((float)c, (float)s);
+  float *at = table + (size_t)t * 128 + (pair >> 1) * 4 + (pair & 1);
+  at[0] = (float)c;
+  at[2] = (float)s;
 }
 
 constexpr int kMaxAlphas = 64;
@@ -171,15 +175,14 @@ __device__ __forceinline__ void split_half2(float x, float y, uint32_t &hi, uint
 
 // One token's 4 channels per lane (channels 4 lane .. 4 lane + 3): rotate by the token's angles.  The
 // partner channel (+-64) sits in lane ^ 16.
-__device__ __forceinline__ void rotate_token(float (&x)[4], const float2 *__restrict__ table_t, int lane) {
-  const int pair0 = (lane & 15) * 4;
+__device__ __forceinline__ void rotate_token(float (&x)[4], const float4 *__restrict__ table_t, int lane) {
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    const float other = __shfl_xor_sync(0xffffffffu, x[e], 16);
-    const float2 cs = table_t[pair0 + e];
+  for (int e = 0; e < 4; e += 2) {
+    const float4 cs = table_t[(lane & 15) * 2 + (e >> 1)];
+    const float o0 = __shfl_xor_sync(0xffffffffu, x[e], 16), o1 = __shfl_xor_sync(0xffffffffu, x[e + 1], 16);
     // lanes 0..15 hold x1 (channel < 64): y1 = x1 c - x2 s;  lanes 16..31 hold x2: y2 = x1 s + x2 c
-    x[e] = lane < 16 ? __fsub_rn(__fmul_rn(x[e], cs.x), __fmul_rn(other, cs.y))
-                     : __fadd_rn(__fmul_rn(other, cs.y), __fmul_rn(x[e], cs.x));
+    x[e] = lane < 16 ? __fsub_rn(__fmul_rn(x[e], cs.x), __fmul_rn(o0, cs.z)) : __fadd_rn(__fmul_rn(o0, cs.z), __fmul_rn(x[e], cs.x));
+    x[e + 1] = lane < 16 ? __fsub_rn(__fmul_rn(x[e + 1], cs.y), __fmul_rn(o1, cs.w)) : __fadd_rn(__fmul_rn(o1, cs.w), __fmul_rn(x[e + 1], cs.y));
   }
 }
 
@@ -198,11 +201,14 @@ __device__ __forceinline__ void quantize_token_centred(float (&x)[4], int bits, 
   const bool plain = s16 >= 0x1p-60f && s16 <= 0x1p60f;  // else: constant token (0 / 0 converts to code 0) or absurd range
   const float y = plain ? __frcp_rn(s16) : 0.f;
   const float half = 0.5f * (float)((1 << bits) - 1);
+  // the chain as one fused multiply-add (see chain_code; 1 / 1 at 16 bit), everything in whole floats
+  const float inv = bits == 2 ? inv_chain_divisor<2>() : bits == 4 ? inv_chain_divisor<4>() : bits == 8 ? inv_chain_divisor<8>() : 1.0f;
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
     const float d = __fsub_rn(x[e], mn);
-    const int c = plain ? code_of_quotient(quotient_rn(d, s16, y)) : min(max(__float2int_rn(__fdiv_rn(d, s16)), 0), 65535);
-    x[e] = (float)shift_chain((uint32_t)c, bits) - half;
+    const float c16 = plain ? __fadd_rn(__fadd_rn(quotient_rn(d, s16, y), 8388608.0f), -8388608.0f)
+                            : (float)min(max(__float2int_rn(__fdiv_rn(d, s16)), 0), 65535);
+    x[e] = __fadd_rn(__fadd_rn(__fmaf_rn(c16, inv, 8388608.0f), -8388608.0f), -half);
   }
   scale = chain_scale(s16, bits);
   zero = fmaf(scale, half, mn);
@@ -230,18 +236,18 @@ __host__ __device__ constexpr int grid_n4(int n_tokens) { return (n_tokens + 3) 
 struct GridPrep {
   const uint16_t *src;     // K or V, bf16 [n_tokens][n_seq][kv_heads][128]
   const float *amax;       // [kv_heads][128]
-  const float2 *table;     // [n_tokens][64]
+  const float4 *table;     // [n_tokens][32]
   const float *alphas;     // those of this batch
   uint8_t *out[kGridMaxBatch];
   float *scale[kGridMaxBatch], *zero[kGridMaxBatch];
   unsigned *vmax;          // per slice, the largest scale (Values)
-  int n_out;               // buffers to fill (alphas of the batch; 1 for Values and for plain Keys)
   int is_key, quantize;    // rotate (and, quantized, equalize); quantize or keep plain
   int n_tokens, n_seq, kv_heads, bits;
   float floor_value;
 };
-// One CTA per (slice, tile): the tile's vectors are read (and rotated) once, a warp on eight of them, and every alpha's
-// version leaves through shared memory as whole 16-byte pieces.
+// One CTA per (slice, tile) and alpha, a warp on eight vectors; they leave through shared memory as whole 16-byte pieces.  (One
+// CTA for the four alphas of a batch reads its Keys once, but the latency of four rounds showed: 38 us per batch of
+// 2048 x 2 x 4 vectors.)
 constexpr int kPrepChunkStride = kGridTile * 16 + 16;  // padded: the 16 channel groups a warp writes fall into different banks
 template <int PLANES>
 __global__ void __launch_bounds__(256) alpha_grid_prep_kernel(const GridPrep p) {
@@ -260,48 +266,48 @@ __global__ void __launch_bounds__(256) alpha_grid_prep_kernel(const GridPrep p) 
   }
   if (p.is_key) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) rotate_token(x0[i], p.table + (size_t)(t0 + min(warp + 8 * i, rows - 1)) * 64, lane);
+    for (int i = 0; i < 8; ++i) rotate_token(x0[i], p.table + (size_t)(t0 + min(warp + 8 * i, rows - 1)) * 32, lane);
   }
-  for (int a = 0; a < p.n_out; ++a) {
-    if (p.is_key && p.quantize && tid < kHeadDim)
+  const int a = blockIdx.y;
+  if (p.is_key && p.quantize) {
+    if (tid < kHeadDim)
       s_inv[tid] = __fdiv_rn(1.0f, powf(fmaxf(p.amax[(size_t)(slice % p.kv_heads) * kHeadDim + tid], p.floor_value), p.alphas[a]));
     __syncthreads();
-    float smax = 0.f;
+  }
+  float smax = 0.f;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int row = warp + 8 * i;
-      float x[4] = {x0[i][0], x0[i][1], x0[i][2], x0[i][3]};
-      if (p.quantize) {
-        if (p.is_key) {
-          const float4 il = *reinterpret_cast<const float4 *>(s_inv + 4 * lane);
-          x[0] = __fmul_rn(x[0], il.x); x[1] = __fmul_rn(x[1], il.y); x[2] = __fmul_rn(x[2], il.z); x[3] = __fmul_rn(x[3], il.w);
-        }
-        float scale, zero;
-        quantize_token_centred(x, p.bits, scale, zero);
-        smax = fmaxf(smax, scale);
-        if (lane == 0) { s_scale[row] = row < rows ? scale : 0.f; s_zero[row] = row < rows ? zero : 0.f; }
+  for (int i = 0; i < 8; ++i) {
+    const int row = warp + 8 * i;
+    float (&x)[4] = x0[i];
+    if (p.quantize) {
+      if (p.is_key) {
+        const float4 il = *reinterpret_cast<const float4 *>(s_inv + 4 * lane);
+        x[0] = __fmul_rn(x[0], il.x); x[1] = __fmul_rn(x[1], il.y); x[2] = __fmul_rn(x[2], il.z); x[3] = __fmul_rn(x[3], il.w);
       }
-      uint2 hi, lo;
-      split_half2(x[0], x[1], hi.x, lo.x);
-      split_half2(x[2], x[3], hi.y, lo.y);
-      const int at = (lane >> 1) * kPrepChunkStride + row * 16 + (lane & 1) * 8;
-      *reinterpret_cast<uint2 *>(&s_tile[0][at]) = hi;
-      if constexpr (PLANES == 2) *reinterpret_cast<uint2 *>(&s_tile[1][at]) = lo;
+      float scale, zero;
+      quantize_token_centred(x, p.bits, scale, zero);
+      smax = fmaxf(smax, scale);
+      if (lane == 0) { s_scale[row] = row < rows ? scale : 0.f; s_zero[row] = row < rows ? zero : 0.f; }
     }
-    if (p.vmax && lane == 0) atomicMax(p.vmax + slice, __float_as_uint(smax));  // scale >= 0: uint order = float order
-    __syncthreads();
-    uint8_t *dst = p.out[a] + ((size_t)slice * p.n_tokens + t0) * (size_t)(256 * PLANES);
+    uint2 hi, lo;
+    split_half2(x[0], x[1], hi.x, lo.x);
+    split_half2(x[2], x[3], hi.y, lo.y);
+    const int at = (lane >> 1) * kPrepChunkStride + row * 16 + (lane & 1) * 8;
+    *reinterpret_cast<uint2 *>(&s_tile[0][at]) = hi;
+    if constexpr (PLANES == 2) *reinterpret_cast<uint2 *>(&s_tile[1][at]) = lo;
+  }
+  if (p.vmax && lane == 0) atomicMax(p.vmax + slice, __float_as_uint(smax));  // scale >= 0: uint order = float order
+  __syncthreads();
+  uint8_t *dst = p.out[a] + ((size_t)slice * p.n_tokens + t0) * (size_t)(256 * PLANES);
 #pragma unroll
-    for (int pl = 0; pl < PLANES; ++pl)
-      for (int i = tid; i < 16 * rows; i += 256) {
-        const int g = i / rows, r = i - g * rows;
-        *reinterpret_cast<uint4 *>(dst + ((size_t)pl * 16 * rows + i) * 16) = *reinterpret_cast<const uint4 *>(&s_tile[pl][g * kPrepChunkStride + r * 16]);
-      }
-    if (p.quantize && tid < grid_n4(rows)) {
-      p.scale[a][(size_t)slice * n4 + t0 + tid] = s_scale[tid];
-      p.zero[a][(size_t)slice * n4 + t0 + tid] = s_zero[tid];
+  for (int pl = 0; pl < PLANES; ++pl)
+    for (int i = tid; i < 16 * rows; i += 256) {
+      const int g = i / rows, r = i - g * rows;
+      *reinterpret_cast<uint4 *>(dst + ((size_t)pl * 16 * rows + i) * 16) = *reinterpret_cast<const uint4 *>(&s_tile[pl][g * kPrepChunkStride + r * 16]);
     }
-    __syncthreads();
+  if (p.quantize && tid < grid_n4(rows)) {
+    p.scale[a][(size_t)slice * n4 + t0 + tid] = s_scale[tid];
+    p.zero[a][(size_t)slice * n4 + t0 + tid] = s_zero[tid];
   }
 }
 
@@ -340,7 +346,7 @@ struct GridAttn {
   const float *k_scale[kGridMaxBatch], *k_zero[kGridMaxBatch], *v_scale, *v_zero;
   const unsigned *vmax;    // per slice
   const float *amax;
-  const float2 *table;
+  const float4 *table;
   const float *alphas;     // those of this batch
   float *o_ref;            // the unquantized outputs, [sequence x head][tile of 128 queries][32 groups of 4 channels][rows][4] fp32
   double *loss_sums;       // those of this batch
@@ -351,10 +357,10 @@ struct GridAttn {
 
 struct GridShared {
   unsigned long long k_full[kGridKSlots], k_free[kGridKSlots], v_full[kGridVSlots], v_free[kGridVSlots], m_full[kGridMetaSlots];
-  unsigned long long q_full[2], s_full[2][2], p_full[2][2], o_done[2];
+  unsigned long long q_full[2], s_full[2][2], p_full[2][2], o_done[2], o_last[2];
   uint32_t tmem_base;
   int abort;
-  float lam[kHeadDim];
+  __align__(16) float lam[kHeadDim];
 };
 
 __device__ __forceinline__ void grid_wait(GridShared &sh, const unsigned long long *bar, uint32_t parity, unsigned *error_word) {
@@ -397,12 +403,16 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
       for (int b = 0; b < 2; ++b) { tc05::mbar_init(tc05::smem_u32(&sh.s_full[q][b]), 1); tc05::mbar_init(tc05::smem_u32(&sh.p_full[q][b]), 4); }
       tc05::mbar_init(tc05::smem_u32(&sh.q_full[q]), 4);
       tc05::mbar_init(tc05::smem_u32(&sh.o_done[q]), 1);
+      tc05::mbar_init(tc05::smem_u32(&sh.o_last[q]), 1);
     }
     sh.abort = 0;
     tc05::mbar_init_fence();
   }
   if (warp == 8) tc05::tmem_alloc(tc05::smem_u32(&sh.tmem_base), 512);
-  if (SCALED && tid < kHeadDim) sh.lam[tid] = powf(fmaxf(p.amax[(size_t)kv_head * kHeadDim + tid], p.floor_value), p.alphas[batch]);
+  if (tid < kHeadDim) {  // what the rotated queries are multiplied by: lambda and the softmax scale in log2 units
+    const float scale_log2 = 1.4426950408889634f * rsqrtf((float)kHeadDim);
+    sh.lam[tid] = SCALED ? powf(fmaxf(p.amax[(size_t)kv_head * kHeadDim + tid], p.floor_value), p.alphas[batch]) * scale_log2 : scale_log2;
+  }
   if (ragged) {  // rows behind the last token stay as they are in the operands: they must be finite
     for (int i = kGridSmemK + 16 * tid; i < kGridSmemBytes; i += 16 * kGridThreads) *reinterpret_cast<uint4 *>(smem + i) = make_uint4(0u, 0u, 0u, 0u);
     tc05::fence_async_smem();
@@ -509,6 +519,8 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
         }
       }
       tc05::mma_commit_elect(tc05::smem_u32(&sh.o_done[q]));
+      // a barrier of its own for the end: a parity wait on o_done there could be two phases off in either direction
+      if (j + 1 == n_mine) tc05::mma_commit_elect(tc05::smem_u32(&sh.o_last[q]));
 #pragma unroll
       for (int pl = 0; pl < PLANES; ++pl) {
         const int a = j * PLANES + pl;
@@ -540,7 +552,6 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
     const int qi = min(first_q + row, n - 1);  // a dead row repeats the last query; its output is dropped
     const bool alive = first_q + row < n;
     const uint32_t t_lane = (uint32_t)((warp & 3) * 32) << 16;
-    const float scale_log2 = 1.4426950408889634f * rsqrtf((float)kHeadDim);
     float sum_q = 0.f, f = 1.f;  // sum of the operand's elements; scores are f times the dot products
     {
       // Four rows at a time: eight lanes share a row, each with the channels of group cg and of its partner group cg + 8 (a row of
@@ -552,7 +563,7 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
       for (int it = 0; it < 8; ++it) {
         const int r = (warp & 3) * 32 + 4 * it + (lane >> 3), t = min(first_q + r, n - 1);
         const uint16_t *src = p.Q + (((size_t)t * p.n_seq + seq) * q_heads + q_head) * kHeadDim + 8 * cg;
-        const float4 *tab = reinterpret_cast<const float4 *>(p.table + (size_t)t * 64 + 8 * cg);
+        const float4 *tab = p.table + (size_t)t * 32 + 4 * cg;
         uint32_t r1[4], r2[4];
         if (aligned) {
           const uint4 u1 = *reinterpret_cast<const uint4 *>(src), u2 = *reinterpret_cast<const uint4 *>(src + 64);
@@ -565,37 +576,39 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
             r2[c] = src[64 + 2 * c] | ((uint32_t)src[64 + 2 * c + 1] << 16);
           }
         }
-        float y1[8], y2[8];
-        float mx = 0.f, sum = 0.f;
+        float2 y1[4], y2[4];
+        float mx = 0.f;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const float4 cs = tab[c];  // (cos, sin) of channels 2 c, 2 c + 1 of the group
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const float x1 = __uint_as_float(e ? (r1[c] & 0xFFFF0000u) : (r1[c] << 16)), x2 = __uint_as_float(e ? (r2[c] & 0xFFFF0000u) : (r2[c] << 16));
-            const float co = e ? cs.z : cs.x, si = e ? cs.w : cs.y;
-            const float l1 = SCALED ? sh.lam[8 * cg + 2 * c + e] : 1.0f, l2 = SCALED ? sh.lam[8 * cg + 2 * c + e + 64] : 1.0f;
-            const float a1 = __fsub_rn(__fmul_rn(x1, co), __fmul_rn(x2, si)) * l1 * scale_log2;
-            const float a2 = __fadd_rn(__fmul_rn(x1, si), __fmul_rn(x2, co)) * l2 * scale_log2;
-            y1[2 * c + e] = a1; y2[2 * c + e] = a2;
-            mx = fmaxf(mx, fmaxf(fabsf(a1), fabsf(a2)));
-          }
+        for (int c = 0; c < 4; ++c) {  // channels 2 c, 2 c + 1 of the group and their partners
+          const float4 cs = tab[c];
+          const float2 co = make_float2(cs.x, cs.y), si = make_float2(cs.z, cs.w);
+          const float2 x1 = make_float2(__uint_as_float(r1[c] << 16), __uint_as_float(r1[c] & 0xFFFF0000u));
+          const float2 x2 = make_float2(__uint_as_float(r2[c] << 16), __uint_as_float(r2[c] & 0xFFFF0000u));
+          const float2 l1 = *reinterpret_cast<const float2 *>(&sh.lam[8 * cg + 2 * c]), l2 = *reinterpret_cast<const float2 *>(&sh.lam[8 * cg + 2 * c + 64]);
+          y1[c] = __fmul2_rn(__ffma2_rn(__fmul2_rn(x2, si), make_float2(-1.f, -1.f), __fmul2_rn(x1, co)), l1);
+          y2[c] = __fmul2_rn(__fadd2_rn(__fmul2_rn(x1, si), __fmul2_rn(x2, co)), l2);
+          mx = fmaxf(fmaxf(mx, fmaxf(fabsf(y1[c].x), fabsf(y1[c].y))), fmaxf(fabsf(y2[c].x), fabsf(y2[c].y)));
         }
 #pragma unroll
         for (int o = 1; o <= 4; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         const int shift = mx > 0.f ? max(-100, min(100, 136 - (int)(__float_as_uint(mx) >> 23))) : 0;  // largest element to [2^9, 2^10)
-        const float up = exp2i(shift);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) { y1[i] *= up; y2[i] *= up; sum += y1[i] + y2[i]; }
-#pragma unroll
-        for (int o = 1; o <= 4; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        const float2 up = make_float2(exp2i(shift), exp2i(shift));
+        float2 sum2 = make_float2(0.f, 0.f);
         uint32_t h[4], l[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) split_half2(y1[2 * c], y1[2 * c + 1], h[c], l[c]);
+        for (int c = 0; c < 4; ++c) {
+          y1[c] = __fmul2_rn(y1[c], up);
+          y2[c] = __fmul2_rn(y2[c], up);
+          sum2 = __fadd2_rn(sum2, __fadd2_rn(y1[c], y2[c]));
+          split_half2(y1[c].x, y1[c].y, h[c], l[c]);
+        }
+        float sum = sum2.x + sum2.y;
+#pragma unroll
+        for (int o = 1; o <= 4; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
         *reinterpret_cast<uint4 *>(q_op + r * 16) = make_uint4(h[0], h[1], h[2], h[3]);
         *reinterpret_cast<uint4 *>(q_op + kGridQBytes + r * 16) = make_uint4(l[0], l[1], l[2], l[3]);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) split_half2(y2[2 * c], y2[2 * c + 1], h[c], l[c]);
+        for (int c = 0; c < 4; ++c) split_half2(y2[c].x, y2[c].y, h[c], l[c]);
         *reinterpret_cast<uint4 *>(q_op + 8 * (kGridQTile * 16) + r * 16) = make_uint4(h[0], h[1], h[2], h[3]);
         *reinterpret_cast<uint4 *>(q_op + kGridQBytes + 8 * (kGridQTile * 16) + r * 16) = make_uint4(l[0], l[1], l[2], l[3]);
         // row L of the warp is lane L's from here on
@@ -611,7 +624,7 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
       const unsigned vm = __ldg(p.vmax + slice);
       if (vm) bias -= (float)max((int)(vm >> 23) - 126, -60);
     }
-    float m = -INFINITY;      // reference; arguments of the exponential are f * t - m_b
+    float m = -INFINITY;      // reference (below every score at first); arguments of the exponential are f * t - m_b
     float m_b = 0.f;          // m - bias
     float2 l2 = make_float2(0.f, 0.f), z2 = make_float2(0.f, 0.f);
     const uint32_t t_o = tmem + kGridTmemO + 128 * q + t_lane;
@@ -646,13 +659,13 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
         for (int k = 0; k < 64; ++k)
           if (j * kGridTile + k > qi) t[k] = -INFINITY;
       }
-      float mx = -INFINITY;
+      float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-      for (int k = 0; k < 64; k += 2) mx = fmaxf(mx, fmaxf(t[k], t[k + 1]));
-      mx *= f;
-      if (__any_sync(0xffffffffu, mx > m + kGridMaxAhead)) {
+      for (int k = 0; k < 64; k += 2) mx[(k >> 1) & 3] = fmaxf(mx[(k >> 1) & 3], fmaxf(t[k], t[k + 1]));
+      const float top = f * fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+      if (__any_sync(0xffffffffu, top > m + kGridMaxAhead)) {
         // key 0 is live for every query and sits in the first tile, so m is finite from the first tile on
-        const float m_new = fmaxf(m, mx);
+        const float m_new = fmaxf(m, top);
         const float corr = ex2_fast(m - m_new);  // 0 on the first tile
         m = m_new;
         m_b = m - bias;
@@ -671,40 +684,41 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
             for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * corr);
             tc05::tmem_st32(t_o + c, o);
           }
-          tc05::wait_st();
         }
       }
-      uint32_t hi[32], lo[32];
       const float2 f2 = make_float2(f, f), nm2 = make_float2(-m_b, -m_b);
 #pragma unroll
-      for (int k = 0; k < 64; k += 4) {
-        float4 sv = make_float4(0.f, 0.f, 0.f, 0.f), zv = sv;
-        if constexpr (SCALED) {
-          sv = *reinterpret_cast<const float4 *>(meta + 2 * kGridTile + k);
-          zv = *reinterpret_cast<const float4 *>(meta + 3 * kGridTile + k);
-        }
+      for (int half = 0; half < 2; ++half) {
+        uint32_t hi[16], lo[16];
 #pragma unroll
-        for (int e = 0; e < 4; e += 2) {
-          const float2 arg = __ffma2_rn(f2, make_float2(t[k + e], t[k + e + 1]), nm2);
-          const float2 pr = make_float2(ex2_fast(arg.x), ex2_fast(arg.y));
-          l2 = __fadd2_rn(l2, pr);
-          float2 w = pr;
+        for (int k = 0; k < 32; k += 4) {
+          float4 sv = make_float4(0.f, 0.f, 0.f, 0.f), zv = sv;
           if constexpr (SCALED) {
-            z2 = __ffma2_rn(pr, e ? make_float2(zv.z, zv.w) : make_float2(zv.x, zv.y), z2);
-            w = __fmul2_rn(pr, e ? make_float2(sv.z, sv.w) : make_float2(sv.x, sv.y));
+            sv = *reinterpret_cast<const float4 *>(meta + 2 * kGridTile + 32 * half + k);
+            zv = *reinterpret_cast<const float4 *>(meta + 3 * kGridTile + 32 * half + k);
           }
-          split_half2(w.x, w.y, hi[(k + e) / 2], lo[(k + e) / 2]);
+#pragma unroll
+          for (int e = 0; e < 4; e += 2) {
+            const float2 arg = __ffma2_rn(f2, make_float2(t[32 * half + k + e], t[32 * half + k + e + 1]), nm2);
+            const float2 pr = make_float2(ex2_fast(arg.x), ex2_fast(arg.y));
+            l2 = __fadd2_rn(l2, pr);
+            float2 w = pr;
+            if constexpr (SCALED) {
+              z2 = __ffma2_rn(pr, e ? make_float2(zv.z, zv.w) : make_float2(zv.x, zv.y), z2);
+              w = __fmul2_rn(pr, e ? make_float2(sv.z, sv.w) : make_float2(sv.x, sv.y));
+            }
+            split_half2(w.x, w.y, hi[(k + e) / 2], lo[(k + e) / 2]);
+          }
         }
+        tc05::tmem_st16(t_s + 16 * half, hi);
+        tc05::tmem_st16(t_s + 32 + 16 * half, lo);
       }
-      tc05::tmem_st32(t_s, hi);
-      tc05::tmem_st32(t_s + 32, lo);
       tc05::wait_st();
       tc05::fence_before_sync();
       warp_arrive(&sh.p_full[q][j & 1], lane);
     }
     // ---- the pass's output: keep it (the unquantized pass) or compare with the kept one ----
-    if (nt[q] > 1) wait(&sh.o_done[q], nt[q] - 2);  // a parity wait must not run two phases ahead
-    wait(&sh.o_done[q], nt[q] - 1);
+    wait(&sh.o_last[q], 0);
     __syncwarp();
     tc05::fence_after_sync();
     const int rows = min(kGridQTile, n - first_q);

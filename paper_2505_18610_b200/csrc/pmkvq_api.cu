@@ -892,7 +892,7 @@ pmkvq_status pmkvq_alpha_grid_search(const void *d_K, const void *d_Q, const voi
   const GridWorkspace w = grid_workspace(n_tokens, n_seq, kv_heads, group);
   uint8_t *ws = static_cast<uint8_t *>(d_workspace);
   float *d_amax = reinterpret_cast<float *>(ws + w.amax);
-  float2 *d_table = reinterpret_cast<float2 *>(ws + w.table);
+  float *d_table = reinterpret_cast<float *>(ws + w.table);
   double *d_loss = reinterpret_cast<double *>(ws + w.loss);
   float *d_alphas = reinterpret_cast<float *>(ws + w.alphas);
   unsigned *d_error = reinterpret_cast<unsigned *>(ws + w.error);
@@ -915,13 +915,13 @@ pmkvq_status pmkvq_alpha_grid_search(const void *d_K, const void *d_Q, const voi
   unsigned *d_vmax = reinterpret_cast<unsigned *>(meta + (2 * kGridMaxBatch + 2) * meta_bytes);
 
   GridPrep prep{};
-  prep.amax = d_amax; prep.table = d_table; prep.n_tokens = n_tokens; prep.n_seq = n_seq; prep.kv_heads = kv_heads;
+  prep.amax = d_amax; prep.table = reinterpret_cast<const float4 *>(d_table); prep.n_tokens = n_tokens; prep.n_seq = n_seq; prep.kv_heads = kv_heads;
   prep.bits = bits; prep.floor_value = floor_value;
   GridAttn attn{};
-  attn.Q = Q; attn.amax = d_amax; attn.table = d_table; attn.o_ref = d_o_ref; attn.error_word = d_error;
+  attn.Q = Q; attn.amax = d_amax; attn.table = prep.table; attn.o_ref = d_o_ref; attn.error_word = d_error;
   attn.n_tokens = n_tokens; attn.n_seq = n_seq; attn.kv_heads = kv_heads; attn.group = group; attn.floor_value = floor_value;
-  auto run_prep = [&](int pl) {
-    const unsigned grid = (unsigned)(slices * (size_t)n_tiles);
+  auto run_prep = [&](int pl, int n_out) {
+    const dim3 grid((unsigned)(slices * (size_t)n_tiles), (unsigned)n_out);
     if (pl == 1) alpha_grid_prep_kernel<1><<<grid, 256, 0, st>>>(prep);
     else alpha_grid_prep_kernel<2><<<grid, 256, 0, st>>>(prep);
   };
@@ -931,18 +931,17 @@ pmkvq_status pmkvq_alpha_grid_search(const void *d_K, const void *d_Q, const voi
     kernel<<<grid, kGridThreads, kGridSmemBytes, st>>>(attn);
   };
   // the unquantized operator
-  prep.n_out = 1;
   prep.src = K; prep.is_key = 1; prep.out[0] = ws + w.region[0];
-  run_prep(2);
+  run_prep(2, 1);
   prep.src = V; prep.is_key = 0; prep.out[0] = ws + w.region[1];
-  run_prep(2);
+  run_prep(2, 1);
   attn.k[0] = ws + w.region[0]; attn.v = ws + w.region[1];
   run_attn(alpha_grid_attn_kernel<2, false>, 1);
   // Eq. 9 at each alpha: the Values once, the Keys of up to four alphas at a time
   if (cudaMemsetAsync(d_vmax, 0, slices * sizeof(unsigned), st) != cudaSuccess) return PMKVQ_ERR_CUDA;
   prep.quantize = 1;
   prep.out[0] = ws + w.region[2]; prep.scale[0] = meta_array(0); prep.zero[0] = meta_array(1); prep.vmax = d_vmax;
-  run_prep(planes);
+  run_prep(planes, 1);
   attn.v = prep.out[0]; attn.v_scale = prep.scale[0]; attn.v_zero = prep.zero[0]; attn.vmax = d_vmax;
   prep.src = K; prep.is_key = 1; prep.vmax = nullptr;
   uint8_t *const buffers[kGridMaxBatch] = {ws + w.region[0], ws + w.region[0] + half, ws + w.region[2] + half, ws + w.region[1]};
@@ -952,12 +951,12 @@ pmkvq_status pmkvq_alpha_grid_search(const void *d_K, const void *d_Q, const voi
     attn.k_zero[i] = prep.zero[i] = meta_array(3 + 2 * i);
   }
   for (int first = 0; first < n_alphas; first += per_batch) {
-    prep.n_out = std::min(per_batch, n_alphas - first);
+    const int count = std::min(per_batch, n_alphas - first);
     prep.alphas = attn.alphas = d_alphas + first;
     attn.loss_sums = d_loss + first;
-    run_prep(planes);
-    if (planes == 1) run_attn(alpha_grid_attn_kernel<1, true>, prep.n_out);
-    else run_attn(alpha_grid_attn_kernel<2, true>, prep.n_out);
+    run_prep(planes, count);
+    if (planes == 1) run_attn(alpha_grid_attn_kernel<1, true>, count);
+    else run_attn(alpha_grid_attn_kernel<2, true>, count);
   }
   if (cudaGetLastError() != cudaSuccess) return PMKVQ_ERR_CUDA;
   unsigned error = 0;
