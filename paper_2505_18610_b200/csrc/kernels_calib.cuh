@@ -143,16 +143,18 @@ __global__ void calib_finish_kernel(float *lambda, int n, float floor_value, flo
 // interpolated RoPE of Eq. 12 from a (cos, sin) table.
 // ---------------------------------------------------------------------------------------------
 
-// cos and sin of pos_scale * t * theta^(-2 pair / 128), rounded from fp64: table[t][pair / 2] = (cos of the even pair, cos of the
-// odd one, sin of the even pair, sin of the odd one), so that packed fp32 instructions find adjacent channels in adjacent
-// registers.
+// cos and sin of pos_scale * t * theta^(-2 pair / 128), rounded from fp64, two pairs to an entry: (cos of the even pair, cos of the odd
+// one, sin of the even pair, sin of the odd one), so that packed fp32 instructions find adjacent channels in adjacent
+// registers.  Entry e (pairs 2 e, 2 e + 1) of a token sits at angle_slot(e): the attention kernel's lanes take groups of eight
+// pairs, lane after lane, and read the same entry of their groups at a time.
+__host__ __device__ constexpr int angle_slot(int e) { return (e & 3) * 8 + (e >> 2); }
 __global__ void rope_table_kernel(float *table, int n_tokens, double pos_scale, double theta) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n_tokens * 64) return;
   const int t = i >> 6, pair = i & 63;
   double s, c;
   sincos((double)t * pos_scale * pow(theta, -2.0 * pair / (double)kHeadDim), &s, &c);
-  float *at = table + (size_t)t * 128 + (pair >> 1) * 4 + (pair & 1);
+  float *at = table + (size_t)t * 128 + angle_slot(pair >> 1) * 4 + (pair & 1);
   at[0] = (float)c;
   at[2] = (float)s;
 }
@@ -178,7 +180,7 @@ __device__ __forceinline__ void split_half2(float x, float y, uint32_t &hi, uint
 __device__ __forceinline__ void rotate_token(float (&x)[4], const float4 *__restrict__ table_t, int lane) {
 #pragma unroll
   for (int e = 0; e < 4; e += 2) {
-    const float4 cs = table_t[(lane & 15) * 2 + (e >> 1)];
+    const float4 cs = table_t[angle_slot((lane & 15) * 2 + (e >> 1))];
     const float o0 = __shfl_xor_sync(0xffffffffu, x[e], 16), o1 = __shfl_xor_sync(0xffffffffu, x[e + 1], 16);
     // lanes 0..15 hold x1 (channel < 64): y1 = x1 c - x2 s;  lanes 16..31 hold x2: y2 = x1 s + x2 c
     x[e] = lane < 16 ? __fsub_rn(__fmul_rn(x[e], cs.x), __fmul_rn(o0, cs.z)) : __fadd_rn(__fmul_rn(o0, cs.z), __fmul_rn(x[e], cs.x));
@@ -357,20 +359,26 @@ struct GridAttn {
 
 struct GridShared {
   unsigned long long k_full[kGridKSlots], k_free[kGridKSlots], v_full[kGridVSlots], v_free[kGridVSlots], m_full[kGridMetaSlots];
-  unsigned long long q_full[2], s_full[2][2], p_full[2][2], o_done[2], o_last[2];
+  unsigned long long q_full[2], s_full[2][2], p_full[2][2], o_done[2][2];  // [query tile][key tile mod 2]: a parity wait is never two phases off
   uint32_t tmem_base;
   int abort;
   __align__(16) float lam[kHeadDim];
 };
 
-__device__ __forceinline__ void grid_wait(GridShared &sh, const unsigned long long *bar, uint32_t parity, unsigned *error_word) {
+// One warp waits for a phase of a barrier.  False if the wait ran out, here or elsewhere in the CTA: the warp then leaves its loop
+// (nothing more is copied, issued or arrived at).
+__device__ __forceinline__ bool grid_wait(GridShared &sh, const unsigned long long *bar, uint32_t parity, unsigned *error_word) {
   const uint32_t addr = tc05::smem_u32(bar);
-  if (tc05::mbar_test_wait(addr, parity & 1u)) return;
-  if (*reinterpret_cast<volatile int *>(&sh.abort)) return;
-  if (!tc05::mbar_wait(addr, parity & 1u)) {
-    sh.abort = 1;
-    atomicOr(error_word, 1u);
+  bool ok = tc05::mbar_test_wait(addr, parity & 1u);
+  if (!ok) {
+    for (uint32_t i = 0; !ok && i < tc05::kWaitLimit && *reinterpret_cast<volatile int *>(&sh.abort) == 0; ++i)
+      ok = tc05::mbar_try_wait_hint(addr, parity & 1u, tc05::kWaitHintNs);
+    if (!ok) {
+      sh.abort = 1;
+      atomicOr(error_word, 1u);
+    }
   }
+  return __all_sync(0xffffffffu, ok);
 }
 
 // PLANES: planes of K and V.  SCALED: quantized tensors with scales and zero-points, whose outputs are compared with o_ref;
@@ -402,8 +410,7 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
     for (int q = 0; q < 2; ++q) {
       for (int b = 0; b < 2; ++b) { tc05::mbar_init(tc05::smem_u32(&sh.s_full[q][b]), 1); tc05::mbar_init(tc05::smem_u32(&sh.p_full[q][b]), 4); }
       tc05::mbar_init(tc05::smem_u32(&sh.q_full[q]), 4);
-      tc05::mbar_init(tc05::smem_u32(&sh.o_done[q]), 1);
-      tc05::mbar_init(tc05::smem_u32(&sh.o_last[q]), 1);
+      for (int b = 0; b < 2; ++b) tc05::mbar_init(tc05::smem_u32(&sh.o_done[q][b]), 1);
     }
     sh.abort = 0;
     tc05::mbar_init_fence();
@@ -422,7 +429,7 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
   tc05::fence_after_sync();
   const uint32_t tmem = sh.tmem_base;
   const uint32_t s_base = tc05::smem_u32(smem);
-  auto wait = [&](const unsigned long long *bar, int phase) { grid_wait(sh, bar, (uint32_t)phase, p.error_word); };
+  auto wait = [&](const unsigned long long *bar, int phase) { return grid_wait(sh, bar, (uint32_t)phase, p.error_word); };
 
   if (warp == 10) {
     // ---- copies ----
@@ -439,17 +446,18 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
       }
       __syncwarp();
     };
-    for (int j = 0; j < n_kt; ++j) {
+    bool go = true;
+    for (int j = 0; go && j < n_kt; ++j) {
       const int rows = min(kGridTile, n - j * kGridTile);
       for (int pl = 0; pl < PLANES; ++pl) {
         const int a = j * PLANES + pl, slot = a % kGridKSlots;
-        if (a >= kGridKSlots) wait(&sh.k_free[slot], a / kGridKSlots - 1);
+        if (!go || (a >= kGridKSlots && !(go = wait(&sh.k_free[slot], a / kGridKSlots - 1)))) break;
         tile_copy(s_base + kGridSmemK + slot * kGridPlaneBytes, k_src + ((size_t)j * kGridTile * PLANES + (size_t)pl * rows) * 256, rows, &sh.k_full[slot]);
       }
       if constexpr (SCALED) {
         // slot j mod 4 was last read for tile j - 4, whose weights were all written before the scores of tile j - 2 that freed
         // this tile's K slot could be issued (a query tile without a tile j - 2 has no tile j - 4 to be read late either)
-        if (lane == 0) {
+        if (lane == 0 && go) {
           const uint32_t b = tc05::smem_u32(&sh.m_full[j % kGridMetaSlots]), bytes = (uint32_t)grid_n4(rows) * 4u;
           const uint32_t dst = s_base + kGridSmemMeta + (j % kGridMetaSlots) * kGridMetaBytes;
           const size_t at = (size_t)slice * n4 + (size_t)j * kGridTile;
@@ -463,7 +471,7 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
       }
       for (int pl = 0; pl < PLANES; ++pl) {
         const int a = j * PLANES + pl, slot = a % kGridVSlots;
-        if (a >= kGridVSlots) wait(&sh.v_free[slot], a / kGridVSlots - 1);
+        if (!go || (a >= kGridVSlots && !(go = wait(&sh.v_free[slot], a / kGridVSlots - 1)))) break;
         tile_copy(s_base + kGridSmemV + slot * kGridPlaneBytes, v_src + ((size_t)j * kGridTile * PLANES + (size_t)pl * rows) * 256, rows, &sh.v_full[slot]);
       }
     }
@@ -473,12 +481,13 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
     constexpr uint32_t idesc_s = tc05::idesc_f16(128, kGridTile, 0), idesc_o = tc05::idesc_f16(128, kHeadDim, 1);
     const uint64_t qh = tc05::smem_desc(s_base + kGridSmemQ + 2 * q * kGridQBytes, kGridQTile * 16, 128);
     const uint64_t ql = tc05::smem_desc(s_base + kGridSmemQ + (2 * q + 1) * kGridQBytes, kGridQTile * 16, 128);
+    bool go = true;
     auto scores = [&](int j) {
 #pragma unroll
-      for (int pl = 0; pl < PLANES; ++pl) wait(&sh.k_full[(j * PLANES + pl) % kGridKSlots], (j * PLANES + pl) / kGridKSlots);
-      if (j >= 2) wait(&sh.o_done[q], j - 2);  // the output MMAs that read this buffer's weights are complete
-      if (j == 0) wait(&sh.q_full[q], 0);
-      __syncwarp();
+      for (int pl = 0; pl < PLANES; ++pl) go = go && wait(&sh.k_full[(j * PLANES + pl) % kGridKSlots], (j * PLANES + pl) / kGridKSlots);
+      // the output MMAs that read this buffer's weights are complete; the query operand is there
+      go = go && (j >= 2 ? wait(&sh.o_done[q][j & 1], (j >> 1) - 1) : j == 0 ? wait(&sh.q_full[q], 0) : true);
+      if (!go) return;
       tc05::fence_after_sync();
       const uint32_t d = tmem + kGridTmemS + 64 * (2 * q + (j & 1));
 #pragma unroll
@@ -502,9 +511,9 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
     };
     auto outputs = [&](int j) {
 #pragma unroll
-      for (int pl = 0; pl < PLANES; ++pl) wait(&sh.v_full[(j * PLANES + pl) % kGridVSlots], (j * PLANES + pl) / kGridVSlots);
-      wait(&sh.p_full[q][j & 1], j >> 1);
-      __syncwarp();
+      for (int pl = 0; pl < PLANES; ++pl) go = go && wait(&sh.v_full[(j * PLANES + pl) % kGridVSlots], (j * PLANES + pl) / kGridVSlots);
+      go = go && wait(&sh.p_full[q][j & 1], j >> 1);
+      if (!go) return;
       tc05::fence_after_sync();
       const uint32_t d = tmem + kGridTmemO + 128 * q, w_hi = tmem + kGridTmemS + 64 * (2 * q + (j & 1)), w_lo = w_hi + 32;
 #pragma unroll
@@ -518,9 +527,7 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
           for (int ks = 0; ks < 4; ++ks) tc05::mma_f16_ts_elect(d, w_lo + 8 * ks, vd + ks * 16, idesc_o, 1u);
         }
       }
-      tc05::mma_commit_elect(tc05::smem_u32(&sh.o_done[q]));
-      // a barrier of its own for the end: a parity wait on o_done there could be two phases off in either direction
-      if (j + 1 == n_mine) tc05::mma_commit_elect(tc05::smem_u32(&sh.o_last[q]));
+      tc05::mma_commit_elect(tc05::smem_u32(&sh.o_done[q][j & 1]));
 #pragma unroll
       for (int pl = 0; pl < PLANES; ++pl) {
         const int a = j * PLANES + pl;
@@ -528,20 +535,20 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
       }
     };
     if (n_mine > 0) scores(0);
-    for (int j = 0; j < n_mine; ++j) {
+    for (int j = 0; go && j < n_mine; ++j) {
       if (j + 1 < n_mine) scores(j + 1);
-      outputs(j);
+      if (go) outputs(j);
     }
     // The key tiles that only the second query tile uses: nothing of this warp reads them.  It gives a slot back once the tile is
     // there (the slot's earlier uses are then all over, so no arrival is counted for the wrong use).
-    for (int a = n_mine * PLANES; n_mine > 0 && a < n_kt * PLANES; ++a) {
+    for (int a = n_mine * PLANES; go && n_mine > 0 && a < n_kt * PLANES; ++a) {
       if (a + kGridKSlots < n_kt * PLANES) {
-        wait(&sh.k_full[a % kGridKSlots], a / kGridKSlots);
-        if (lane == 0) tc05::mbar_arrive(tc05::smem_u32(&sh.k_free[a % kGridKSlots]));
+        go = go && wait(&sh.k_full[a % kGridKSlots], a / kGridKSlots);
+        if (lane == 0 && go) tc05::mbar_arrive(tc05::smem_u32(&sh.k_free[a % kGridKSlots]));
       }
       if (a + kGridVSlots < n_kt * PLANES) {
-        wait(&sh.v_full[a % kGridVSlots], a / kGridVSlots);
-        if (lane == 0) tc05::mbar_arrive(tc05::smem_u32(&sh.v_free[a % kGridVSlots]));
+        go = go && wait(&sh.v_full[a % kGridVSlots], a / kGridVSlots);
+        if (lane == 0 && go) tc05::mbar_arrive(tc05::smem_u32(&sh.v_free[a % kGridVSlots]));
       }
       __syncwarp();
     }
@@ -554,66 +561,78 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
     const uint32_t t_lane = (uint32_t)((warp & 3) * 32) << 16;
     float sum_q = 0.f, f = 1.f;  // sum of the operand's elements; scores are f times the dot products
     {
-      // Four rows at a time: eight lanes share a row, each with the channels of group cg and of its partner group cg + 8 (a row of
-      // 256 bytes is then read in whole lines; thread = row would touch 32 lines per load and took 60 000 cycles here).
-      const int cg = lane & 7;
+      // Eight rows at a time, four lanes on a row, each with the channels of two groups and of their partner groups (+ 8).  Loads then
+      // take whole 64-byte pieces (thread = row would touch 32 lines per load and took 60 000 cycles), and the eight lanes
+      // of a store phase write eight consecutive rows of the operand (eight lanes on a row write groups 2 KB apart, a bank
+      // conflict of eight).  The loop is not unrolled: straight-line code that a CTA runs once costs more to fetch than to run.
       const bool aligned = (reinterpret_cast<uintptr_t>(p.Q) & 15) == 0;
-      uint8_t *q_op = smem + kGridSmemQ + 2 * q * kGridQBytes + cg * (kGridQTile * 16);
-#pragma unroll 2
-      for (int it = 0; it < 8; ++it) {
-        const int r = (warp & 3) * 32 + 4 * it + (lane >> 3), t = min(first_q + r, n - 1);
-        const uint16_t *src = p.Q + (((size_t)t * p.n_seq + seq) * q_heads + q_head) * kHeadDim + 8 * cg;
-        const float4 *tab = p.table + (size_t)t * 32 + 4 * cg;
-        uint32_t r1[4], r2[4];
-        if (aligned) {
-          const uint4 u1 = *reinterpret_cast<const uint4 *>(src), u2 = *reinterpret_cast<const uint4 *>(src + 64);
-          r1[0] = u1.x; r1[1] = u1.y; r1[2] = u1.z; r1[3] = u1.w;
-          r2[0] = u2.x; r2[1] = u2.y; r2[2] = u2.z; r2[3] = u2.w;
-        } else {
+#pragma unroll 1
+      for (int rg = 0; rg < 4; ++rg) {
+        const int r = (warp & 3) * 32 + 8 * rg + (lane & 7), t = min(first_q + r, n - 1);
+        const uint16_t *src = p.Q + (((size_t)t * p.n_seq + seq) * q_heads + q_head) * kHeadDim + 8 * (lane >> 3);
+        const float4 *tab = p.table + (size_t)t * 32 + (lane >> 3);
+        uint4 raw[2][2];  // [half of the groups][channels, partners]
+        float4 cs[2][4];
 #pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            r1[c] = src[2 * c] | ((uint32_t)src[2 * c + 1] << 16);
-            r2[c] = src[64 + 2 * c] | ((uint32_t)src[64 + 2 * c + 1] << 16);
+        for (int g = 0; g < 2; ++g) {
+          if (aligned) {
+            raw[g][0] = __ldg(reinterpret_cast<const uint4 *>(src + 32 * g));
+            raw[g][1] = __ldg(reinterpret_cast<const uint4 *>(src + 32 * g + 64));
+          } else {
+            uint32_t w[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+              const uint16_t *at = src + 32 * g + 2 * (c & 3) + 64 * (c >> 2);
+              w[c] = at[0] | ((uint32_t)at[1] << 16);
+            }
+            raw[g][0] = make_uint4(w[0], w[1], w[2], w[3]);
+            raw[g][1] = make_uint4(w[4], w[5], w[6], w[7]);
           }
+#pragma unroll
+          for (int c = 0; c < 4; ++c) cs[g][c] = __ldg(tab + 4 * g + 8 * c);  // entries 4 group + c
         }
-        float2 y1[4], y2[4];
+        float2 y1[2][4], y2[2][4];
         float mx = 0.f;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {  // channels 2 c, 2 c + 1 of the group and their partners
-          const float4 cs = tab[c];
-          const float2 co = make_float2(cs.x, cs.y), si = make_float2(cs.z, cs.w);
-          const float2 x1 = make_float2(__uint_as_float(r1[c] << 16), __uint_as_float(r1[c] & 0xFFFF0000u));
-          const float2 x2 = make_float2(__uint_as_float(r2[c] << 16), __uint_as_float(r2[c] & 0xFFFF0000u));
-          const float2 l1 = *reinterpret_cast<const float2 *>(&sh.lam[8 * cg + 2 * c]), l2 = *reinterpret_cast<const float2 *>(&sh.lam[8 * cg + 2 * c + 64]);
-          y1[c] = __fmul2_rn(__ffma2_rn(__fmul2_rn(x2, si), make_float2(-1.f, -1.f), __fmul2_rn(x1, co)), l1);
-          y2[c] = __fmul2_rn(__fadd2_rn(__fmul2_rn(x1, si), __fmul2_rn(x2, co)), l2);
-          mx = fmaxf(fmaxf(mx, fmaxf(fabsf(y1[c].x), fabsf(y1[c].y))), fmaxf(fabsf(y2[c].x), fabsf(y2[c].y)));
-        }
+        for (int g = 0; g < 2; ++g) {
+          const int ch = 8 * (4 * g + (lane >> 3));
+          const uint32_t r1[4] = {raw[g][0].x, raw[g][0].y, raw[g][0].z, raw[g][0].w}, r2[4] = {raw[g][1].x, raw[g][1].y, raw[g][1].z, raw[g][1].w};
 #pragma unroll
-        for (int o = 1; o <= 4; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+          for (int c = 0; c < 4; ++c) {  // channels 2 c, 2 c + 1 of the group and their partners
+            const float2 co = make_float2(cs[g][c].x, cs[g][c].y), si = make_float2(cs[g][c].z, cs[g][c].w);
+            const float2 x1 = make_float2(__uint_as_float(r1[c] << 16), __uint_as_float(r1[c] & 0xFFFF0000u));
+            const float2 x2 = make_float2(__uint_as_float(r2[c] << 16), __uint_as_float(r2[c] & 0xFFFF0000u));
+            const float2 l1 = *reinterpret_cast<const float2 *>(&sh.lam[ch + 2 * c]), l2 = *reinterpret_cast<const float2 *>(&sh.lam[ch + 2 * c + 64]);
+            y1[g][c] = __fmul2_rn(__ffma2_rn(__fmul2_rn(x2, si), make_float2(-1.f, -1.f), __fmul2_rn(x1, co)), l1);
+            y2[g][c] = __fmul2_rn(__fadd2_rn(__fmul2_rn(x1, si), __fmul2_rn(x2, co)), l2);
+            mx = fmaxf(fmaxf(mx, fmaxf(fabsf(y1[g][c].x), fabsf(y1[g][c].y))), fmaxf(fabsf(y2[g][c].x), fabsf(y2[g][c].y)));
+          }
+        }
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
         const int shift = mx > 0.f ? max(-100, min(100, 136 - (int)(__float_as_uint(mx) >> 23))) : 0;  // largest element to [2^9, 2^10)
         const float2 up = make_float2(exp2i(shift), exp2i(shift));
         float2 sum2 = make_float2(0.f, 0.f);
-        uint32_t h[4], l[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          y1[c] = __fmul2_rn(y1[c], up);
-          y2[c] = __fmul2_rn(y2[c], up);
-          sum2 = __fadd2_rn(sum2, __fadd2_rn(y1[c], y2[c]));
-          split_half2(y1[c].x, y1[c].y, h[c], l[c]);
+        for (int g = 0; g < 2; ++g) {
+          uint8_t *q_op = smem + kGridSmemQ + 2 * q * kGridQBytes + (4 * g + (lane >> 3)) * (kGridQTile * 16) + r * 16;
+          uint32_t h1[4], o1[4], h2[4], o2[4];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            const float2 a = __fmul2_rn(y1[g][c], up), b = __fmul2_rn(y2[g][c], up);
+            sum2 = __fadd2_rn(sum2, __fadd2_rn(a, b));
+            split_half2(a.x, a.y, h1[c], o1[c]);
+            split_half2(b.x, b.y, h2[c], o2[c]);
+          }
+          *reinterpret_cast<uint4 *>(q_op) = make_uint4(h1[0], h1[1], h1[2], h1[3]);
+          *reinterpret_cast<uint4 *>(q_op + kGridQBytes) = make_uint4(o1[0], o1[1], o1[2], o1[3]);
+          *reinterpret_cast<uint4 *>(q_op + 8 * (kGridQTile * 16)) = make_uint4(h2[0], h2[1], h2[2], h2[3]);
+          *reinterpret_cast<uint4 *>(q_op + kGridQBytes + 8 * (kGridQTile * 16)) = make_uint4(o2[0], o2[1], o2[2], o2[3]);
         }
         float sum = sum2.x + sum2.y;
-#pragma unroll
-        for (int o = 1; o <= 4; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        *reinterpret_cast<uint4 *>(q_op + r * 16) = make_uint4(h[0], h[1], h[2], h[3]);
-        *reinterpret_cast<uint4 *>(q_op + kGridQBytes + r * 16) = make_uint4(l[0], l[1], l[2], l[3]);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) split_half2(y2[c].x, y2[c].y, h[c], l[c]);
-        *reinterpret_cast<uint4 *>(q_op + 8 * (kGridQTile * 16) + r * 16) = make_uint4(h[0], h[1], h[2], h[3]);
-        *reinterpret_cast<uint4 *>(q_op + kGridQBytes + 8 * (kGridQTile * 16) + r * 16) = make_uint4(l[0], l[1], l[2], l[3]);
-        // row L of the warp is lane L's from here on
-        const float s_row = __shfl_sync(0xffffffffu, sum, (lane & 3) * 8), f_row = __shfl_sync(0xffffffffu, exp2i(-shift), (lane & 3) * 8);
-        if ((lane >> 2) == it) { sum_q = s_row; f = f_row; }
+        sum += __shfl_xor_sync(0xffffffffu, sum, 8);
+        sum += __shfl_xor_sync(0xffffffffu, sum, 16);
+        if ((lane >> 3) == rg) { sum_q = sum; f = exp2i(-shift); }  // row L of the warp is lane L's from here on
       }
       tc05::fence_async_smem();
       warp_arrive(&sh.q_full[q], lane);
@@ -628,12 +647,13 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
     float m_b = 0.f;          // m - bias
     float2 l2 = make_float2(0.f, 0.f), z2 = make_float2(0.f, 0.f);
     const uint32_t t_o = tmem + kGridTmemO + 128 * q + t_lane;
+    bool go = true;
     for (int j = 0; j < nt[q]; ++j) {
       const uint32_t t_s = tmem + kGridTmemS + 64 * (2 * q + (j & 1)) + t_lane;
       const float *meta = reinterpret_cast<const float *>(smem + kGridSmemMeta + (j % kGridMetaSlots) * kGridMetaBytes);
-      wait(&sh.s_full[q][j & 1], j >> 1);
-      if constexpr (SCALED) wait(&sh.m_full[j % kGridMetaSlots], j / kGridMetaSlots);
-      __syncwarp();
+      go = wait(&sh.s_full[q][j & 1], j >> 1);
+      if constexpr (SCALED) go = go && wait(&sh.m_full[j % kGridMetaSlots], j / kGridMetaSlots);
+      if (!go) break;
       tc05::fence_after_sync();
       float t[64];
       {
@@ -672,8 +692,7 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
         l2 = __fmul2_rn(l2, make_float2(corr, corr));
         z2 = __fmul2_rn(z2, make_float2(corr, corr));
         if (j > 0) {  // this thread's row of the outputs, once all output MMAs issued so far are complete
-          wait(&sh.o_done[q], j - 1);
-          __syncwarp();
+          if (!(go = wait(&sh.o_done[q][(j - 1) & 1], (j - 1) >> 1))) break;
           tc05::fence_after_sync();
 #pragma unroll 1
           for (int c = 0; c < 128; c += 32) {
@@ -718,15 +737,14 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
       warp_arrive(&sh.p_full[q][j & 1], lane);
     }
     // ---- the pass's output: keep it (the unquantized pass) or compare with the kept one ----
-    wait(&sh.o_last[q], 0);
-    __syncwarp();
+    go = go && wait(&sh.o_done[q][(nt[q] - 1) & 1], (nt[q] - 1) >> 1);
     tc05::fence_after_sync();
     const int rows = min(kGridQTile, n - first_q);
     float4 *kept = reinterpret_cast<float4 *>(p.o_ref) + (((size_t)seq * q_heads + q_head) * n + first_q) * (kHeadDim / 4) + row;
     const float inv_l = __fdiv_rn(1.0f, l2.x + l2.y), zs = z2.x + z2.y;
     float err = 0.f;
 #pragma unroll 1
-    for (int c = 0; c < 128; c += 32) {
+    for (int c = 0; go && c < 128; c += 32) {
       uint32_t o[32];
       tc05::tmem_ld32(t_o + c, o);
       tc05::wait_ld();
