@@ -737,29 +737,36 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
       warp_arrive(&sh.p_full[q][j & 1], lane);
     }
     // ---- the pass's output: keep it (the unquantized pass) or compare with the kept one ----
-    go = go && wait(&sh.o_done[q][(nt[q] - 1) & 1], (nt[q] - 1) >> 1);
-    tc05::fence_after_sync();
     const int rows = min(kGridQTile, n - first_q);
     float4 *kept = reinterpret_cast<float4 *>(p.o_ref) + (((size_t)seq * q_heads + q_head) * n + first_q) * (kHeadDim / 4) + row;
     const float inv_l = __fdiv_rn(1.0f, l2.x + l2.y), zs = z2.x + z2.y;
     float err = 0.f;
 #pragma unroll 1
-    for (int c = 0; go && c < 128; c += 32) {
-      uint32_t o[32];
-      tc05::tmem_ld32(t_o + c, o);
-      tc05::wait_ld();
-      if (alive) {
+    for (int c0 = 0; go && c0 < 128; c0 += 64) {
+      float4 ref[16];  // half of the query's kept outputs, the first half asked for before the last output MMAs are complete
+      if (SCALED && alive) {
 #pragma unroll
-        for (int i = 0; i < 32; i += 4) {
-          float4 *at = kept + (size_t)((c + i) >> 2) * rows;
-          float4 v = make_float4((__uint_as_float(o[i]) + zs) * inv_l, (__uint_as_float(o[i + 1]) + zs) * inv_l,
-                                 (__uint_as_float(o[i + 2]) + zs) * inv_l, (__uint_as_float(o[i + 3]) + zs) * inv_l);
-          if constexpr (SCALED) {
-            const float4 r = *at;
-            v.x -= r.x; v.y -= r.y; v.z -= r.z; v.w -= r.w;
-            err = fmaf(v.x, v.x, err); err = fmaf(v.y, v.y, err); err = fmaf(v.z, v.z, err); err = fmaf(v.w, v.w, err);
-          } else {
-            *at = v;
+        for (int i = 0; i < 16; ++i) ref[i] = kept[(size_t)(c0 / 4 + i) * rows];
+      }
+      if (c0 == 0 && !(go = wait(&sh.o_done[q][(nt[q] - 1) & 1], (nt[q] - 1) >> 1))) break;
+      tc05::fence_after_sync();
+#pragma unroll
+      for (int c = 0; c < 64; c += 32) {
+        uint32_t o[32];
+        tc05::tmem_ld32(t_o + c0 + c, o);
+        tc05::wait_ld();
+        if (alive) {
+#pragma unroll
+          for (int i = 0; i < 32; i += 4) {
+            float4 v = make_float4((__uint_as_float(o[i]) + zs) * inv_l, (__uint_as_float(o[i + 1]) + zs) * inv_l,
+                                   (__uint_as_float(o[i + 2]) + zs) * inv_l, (__uint_as_float(o[i + 3]) + zs) * inv_l);
+            if constexpr (SCALED) {
+              const float4 r = ref[(c + i) / 4];
+              v.x -= r.x; v.y -= r.y; v.z -= r.z; v.w -= r.w;
+              err = fmaf(v.x, v.x, err); err = fmaf(v.y, v.y, err); err = fmaf(v.z, v.z, err); err = fmaf(v.w, v.w, err);
+            } else {
+              kept[(size_t)((c0 + c + i) / 4) * rows] = v;
+            }
           }
         }
       }
