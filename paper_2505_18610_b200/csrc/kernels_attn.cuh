@@ -7,10 +7,9 @@
 // empty units that stand for the fixed cost of a segment.  All units of all slices form one
 // line that is cut into equal contiguous pieces, one per CTA of a persistent grid (one CTA of 16
 // warps per SM), so every CTA streams the same number of bytes whatever the shape.  The part of a
-// CTA's piece that lies in one slice is a "segment": its 16 warps draw the segment's tiles from a
-// shared counter (INT16 tiles first, then body tiles, the accumulators changing units in between),
-// so they finish together however the SM shares its issue slots among them; each warp keeps its
-// own running (max, sum, accumulator), the warps are merged in shared memory and the segment
+// CTA's piece that lies in one slice is a "segment": its 16 warps share the segment's body and INT16
+// tiles (the accumulators change units in between), so that they finish
+// together however the SM shares its issue slots among them; each warp keeps its own running (max, sum, accumulator), the warps are merged in shared memory and the segment
 // publishes one partial (m, l, o[128]) per head.  The CTA that publishes the
 // last partial of a slice (atomic ticket, nobody waits) merges the slice and writes the output.
 //
@@ -118,6 +117,10 @@ __device__ __forceinline__ int claim_next(int *ctr, int lane) {
       : "r"(addr), "r"(lane)
       : "memory");
   return __shfl_sync(0xffffffffu, j, 0);
+}
+// asks for a run of bytes (16-byte aligned, a multiple of 16) to be brought into L2; one lane
+__device__ __forceinline__ void prefetch_l2(const void *ptr, uint32_t bytes, int lane) {
+  if (lane == 0) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(ptr), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
@@ -578,6 +581,9 @@ __device__ __forceinline__ float slice_sigma16(const AttnParams &p, int slice) {
   return s16 ? exp2i(max(-126, (int)(s16 >> 23) - 126)) : 1.0f;
 }
 
+__device__ __forceinline__ const uint8_t *int16_tile(const AttnParams &p, const uint8_t *slice_base, int it) {
+  return slice_base + (it < p.sink_tiles ? (size_t)it * tile_bytes(16) : p.geom.ring_off + (size_t)(it - p.sink_tiles) * tile_bytes(16));
+}
 // The INT16 tiles [a_lo, a_hi) of a slice (sink tiles, then the window ring), drawn from the shared
 // counter s_ctr[0] by the warps of the CTA.
 __device__ __forceinline__ void run_int16_tiles(const AttnParams &p, const uint8_t *slice_base, int a_lo, int a_hi,
@@ -594,14 +600,12 @@ __device__ __forceinline__ void run_int16_tiles(const AttnParams &p, const uint8
   const int first_slot = n_win > 0 ? (p.win_start - p.geom.n_sink) % p.geom.ring_tokens : 0;
   do {
     uint32_t mask;
-    const uint8_t *tile;
+    const uint8_t *tile = int16_tile(p, slice_base, it);
     if (it < p.sink_tiles) {
       const int live = max(0, min(16, p.n_sink_eff - 16 * it));
       mask = (1u << live) - 1u;
-      tile = slice_base + (size_t)it * tile_bytes(16);
     } else {
       const int rt = it - p.sink_tiles;
-      tile = slice_base + p.geom.ring_off + (size_t)rt * tile_bytes(16);
       int d = rt * 16 + (lane & 15) - first_slot;  // lane r looks at row r of the tile
       if (d < 0) d += p.geom.ring_tokens;
       mask = __ballot_sync(0xffffffffu, d < n_win) & 0xFFFFu;
@@ -708,8 +712,7 @@ __device__ __forceinline__ void publish_segment(const AttnParams &p, int slice, 
 // warp each took four passes and the merge 3 of a short segment's 9 us).
 constexpr int kMergeRow = kHeadDim + 8;
 constexpr int kMergeBytes = kAttnWarps * kMaxGroup * kMergeRow * 4;
-template <class FactorOf>
-__device__ __forceinline__ void merge_warps(const AttnParams &p, int slice, const WarpState &st, FactorOf f_of,
+__device__ __forceinline__ void merge_warps(const AttnParams &p, int slice, const WarpState &st, float unit,
                                             float (*s_o)[kMaxGroup][kMergeRow], float *s_ml, int *s_ctr) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, tig = lane & 3;
   float l_sum, zs_sum;
@@ -727,16 +730,15 @@ __device__ __forceinline__ void merge_warps(const AttnParams &p, int slice, cons
   }
   const float f_mine = ex2(st.m - M);
   const float z_mine = zs_sum * f_mine;
-  const float f0 = __shfl_sync(0xffffffffu, f_mine, (2 * tig) * 4), f1 = __shfl_sync(0xffffffffu, f_mine, (2 * tig + 1) * 4);
+  const float f0 = unit * __shfl_sync(0xffffffffu, f_mine, (2 * tig) * 4), f1 = unit * __shfl_sync(0xffffffffu, f_mine, (2 * tig + 1) * 4);
   const float zs0 = __shfl_sync(0xffffffffu, z_mine, (2 * tig) * 4), zs1 = __shfl_sync(0xffffffffu, z_mine, (2 * tig + 1) * 4);
 #pragma unroll
   for (int mt = 0; mt < 8; ++mt) {
 #pragma unroll
     for (int rr = 0; rr < 2; ++rr) {
-      const float f = f_of(2 * mt + rr);
       const int ch = 16 * mt + 8 * rr + g;
-      s_o[warp][2 * tig][ch] = fmaf(st.acc[mt][2 * rr], f * f0, zs0);
-      s_o[warp][2 * tig + 1][ch] = fmaf(st.acc[mt][2 * rr + 1], f * f1, zs1);
+      s_o[warp][2 * tig][ch] = fmaf(st.acc[mt][2 * rr], f0, zs0);
+      s_o[warp][2 * tig + 1][ch] = fmaf(st.acc[mt][2 * rr + 1], f1, zs1);
     }
   }
   float *part = partial_slot(p, slice);
@@ -783,11 +785,16 @@ __device__ __forceinline__ void segment_ranges(const AttnParams &p, int u_lo, in
 }
 
 // One segment on the warp-level MMA path: the part [u_lo, u_hi) (units relative to the slice) of one slice
-// that this CTA owns.  Builds the slice's query, runs the INT16 tiles and then the body tiles (width
-// BITS) of the range, merges the warps and publishes one partial per head.  The warps of the CTA draw
-// work from two shared counters (INT16 tiles, then body steps of NT tiles), so they all finish together
-// whatever share of the issue slots each of them gets.  `ring` is the CTA's dynamic shared memory: the
-// per-warp cp.async stages while tiles stream, then the warps' outputs.
+// that this CTA owns.  Builds the slice's query, runs the body tiles (width BITS) and the INT16 tiles of the range, merges
+// the warps and publishes one partial per head.  How the work reaches the warps depends on what bounds it.
+//   2 and 4 bit, bound by instructions: warp w takes body steps w, w + 16, ..., which keeps it inside one stream, so its next
+//     copy is one addition away and only the ends of the range need checks.  The INT16 tiles come last, drawn from a shared
+//     counter, so they even out what the warps finished apart (64 slices x 32K tokens, 4 blocks: 199 -> 185 us at 2 bit and
+//     220 -> 205 us at 4 bit, against everything from counters); they are asked into L2 when the segment begins, and
+//     a launch behind the decode step's append waits for it only there.
+//   8 and 16 bit, bound by memory: INT16 tiles first, then body steps, both from counters, which keep the SM's share of the
+//     memory busy however the warps drift apart (dealt out as above: 2 % slower).
+// `ring` is the CTA's dynamic shared memory: the per-warp cp.async stages while tiles stream, then the warps' outputs.
 template <int BITS>
 __device__ __forceinline__ void run_segment(const AttnParams &p, int slice, int u_lo, int u_hi,
                                             float (*s_q)[kHeadDim], float *s_stat, int *s_ctr, uint4 *s_frag,
@@ -798,56 +805,66 @@ __device__ __forceinline__ void run_segment(const AttnParams &p, int slice, int 
   const int b = slice / p.kv_heads, hkv = slice - b * p.kv_heads;
 
   // (the previous segment ended with a CTA-wide barrier after its last use of s_q / s_stat / s_ctr / ring)
+  constexpr bool kDealt = BITS <= 4;
   if (tid == 0) s_ctr[0] = s_ctr[1] = 0;
-  __syncthreads();
+  if constexpr (!kDealt) __syncthreads();
   int a_lo, a_hi, t_lo, t_hi;
   segment_ranges<BITS>(p, u_lo, u_hi, a_lo, a_hi, t_lo, t_hi);
   const uint8_t *slice_base = p.geom.base + (size_t)slice * p.geom.slice_stride;
 
-  // ---- body stream set-up: claim the first steps and start their copies before anything else ----
+  // ---- this warp's body steps; the first copy starts before anything else ----
   constexpr int TB = tile_bytes(BITS);
-  constexpr int NT = F::NT, S = F::SLOTS > 0 ? F::SLOTS : 1, SB = NT * TB;
-  const uint8_t *body = slice_base + p.geom.body_off;
-  const size_t stream_stride = p.geom.stream_stride;
-  // A step is NT tiles.  With NT = 2 these are the tiles 16 G + s and 16 G + 8 + s: neighbours in stream s, one
-  // contiguous run of 2 TB bytes (attention does not care about the order of the tokens).  The first and
-  // the last group of 16 tiles of a segment may reach beyond [t_lo, t_hi): such tiles are left out.
-  const int g_lo = t_lo >> 4;
-  const int n_steps = t_hi <= t_lo ? 0 : (NT == 2 ? 8 * (((t_hi - 1) >> 4) - g_lo + 1) : t_hi - t_lo);
-  auto step_tile = [&](int j, int k) { return NT == 2 ? 16 * (g_lo + (j >> 3)) + (j & 7) + 8 * k : t_lo + j; };
+  constexpr int NT = F::NT, SB = NT * TB;
+  static_assert(kDealt == (NT == 2) && (F::SLOTS == 0 || F::SLOTS == 2), "one step in flight while another is worked on");
+  // A step is NT tiles.  With NT = 2 these are the tiles 16 u + s and 16 u + 8 + s, s = warp mod 8: neighbours in stream s, one
+  // contiguous run of 2 TB bytes (attention does not care about the order of the tokens); the first and the last group of 16
+  // tiles of a segment may reach beyond [t_lo, t_hi), and such tiles are left out.  With NT = 1 a step is tile u.
+  const int tail_rows = p.n_body & 15;
+  const int tail_tile = tail_rows ? p.body_tiles - 1 : kNoTiles;  // the one tile with dead rows
+  const int s = warp & 7;
+  auto first_tile = [&](int u) { return NT == 2 ? 16 * u + s : u; };
+  const int u_end = NT == 2 ? (t_hi > t_lo ? (t_hi + 15) >> 4 : 0) : t_hi;
+  // steps [fast_lo, fast_hi) consist of whole live tiles that may be read at once
+  const int t_fast = min(t_hi, min(tail_tile, p.clean_tiles));
+  const int fast_lo = NT == 2 ? (max(t_lo - s, 0) + 15) >> 4 : t_lo;
+  const int fast_hi = NT == 2 ? (t_fast - s - 8 + 15) >> 4 : t_fast;  // 16 u + s + 8 < t_fast
+  auto fast = [&](int v) { return v >= fast_lo && v < fast_hi; };
   auto live = [&](int t) { return t >= t_lo && t < t_hi; };
-  uint8_t *my_ring = ring + (size_t)warp * S * SB;
-  const uint32_t ring_addr = (uint32_t)__cvta_generic_to_shared(my_ring);
-  auto claim = [&](int which) { return claim_next(s_ctr + which, lane); };
-  auto issue = [&](int j, int slot) {
+  const uint8_t *body = slice_base + p.geom.body_off;
+  auto step_src = [&](int v) { return body + body_tile_offset(first_tile(v), BITS, p.geom.stream_stride); };
+  auto claim_step = [&]() { return t_lo + claim_next(s_ctr + 1, lane); };
+  constexpr int DU = kAttnWarps / 8;                                  // dealt steps: from one of a warp's to its next
+  constexpr size_t kSrcStep = (size_t)(kAttnWarps * NT / 8) * TB;
+  uint8_t *my_ring = ring + (size_t)warp * 2 * SB;
+  const uint32_t ring_addr = (uint32_t)__cvta_generic_to_shared(my_ring) + lane * 16;
+  auto issue = [&](int v, const uint8_t *from, int slot) {
     constexpr int CPT = TB / 16;  // 16-byte chunks per tile: lane l copies chunks l, l + 32, ...
-    const int ta = step_tile(j, 0);
-    const uint8_t *src = body + body_tile_offset(ta, BITS, stream_stride) + lane * 16;
-    const uint32_t dst = ring_addr + slot * SB + lane * 16;
-    if (NT == 2 && (NT * CPT) % 32 == 0 && live(ta) && live(ta + 8)) {  // the whole step, every lane the same number of chunks
-      cp_async_run<NT * CPT / 32>(dst, src);
+    const uint32_t dst = ring_addr + slot * SB;
+    from += lane * 16;
+    if (fast(v)) {  // the whole step is one run
+      cp_async_run<NT * CPT / 32>(dst, from);
+      if ((NT * CPT) % 32 != 0 && lane < (NT * CPT) % 32) cp_async16_at<(NT * CPT / 32) * 512>(dst, from);
     } else {
+      if (first_tile(v) + 8 * (NT - 1) >= p.clean_tiles) pdl_wait();
 #pragma unroll
       for (int k = 0; k < NT; ++k) {
-        if (live(step_tile(j, k))) {
-          cp_async_run<CPT / 32>(dst + k * TB, src + k * TB);
-          if (CPT % 32 != 0 && lane < CPT % 32) cp_async16_at<(CPT / 32) * 512>(dst + k * TB, src + k * TB);
+        if (live(first_tile(v) + 8 * k)) {
+          cp_async_run<CPT / 32>(dst + k * TB, from + k * TB);
+          if (CPT % 32 != 0 && lane < CPT % 32) cp_async16_at<(CPT / 32) * 512>(dst + k * TB, from + k * TB);
         }
       }
     }
   };
-  int pending[S];  // steps claimed and in flight, oldest first (>= n_steps: none)
+  int u = 0;
+  const uint8_t *src = nullptr;
   if constexpr (F::SLOTS > 0) {
-#pragma unroll
-    for (int i = 0; i < S - 1; ++i) {
-      pending[i] = n_steps > 0 ? claim(1) : 0;
-      if (pending[i] < n_steps) {
-        if (step_tile(pending[i], NT - 1) >= p.clean_tiles) pdl_wait();
-        issue(pending[i], i);
-      }
-      cp_async_commit();
-    }
+    u = kDealt ? (t_lo >> 4) + (warp >> 3) : u_end > t_lo ? claim_step() : u_end;
+    src = step_src(u);
+    if (u < u_end) issue(u, src, 0);
+    cp_async_commit();
   }
+  if constexpr (kDealt)
+    for (int it = a_lo + warp; it < a_hi; it += kAttnWarps) prefetch_l2(int16_tile(p, slice_base, it), tile_bytes(16), lane);
 
   build_query(p, b, hkv, s_q, s_stat);
   const int e_g = (int)s_stat[g];
@@ -855,83 +872,100 @@ __device__ __forceinline__ void run_segment(const AttnParams &p, int slice, int 
   fill_q_fragments<16>(s_frag, s_q, s_stat);  // half of the threads each
   if constexpr (BITS != 16) fill_q_fragments<BITS>(s_frag + 256, s_q, s_stat, 256);
   __syncthreads();
-  pdl_wait();  // from here on the segment reads what the append in front of this launch may have written
-  const float sigma16 = slice_sigma16(p, slice);
 
   WarpState st;
   st.m = kNegBig; st.l = make_float2(0.f, 0.f); st.zs = make_float2(0.f, 0.f);
 #pragma unroll
   for (int mt = 0; mt < 8; ++mt) st.acc[mt][0] = st.acc[mt][1] = st.acc[mt][2] = st.acc[mt][3] = 0.f;
 
-  // ---- INT16 tiles (sink + window ring) ----
-  if (a_hi > a_lo) {
-    run_int16_tiles(p, slice_base, a_lo, a_hi, st, s_frag, s_ctr, e_g, sumq, sigma16, lane);
-    if constexpr (BITS != 16) {
-      // accumulator units change with the width: INT16 units -> body units (exact powers of two)
+  // accumulator units change with the width (exact powers of two)
+  auto change_units = [&](bool to_int16, float ratio) {
 #pragma unroll
-      for (int mt = 0; mt < 8; ++mt) {
+    for (int mt = 0; mt < 8; ++mt) {
 #pragma unroll
-        for (int rr = 0; rr < 2; ++rr) {
-          const float f = exp2i(F::EP - F16::EP + F::pos((2 * mt + rr) % F::N) - F::SIGMA_LOG2);
-          st.acc[mt][2 * rr] *= f;
-          st.acc[mt][2 * rr + 1] *= f;
-        }
+      for (int rr = 0; rr < 2; ++rr) {
+        const int e = F::EP - F16::EP + F::pos((2 * mt + rr) % F::N) - F::SIGMA_LOG2;
+        const float f = exp2i(to_int16 ? -e : e) * ratio;
+        st.acc[mt][2 * rr] *= f;
+        st.acc[mt][2 * rr + 1] *= f;
       }
+    }
+  };
+  // ---- INT16 tiles (sink + window ring) before the body ----
+  if constexpr (!kDealt) pdl_wait();  // they are what the append in front of this launch may have written
+  // The slice's largest INT16 V scale; at 2 and 4 bit perhaps before that append has raised it: every body token is older.
+  const float sigma_body = slice_sigma16(p, slice);
+  if constexpr (!kDealt) {
+    if (a_hi > a_lo) {
+      run_int16_tiles(p, slice_base, a_lo, a_hi, st, s_frag, s_ctr, e_g, sumq, sigma_body, lane);
+      if constexpr (BITS != 16) change_units(false, 1.0f);
     }
   }
 
   // ---- body tiles ----
-  const float sigma_u = sigma16 * exp2i(F::SIGMA_LOG2);
-  if (n_steps > 0) {
+  if (t_hi > t_lo) {
     QFrag qa;
     qa.mine = (BITS != 16 ? s_frag + 256 : s_frag) + lane;
     const float mu = exp2i(24 - F::EQ + e_g);
-    const float inv_sigma_e = exp2i(F::EP) / sigma_u;
-    const uint32_t tail_mask = (p.n_body & 15) ? (1u << (p.n_body & 15)) - 1u : 0xFFFFu;
-    const int tail_tile = tail_mask != 0xFFFFu ? p.body_tiles - 1 : -1;  // the one tile with dead rows
+    const float inv_sigma_e = exp2i(F::EP) / (sigma_body * exp2i(F::SIGMA_LOG2));
+    const uint32_t tail_mask = (1u << tail_rows) - 1u;
     if constexpr (F::SLOTS == 0) {
-      for (int t = t_lo + claim(1); t < t_hi; t = t_lo + claim(1)) {
-        const uint8_t *tile = body + body_tile_offset(t, BITS, stream_stride);
-        if (t == tail_tile) process_tiles<BITS, 1, true>(tile, tail_mask, st, qa, mu, sumq, inv_sigma_e, lane);
-        else process_tiles<BITS, 1, false>(tile, 0xFFFFu, st, qa, mu, sumq, inv_sigma_e, lane);
+      for (u = claim_step(); u < u_end; u = claim_step()) {
+        src = step_src(u);
+        if (u == tail_tile) process_tiles<BITS, 1, true>(src, tail_mask, st, qa, mu, sumq, inv_sigma_e, lane);
+        else process_tiles<BITS, 1, false>(src, 0xFFFFu, st, qa, mu, sumq, inv_sigma_e, lane);
       }
     } else {
-      int slot = 0, fill = S - 1;
-      while (pending[0] < n_steps) {
-        const int nxt = claim(1);
-        if (nxt < n_steps) issue(nxt, fill);
+      for (int slot = 0; u < u_end; slot ^= 1) {
+        int next;
+        if constexpr (kDealt) {
+          next = u + DU;
+          src += kSrcStep;
+        } else {
+          next = claim_step();
+          src = step_src(next);
+        }
+        if (next < u_end) issue(next, src, slot ^ 1);
         cp_async_commit();
-        cp_async_wait<S - 1>();
+        cp_async_wait<1>();
         __syncwarp();
         const uint8_t *tile = my_ring + slot * SB;
-        const int t = step_tile(pending[0], 0);
-        if (NT == 2 && live(t) && live(t + 8) && t != tail_tile && t + 8 != tail_tile) {
+        if (fast(u)) {
           process_tiles<BITS, NT, false>(tile, 0xFFFFu, st, qa, mu, sumq, inv_sigma_e, lane);
         } else {
-#pragma unroll
+#pragma unroll 1
           for (int k = 0; k < NT; ++k) {
-            const int tk = step_tile(pending[0], k);
+            const int tk = first_tile(u) + 8 * k;
             if (!live(tk)) continue;
-            if (tk == tail_tile)
-              process_tiles<BITS, 1, true>(tile + k * TB, tail_mask, st, qa, mu, sumq, inv_sigma_e, lane);
-            else
-              process_tiles<BITS, 1, false>(tile + k * TB, 0xFFFFu, st, qa, mu, sumq, inv_sigma_e, lane);
+            if (tk == tail_tile) process_tiles<BITS, 1, true>(tile + k * TB, tail_mask, st, qa, mu, sumq, inv_sigma_e, lane);
+            else process_tiles<BITS, 1, false>(tile + k * TB, 0xFFFFu, st, qa, mu, sumq, inv_sigma_e, lane);
           }
         }
         __syncwarp();
-#pragma unroll
-        for (int i = 0; i + 2 < S; ++i) pending[i] = pending[i + 1];
-        pending[S - 2] = nxt;
-        fill = slot;
-        slot = (slot + 1 == S) ? 0 : slot + 1;
+        u = next;
       }
     }
   }
   if constexpr (F::SLOTS > 0) cp_async_wait<0>();
 
+  // ---- INT16 tiles behind the body ----
+  float unit = sigma_body * exp2i(24 - F16::EP);
+  if constexpr (kDealt) {
+    pdl_wait();
+    float sigma16 = sigma_body, ratio = 1.0f;
+    if (p.clean_tiles != kNoTiles) {  // (a ratio beyond 2^60 means constant Values so far: the sums are zero)
+      sigma16 = slice_sigma16(p, slice);
+      ratio = fminf(sigma_body / sigma16, 0x1p60f);
+    }
+    change_units(true, ratio);
+    if (a_hi > a_lo) run_int16_tiles(p, slice_base, a_lo, a_hi, st, s_frag, s_ctr, e_g, sumq, sigma16, lane);
+    unit = sigma16 * exp2i(24 - F16::EP);
+  } else if constexpr (BITS != 16) {
+    change_units(true, 1.0f);
+  }
+
   // ---- the warps' states become the segment's partial, in real units (the ring's memory is reused) ----
-  merge_warps(p, slice, st, [&](int J) { return sigma_u * exp2i(24 - F::EP - F::pos(J % F::N)); },
-              reinterpret_cast<float(*)[kMaxGroup][kMergeRow]>(ring), s_stat + 16, s_ctr);
+  merge_warps(p, slice, st, unit, reinterpret_cast<float(*)[kMaxGroup][kMergeRow]>(ring), s_stat + 16, s_ctr);
 }
 
 }  // namespace pmkvq
