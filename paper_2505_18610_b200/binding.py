@@ -1,7 +1,8 @@
 """Thin ctypes binding of the C ABI in ``include/pmkvq.h`` (same call names, argument
 marshalling only).  PyTorch supplies device memory (the arena, inputs, outputs) and the stream;
-every step of the path runs inside ``libpmkvq.so``.  There is no fallback: if the library is
-missing it is built with nvcc, and if that fails the import raises.
+every step of the path runs inside ``libpmkvq.so``.  The calls of the token loop (append, decode_attention, decode_step,
+restore_layer_state) reach it through ``_host_calls.so``, which does their checks and marshalling natively.  There is no
+fallback: if a library is missing it is built, and if that fails the import raises.
 """
 from __future__ import annotations
 
@@ -45,6 +46,10 @@ def load_library() -> ctypes.CDLL:
     if _build.needs_build():
         _build.build()
     lib = ctypes.CDLL(_LIB_PATH)
+    from . import _host_calls   # linked to the same library file
+    _host_calls.set_error(PmkvqError)
+    global _calls
+    _calls = _host_calls
     vp, i32, u64p, i32p = ctypes.c_void_p, ctypes.c_int32, ctypes.POINTER(ctypes.c_uint64), ctypes.POINTER(ctypes.c_int32)
     lib.pmkvq_arena_bytes_required.restype = ctypes.c_size_t
     lib.pmkvq_arena_bytes_required.argtypes = [ctypes.POINTER(_Config)]
@@ -98,6 +103,7 @@ def load_library() -> ctypes.CDLL:
 
 
 _lib: Optional[ctypes.CDLL] = None
+_calls = None   # the extension module, loaded with the library
 
 
 def lib() -> ctypes.CDLL:
@@ -108,8 +114,7 @@ def lib() -> ctypes.CDLL:
 
 
 def _stream_ptr(stream: Optional[torch.cuda.Stream]) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    return _calls.current_stream() if stream is None else stream.cuda_stream
 
 
 def calibrate_lambda(k_pre: torch.Tensor, pos_scale: float = 1.0, theta: float = 10000.0, alpha: float = 0.5,
@@ -180,6 +185,7 @@ class Cache:
                  device: str = "cuda:0", shift_variant: int = 0, attention_path: int = 0, slack_bytes: int = 0,
                  fill_byte: Optional[int] = None):
         self._h = None
+        self._handle = 0    # the same as an integer
         self.layers, self.q_heads, self.kv_heads, self.batch = layers, q_heads, kv_heads, batch
         self._fbit = (ctypes.c_uint8 * layers)(*[int(b) for b in fbit])
         self._budget = None if budget_bytes is None else (ctypes.c_uint64 * layers)(*[int(b) for b in budget_bytes])
@@ -213,12 +219,13 @@ class Cache:
             st = lib().pmkvq_cache_create(ctypes.byref(cfg), ctypes.byref(h))
         if st != OK:
             raise PmkvqError(st, "pmkvq_cache_create")
-        self._h = h
+        self._h, self._handle = h, h.value
+        self._token = batch * kv_heads * 128    # numbers in one token's K
 
     def close(self):
         if self._h is not None:
             lib().pmkvq_cache_destroy(self._h)
-            self._h = None
+            self._h, self._handle = None, 0
 
     def __del__(self):
         try:
@@ -233,11 +240,7 @@ class Cache:
 
     def append(self, layer: int, k: torch.Tensor, v: torch.Tensor, stream=None, check: bool = True) -> int:
         """k, v: bf16 [n_new, batch, kv_heads, 128] (or [batch, kv_heads, 128] for one token)."""
-        self._check(k, torch.bfloat16, "k"); self._check(v, torch.bfloat16, "v")
-        n_new = 1 if k.dim() == 3 else k.shape[0]
-        if k.numel() != n_new * self.batch * self.kv_heads * 128 or v.numel() != k.numel():
-            raise ValueError("bad K/V shape")
-        st = lib().pmkvq_append(self._h, layer, k.data_ptr(), v.data_ptr(), n_new, _stream_ptr(stream))
+        st = _calls.append(self._handle, layer, k, v, self._token, stream)
         if check and st != OK:
             raise PmkvqError(st, "pmkvq_append")
         return st
@@ -250,16 +253,7 @@ class Cache:
 
     def decode_attention(self, layer: int, q: torch.Tensor, out: Optional[torch.Tensor] = None, stream=None):
         """q: bf16 [batch, q_heads, 128] -> fp32 [batch, q_heads, 128]."""
-        self._check(q, torch.bfloat16, "q")
-        if q.numel() != self.batch * self.q_heads * 128:
-            raise ValueError("bad Q shape")
-        if out is None:
-            out = torch.empty(self.batch, self.q_heads, 128, dtype=torch.float32, device=q.device)
-        self._check(out, torch.float32, "out")
-        st = lib().pmkvq_decode_attention(self._h, layer, q.data_ptr(), out.data_ptr(), _stream_ptr(stream))
-        if st != OK:
-            raise PmkvqError(st, "pmkvq_decode_attention")
-        return out
+        return _calls.decode_attention(self._handle, layer, q, self.batch, self.q_heads, out, stream)
 
     def decode_attention_static(self, layer: int, q: torch.Tensor, out: torch.Tensor, stream=None, check: bool = True):
         """pmkvq_decode_attention_static: same result as decode_attention, split-K workspace inside the
@@ -276,19 +270,7 @@ class Cache:
                     stream=None):
         """One decode step over all blocks.  k, v: bf16 [layers, batch, kv_heads, 128]; q: bf16
         [layers, batch, q_heads, 128] -> fp32 [layers, batch, q_heads, 128]."""
-        self._check(k, torch.bfloat16, "k"); self._check(v, torch.bfloat16, "v"); self._check(q, torch.bfloat16, "q")
-        if (k.numel() != self.layers * self.batch * self.kv_heads * 128 or v.numel() != k.numel()
-                or q.numel() != self.layers * self.batch * self.q_heads * 128):
-            raise ValueError("bad K/V/Q shape")
-        if out is None:
-            out = torch.empty(self.layers, self.batch, self.q_heads, 128, dtype=torch.float32, device=q.device)
-        self._check(out, torch.float32, "out")
-        if out.numel() != q.numel():
-            raise ValueError("bad out shape")
-        st = lib().pmkvq_decode_step(self._h, k.data_ptr(), v.data_ptr(), q.data_ptr(), out.data_ptr(), _stream_ptr(stream))
-        if st != OK:
-            raise PmkvqError(st, "pmkvq_decode_step")
-        return out
+        return _calls.decode_step(self._handle, k, v, q, self.layers, self.batch, self.kv_heads, self.q_heads, out, stream)
 
     def decode_attention_all(self, q: torch.Tensor, out: Optional[torch.Tensor] = None, stream=None):
         """Attention of all blocks in one launch, nothing appended.  q: bf16 [layers, batch, q_heads, 128]
@@ -323,9 +305,7 @@ class Cache:
         return int(got.value)
 
     def restore_layer_state(self, layer: int, n_tokens: int, cur_bits: int):
-        st = lib().pmkvq_restore_layer_state(self._h, layer, int(n_tokens), int(cur_bits))
-        if st != OK:
-            raise PmkvqError(st, "pmkvq_restore_layer_state")
+        _calls.restore_layer_state(self._handle, layer, int(n_tokens), int(cur_bits))
 
     def arena_layout(self, layer: int):
         out = (ctypes.c_uint64 * 10)()

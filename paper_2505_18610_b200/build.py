@@ -1,13 +1,19 @@
-"""In-tree build of the CUDA library: nvcc -> paper_2505_18610_b200/libpmkvq.so (sm_100a only)."""
+"""In-tree build: nvcc -> paper_2505_18610_b200/libpmkvq.so (the CUDA library, sm_100a only) and the host compiler ->
+paper_2505_18610_b200/_host_calls.so (the Python extension for the calls of the token loop, linked to the former)."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
+
+import torch
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 SRC = os.path.join(HERE, "csrc", "pmkvq_api.cu")
 LIB = os.path.join(HERE, "libpmkvq.so")
+HOST_SRC = os.path.join(HERE, "csrc", "host_calls.cpp")
+HOST_LIB = os.path.join(HERE, "_host_calls.so")
 DEPS = [os.path.join(HERE, "csrc", f) for f in os.listdir(os.path.join(HERE, "csrc"))] + [
     os.path.join(os.path.dirname(HERE), "include", "pmkvq.h")]
 
@@ -19,10 +25,24 @@ NVCC_FLAGS = [
 
 
 def needs_build() -> bool:
-    if not os.path.exists(LIB):
+    if not (os.path.exists(LIB) and os.path.exists(HOST_LIB)):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(HOST_LIB))
     return any(os.path.getmtime(d) > t for d in DEPS)
+
+
+def _build_host_calls() -> None:
+    at = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+    include = [os.path.join(at, "include"), sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
+    cmd = ([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}"] + ["-I" + i for i in include]
+           + ["-o", HOST_LIB, HOST_SRC, "-L" + HERE, "-l:libpmkvq.so", "-Wl,-rpath,$ORIGIN", "-L" + os.path.join(at, "lib"),
+              "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10"])
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        sys.stderr.write(res.stdout + res.stderr)
+        raise RuntimeError("the host compiler failed building _host_calls.so")
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -36,6 +56,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         raise RuntimeError("nvcc failed building libpmkvq.so")
     if verbose:
         sys.stderr.write(res.stderr)
+    _build_host_calls()
     return LIB
 
 

@@ -1,0 +1,76 @@
+"""The native host path of the token loop: which arguments it refuses and with which exception, the caller's own output and
+stream."""
+import pytest
+import torch
+
+from paper_2505_18610_b200 import binding as B
+
+
+def test_refusals_without_a_device():
+    B.lib()
+    x = torch.zeros(1, 1, 128, dtype=torch.bfloat16)
+    with pytest.raises(ValueError, match="k must be a contiguous CUDA tensor of torch.bfloat16"):
+        B._calls.append(0, 0, x, x, 128, None)
+    with pytest.raises(ValueError, match="q must be a contiguous CUDA tensor"):
+        B._calls.decode_attention(0, 0, x, 1, 1, None, None)
+    with pytest.raises(TypeError):
+        B._calls.append(0, 0, None, x, 128, None)
+    with pytest.raises(TypeError):
+        B._calls.append(0, 0.5, x, x, 128, None)
+    with pytest.raises(TypeError):
+        B._calls.append(0, 0, x, x, 128)
+    with pytest.raises(B.PmkvqError) as e:
+        B._calls.restore_layer_state(0, 0, 1, 16)
+    assert e.value.status == B.INVALID_ARG and "pmkvq_restore_layer_state" in str(e.value)
+
+
+@pytest.mark.gpu
+def test_shapes_outputs_and_streams():
+    # which warp takes which tile may differ from call to call: the probabilities' 11 significant bits are rounded against another
+    # maximum, 2^-11 of Values of magnitude 4 at most
+    def same(a, b):
+        torch.testing.assert_close(a, b, rtol=0, atol=4 * 2.0 ** -11)
+
+    c = B.Cache(2, 8, 2, 3, 64, [4, 4], window=16)
+    g = torch.Generator(device="cuda").manual_seed(1)
+    k, v = (torch.randn(20, 3, 2, 128, device="cuda", generator=g).bfloat16() for _ in range(2))
+    q = torch.randn(2, 3, 8, 128, device="cuda", generator=g).bfloat16()
+    for bad_k, bad_v in ((k[:, :, :1].contiguous(), v), (k, v[:19]), (k[0, 0, 0], v[0, 0, 0])):
+        with pytest.raises(ValueError, match="bad K/V shape"):
+            c.append(0, bad_k, bad_v)
+    for bad in (k.transpose(1, 2), k.float(), k.cpu()):
+        with pytest.raises(ValueError, match="k must be"):
+            c.append(0, bad, v)
+    with pytest.raises(IndexError):
+        c.append(0, k[0, 0, 0, 0], v[0, 0, 0, 0])
+    with pytest.raises(B.PmkvqError) as e:
+        c.append(2, k, v)
+    assert e.value.status == B.INVALID_ARG and c.append(2, k, v, check=False) == B.INVALID_ARG
+    assert c.append(0, k, v) == B.OK and c.append(1, k, v) == B.OK
+    with pytest.raises(ValueError, match="bad Q shape"):
+        c.decode_attention(0, q)
+    with pytest.raises(ValueError, match="out must be a contiguous CUDA tensor of torch.float32"):
+        c.decode_attention(0, q[0], out=q[0])
+    with pytest.raises(ValueError, match="bad K/V/Q shape"):
+        c.decode_step(k[:1], v[:1], q)
+    with pytest.raises(ValueError, match="bad out shape"):
+        c.decode_step(k[:2], v[:2], q, out=torch.empty(1, 3, 8, 128, device="cuda"))
+    want = c.decode_attention(1, q[1])
+    assert want.shape == (3, 8, 128) and want.dtype == torch.float32 and want.device == q.device
+    mine = torch.full_like(want, float("nan"))
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    assert c.decode_attention(1, q[1], out=mine, stream=side) is mine
+    side.synchronize()
+    same(mine, want)
+    with torch.cuda.stream(side):       # the current stream is the caller's, not the default one
+        step = c.decode_step(k[:2], v[:2], q)
+        assert c.layer_state(1)["n_tokens"] == 21
+        c.restore_layer_state(0, 20, 16), c.restore_layer_state(1, 20, 16)
+        mine = torch.empty_like(step)
+        assert c.decode_step(k[:2], v[:2], q, out=mine) is mine
+    side.synchronize()
+    same(mine, step)
+    c.close()
+    with pytest.raises(B.PmkvqError):
+        c.append(0, k, v)
