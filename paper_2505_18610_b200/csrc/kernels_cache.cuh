@@ -3,6 +3,7 @@
 // with explicit round-to-nearest intrinsics so that codes, scales and zero-points have exactly
 // one bit pattern.
 #pragma once
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <cstdint>
 
@@ -314,81 +315,110 @@ __global__ void __launch_bounds__(128) append_kernel(const uint16_t *__restrict_
              n_new);
 }
 
-// Bulk appends (prefill): body tiles that consist of new tokens only are built whole, one warp per
-// (tile, slice, K|V).  Every lane loads exactly the elements whose codes the tile layout makes it own
-// (K part: tokens {g, g+8} x channels {8W + 2 tig + h}; V part: tokens {2 tig + 8r + h} x channels
-// {8J + g}), so a token's minimum and maximum meet inside a quad (K) or across the eight lanes of equal
-// tig (V), the codes are packed in registers (Eq. 3 chain to the body width included) and leave as the
-// lane's own 16-byte chunks: coalesced 128-bit stores, no shared memory.  The strided 2- and 4-byte
-// loads of one warp cover whole 4 KB of input; the sectors they share are served by L1.
+__device__ __forceinline__ float min3(float a, float b, float c) {
+  float r;
+  asm("min.f32 %0, %1, %2, %3;\n" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;\n" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+template <int BYTES>
+__device__ __forceinline__ void copy_async(uint32_t to, const void *from) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(to), "l"(from), "n"(BYTES) : "memory");
+}
+// four 8 x 8 matrices of 16-bit values from shared memory; lane l gives the address of row l & 7 of matrix l >> 3
+template <bool TRANSPOSED>
+__device__ __forceinline__ void load_matrices(uint32_t addr, uint32_t *out) {
+  if constexpr (TRANSPOSED)
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];\n" : "=r"(out[0]), "=r"(out[1]), "=r"(out[2]), "=r"(out[3]) : "r"(addr) : "memory");
+  else
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];\n" : "=r"(out[0]), "=r"(out[1]), "=r"(out[2]), "=r"(out[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ __nv_bfloat162 as_bf162(uint32_t x) { return *reinterpret_cast<const __nv_bfloat162 *>(&x); }
 
-// Eq. 1-2 at 16 bit on N values of one token that a lane holds, given the token's min and max; the
-// values are replaced by their codes at `BITS` (Eq. 3 chain).  Returns the INT16 scale.  With CLEAN = false only the low
-// BITS (at 16 bit: 16) bits of a result are the code and bits 16 .. 23 are zero; what sits above may be anything.
-template <int BITS, int N, bool CLEAN>
-__device__ __forceinline__ float quantize_owned(float (&x)[N], float mn, float mx, int variant) {
-  const float scale = __fdiv_rn(__fsub_rn(mx, mn), 65535.0f);
-  if (scale >= 0x1p-60f && scale <= 0x1p60f) {  // one scale per token: the branch is uniform in the warp
-    // two values per instruction (packed fp32 pairs, each component rounded to nearest like the scalar form):
-    // x - mn as x + (-mn), the residual d - q s as q (-s) + d
-    static_assert(N % 2 == 0, "values are taken in pairs");
-    const float y = __frcp_rn(scale);
-    const float2 y2 = make_float2(y, y), ns2 = make_float2(-scale, -scale), nmn2 = make_float2(-mn, -mn);
-#pragma unroll
-    for (int i = 0; i < N; i += 2) {
-      const float2 d = __fadd2_rn(make_float2(x[i], x[i + 1]), nmn2);
-      float2 q = __fmul2_rn(d, y2);
-      float2 r = __ffma2_rn(q, ns2, d);
-      q = __ffma2_rn(r, y2, q);
-      r = __ffma2_rn(q, ns2, d);
-      q = __ffma2_rn(r, y2, q);
-      const float2 c = __fadd2_rn(q, make_float2(8388608.0f, 8388608.0f));  // code_of_quotient, both at once
-      if constexpr (BITS == 16) {  // the code is the low half of the sum's bit pattern; the packing keeps only that
-        x[i] = c.x;
-        x[i + 1] = c.y;
-      } else if (variant == kShiftEquivalent) {  // chain_code on both
-        const float2 c16 = __fadd2_rn(c, make_float2(-8388608.0f, -8388608.0f));
-        constexpr float inv = inv_chain_divisor<BITS>();
-        const float2 cb = __ffma2_rn(c16, make_float2(inv, inv), make_float2(8388608.0f, 8388608.0f));
-        x[i] = CLEAN ? __uint_as_float(__float_as_uint(cb.x) & 0xFFu) : cb.x;
-        x[i + 1] = CLEAN ? __uint_as_float(__float_as_uint(cb.y) & 0xFFu) : cb.y;
-      } else {
-        x[i] = __uint_as_float((uint32_t)(__float_as_int(c.x) - 0x4B000000) >> (16 - BITS));
-        x[i + 1] = __uint_as_float((uint32_t)(__float_as_int(c.y) - 0x4B000000) >> (16 - BITS));
-      }
-    }
-  } else {  // constant tokens (0 / 0 converts to code 0) and scales far outside any real tensor's range
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-      const int c = min(max(__float2int_rn(__fdiv_rn(__fsub_rn(x[i], mn), scale)), 0), 65535);
-      x[i] = __uint_as_float(chain_code<BITS>((uint32_t)c, variant));
-    }
+// Bulk appends (prefill): whole tiles (or masked ones, see append_tile_half), one warp per (tile, slice, K|V).
+
+// Eq. 1-2 at 16 bit and the Eq. 3 chain to BITS on two values at once.  Two values per instruction (packed fp32 pairs, each
+// component rounded to nearest like the scalar form): x - mn as x + (-mn), the residual d - q s as q (-s) + d.
+// The quotient starts from the reciprocal in two parts, y + yl = 1 / s to 2^-47: q = d y + (d yl) is faithful, and one
+// correction with the correctly rounded y makes it the correctly rounded quotient (Markstein, as in quotient_rn, which
+// spends a correction more on getting there).
+struct TokenScale {
+  float2 nmn, s, ns, y, yl;  // -min, S, -S, 1 / S rounded, what the rounding left
+  bool plain;             // false: constant tokens and scales far outside any real tensor's range
+};
+// d / 65535 rounded to nearest: the rounded reciprocal is off by 2^-32 of itself, so d y is faithful and one correction makes
+// it exact while no residual can underflow
+__device__ __forceinline__ float range_scale(float d) {
+  constexpr float y = 1.0f / 65535.0f;
+  const float q = __fmul_rn(d, y);
+  if (d >= 0x1p-60f && d <= 0x1p100f) return __fmaf_rn(__fmaf_rn(-q, 65535.0f, d), y, q);
+  return __fdiv_rn(d, 65535.0f);
+}
+__device__ __forceinline__ void token_scale(float mn, float mx, float &nmn, float &s, float &ns, float &y, float &yl) {
+  s = range_scale(__fsub_rn(mx, mn));
+  nmn = -mn;
+  ns = -s;
+  y = __frcp_rn(s);
+  yl = __fmul_rn(__fmaf_rn(ns, y, 1.f), y);
+}
+__device__ __forceinline__ TokenScale one_token(float mn, float mx) {
+  TokenScale t;
+  token_scale(mn, mx, t.nmn.x, t.s.x, t.ns.x, t.y.x, t.yl.x);
+  t.nmn.y = t.nmn.x; t.s.y = t.s.x; t.ns.y = t.ns.x; t.y.y = t.y.x; t.yl.y = t.yl.x;
+  t.plain = t.s.x >= 0x1p-60f && t.s.x <= 0x1p60f;
+  return t;
+}
+__device__ __forceinline__ TokenScale two_tokens(float2 mn, float2 mx) {
+  TokenScale t;
+  token_scale(mn.x, mx.x, t.nmn.x, t.s.x, t.ns.x, t.y.x, t.yl.x);
+  token_scale(mn.y, mx.y, t.nmn.y, t.s.y, t.ns.y, t.y.y, t.yl.y);
+  t.plain = fminf(t.s.x, t.s.y) >= 0x1p-60f && fmaxf(t.s.x, t.s.y) <= 0x1p60f;
+  return t;
+}
+// the codes of both values, one in each half of the result
+template <int BITS, int VARIANT>
+__device__ __forceinline__ uint32_t pair_codes(float2 x, const TokenScale &t) {
+  const float2 d = __fadd2_rn(x, t.nmn);
+  float2 q = __ffma2_rn(d, t.y, __fmul2_rn(d, t.yl));
+  const float2 r = __ffma2_rn(q, t.ns, d);
+  q = __ffma2_rn(r, t.y, q);
+  const float2 magic = make_float2(8388608.0f, 8388608.0f);
+  float2 c = __fadd2_rn(q, magic);  // code_of_quotient: the code is the low half of the sum's bit pattern
+  if constexpr (BITS < 16 && VARIANT == kShiftEquivalent) {  // chain_code on both
+    constexpr float inv = inv_chain_divisor<BITS>();
+    c = __ffma2_rn(__fadd2_rn(c, make_float2(-8388608.0f, -8388608.0f)), make_float2(inv, inv), magic);
   }
-  return scale;
+  const uint32_t both = __byte_perm(__float_as_uint(c.x), __float_as_uint(c.y), 0x5410);
+  if constexpr (BITS < 16 && VARIANT != kShiftEquivalent) return (both >> (16 - BITS)) & (((1u << BITS) - 1) * 0x10001u);
+  return both;
+}
+__device__ __forceinline__ uint32_t rare_code(float x, float mn, float scale) {  // 0 / 0 converts to code 0
+  return (uint32_t)min(max(__float2int_rn(__fdiv_rn(__fsub_rn(x, mn), scale)), 0), 65535);
 }
 
-// Lane-words of one token pair: word w holds codes idx = w n + j (n = 16 / BITS) of the token (or
-// channel) in half 0 and of its partner in half 1.  lo / hi: the 16 codes (as bit patterns) of the halves,
-// `step` entries apart.
-template <int BITS>
-__device__ __forceinline__ void pack_words(const float *lo, const float *hi, int step, uint32_t *words) {
-  constexpr int n = 16 / BITS;
-  if constexpr (BITS == 16) {  // one code per half; only the low 16 bits of a pattern are the code
+// The same on N values of one token that a lane holds, given the token's min and max; the values are replaced by their
+// codes at `BITS`.  Returns the INT16 scale.
+template <int BITS, int N>
+__device__ __forceinline__ float quantize_owned(float (&x)[N], float mn, float mx, int variant) {
+  static_assert(N % 2 == 0, "values are taken in pairs");
+  const TokenScale t = one_token(mn, mx);
+  if (t.plain) {  // one scale per token: the branch is uniform in the warp
 #pragma unroll
-    for (int w = 0; w < 16; ++w) words[w] = __byte_perm(__float_as_uint(lo[w * step]), __float_as_uint(hi[w * step]), 0x5410);
+    for (int i = 0; i < N; i += 2) {
+      const float2 pair = make_float2(x[i], x[i + 1]);
+      const uint32_t c = variant == kShiftEquivalent ? pair_codes<BITS, kShiftEquivalent>(pair, t) : pair_codes<BITS, kShiftModified>(pair, t);
+      x[i] = __uint_as_float(c & 0xFFFFu);
+      x[i + 1] = __uint_as_float(c >> 16);
+    }
   } else {
 #pragma unroll
-    for (int w = 0; w < BITS; ++w) {
-      uint32_t a = 0, b = 0;
-#pragma unroll
-      for (int j = 0; j < n; ++j) {
-        // a sum: what sits above bit 23 of a pattern only moves further up
-        a += __float_as_uint(lo[(w * n + j) * step]) << (j * BITS);
-        b += __float_as_uint(hi[(w * n + j) * step]) << (j * BITS);
-      }
-      words[w] = __byte_perm(a, b, 0x5410);
-    }
+    for (int i = 0; i < N; ++i) x[i] = __uint_as_float(chain_code<BITS>(rare_code(x[i], mn, t.s.x), variant));
   }
+  return t.s.x;
 }
 
 // The lane's words lw = r BITS .. r BITS + BITS - 1 (lane-word lw sits in chunk lw / 4 at word lw % 4).
@@ -418,114 +448,167 @@ __device__ __forceinline__ void store_word_halves(uint8_t *part, int r, int lane
 }
 constexpr uint32_t kAllRows = 0xFFFFu;
 
-constexpr int kStageRowBytes = 272;  // a staged bf16 row of 128 channels plus 16 bytes: the owner-mapped reads below hit 32 different banks
-// Rows [row_lo, row_hi) of the tile are new tokens and may be loaded; the rows of `keep` are written, the tile's others left
-// alone.
+constexpr int kStageRowBytes = 272;  // a staged bf16 row of 128 channels plus 16 bytes: eight rows of a matrix load hit 32 different banks
+
+// 16 pairs of values of one token half of the lane (token and channels: see append_tile_half) -> its words of round r.
+// pair_at(i): pair i once more, for the rare branch, which is a loop so as not to cost the common one registers.
+template <int BITS, class PairAt>
+__device__ __forceinline__ void words_of_pairs(const float2 (&x)[16], const TokenScale &t, int variant, uint32_t (&words)[BITS],
+                                               PairAt pair_at) {
+  constexpr int n = 16 / BITS;
+  auto pack = [&](auto code) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const uint32_t c = code(x[i]);
+      words[i / n] = i % n == 0 ? c : words[i / n] + (c << (i % n * BITS));
+    }
+  };
+  if (t.plain && (BITS == 16 || variant == kShiftEquivalent)) {
+    pack([&](float2 v) { return pair_codes<BITS, kShiftEquivalent>(v, t); });
+  } else if (t.plain) {
+    pack([&](float2 v) { return pair_codes<BITS, kShiftModified>(v, t); });
+  } else {
+    uint32_t slow[BITS];
+#pragma unroll 1
+    for (int w = 0; w < BITS; ++w) {
+      uint32_t a = 0;
+#pragma unroll 1
+      for (int j = 0; j < n; ++j) {
+        const float2 v = pair_at(w * n + j);
+        const uint32_t lo = chain_code<BITS>(rare_code(v.x, -t.nmn.x, t.s.x), variant), hi = chain_code<BITS>(rare_code(v.y, -t.nmn.y, t.s.y), variant);
+        a |= (lo | hi << 16) << (j * BITS);
+      }
+      slow[w] = a;
+    }
+#pragma unroll
+    for (int w = 0; w < BITS; ++w) words[w] = slow[w];
+  }
+}
+
+// Half (K or V) of the rows `keep` of a lane-owned tile, by one warp; the tile's other rows are left alone.  Rows
+// [row_lo, row_hi) are new tokens and may be loaded.
+// Lane 4 g + tig owns, in round r, K of token g + 8 r at channels 8 W + 2 tig + h, or V of tokens 2 tig + 8 r + h at channels
+// 8 J + g: fragments of 8 x 8 matrices, as they are for K and transposed for V, so the staged rows come back with four
+// 16-byte matrix loads per round, as the pairs (h = 0, 1) that end in the two halves of a word.  A token's
+// minimum and maximum meet inside a quad (K) or across the eight lanes of equal tig (V); the codes are packed in
+// registers (Eq. 3 chain to the body width included) and leave as the lane's own 16-byte chunks.
 template <int BITS>
 __device__ __forceinline__ void append_tile_half(const uint16_t *__restrict__ src, size_t row_stride,
                                                  const float *__restrict__ il, uint8_t *dst_tile, int is_value,
                                                  unsigned *vmax_slot, int lane, int variant, uint8_t *stage, int row_lo = 0,
                                                  int row_hi = kTileTokens, uint32_t keep = kAllRows) {
   const int g = lane >> 2, tig = lane & 3;
-  uint32_t words[BITS];
-  // the tile's 16 rows of 256 bytes come in with eight coalesced 16-byte loads per lane, all in flight at once
+  // the rows of 256 bytes come in with four coalesced 16-byte copies per lane and round, all in flight at once
+  const uint32_t stage_s = (uint32_t)__cvta_generic_to_shared(stage);
   {
+    const uint32_t to = stage_s + (lane >> 4) * kStageRowBytes + (lane & 15) * 16;
+    // a row that may not be loaded stands in as a copy of one that may (zeros would send the whole warp through
+    // the quantizer's rare branch)
+    auto row_at = [&](int row) { return src + (ptrdiff_t)max(row_lo, min(row, row_hi - 1)) * (ptrdiff_t)row_stride + (lane & 15) * 8; };
     const bool aligned = (reinterpret_cast<uintptr_t>(src) & 15) == 0;
-    uint4 v[8];
+    if (aligned && row_lo == 0 && row_hi == kTileTokens) {
+      const uint16_t *from = src + (size_t)(lane >> 4) * row_stride + (lane & 15) * 8;
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const int id = lane + 32 * c;
-      // a row that may not be loaded stands in as a copy of one that may (zeros would send the whole warp through
-      // the quantizer's rare branch)
-      const int row = max(row_lo, min(id >> 4, row_hi - 1));
-      const uint16_t *from = src + (ptrdiff_t)row * (ptrdiff_t)row_stride + (id & 15) * 8;
-      if (aligned) {
-        v[c] = *reinterpret_cast<const uint4 *>(from);
-      } else {  // inputs on an 8-byte boundary
-        const uint2 a = *reinterpret_cast<const uint2 *>(from), b = *reinterpret_cast<const uint2 *>(from + 4);
-        v[c] = make_uint4(a.x, a.y, b.x, b.y);
+      for (int r = 0; r < 2; ++r) {
+        if ((keep >> (8 * r)) & 0xFFu) {
+#pragma unroll
+          for (int c = 0; c < 4; ++c) copy_async<16>(to + (8 * r + 2 * c) * kStageRowBytes, from + (size_t)(8 * r + 2 * c) * row_stride);
+        }
+      }
+    } else {
+#pragma unroll 1
+      for (int c = 0; c < 8; ++c) {
+        const uint16_t *from = row_at((lane >> 4) + 2 * c);
+        if (aligned) {
+          copy_async<16>(to + 2 * c * kStageRowBytes, from);
+        } else {  // inputs on an 8-byte boundary
+          copy_async<8>(to + 2 * c * kStageRowBytes, from);
+          copy_async<8>(to + 2 * c * kStageRowBytes + 8, from + 4);
+        }
       }
     }
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const int id = lane + 32 * c;
-      *reinterpret_cast<uint4 *>(stage + (id >> 4) * kStageRowBytes + (id & 15) * 16) = v[c];
-    }
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
     __syncwarp();
   }
-  if (!is_value) {
+  const uint32_t from = stage_s + (lane & 7) * kStageRowBytes + (lane >> 3) * 16;
+  float smax = 0.f;
 #pragma unroll 1
-    for (int r = 0; r < 2; ++r) {  // token g + 8 r
-      float x[32];                 // [2 W + h]
-      const uint8_t *row = stage + (g + 8 * r) * kStageRowBytes + 4 * tig;
+  for (int r = 0; r < 2; ++r) {
+    const uint32_t keep8 = (keep >> (8 * r)) & 0xFFu;
+    if (keep8 == 0) continue;
+    uint32_t raw[16], words[BITS];
+    float2 x[16];
+    TokenScale t;
+    uint8_t *part = dst_tile;
+    int row0, row1;  // tokens of the words' halves
+    if (!is_value) {
 #pragma unroll
-      for (int W = 0; W < 16; ++W) {
-        const uint32_t raw = *reinterpret_cast<const uint32_t *>(row + 16 * W);
-        const float2 l2 = __ldg(reinterpret_cast<const float2 *>(il + 8 * W + 2 * tig));  // Lambda^-1, L1-resident
-        const float2 xl = __fmul2_rn(make_float2(__uint_as_float(raw << 16), __uint_as_float(raw & 0xFFFF0000u)), l2);
-        x[2 * W] = xl.x;
-        x[2 * W + 1] = xl.y;
+      for (int m = 0; m < 4; ++m) {
+        load_matrices<false>(from + r * 8 * kStageRowBytes + m * 64, raw);
+#pragma unroll
+        for (int W = 4 * m; W < 4 * m + 4; ++W) {
+          const float2 l2 = __ldg(reinterpret_cast<const float2 *>(il + 8 * W + 2 * tig));  // Lambda^-1, L1-resident
+          x[W] = __fmul2_rn(make_float2(__uint_as_float(raw[W & 3] << 16), __uint_as_float(raw[W & 3] & 0xFFFF0000u)), l2);
+        }
       }
-      float mn = x[0], mx = x[0];
+      float lo = fminf(x[0].x, x[0].y), hi = fmaxf(x[0].x, x[0].y);
 #pragma unroll
-      for (int i = 1; i < 32; ++i) { mn = fminf(mn, x[i]); mx = fmaxf(mx, x[i]); }
+      for (int W = 1; W < 16; ++W) { lo = min3(lo, x[W].x, x[W].y); hi = max3(hi, x[W].x, x[W].y); }
 #pragma unroll
       for (int o = 1; o <= 2; o <<= 1) {
-        mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
       }
-      const float s16 = quantize_owned<BITS, 32, false>(x, mn, mx, variant);
-      pack_words<BITS>(x, x + 1, 2, words);  // halves of a word: channels h = 0, 1 of the token
-      const bool kept = (keep >> (g + 8 * r)) & 1u;
-      if (keep == kAllRows) store_words<BITS>(dst_tile, r, lane, words);
-      else store_word_halves<BITS>(dst_tile, r, lane, words, kept, kept);
-      // metadata record g / 2 holds tokens {2t, 2t+1, 8+2t, 9+2t} at entries {0, 1, 2, 3}
-      if (tig == 0 && kept) {
-        float *rec = reinterpret_cast<float *>(dst_tile + meta_offset(BITS) + (g >> 1) * 64) + 2 * r + (g & 1);
-        rec[0] = chain_scale(s16, BITS, variant);
-        rec[4] = chain_zero(mn, s16, BITS, variant);
+      t = one_token(lo, hi);
+      row0 = row1 = g;
+    } else {
+#pragma unroll
+      for (int m = 0; m < 4; ++m) load_matrices<true>(from + r * 8 * kStageRowBytes + m * 64, &raw[4 * m]);
+      // bf16 pairs: minimum and maximum of both tokens at once
+      __nv_bfloat162 lo = as_bf162(raw[0]), hi = lo;
+#pragma unroll
+      for (int J = 1; J < 16; ++J) { lo = __hmin2(lo, as_bf162(raw[J])); hi = __hmax2(hi, as_bf162(raw[J])); }
+#pragma unroll
+      for (int o = 4; o <= 16; o <<= 1) {
+        lo = __hmin2(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = __hmax2(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+      }
+      t = two_tokens(__bfloat1622float2(lo), __bfloat1622float2(hi));
+#pragma unroll
+      for (int J = 0; J < 16; ++J) x[J] = make_float2(__uint_as_float(raw[J] << 16), __uint_as_float(raw[J] & 0xFFFF0000u));
+      part += v_part_offset(BITS);
+      row0 = 2 * tig;
+      row1 = row0 + 1;
+    }
+    words_of_pairs<BITS>(x, t, variant, words, [&](int i) {
+      const uint8_t *at = stage + (8 * r + row0) * kStageRowBytes + 16 * i;
+      if (is_value) {
+        const uint32_t a = *reinterpret_cast<const uint16_t *>(at + 2 * g), b = *reinterpret_cast<const uint16_t *>(at + kStageRowBytes + 2 * g);
+        return make_float2(__uint_as_float(a << 16), __uint_as_float(b << 16));
+      }
+      const uint32_t a = *reinterpret_cast<const uint32_t *>(at + 4 * tig);
+      const float2 l2 = __ldg(reinterpret_cast<const float2 *>(il + 8 * i + 2 * tig));
+      return __fmul2_rn(make_float2(__uint_as_float(a << 16), __uint_as_float(a & 0xFFFF0000u)), l2);
+    });
+    const bool kept0 = (keep8 >> row0) & 1u, kept1 = (keep8 >> row1) & 1u;
+    if (keep8 == 0xFFu) store_words<BITS>(part, r, lane, words);
+    else store_word_halves<BITS>(part, r, lane, words, kept0, kept1);
+    // metadata record t holds tokens {2t, 2t+1, 8+2t, 9+2t} at entries {0, 1, 2, 3}: S_K at bytes 0.., Z_K 16.., S_V 32.., Z_V 48..
+    float *rec = reinterpret_cast<float *>(dst_tile + meta_offset(BITS) + (row0 >> 1) * 64 + (is_value ? 32 : 0)) + 2 * r + (row0 & 1);
+    const bool writer = is_value ? g == 0 : tig == 0;
+    if (writer && kept0) {
+      rec[0] = chain_scale(t.s.x, BITS, variant);
+      rec[4] = chain_zero(-t.nmn.x, t.s.x, BITS, variant);
+    }
+    if (is_value) {
+      smax = fmaxf(smax, fmaxf(t.s.x, t.s.y));
+      if (writer && kept1) {
+        rec[1] = chain_scale(t.s.y, BITS, variant);
+        rec[5] = chain_zero(-t.nmn.y, t.s.y, BITS, variant);
       }
     }
-  } else {
-    float smax = 0.f;
-#pragma unroll 1
-    for (int r = 0; r < 2; ++r) {  // tokens 2 tig + 8 r + h, h = 0, 1
-      float x[2][16];              // [h][J]
-      const uint8_t *row = stage + (2 * tig + 8 * r) * kStageRowBytes + 2 * g;
-#pragma unroll
-      for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int J = 0; J < 16; ++J)
-          x[h][J] = __uint_as_float((uint32_t)*reinterpret_cast<const uint16_t *>(row + h * kStageRowBytes + 16 * J) << 16);
-      float S[2], Z[2];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        float mn = x[h][0], mx = x[h][0];
-#pragma unroll
-        for (int i = 1; i < 16; ++i) { mn = fminf(mn, x[h][i]); mx = fmaxf(mx, x[h][i]); }
-#pragma unroll
-        for (int o = 4; o <= 16; o <<= 1) {
-          mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-          mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        }
-        S[h] = quantize_owned<BITS, 16, false>(x[h], mn, mx, variant);
-        Z[h] = mn;
-        smax = fmaxf(smax, S[h]);
-      }
-      pack_words<BITS>(x[0], x[1], 1, words);  // halves of a word: tokens h = 0, 1 of one channel
-      const bool kept0 = (keep >> (2 * tig + 8 * r)) & 1u, kept1 = (keep >> (2 * tig + 8 * r + 1)) & 1u;
-      if (keep == kAllRows) store_words<BITS>(dst_tile + v_part_offset(BITS), r, lane, words);
-      else store_word_halves<BITS>(dst_tile + v_part_offset(BITS), r, lane, words, kept0, kept1);
-      if (g == 0) {  // record tig: S_V at bytes 32.., Z_V at 48.., entries 2 r + h
-        float *rec = reinterpret_cast<float *>(dst_tile + meta_offset(BITS) + tig * 64 + 32) + 2 * r;
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-          if (h == 0 ? kept0 : kept1) {
-            rec[h] = chain_scale(S[h], BITS, variant);
-            rec[4 + h] = chain_zero(Z[h], S[h], BITS, variant);
-          }
-      }
-    }
+  }
+  if (is_value) {
     smax = fmaxf(smax, __shfl_xor_sync(0xffffffffu, smax, 1));  // the four tig groups hold different tokens
     smax = fmaxf(smax, __shfl_xor_sync(0xffffffffu, smax, 2));
     if (lane == 0) atomicMax(vmax_slot, __float_as_uint(smax));  // scale >= 0: uint order = float order
@@ -574,7 +657,7 @@ __device__ __forceinline__ void append_tile_half_row(const uint16_t *__restrict_
       mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
       mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     }
-    const float s16 = quantize_owned<BITS, 32, true>(x, mn, mx, variant);
+    const float s16 = quantize_owned<BITS, 32>(x, mn, mx, variant);
     if (!is_value) {
       uint32_t words[words_per_lane];
 #pragma unroll
@@ -727,7 +810,8 @@ __device__ __forceinline__ void evict_tile_half(const uint8_t *src_tile, uint8_t
   uint8_t *dst = dst_tile + (is_value ? v_part_offset(BITS) : 0);
   uint4 in[8];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) in[q] = *reinterpret_cast<const uint4 *>(src + (q * 32 + lane) * 16);
+  for (int q = 0; q < 8; ++q)
+    if ((keep >> (8 * (q >> 2))) & 0xFFu) in[q] = *reinterpret_cast<const uint4 *>(src + (q * 32 + lane) * 16);
   const float *smeta = reinterpret_cast<const float *>(src_tile + meta_offset(16));
   float s16 = 0.f, z16 = 0.f;
   const int kind = is_value ? 2 : 0, row = lane & 15;
@@ -737,6 +821,8 @@ __device__ __forceinline__ void evict_tile_half(const uint8_t *src_tile, uint8_t
   }
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
+    const uint32_t keep8 = (keep >> (8 * r)) & 0xFFu;
+    if (keep8 == 0) continue;
     uint32_t words[BITS];
 #pragma unroll
     for (int w = 0; w < BITS; ++w) {
@@ -751,11 +837,11 @@ __device__ __forceinline__ void evict_tile_half(const uint8_t *src_tile, uint8_t
       }
       words[w] = __byte_perm(a, b, 0x5410);
     }
-    if (keep == kAllRows) {
+    if (keep8 == 0xFFu) {
       store_words<BITS>(dst, r, lane, words);
     } else {
-      const int g = lane >> 2, tig = lane & 3, row0 = is_value ? 2 * tig + 8 * r : g + 8 * r, row1 = is_value ? row0 + 1 : row0;
-      store_word_halves<BITS>(dst, r, lane, words, (keep >> row0) & 1u, (keep >> row1) & 1u);
+      const int g = lane >> 2, tig = lane & 3, row0 = is_value ? 2 * tig : g, row1 = is_value ? row0 + 1 : row0;
+      store_word_halves<BITS>(dst, r, lane, words, (keep8 >> row0) & 1u, (keep8 >> row1) & 1u);
     }
   }
   if (lane < 16 && ((keep >> row) & 1u)) store_meta(dst_tile, BITS, row, is_value, s16, z16, variant, false);
@@ -781,13 +867,18 @@ __device__ __forceinline__ void evict_tile_one(int is_value, int slice, int grou
 // leaving rows' own item leaves them out.
 // (Before, the window and the ragged ends went token by token, 16 times the warps, in three to four launches: 16.8 us per block
 // for a 2537-token prompt, 35 us for a chunk of 2048 tokens x 32 slices.)
+// What bounds it: a single wave is one chain of about 1000 instructions per warp, hence the split in parts and the 72
+// registers (with 64 the loop over the rounds spills: 7.9 against 6.4 us for 2537 tokens x 4 slices, one part). Large
+// prompts are bound by the fp32 pipe next to memory: 8192 tokens x 32 slices 49 us at 16 bit (5.5 TB/s), 47 us at 4 bit, where five
+// to eight CTAs per SM make no difference.  Persistent warps that load a tile ahead: 71 us.
 struct BulkParams {
   int n_old, n_after, win_start;  // tokens before and after, first token of the window afterwards
   int ev_first, ev_end;           // tokens that leave the window
   int ring_lo, body_lo, evict_lo; // first group of each kind, and the items of this and the kinds before it (ring items
   int ring_end, body_end, evict_end, sink_end;  // take longest and go first)
+  int parts;                      // warps per half item: 1, or 2 that take its rows 0 .. 7 and 8 .. 15
 };
-__global__ void __launch_bounds__(128, 8) append_bulk_kernel(const uint16_t *__restrict__ K, const uint16_t *__restrict__ V,
+__global__ void __launch_bounds__(128, 7) append_bulk_kernel(const uint16_t *__restrict__ K, const uint16_t *__restrict__ V,
                                                              const float *__restrict__ inv_lambda, unsigned *vmax_bits,
                                                              const LayerGeom geom, int n_slices, int kv_heads, int cur_bits,
                                                              const BulkParams bp) {
@@ -795,10 +886,13 @@ __global__ void __launch_bounds__(128, 8) append_bulk_kernel(const uint16_t *__r
   pdl_launch_next();
   pdl_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long wid = (long long)blockIdx.x * 4 + warp, per = 2ll * n_slices;
+  // (2^32 warps would move more than a terabyte)
+  const uint32_t wid = blockIdx.x * 4u + warp, per = bp.parts * 2u * n_slices;
   if (wid >= per * bp.sink_end) return;
   const int item = (int)(wid / per);
-  const int in_item = (int)(wid - item * per), is_value = in_item & 1, slice = in_item >> 1;
+  const int in_item = (int)(wid - item * per), is_value = in_item & 1, part = bp.parts == 2 ? (in_item >> 1) & 1 : 0;
+  const int slice = in_item >> bp.parts;
+  const uint32_t part_rows = bp.parts == 2 ? 0xFFu << (8 * part) : kAllRows;
   const int ring = geom.ring_tokens, ring_tiles = ring >> 4, first_new = max(bp.n_old, bp.win_start);  // first new window token
   const int row = lane & 15;
   if (item < bp.body_end) {
@@ -806,14 +900,15 @@ __global__ void __launch_bounds__(128, 8) append_bulk_kernel(const uint16_t *__r
     const int group = to_ring ? bp.ring_lo + item : bp.body_lo + item - bp.ring_end;
     const int t0 = geom.n_sink + group * kTileTokens, i0 = t0 - bp.n_old, t = t0 + row;
     const bool mine = to_ring ? t >= first_new && t < bp.n_after : t >= bp.n_old && t < bp.win_start;
-    const uint32_t keep = __ballot_sync(0xffffffffu, mine) & kAllRows;
+    const uint32_t keep = __ballot_sync(0xffffffffu, mine) & part_rows;
+    if (keep == 0) return;
     uint8_t *dst = geom.base + (size_t)slice * geom.slice_stride;
     int bits = 16;
     if (to_ring) {
       dst += geom.ring_off + (size_t)(group % ring_tiles) * tile_bytes(16);
       // the last group before this append in the same ring tile: its rows that leave the window and are overwritten here
       const int old = group - (max(i0, 0) / ring + 1) * ring_tiles, t_old = geom.n_sink + old * kTileTokens + row;
-      const uint32_t out = __ballot_sync(0xffffffffu, mine && t_old >= bp.ev_first && t_old < bp.ev_end) & kAllRows;
+      const uint32_t out = __ballot_sync(0xffffffffu, mine && t_old >= bp.ev_first && t_old < bp.ev_end) & part_rows;
       if (out) evict_tile_one(is_value, slice, old, geom, cur_bits, lane, out);
       __syncwarp();
     } else {
@@ -825,10 +920,10 @@ __global__ void __launch_bounds__(128, 8) append_bulk_kernel(const uint16_t *__r
   } else if (item < bp.evict_end) {
     const int group = bp.evict_lo + item - bp.body_end, t = geom.n_sink + group * kTileTokens + row;
     const int taker = t + max(1, (first_new - t + ring - 1) / ring) * ring;  // the new window token that lands in t's slot, if any
-    const uint32_t out = __ballot_sync(0xffffffffu, t >= bp.ev_first && t < bp.ev_end && taker >= bp.n_after) & kAllRows;
+    const uint32_t out = __ballot_sync(0xffffffffu, t >= bp.ev_first && t < bp.ev_end && taker >= bp.n_after) & part_rows;
     if (out) evict_tile_one(is_value, slice, group, geom, cur_bits, lane, out);
-  } else {
-    append_one(in_item, reinterpret_cast<uint16_t *>(s_scratch[warp]), lane, K, V, inv_lambda, vmax_bits, geom, n_slices, kv_heads, bp.n_old,
+  } else if (part == 0) {
+    append_one(slice * 2 + is_value, reinterpret_cast<uint16_t *>(s_scratch[warp]), lane, K, V, inv_lambda, vmax_bits, geom, n_slices, kv_heads, bp.n_old,
                bp.win_start, cur_bits, item - bp.evict_end, 1);
   }
 }

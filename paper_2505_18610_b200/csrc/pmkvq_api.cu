@@ -51,6 +51,7 @@ struct pmkvq_cache {
   size_t off_error;  // one word: bits set by a device-side wait that ran out
   int sink_tiles, ring_tiles, user_ctas;
   int resident_ctas[4];  // one wave of the attention kernel at body width 16, 8, 4, 2
+  int sms;
   int resident_fused;    // one wave of the all-blocks attention kernel
   uint64_t launches = 0;  // kernels launched so far
   std::vector<Layer> L;
@@ -225,6 +226,7 @@ cudaError_t attention_setup(pmkvq_cache *k) {
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  k->sms = sms;
   if (e == cudaSuccess) e = k->rows ? attention_setup_path<true>(k, sms) : attention_setup_path<false>(k, sms);
   return e;
 }
@@ -385,6 +387,10 @@ static BulkParams bulk_items(const pmkvq_cache &k, int n_old, int n_after, int w
   bp.body_end = bp.ring_end + groups(n_old, win_start, bp.body_lo);
   bp.evict_end = bp.body_end + groups(bp.ev_first, bp.ev_end, bp.evict_lo);
   bp.sink_end = bp.evict_end + std::max(0, std::min(n_after, k.n_sink) - n_old);
+  // Up to 24 warps per SM a half tile's two rounds of eight rows go to a warp each: nothing else fills the SM then, and a warp is
+  // one long chain (4 slices x 2537 tokens: 4.4 us against 6.4; x 6000, 20 warps per SM: 6.3 against 7.0; 32 slices x 700,
+  // 27 per SM: 7.3 against 7.9, but 4 x 8000, 27 per SM: 7.6 against 7.2, and 32 x 1000: 9.0 against 8.0).
+  bp.parts = 2ll * k.n_slices * bp.sink_end <= 24ll * k.sms ? 2 : 1;
   return bp;
 }
 
@@ -419,7 +425,7 @@ pmkvq_status pmkvq_append(pmkvq_cache *k, int32_t layer, const void *d_K, const 
                k->n_slices, k->kv_heads, n_old, new_win_start, l.cur_bits, ev_first, n_evict);
   } else if (!k->rows) {
     const BulkParams bp = bulk_items(*k, n_old, n_after, new_win_start, ev_first, n_evict);
-    e = launch(k->launches, append_bulk_kernel, four_warp_ctas(2ll * k->n_slices * bp.sink_end), 128, 0, st, K, V, inv_lam, vmax, g, k->n_slices,
+    e = launch(k->launches, append_bulk_kernel, four_warp_ctas(2ll * bp.parts * k->n_slices * bp.sink_end), 128, 0, st, K, V, inv_lam, vmax, g, k->n_slices,
                k->kv_heads, l.cur_bits, bp);
   } else {
     // row tiles: Values are inserted by read-modify-write of half-words that the tokens of a tile share, so the

@@ -79,3 +79,26 @@ def test_back_to_back_decode_steps_equal_separate_calls(context, batch, evict_ch
             for is_v in (False, True):
                 for x, y in zip(a.cache.export_slice(l, s // kvh, s % kvh, is_v), b.cache.export_slice(l, s // kvh, s % kvh, is_v)):
                     assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("shift_variant", [0, 1])
+@pytest.mark.parametrize("bits", [2, 4, 8, 16])
+@pytest.mark.parametrize("batch,sizes", [(1, (37, 250)), (32, (37, 700, 90, 513))])
+def test_appends_of_one_and_of_two_warps_per_half_tile(bits, batch, sizes, shift_variant):
+    """32 x 4 slices x 700 tokens take one warp per half tile, the rest two; constant tokens and scales outside the plain
+    quotient's range, alone and beside ordinary ones in a tile."""
+    total, kvh = sum(sizes), 4
+    k, v = make_inputs(11, 0, total, batch, kvh)
+    for t in (3, 40, 41, 130, 200):
+        k[t], v[t] = 0.75, -1.5
+    for t, f in ((5, 1e-25), (44, 1e25), (131, 1e-30), (201, 1e-36)):
+        k[t], v[t] = k[t] * f, v[t] * f
+    m = Mirror(1, kvh, kvh, batch, total, [bits], slices=sorted({0, 1, batch * kvh // 2, batch * kvh - 1}), window=64, evict_chunk=8,
+               shift_variant=shift_variant)
+    m.cache.restore_layer_state(0, 0, bits)
+    m.oracles[0].p.cur_bits = bits
+    done = 0
+    for n in sizes:
+        m.append(0, k[done:done + n], v[done:done + n])
+        done += n
+        m.check_state(0)
