@@ -76,7 +76,7 @@ struct AttnParams {
   int unit_weight;            // fine units per unit
   int cta_origin;             // first CTA that touches this block (partials are numbered from it)
   long long per_cta;          // fine units of a CTA's piece, and its reciprocal
-  double inv_per_cta;
+  unsigned long long inv_per_cta;
   float qk_scale;             // sm_scale * log2(e)
   int clean_tiles;            // body tiles below this one may be read before pdl_wait()
 };
@@ -443,14 +443,13 @@ __device__ __forceinline__ void process_tiles(const uint8_t *tile0, uint32_t mas
 // ---- where the partials of a slice live ------------------------------------------------------
 // Slice s covers units [s U, (s+1) U); the segment of CTA c in it publishes partial number (c - cta_origin) + s.
 // A unit belongs to the CTA whose piece holds the unit's first fine unit (per_cta counts fine units).  Fine units
-// are 64-bit numbers below 2^53: their quotients are taken as a double product (off by one at most) and put
-// right, a handful of instructions where a 64-bit division is a call of a hundred.
-__device__ __forceinline__ long long floor_div(long long x, long long d, double inv_d) {
-  long long q = (long long)((double)x * inv_d);
-  const long long r = x - q * d;
-  if (r < 0) --q;
-  else if (r >= d) ++q;
-  return q;
+// are 64-bit numbers below 2^53: their quotients are the high half of a product with the divisor's 64-bit reciprocal (one
+// too low at most) and put right, a dozen instructions where a 64-bit division is a call of a hundred (as a double
+// product two of them took 0.4 us at the start of every CTA).
+__host__ __device__ constexpr unsigned long long reciprocal64(unsigned long long d) { return ~0ull / d; }
+__device__ __forceinline__ long long floor_div(long long x, long long d, unsigned long long inv_d) {
+  const unsigned long long q = __umul64hi((unsigned long long)x, inv_d);
+  return (long long)q + ((unsigned long long)x - q * (unsigned long long)d >= (unsigned long long)d ? 1 : 0);
 }
 __device__ __forceinline__ int unit_owner(const AttnParams &p, int unit) {
   return (int)floor_div(p.line_origin + (long long)unit * p.unit_weight, p.per_cta, p.inv_per_cta);
@@ -462,10 +461,10 @@ __device__ __forceinline__ void slice_ctas(const AttnParams &p, int slice, int &
 }
 
 // Log-sum-exp merge of the n_parts partials of one slice (all published), the first one at `base`.  Warp w
-// merges head w; a lane owns 4 channels.  Partials are taken eight at a time with all their loads in flight
-// together, so up to eight cost one round trip to L2.
+// merges head w; a lane owns 4 channels.  Partials are taken sixteen at a time with all their loads in flight
+// together, so up to sixteen cost one round trip to L2; lane j looks after the reference and the sum of partial j.
 __device__ __forceinline__ void combine_slice(const AttnParams &p, int slice, const float *base, int n_parts) {
-  constexpr int kAtOnce = 8;
+  constexpr int kAtOnce = 16;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int b = slice / p.kv_heads, hkv = slice - b * p.kv_heads;
   for (int h = warp; h < p.group; h += kAttnWarps) {
@@ -473,28 +472,29 @@ __device__ __forceinline__ void combine_slice(const AttnParams &p, int slice, co
     float M = kNegBig, den = 0.f;
     float4 num = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int c0 = 0; c0 < n_parts; c0 += kAtOnce) {
-      float2 ml[kAtOnce];
+      const int n = min(kAtOnce, n_parts - c0);
+      const float *pc = ph + (size_t)c0 * (kMaxGroup * kPartialStride);
+      const float2 ml = __ldcg(reinterpret_cast<const float2 *>(pc + (size_t)min(lane, n - 1) * (kMaxGroup * kPartialStride)));
       float4 o4[kAtOnce];
 #pragma unroll
-      for (int j = 0; j < kAtOnce; ++j) {
-        const float *pc = ph + (size_t)min(c0 + j, n_parts - 1) * (kMaxGroup * kPartialStride);
-        ml[j] = __ldcg(reinterpret_cast<const float2 *>(pc));
-        o4[j] = __ldcg(reinterpret_cast<const float4 *>(pc + 4) + lane);
-      }
-      float m_new = M;
+      for (int j = 0; j < kAtOnce; ++j)
+        o4[j] = __ldcg(reinterpret_cast<const float4 *>(pc + (size_t)min(j, n - 1) * (kMaxGroup * kPartialStride) + 4) + lane);
+      float m_new = fmaxf(M, ml.x);  // (lanes beyond n hold the last partial again)
 #pragma unroll
-      for (int j = 0; j < kAtOnce; ++j) m_new = fmaxf(m_new, ml[j].x);
-      const float f = ex2(M - m_new);
-      den *= f; num.x *= f; num.y *= f; num.z *= f; num.w *= f;
+      for (int o = 16; o; o >>= 1) m_new = fmaxf(m_new, __shfl_xor_sync(0xffffffffu, m_new, o));
+      const float f = ex2(M - m_new), w_mine = lane < n ? ex2(ml.x - m_new) : 0.f;
       M = m_new;
+      den = fmaf(w_mine, ml.y, den * f);
+      num.x *= f; num.y *= f; num.z *= f; num.w *= f;
 #pragma unroll
       for (int j = 0; j < kAtOnce; ++j) {
-        const float w = c0 + j < n_parts ? ex2(ml[j].x - M) : 0.f;
-        den = fmaf(w, ml[j].y, den);
+        const float w = __shfl_sync(0xffffffffu, w_mine, j);  // 0 beyond n
         num.x = fmaf(w, o4[j].x, num.x); num.y = fmaf(w, o4[j].y, num.y);
         num.z = fmaf(w, o4[j].z, num.z); num.w = fmaf(w, o4[j].w, num.w);
       }
     }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) den += __shfl_xor_sync(0xffffffffu, den, o);
     const float inv = 1.0f / den;
     float4 *dst = reinterpret_cast<float4 *>(p.out + ((size_t)b * p.q_heads + hkv * p.group + h) * kHeadDim) + lane;
     *dst = make_float4(num.x * inv, num.y * inv, num.z * inv, num.w * inv);
@@ -536,27 +536,39 @@ __device__ __forceinline__ void fill_q_fragments(uint4 *s_frag, const float (*s_
 
 // ---- pieces of a segment that both contraction paths share --------------------------------------
 
+// The inputs of a segment's query, on their way: warp h < group holds head h, four channels per lane.  They are asked for
+// before the first tiles: 70 KB of tiles in front of them in the SM's queue delayed every segment by 1.2 us.
+struct QueryLoad {
+  uint2 raw;
+  float4 lam;
+};
+__device__ __forceinline__ QueryLoad load_query(const AttnParams &p, int b, int hkv) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  QueryLoad q;
+  q.raw = make_uint2(0u, 0u);
+  q.lam = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (warp < p.group) {
+    const uint16_t *src = p.Q + ((size_t)b * p.q_heads + hkv * p.group + warp) * kHeadDim + 4 * lane;
+    if ((reinterpret_cast<uintptr_t>(p.Q) & 7) == 0) {
+      q.raw = *reinterpret_cast<const uint2 *>(src);
+    } else {  // a caller's query tensor may sit at any bf16 address
+      q.raw.x = src[0] | ((uint32_t)src[1] << 16);
+      q.raw.y = src[2] | ((uint32_t)src[3] << 16);
+    }
+    q.lam = *reinterpret_cast<const float4 *>(p.lambda + hkv * kHeadDim + 4 * lane);
+  }
+  return q;
+}
 // Q'' = Q * lambda * sm_scale * log2(e)  (Eq. 9: the equalization scale migrates into Q), per-head
-// exponent of max |q''| and sum of q''.  Warp h takes head h, four channels per lane.  Ends with a CTA-wide barrier.
-__device__ __forceinline__ void build_query(const AttnParams &p, int b, int hkv, float (*s_q)[kHeadDim], float *s_stat) {
+// exponent of max |q''| and sum of q''.  Ends with a CTA-wide barrier.
+__device__ __forceinline__ void build_query(const AttnParams &p, const QueryLoad &q, float (*s_q)[kHeadDim], float *s_stat) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (warp < kMaxGroup) {
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (warp < p.group) {
-      const uint16_t *src = p.Q + ((size_t)b * p.q_heads + hkv * p.group + warp) * kHeadDim + 4 * lane;
-      uint2 raw;
-      if ((reinterpret_cast<uintptr_t>(p.Q) & 7) == 0) {
-        raw = *reinterpret_cast<const uint2 *>(src);
-      } else {  // a caller's query tensor may sit at any bf16 address
-        raw.x = src[0] | ((uint32_t)src[1] << 16);
-        raw.y = src[2] | ((uint32_t)src[3] << 16);
-      }
-      const float4 lam = *reinterpret_cast<const float4 *>(p.lambda + hkv * kHeadDim + 4 * lane);
-      v.x = __fmul_rn(__fmul_rn(__uint_as_float(raw.x << 16), lam.x), p.qk_scale);
-      v.y = __fmul_rn(__fmul_rn(__uint_as_float(raw.x & 0xFFFF0000u), lam.y), p.qk_scale);
-      v.z = __fmul_rn(__fmul_rn(__uint_as_float(raw.y << 16), lam.z), p.qk_scale);
-      v.w = __fmul_rn(__fmul_rn(__uint_as_float(raw.y & 0xFFFF0000u), lam.w), p.qk_scale);
-    }
+    float4 v;
+    v.x = __fmul_rn(__fmul_rn(__uint_as_float(q.raw.x << 16), q.lam.x), p.qk_scale);
+    v.y = __fmul_rn(__fmul_rn(__uint_as_float(q.raw.x & 0xFFFF0000u), q.lam.y), p.qk_scale);
+    v.z = __fmul_rn(__fmul_rn(__uint_as_float(q.raw.y << 16), q.lam.z), p.qk_scale);
+    v.w = __fmul_rn(__fmul_rn(__uint_as_float(q.raw.y & 0xFFFF0000u), q.lam.w), p.qk_scale);
     *reinterpret_cast<float4 *>(&s_q[warp][4 * lane]) = v;
     float mx = fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
     float sm = (v.x + v.y) + (v.z + v.w);
@@ -658,19 +670,20 @@ __device__ __forceinline__ float *partial_slot(const AttnParams &p, int slice) {
 }
 
 // The segment's partial is written (by all threads): count it, and let the CTA that publishes the slice's last
-// partial merge the slice (nobody waits).  One thread's fence after the CTA-wide barrier covers the whole CTA's
-// stores (barrier and fence order them cumulatively); a fence in every thread costs a microsecond.
+// partial merge the slice (nobody waits).  One thread's release after the CTA-wide barrier covers the whole CTA's
+// stores (barrier and release order them cumulatively); a fence in every thread costs a microsecond.
 __device__ __forceinline__ void publish_partial(const AttnParams &p, int slice, int *s_ctr) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned t = atomicAdd(p.tickets + slice, 1u);
+  if (threadIdx.x == 32) {
     int cf, cl;
     slice_ctas(p, slice, cf, cl);
-    s_ctr[2] = (t + 1u == (unsigned)(cl - cf + 1)) ? 1 : 0;
     s_ctr[3] = cl - cf + 1;
     s_ctr[4] = cf;
-    __threadfence();
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned t;
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;\n" : "=r"(t) : "l"(p.tickets + slice) : "memory");
+    s_ctr[2] = t + 1u == (unsigned)s_ctr[3] ? 1 : 0;
   }
   __syncthreads();
   if (s_ctr[2]) {
@@ -855,6 +868,7 @@ __device__ __forceinline__ void run_segment(const AttnParams &p, int slice, int 
       }
     }
   };
+  const QueryLoad query = load_query(p, b, hkv);
   int u = 0;
   const uint8_t *src = nullptr;
   if constexpr (F::SLOTS > 0) {
@@ -866,7 +880,7 @@ __device__ __forceinline__ void run_segment(const AttnParams &p, int slice, int 
   if constexpr (kDealt)
     for (int it = a_lo + warp; it < a_hi; it += kAttnWarps) prefetch_l2(int16_tile(p, slice_base, it), tile_bytes(16), lane);
 
-  build_query(p, b, hkv, s_q, s_stat);
+  build_query(p, query, s_q, s_stat);
   const int e_g = (int)s_stat[g];
   const float sumq = s_stat[8 + g];
   fill_q_fragments<16>(s_frag, s_q, s_stat);  // half of the threads each
@@ -995,7 +1009,7 @@ __device__ __forceinline__ void run_segment_tc(const AttnParams &p, int slice, i
   segment_ranges<BITS>(p, u_lo, u_hi, a_lo, a_hi, t_lo, t_hi);
   const uint8_t *slice_base = p.geom.base + (size_t)slice * p.geom.slice_stride;
 
-  build_query(p, b, hkv, s_q, s_stat);
+  build_query(p, load_query(p, b, hkv), s_q, s_stat);
   if (a_hi > a_lo) fill_q_fragments<16>(s_frag, s_q, s_stat);
   if (t_hi > t_lo) {
     fill_q_operand<BITS>(tc.q_operand, s_q, s_stat);
@@ -1139,7 +1153,7 @@ struct FusedParams {
   int behind_append;
   float qk_scale;
   long long per_cta, total;              // fine units
-  double inv_per_cta;
+  unsigned long long inv_per_cta;
   long long start[kMaxFusedLayers + 1];  // fine units before each block
   int n_tokens[kMaxFusedLayers], n_body[kMaxFusedLayers];
   short cta_origin[kMaxFusedLayers];     // first CTA whose piece reaches into the block
@@ -1156,7 +1170,9 @@ __host__ __device__ constexpr int tile_weight(int bits) { return bits == 16 ? 15
 // body tiles of each width: about 12 us at the measured per-SM tile rates.
 __host__ __device__ constexpr int segment_cost_tiles(int bits) { return bits == 16 ? 48 : bits == 8 ? 96 : bits == 4 ? 176 : 160; }
 __host__ __device__ constexpr int int16_units(int bits) { return (tile_bytes(16) + tile_bytes(bits) - 1) / tile_bytes(bits); }
-__device__ __forceinline__ double inv_tile_weight(int bits) { return bits == 16 ? 1.0 / tile_weight(16) : bits == 8 ? 1.0 / tile_weight(8) : bits == 4 ? 1.0 / tile_weight(4) : 1.0 / tile_weight(2); }
+__device__ __forceinline__ unsigned long long inv_tile_weight(int bits) {
+  return bits == 16 ? reciprocal64(tile_weight(16)) : bits == 8 ? reciprocal64(tile_weight(8)) : bits == 4 ? reciprocal64(tile_weight(4)) : reciprocal64(tile_weight(2));
+}
 
 __device__ __forceinline__ void fused_layer_params(const FusedParams &fp, int l, AttnParams &p) {
   const int n = fp.n_tokens[l], bits = fp.bits[l];
@@ -1209,7 +1225,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) decode_attn_fused_kernel(cons
     fused_layer_params(fp, l, p);
     // units of this block whose first fine unit lies in the piece
     const int w = p.unit_weight;
-    const double inv_w = inv_tile_weight(p.cur_bits);
+    const unsigned long long inv_w = inv_tile_weight(p.cur_bits);
     const int u_begin = (int)floor_div(max(f_begin - p.line_origin, 0ll) + w - 1, w, inv_w);
     const int u_end = (int)floor_div(min(f_end, fp.start[l + 1]) - p.line_origin + w - 1, w, inv_w);
     int slice = u_begin / p.units_slice;

@@ -492,7 +492,7 @@ static pmkvq_status attn_params(pmkvq_cache *k, int32_t layer, const void *d_Q, 
   const int width_idx = l.cur_bits == 16 ? 0 : l.cur_bits == 8 ? 1 : l.cur_bits == 4 ? 2 : 3;
   const int want = k->user_ctas > 0 ? k->user_ctas : k->resident_ctas[width_idx];
   p.per_cta = std::max<long long>((total + want - 1) / want, k->user_ctas > 0 ? 1 : kMinUnitsPerCta);
-  p.inv_per_cta = 1.0 / (double)p.per_cta;
+  p.inv_per_cta = reciprocal64((unsigned long long)p.per_cta);
   p.line_origin = 0;
   p.unit_weight = 1;
   p.cta_origin = 0;
@@ -569,7 +569,7 @@ static pmkvq_status attention_all_blocks(pmkvq_cache *k, const void *d_Q, float 
   // partial, which is what the slice's ticket count expects.
   fp.per_cta = std::max<long long>((total + want - 1) / want,
                                    k->user_ctas > 0 ? (long long)tile_weight(16) : 50ll * kMinUnitsPerCta);
-  fp.inv_per_cta = 1.0 / (double)fp.per_cta;
+  fp.inv_per_cta = reciprocal64((unsigned long long)fp.per_cta);
   const unsigned n_ctas = (unsigned)((total + fp.per_cta - 1) / fp.per_cta);
   for (int l = 0; l < k->layers; ++l) fp.cta_origin[l] = (short)(fp.start[l] / fp.per_cta);
   int l0 = 0;
