@@ -1100,8 +1100,13 @@ __device__ __forceinline__ void tc_teardown(TcCtx &tc) {
   if ((threadIdx.x >> 5) == 0) tc05::tmem_dealloc(tc.tmem_base, kTmemCols);
 }
 
+// Registers: with 128 per thread a CTA holds all of an SM's, and the append behind or in front of it gets no SM until
+// it has left; 112 leave room for one of its CTAs (64 registers, one warp per scheduler).  16 slices x 9K tokens at 16 bit block by
+// block: 25.0 -> 24.8 us per append and attention; 28 blocks x 4 slices x 3K tokens 42.7 -> 42.3 us per step.  At 4 and 2 bit the 16
+// registers are worth more (128 slices x 64K tokens at 2 bit, append and attention: 196 us, 203 with 112).
+constexpr int attn_registers(int bits) { return bits >= 8 ? 112 : 128; }
 template <int BODY_BITS, bool ROWS>
-__global__ void __launch_bounds__(kAttnThreads, 1) decode_attn_splitk_kernel(const AttnParams p, unsigned *error_word) {
+__global__ void __maxnreg__(attn_registers(BODY_BITS)) decode_attn_splitk_kernel(const AttnParams p, unsigned *error_word) {
   __shared__ __align__(16) float s_q[kMaxGroup][kHeadDim];
   __shared__ __align__(16) float s_stat[16 + 2 * kParts * kMaxGroup];  // head stats, per-partial (m, l)
   __shared__ int s_ctr[5];                                // work counters (INT16 tiles, body tiles), combine flag and range
@@ -1206,7 +1211,7 @@ __device__ __forceinline__ void fused_layer_params(const FusedParams &fp, int l,
 }
 
 template <bool ROWS>
-__global__ void __launch_bounds__(kAttnThreads, 1) decode_attn_fused_kernel(const __grid_constant__ FusedParams fp) {
+__global__ void __maxnreg__(112) decode_attn_fused_kernel(const __grid_constant__ FusedParams fp) {
   __shared__ __align__(16) float s_q[kMaxGroup][kHeadDim];
   __shared__ __align__(16) float s_stat[16 + 2 * kParts * kMaxGroup];
   __shared__ int s_ctr[5];
