@@ -1168,8 +1168,10 @@ struct FusedParams {
 static_assert(kMaxFusedLayers <= 256 && sizeof(FusedParams) <= 4096, "block numbers are bytes; kernel parameters fit one 4 KB bank");
 
 // What a tile of each width weighs, in fine units, and the lead of a slice in tiles (see segment_cost_tiles).
-// Time per 16-token tile at each width, in fiftieths of a 2-bit tile's (measured: 52.6 / 55.4 / 84.1 us per
-// block of 130 560 tiles at 2 / 4 / 8 bit, about 160 us at 16 bit).
+// Time per 16-token tile at each width, in fiftieths of a 2-bit tile's, at the clock a long run settles at under the power cap
+// (2 and 4 bit, bound by instructions, slow down with it).  The ratios at full clock (45.2 / 49.7 / 80.6 / 157.7 us per block of
+// 130 560 tiles at 2 / 4 / 8 / 16 bit, i.e. 50 / 55 / 89 / 174) make mixed launches slower: 20 blocks at 2 and 8 at 4 bit
+// 2965 -> 2982 us for two steps, 8 and 4 bit mixed 756 -> 764 us for four.
 __host__ __device__ constexpr int tile_weight(int bits) { return bits == 16 ? 152 : bits == 8 ? 80 : bits == 4 ? 53 : 50; }
 // Fixed cost of one more segment (set-up, warp merge, publish, its share of the slice combine), in
 // body tiles of each width: about 12 us at the measured per-SM tile rates.
