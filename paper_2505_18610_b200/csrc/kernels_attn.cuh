@@ -907,8 +907,9 @@ __device__ __forceinline__ void run_segment(const AttnParams &p, int slice, int 
   };
   // ---- INT16 tiles (sink + window ring) before the body ----
   if constexpr (!kDealt) pdl_wait();  // they are what the append in front of this launch may have written
-  // The slice's largest INT16 V scale; at 2 and 4 bit perhaps before that append has raised it: every body token is older.
-  const float sigma_body = slice_sigma16(p, slice);
+  // The slice's largest INT16 V scale; at 2 and 4 bit perhaps before that append has raised it: with a window every body token is
+  // older (without one the launch has waited).  One lane's reading for the warp: its lanes' weights meet in one sum.
+  const float sigma_body = __shfl_sync(0xffffffffu, slice_sigma16(p, slice), 0);
   if constexpr (!kDealt) {
     if (a_hi > a_lo) {
       run_int16_tiles(p, slice_base, a_lo, a_hi, st, s_frag, s_ctr, e_g, sumq, sigma_body, lane);
@@ -1153,8 +1154,8 @@ struct FusedParams {
   size_t partial_stride;
   int layers, kv_heads, group, q_heads, n_slices, batch;
   int n_sink, sink_tiles, aux_tiles, evict_chunk;
-  // 1: this launch sits right behind append_step_kernel in its stream.  That kernel lets us start only once everything
-  // before it is complete, so the queries and the tiles it cannot touch may be read while it still runs.
+  // 1: this launch sits right behind append_step_kernel in its stream, in a cache with a window.  That kernel lets us start only
+  // once everything before it is complete, so the queries and the tiles it cannot touch may be read while it still runs.
   int behind_append;
   float qk_scale;
   long long per_cta, total;              // fine units

@@ -545,7 +545,9 @@ static pmkvq_status attention_all_blocks(pmkvq_cache *k, const void *d_Q, float 
   fp.layers = k->layers; fp.kv_heads = k->kv_heads; fp.group = k->group; fp.q_heads = k->q_heads;
   fp.n_slices = k->n_slices; fp.batch = k->batch;
   fp.n_sink = k->n_sink; fp.evict_chunk = k->evict_chunk;
-  fp.behind_append = behind_append ? 1 : 0;
+  // Without a window the append puts the new token straight into the body and raises the slice's largest V scale, which the
+  // body's unit at 2 and 4 bit is taken from before the wait: the launch then waits at its start.
+  fp.behind_append = behind_append && k->window > 0 ? 1 : 0;
   fp.sink_tiles = k->sink_tiles; fp.aux_tiles = k->sink_tiles + k->ring_tiles;
   fp.qk_scale = k->sm_scale * 1.4426950408889634f;
   long long total = 0;
