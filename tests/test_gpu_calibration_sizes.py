@@ -24,3 +24,16 @@ def test_absmax_work_split_edges(n_tokens, n_seq, kv_heads, offset):
     got = B.calibrate_lambda(k, pos_scale=2.0, alpha=1.0).cpu().numpy()
     # fp32 rotation from correctly rounded angles: two products and a sum, each within half an ulp, and the power
     assert np.allclose(got, want, rtol=2e-6, atol=0)
+
+
+def test_calibration_reads_a_nan_as_a_channel_without_a_maximum():
+    """A channel that saw a NaN gets the floor, whatever else it saw; the others keep their maxima."""
+    from paper_2505_18610_b200 import binding as B
+    k = torch.randn(9, 5, 3, 128, generator=torch.Generator().manual_seed(4)).bfloat16()
+    clean = B.calibrate_lambda(k.cuda(), alpha=1.0, floor_value=0.125).cpu()
+    k[0, 2, 1, 7] = float("nan")                     # channels 7 and 71 are rotated into one another
+    k[8, 4, 2, 100] = float("nan")
+    got = B.calibrate_lambda(k.cuda(), alpha=1.0, floor_value=0.125).cpu()
+    want = clean.clone()
+    want[1, 7] = want[1, 71] = want[2, 36] = want[2, 100] = 0.125
+    assert torch.equal(got, want)
