@@ -376,7 +376,8 @@ __device__ __forceinline__ TokenScale two_tokens(float2 mn, float2 mx) {
   TokenScale t;
   token_scale(mn.x, mx.x, t.nmn.x, t.s.x, t.ns.x, t.y.x, t.yl.x);
   token_scale(mn.y, mx.y, t.nmn.y, t.s.y, t.ns.y, t.y.y, t.yl.y);
-  t.plain = fminf(t.s.x, t.s.y) >= 0x1p-60f && fmaxf(t.s.x, t.s.y) <= 0x1p60f;
+  // each on its own: the minimum and the maximum of the two would pass over a NaN (infinities only, NaNs only)
+  t.plain = t.s.x >= 0x1p-60f && t.s.x <= 0x1p60f && t.s.y >= 0x1p-60f && t.s.y <= 0x1p60f;
   return t;
 }
 // the codes of both values, one in each half of the result

@@ -6,6 +6,7 @@ import numpy as np
 import pytest
 import torch
 
+from paper_2505_18610_b200 import binding as B
 from paper_2505_18610_b200 import synth
 from tests.helpers import Mirror, make_inputs
 
@@ -102,3 +103,24 @@ def test_appends_of_one_and_of_two_warps_per_half_tile(bits, batch, sizes, shift
         m.append(0, k[done:done + n], v[done:done + n])
         done += n
         m.check_state(0)
+
+
+@pytest.mark.parametrize("bits", [2, 4, 8, 16])
+@pytest.mark.parametrize("value", [float("inf"), -float("inf"), float("nan")])
+def test_bulk_append_of_a_token_without_a_scale(bits, value):
+    """A Value vector of infinities or NaNs has no scale: its codes are 0 as in the token-by-token append, and the token it shares
+    words with is not touched."""
+    n = 40
+    k, v = make_inputs(33, 0, n, 1, 1)
+    v[5], v[36] = value, value                       # one in the body, one in the window
+    v[20], v[21] = value, 0.25                       # beside a constant token
+    caches = [B.Cache(1, 1, 1, 1, n, [bits], window=16) for _ in range(2)]
+    for c in caches:
+        c.restore_layer_state(0, 0, bits)
+    k, v = k.cuda(), v.cuda()
+    caches[0].append(0, k, v)
+    for t in range(n):
+        caches[1].append(0, k[t], v[t])
+    for is_v in (False, True):
+        for x, y in zip(*(c.export_slice(0, 0, 0, is_v) for c in caches)):
+            assert np.array_equal(x, y, equal_nan=x.dtype.kind == "f")
