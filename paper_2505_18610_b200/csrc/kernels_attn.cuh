@@ -587,10 +587,11 @@ __device__ __forceinline__ void build_query(const AttnParams &p, const QueryLoad
   __syncthreads();
 }
 
-// unit of the V accumulators: a power of two >= every INT16 V scale of this slice
+// unit of the V accumulators: a power of two >= every INT16 V scale of this slice; 1 when there is none, or when a Value that was
+// not finite has been here (the largest scale outlives a token that is rolled back)
 __device__ __forceinline__ float slice_sigma16(const AttnParams &p, int slice) {
   const unsigned s16 = __ldcg(p.vmax_bits + slice);  // a non-negative float's bit pattern
-  return s16 ? exp2i(max(-126, (int)(s16 >> 23) - 126)) : 1.0f;
+  return s16 && s16 < 0x7F800000u ? exp2i(max(-126, (int)(s16 >> 23) - 126)) : 1.0f;
 }
 
 __device__ __forceinline__ const uint8_t *int16_tile(const AttnParams &p, const uint8_t *slice_base, int it) {
