@@ -578,8 +578,8 @@ __device__ __forceinline__ void build_query(const AttnParams &p, const QueryLoad
       sm += __shfl_xor_sync(0xffffffffu, sm, o);
     }
     if (lane == 0) {
-      // mx = f * 2^e, f in [0.5, 1); the bounds keep every power of two built from e a normal number
-      const int e = mx > 0.f ? max(-100, min(110, (int)(__float_as_uint(mx) >> 23) - 126)) : 0;
+      // mx = f * 2^e, f in [0.5, 1); the bounds keep every power of two built from e a normal number (24 - EQ + e <= 127)
+      const int e = mx > 0.f ? max(-100, min(117, (int)(__float_as_uint(mx) >> 23) - 126)) : 0;
       s_stat[warp] = (float)e;
       s_stat[8 + warp] = sm;
     }

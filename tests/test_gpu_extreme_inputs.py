@@ -1,5 +1,6 @@
 """Numbers at the ends of their range in decode attention: Values that are not finite, queries near the largest exponent the kernels
 carry."""
+import numpy as np
 import pytest
 import torch
 
@@ -23,3 +24,17 @@ def test_rolled_back_token_with_infinite_value(bits, attention_path):
     m.cache.restore_layer_state(0, n, bits)
     q = torch.randn(1, group * kvh, 128, generator=torch.Generator().manual_seed(3)).bfloat16()
     m.check_attention(0, q)
+
+
+@pytest.mark.parametrize("bits", [2, 4, 8, 16])
+@pytest.mark.parametrize("d", [0, 3, 5])
+def test_queries_up_to_two_to_the_116(bits, d, attention_path):
+    """Tiny Keys and huge queries whose scores are ordinary: Q * lambda * scale * log2(e) reaches 2^(110 + d) and the cache holds
+    Keys of 2^-(112 + d), INT16 scales around 2^-(122 + d)."""
+    n, kvh, group = 500, 1, 4
+    k, v = make_inputs(31, 0, n, 1, kvh)
+    q = torch.randn(1, group, 128, generator=torch.Generator().manual_seed(2))
+    m = Mirror(1, group, kvh, 1, n, [bits], lam=np.full((1, kvh, 128), 2.0 ** 10, np.float32), window=32, attention_path=attention_path)
+    m.append(0, (k.float() * 2.0 ** -(102 + d)).to(torch.bfloat16), v)
+    m.check_state(0)
+    m.check_attention(0, (q * 2.0 ** (102 + d)).to(torch.bfloat16))
