@@ -91,9 +91,11 @@ __global__ void __launch_bounds__(kAbsmaxThreads, 3) calib_absmax_kernel(const u
             for (int v = 0; v < 2; ++v) {
               const float2 x1 = make_float2(__uint_as_float(a[v][j] << 16), __uint_as_float(a[v][j] & 0xFFFF0000u));
               const float2 x2 = make_float2(__uint_as_float(b[v][j] << 16), __uint_as_float(b[v][j] & 0xFFFF0000u));
-              const float2 xs = __fmul2_rn(x2, sn[j]);
-              y1[v] = __fadd2_rn(__fmul2_rn(x1, cs[j]), make_float2(-xs.x, -xs.y));  // Eq. 11 with the scaled position
-              y2[v] = __fadd2_rn(__fmul2_rn(x1, sn[j]), __fmul2_rn(x2, cs[j]));
+              // Eq. 11 with the scaled position; the sums one by one, since a packed sum of packed products comes out as a fused
+              // multiply-add, which is another number than the sum of two rounded products
+              const float2 c1 = __fmul2_rn(x1, cs[j]), s2 = __fmul2_rn(x2, sn[j]), s1 = __fmul2_rn(x1, sn[j]), c2 = __fmul2_rn(x2, cs[j]);
+              y1[v] = make_float2(__fsub_rn(c1.x, s2.x), __fsub_rn(c1.y, s2.y));
+              y2[v] = make_float2(__fadd_rn(s1.x, c2.x), __fadd_rn(s1.y, c2.y));
             }
             m1[j].x = max_abs_or_nan(m1[j].x, y1[0].x, y1[1].x); m1[j].y = max_abs_or_nan(m1[j].y, y1[0].y, y1[1].y);
             m2[j].x = max_abs_or_nan(m2[j].x, y2[0].x, y2[1].x); m2[j].y = max_abs_or_nan(m2[j].y, y2[0].y, y2[1].y);

@@ -37,3 +37,18 @@ def test_calibration_reads_a_nan_as_a_channel_without_a_maximum():
     want = clean.clone()
     want[1, 7] = want[1, 71] = want[2, 36] = want[2, 100] = 0.125
     assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("t", [1, 5, 100, 1500])
+def test_rotation_of_one_token_bit_for_bit(t):
+    """Two products, each rounded, and their rounded sum: the Key that pmkvq_append would be given."""
+    from paper_2505_18610_b200 import binding as B
+    k = torch.zeros(t + 1, 1, 8, 128)
+    k[t] = torch.randn(1, 8, 128, generator=torch.Generator().manual_seed(t))
+    k = k.bfloat16()
+    angle = np.float64(t) * 10000.0 ** (-2.0 * np.arange(64) / 128)
+    c, s = np.cos(angle).astype(np.float32), np.sin(angle).astype(np.float32)
+    x1, x2 = k[t, 0, :, :64].float().numpy(), k[t, 0, :, 64:].float().numpy()
+    want = np.abs(np.concatenate([x1 * c - x2 * s, x1 * s + x2 * c], -1))
+    got = B.calibrate_lambda(k.cuda(), alpha=1.0, floor_value=1e-30).cpu().numpy()
+    assert np.array_equal(got, want)
