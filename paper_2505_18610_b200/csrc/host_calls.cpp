@@ -110,6 +110,7 @@ PyObject *decode_attention(PyObject *, PyObject *const *a, Py_ssize_t n) {
   const at::Tensor *out = &made;
   if (a[5] == Py_None) made = at::empty({batch, heads, 128}, q->options().dtype(at::kFloat));
   else if (!(out = tensor_arg(a[5], at::kFloat, "out"))) return nullptr;
+  if (out->numel() < q->numel()) return value_error("bad out shape");  // (a larger one has always been taken: its head is written)
   if (!stream_arg(a[6], st)) return nullptr;
   const void *qp = q->data_ptr();
   float *op = static_cast<float *>(out->data_ptr());

@@ -74,3 +74,21 @@ def test_shapes_outputs_and_streams():
     c.close()
     with pytest.raises(B.PmkvqError):
         c.append(0, k, v)
+
+
+@pytest.mark.gpu
+def test_an_output_too_small_for_the_result_is_refused():
+    c = B.Cache(1, 8, 2, 3, 64, [4], window=16)
+    k = torch.randn(20, 3, 2, 128, device="cuda").bfloat16()
+    q = torch.randn(3, 8, 128, device="cuda").bfloat16()
+    c.append(0, k, k)
+    launches = c.launch_count()
+    for shape in ((3, 8, 127), (2, 8, 128), (0,)):
+        with pytest.raises(ValueError, match="bad out shape"):
+            c.decode_attention(0, q, out=torch.empty(shape, device="cuda"))
+    assert c.launch_count() == launches
+    want = c.decode_attention(0, q)
+    large = torch.zeros(4 * 8 * 128, device="cuda")
+    assert c.decode_attention(0, q, out=large) is large
+    torch.testing.assert_close(large[:want.numel()], want.flatten(), rtol=0, atol=4 * 2.0 ** -11)   # as in `same` above
+    assert not large[want.numel():].any()
