@@ -101,7 +101,8 @@ pmkvq_status pmkvq_progressive_reduce(pmkvq_cache *cache, int32_t layer, void *s
 
 /* Decode-step attention of one block over all cached tokens (the one just appended included):
  * out = softmax(sm_scale * (Q Lambda) dequant(K Lambda^-1)^T) dequant(V)  (Eq. 9 with GQA).
- *   d_Q_bf16: DEVICE bf16 [batch][q_heads][128]; d_out: DEVICE fp32 [batch][q_heads][128].
+ *   d_Q_bf16: DEVICE bf16 [batch][q_heads][128]; d_out: DEVICE fp32 [batch][q_heads][128], on a 16-byte boundary
+ *   (INVALID_ARG otherwise, here and in the calls below; nothing is launched or appended).
  * A block without any cached token has no softmax to take: INVALID_ARG, nothing is launched. */
 pmkvq_status pmkvq_decode_attention(pmkvq_cache *cache, int32_t layer, const void *d_Q_bf16, float *d_out,
                                     void *stream);

@@ -458,10 +458,13 @@ pmkvq_status pmkvq_append(pmkvq_cache *k, int32_t layer, const void *d_K, const 
 
 }  // extern "C"
 
+// The outputs are written sixteen bytes at a time.
+static bool output_address(const float *d_out) { return d_out && (reinterpret_cast<uintptr_t>(d_out) & 15) == 0; }
+
 // Everything of one attention launch except where its split-K scratch lives.
 static pmkvq_status attn_params(pmkvq_cache *k, int32_t layer, const void *d_Q, float *d_out, AttnParams &p,
                                 unsigned &n_ctas) {
-  if (!k || layer < 0 || layer >= k->layers || !d_Q || !d_out) return PMKVQ_ERR_INVALID_ARG;
+  if (!k || layer < 0 || layer >= k->layers || !d_Q || !output_address(d_out)) return PMKVQ_ERR_INVALID_ARG;
   const Layer &l = k->L[layer];
   if (l.n_tokens <= 0) return PMKVQ_ERR_INVALID_ARG;
   p.geom = k->geom(l);
@@ -613,7 +616,7 @@ pmkvq_status pmkvq_decode_attention_static(pmkvq_cache *k, int32_t layer, const 
 
 pmkvq_status pmkvq_decode_step(pmkvq_cache *k, const void *d_K, const void *d_V, const void *d_Q, float *d_out,
                                void *stream) {
-  if (!k || !d_K || !d_V || !d_Q || !d_out) return PMKVQ_ERR_INVALID_ARG;
+  if (!k || !d_K || !d_V || !d_Q || !output_address(d_out)) return PMKVQ_ERR_INVALID_ARG;
   if ((reinterpret_cast<uintptr_t>(d_K) | reinterpret_cast<uintptr_t>(d_V)) & 7) return PMKVQ_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t kv_stride = (size_t)k->n_slices * kHeadDim * 2;            // bytes of one block's bf16 K (or V)
@@ -665,7 +668,7 @@ pmkvq_status pmkvq_decode_step(pmkvq_cache *k, const void *d_K, const void *d_V,
 }
 
 pmkvq_status pmkvq_decode_attention_all(pmkvq_cache *k, const void *d_Q, float *d_out, void *stream) {
-  if (!k || !d_Q || !d_out) return PMKVQ_ERR_INVALID_ARG;
+  if (!k || !d_Q || !output_address(d_out)) return PMKVQ_ERR_INVALID_ARG;
   if (k->layers > kMaxFusedLayers) return PMKVQ_ERR_INVALID_ARG;
   return attention_all_blocks(k, d_Q, d_out, static_cast<cudaStream_t>(stream), false);
 }

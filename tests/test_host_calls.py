@@ -92,3 +92,24 @@ def test_an_output_too_small_for_the_result_is_refused():
     assert c.decode_attention(0, q, out=large) is large
     torch.testing.assert_close(large[:want.numel()], want.flatten(), rtol=0, atol=4 * 2.0 ** -11)   # as in `same` above
     assert not large[want.numel():].any()
+
+
+@pytest.mark.gpu
+def test_an_output_off_a_16_byte_boundary_is_refused():
+    c = B.Cache(2, 2, 1, 1, 64, [4, 4])
+    k = torch.randn(20, 1, 1, 128, device="cuda").bfloat16()
+    q = torch.randn(2, 1, 2, 128, device="cuda").bfloat16()
+    for layer in range(2):
+        c.append(layer, k, k)
+    launches = c.launch_count()
+    buf = torch.zeros(2 * 2 * 128 + 4, device="cuda")
+    for off in (1, 2, 3):
+        one, two = buf[off:off + 256].view(1, 2, 128), buf[off:off + 512].view(2, 1, 2, 128)
+        for call in (lambda: c.decode_attention(0, q[0], out=one), lambda: c.decode_attention_static(0, q[0], one),
+                     lambda: c.decode_attention_all(q, out=two), lambda: c.decode_step(k[:2], k[:2], q, out=two)):
+            with pytest.raises(B.PmkvqError) as e:
+                call()
+            assert e.value.status == B.INVALID_ARG
+    assert c.launch_count() == launches and c.layer_state(0)["n_tokens"] == c.layer_state(1)["n_tokens"] == 20
+    got = c.decode_attention_all(q, out=buf[4:].view(2, 1, 2, 128))
+    torch.testing.assert_close(got, c.decode_attention_all(q), rtol=0, atol=4 * 2.0 ** -11)
