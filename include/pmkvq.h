@@ -229,7 +229,7 @@ pmkvq_status pmkvq_calibrate_lambda(const void *d_K_pre_bf16, int32_t n_tokens, 
  * alphas (per alpha at 16 bit).  The attention launches wait on hardware barriers with a limit, as pmkvq_device_status
  * describes: a wait that runs out returns PMKVQ_ERR_DEVICE_WAIT here.
  *   d_K_pre_bf16, d_V_bf16  DEVICE bf16 [n_tokens][n_seq][kv_heads][128]; Keys before RoPE, token t at position t
- *   d_Q_pre_bf16            DEVICE bf16 [n_tokens][n_seq][kv_heads * group][128], before RoPE
+ *   d_Q_pre_bf16            DEVICE bf16 [n_tokens][n_seq][kv_heads * group][128], before RoPE; all three at any bf16 address
  *   bits                    2, 4, 8 or 16: the width whose loss is minimised (the block's Fbit)
  *   h_alphas                HOST [n_alphas], 1 <= n_alphas <= 64 (the section's grid: j / 20, j = 0..19)
  *   d_workspace             DEVICE, 256-byte aligned, pmkvq_alpha_grid_workspace_bytes(...) bytes of the same sizes

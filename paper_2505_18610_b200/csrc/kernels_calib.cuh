@@ -231,8 +231,10 @@ __device__ __forceinline__ void quantize_token_centred(float (&x)[4], int bits, 
   zero = fmaf(scale, half, mn);
 }
 
-__device__ __forceinline__ void load_bf16x4(const uint16_t *src, float (&x)[4]) {
-  const uint2 raw = *reinterpret_cast<const uint2 *>(src);
+__device__ __forceinline__ void load_bf16x4(const uint16_t *src, bool aligned, float (&x)[4]) {
+  uint2 raw;
+  if (aligned) raw = *reinterpret_cast<const uint2 *>(src);
+  else raw = make_uint2(src[0] | ((uint32_t)src[1] << 16), src[2] | ((uint32_t)src[3] << 16));  // a caller's tensor may sit at any bf16 address
   x[0] = __uint_as_float(raw.x << 16);
   x[1] = __uint_as_float(raw.x & 0xFFFF0000u);
   x[2] = __uint_as_float(raw.y << 16);
@@ -275,11 +277,12 @@ __global__ void __launch_bounds__(256) alpha_grid_prep_kernel(const GridPrep p) 
   const int n_tiles = (p.n_tokens + kGridTile - 1) / kGridTile;
   const int tile = (int)(blockIdx.x % (unsigned)n_tiles), slice = (int)(blockIdx.x / (unsigned)n_tiles), n_slices = p.n_seq * p.kv_heads;
   const int t0 = tile * kGridTile, rows = min(kGridTile, p.n_tokens - t0), n4 = grid_n4(p.n_tokens);
+  const bool aligned = (reinterpret_cast<uintptr_t>(p.src) & 7) == 0;
   float x0[8][4];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const int t = t0 + min(warp + 8 * i, rows - 1);
-    load_bf16x4(p.src + ((size_t)t * n_slices + slice) * kHeadDim + 4 * lane, x0[i]);
+    load_bf16x4(p.src + ((size_t)t * n_slices + slice) * kHeadDim + 4 * lane, aligned, x0[i]);
   }
   if (p.is_key) {
 #pragma unroll

@@ -40,3 +40,18 @@ def test_sixteen_bit_codes_lose_next_to_nothing(n_tokens):
     _, l8 = B.alpha_grid_search(k, q, v, 8, alphas=[0.0, 0.5])
     # the step is 257 times finer; what is left is that and the arithmetic's 2^-20 of unit outputs
     assert np.all(l16 >= 0) and np.all(l16 < l8 / 100.0)
+
+
+@pytest.mark.parametrize("offset", [1, 2, 4])
+@pytest.mark.parametrize("bits", [4, 16])
+def test_tensors_at_any_bf16_address(offset, bits):
+    from paper_2505_18610_b200 import binding as B
+    at_0 = [t.cuda() for t in _tensors(70, 2, 2, 2, 3)]
+    shifted = []
+    for t in at_0:
+        buf = torch.zeros(t.numel() + 8, dtype=torch.bfloat16, device="cuda")
+        buf[offset:offset + t.numel()] = t.flatten()
+        shifted.append(buf[offset:offset + t.numel()].view(t.shape))
+    _, want = B.alpha_grid_search(*at_0, bits, alphas=[0.0, 0.5])
+    _, got = B.alpha_grid_search(*shifted, bits, alphas=[0.0, 0.5])
+    assert np.allclose(got, want, rtol=1e-12, atol=0)     # the same numbers, summed in fp64 in another order
