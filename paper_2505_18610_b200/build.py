@@ -24,11 +24,26 @@ NVCC_FLAGS = [
 ]
 
 
-def needs_build() -> bool:
-    if not (os.path.exists(LIB) and os.path.exists(HOST_LIB)):
+# The extension uses torch's C++ classes and CPython's structures, so it belongs to one torch and one Python; it carries this text.
+HOST_FOR = f"built for torch {torch.__version__}, {sysconfig.get_config_var('SOABI')}"
+
+
+def _stale(lib: str) -> bool:
+    if not os.path.exists(lib):
         return True
-    t = min(os.path.getmtime(LIB), os.path.getmtime(HOST_LIB))
+    t = os.path.getmtime(lib)
     return any(os.path.getmtime(d) > t for d in DEPS)
+
+
+def _host_stale() -> bool:
+    if _stale(HOST_LIB):
+        return True
+    with open(HOST_LIB, "rb") as f:
+        return HOST_FOR.encode() not in f.read()
+
+
+def needs_build() -> bool:
+    return _stale(LIB) or _host_stale()
 
 
 def _build_host_calls() -> None:
@@ -36,7 +51,7 @@ def _build_host_calls() -> None:
     cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
     include = [os.path.join(at, "include"), sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
     cmd = ([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
-            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}"] + ["-I" + i for i in include]
+            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}", f'-DHOST_FOR="{HOST_FOR}"'] + ["-I" + i for i in include]
            + ["-o", HOST_LIB, HOST_SRC, "-L" + HERE, "-l:libpmkvq.so", "-Wl,-rpath,$ORIGIN", "-L" + os.path.join(at, "lib"),
               "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10"])
     res = subprocess.run(cmd, capture_output=True, text=True)
@@ -45,9 +60,7 @@ def _build_host_calls() -> None:
         raise RuntimeError("the host compiler failed building _host_calls.so")
 
 
-def build(force: bool = False, verbose: bool = False) -> str:
-    if not force and not needs_build():
-        return LIB
+def _build_library(verbose: bool) -> None:
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     cmd = [nvcc] + NVCC_FLAGS + ["-o", LIB, SRC]
     res = subprocess.run(cmd, capture_output=True, text=True)
@@ -56,7 +69,13 @@ def build(force: bool = False, verbose: bool = False) -> str:
         raise RuntimeError("nvcc failed building libpmkvq.so")
     if verbose:
         sys.stderr.write(res.stderr)
-    _build_host_calls()
+
+
+def build(force: bool = False, verbose: bool = False) -> str:
+    if force or _stale(LIB):
+        _build_library(verbose)
+    if force or _host_stale():
+        _build_host_calls()
     return LIB
 
 

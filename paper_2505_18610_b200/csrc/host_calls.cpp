@@ -12,6 +12,9 @@
 
 namespace {
 
+// what this was compiled against, read by build.py from the file
+__attribute__((used)) const char kBuiltFor[] = HOST_FOR;
+
 PyObject *g_error = nullptr;     // PmkvqError(status, what)
 PyObject *g_stream_attr = nullptr;  // "cuda_stream"
 

@@ -4,6 +4,19 @@ import pytest
 import torch
 
 from paper_2505_18610_b200 import binding as B
+from paper_2505_18610_b200 import build
+
+
+def test_the_extension_is_rebuilt_for_another_torch(monkeypatch):
+    build.build()
+    assert not build.needs_build()
+    made = []
+    monkeypatch.setattr(build, "_build_library", lambda verbose: made.append("library"))
+    monkeypatch.setattr(build, "_build_host_calls", lambda: made.append("extension"))
+    monkeypatch.setattr(build, "HOST_FOR", build.HOST_FOR.replace(torch.__version__, "2.0.0+cu118"))
+    assert build.needs_build()
+    build.build()
+    assert made == ["extension"]                  # the CUDA library does not depend on torch
 
 
 def test_refusals_without_a_device():
