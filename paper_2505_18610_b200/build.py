@@ -3,6 +3,7 @@ paper_2505_18610_b200/_host_calls.so (the Python extension for the calls of the 
 from __future__ import annotations
 
 import os
+import shutil
 import subprocess
 import sys
 import sysconfig
@@ -46,10 +47,17 @@ def needs_build() -> bool:
     return _stale(LIB) or _host_stale()
 
 
+def _nvcc() -> str:
+    return os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")   # a path, or a name to be found on PATH
+
+
+def _cuda_home() -> str:
+    return os.path.dirname(os.path.dirname(os.path.realpath(shutil.which(_nvcc()) or _nvcc())))
+
+
 def _build_host_calls() -> None:
     at = os.path.dirname(torch.__file__)
-    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
-    include = [os.path.join(at, "include"), sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
+    include = [os.path.join(at, "include"), sysconfig.get_paths()["include"], os.path.join(_cuda_home(), "include")]
     cmd = ([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
             f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}", f'-DHOST_FOR="{HOST_FOR}"'] + ["-I" + i for i in include]
            + ["-o", HOST_LIB, HOST_SRC, "-L" + HERE, "-l:libpmkvq.so", "-Wl,-rpath,$ORIGIN", "-L" + os.path.join(at, "lib"),
@@ -61,8 +69,7 @@ def _build_host_calls() -> None:
 
 
 def _build_library(verbose: bool) -> None:
-    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
-    cmd = [nvcc] + NVCC_FLAGS + ["-o", LIB, SRC]
+    cmd = [_nvcc()] + NVCC_FLAGS + ["-o", LIB, SRC]
     res = subprocess.run(cmd, capture_output=True, text=True)
     if res.returncode != 0:
         sys.stderr.write(res.stdout + res.stderr)

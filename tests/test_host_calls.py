@@ -19,6 +19,22 @@ def test_the_extension_is_rebuilt_for_another_torch(monkeypatch):
     assert made == ["extension"]                  # the CUDA library does not depend on torch
 
 
+def test_nvcc_may_be_a_name_on_the_path(monkeypatch, tmp_path):
+    home = tmp_path / "toolkit"
+    (home / "bin").mkdir(parents=True)
+    (home / "bin" / "nvcc").write_text("#!/bin/sh\n")
+    (home / "bin" / "nvcc").chmod(0o755)
+    (tmp_path / "bin").mkdir()
+    (tmp_path / "bin" / "nvcc").symlink_to(home / "bin" / "nvcc")
+    monkeypatch.setenv("PATH", str(tmp_path / "bin"))
+    ran = []
+    monkeypatch.setattr(build.subprocess, "run", lambda cmd, **kw: ran.append(cmd) or build.subprocess.CompletedProcess(cmd, 0, "", ""))
+    for name in ("nvcc", str(tmp_path / "bin" / "nvcc"), str(home / "bin" / "nvcc")):
+        monkeypatch.setenv("NVCC", name)
+        build._build_host_calls()
+        assert "-I" + str(home / "include") in ran[-1]
+
+
 def test_refusals_without_a_device():
     B.lib()
     x = torch.zeros(1, 1, 128, dtype=torch.bfloat16)
