@@ -537,7 +537,9 @@ __device__ __forceinline__ void fill_q_fragments(uint4 *s_frag, const float (*s_
 // ---- pieces of a segment that both contraction paths share --------------------------------------
 
 // The inputs of a segment's query, on their way: warp h < group holds head h, four channels per lane.  They are asked for
-// before the first tiles: 70 KB of tiles in front of them in the SM's queue delayed every segment by 1.2 us.
+// before the first tiles: 70 KB of tiles in front of them in the SM's queue delayed every segment by 1.2 us.  Past L1, because
+// in the launch that starts under its append they are read before the wait that makes other kernels' writes visible: the kernel that
+// wrote the queries is complete by then, but a line of an earlier step may still sit in this SM's L1.
 struct QueryLoad {
   uint2 raw;
   float4 lam;
@@ -550,12 +552,12 @@ __device__ __forceinline__ QueryLoad load_query(const AttnParams &p, int b, int 
   if (warp < p.group) {
     const uint16_t *src = p.Q + ((size_t)b * p.q_heads + hkv * p.group + warp) * kHeadDim + 4 * lane;
     if ((reinterpret_cast<uintptr_t>(p.Q) & 7) == 0) {
-      q.raw = *reinterpret_cast<const uint2 *>(src);
+      q.raw = __ldcg(reinterpret_cast<const uint2 *>(src));
     } else {  // a caller's query tensor may sit at any bf16 address
-      q.raw.x = src[0] | ((uint32_t)src[1] << 16);
-      q.raw.y = src[2] | ((uint32_t)src[3] << 16);
+      q.raw.x = __ldcg(src) | ((uint32_t)__ldcg(src + 1) << 16);
+      q.raw.y = __ldcg(src + 2) | ((uint32_t)__ldcg(src + 3) << 16);
     }
-    q.lam = *reinterpret_cast<const float4 *>(p.lambda + hkv * kHeadDim + 4 * lane);
+    q.lam = __ldcg(reinterpret_cast<const float4 *>(p.lambda + hkv * kHeadDim + 4 * lane));
   }
   return q;
 }
