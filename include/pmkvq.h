@@ -225,8 +225,7 @@ pmkvq_status pmkvq_calibrate_lambda(const void *d_K_pre_bf16, int32_t n_tokens, 
  * Arithmetic: rotation, equalization and quantizer decisions in fp32 (as in pmkvq_append); the attention
  * contractions run on the tensor cores with every operand carried exactly (codes) or as the sum of two fp16
  * numbers (22 significant bits) and fp32 accumulation; softmax in fp32; sums of squared errors in fp64.
- * Launches: abs-max, rotation table, three for the unquantized operator, one for the quantized Values and two per four
- * alphas (per alpha at 16 bit).  The attention launches wait on hardware barriers with a limit, as pmkvq_device_status
+ * Launches: abs-max, rotation table, two for the unquantized operator and two per four alphas (per alpha at 16 bit).  The attention launches wait on hardware barriers with a limit, as pmkvq_device_status
  * describes: a wait that runs out returns PMKVQ_ERR_DEVICE_WAIT here.
  *   d_K_pre_bf16, d_V_bf16  DEVICE bf16 [n_tokens][n_seq][kv_heads][128]; Keys before RoPE, token t at position t
  *   d_Q_pre_bf16            DEVICE bf16 [n_tokens][n_seq][kv_heads * group][128], before RoPE; all three at any bf16 address

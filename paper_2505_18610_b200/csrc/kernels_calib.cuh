@@ -169,6 +169,7 @@ __global__ void rope_table_kernel(float *table, int n_tokens, double pos_scale, 
   const int t = i >> 6, pair = i & 63;
   double s, c;
   sincos((double)t * pos_scale * pow(theta, -2.0 * pair / (double)kHeadDim), &s, &c);
+  pdl_wait();  // the angles are made while the abs-max in front of this launch runs
   float *at = table + (size_t)t * 128 + angle_slot(pair >> 1) * 4 + (pair & 1);
   at[0] = (float)c;
   at[2] = (float)s;
@@ -253,23 +254,24 @@ constexpr int kGridMaxBatch = 4;  // alphas whose Keys sit in the workspace side
 __host__ __device__ constexpr int grid_n4(int n_tokens) { return (n_tokens + 3) & ~3; }
 
 struct GridPrep {
-  const uint16_t *src;     // K or V, bf16 [n_tokens][n_seq][kv_heads][128]
   const float *amax;       // [kv_heads][128]
   const float4 *table;     // [n_tokens][32]
-  const float *alphas;     // those of this batch
-  uint8_t *out[kGridMaxBatch];
-  float *scale[kGridMaxBatch], *zero[kGridMaxBatch];
-  unsigned *vmax;          // per slice, the largest scale (Values)
-  int is_key, quantize;    // rotate (and, quantized, equalize); quantize or keep plain
+  const uint16_t *k, *v;   // bf16 [n_tokens][n_seq][kv_heads][128]
+  int n_keys;              // outputs 0 .. n_keys - 1 are Keys (rotated and, quantized, equalized), one per alpha; the one behind them Values
+  float alphas[kGridMaxBatch];
+  uint8_t *out[kGridMaxBatch + 1];
+  float *scale[kGridMaxBatch + 1], *zero[kGridMaxBatch + 1];
+  unsigned *vmax;          // per slice, the largest scale of the Values
+  int quantize;            // or keep plain
   int n_tokens, n_seq, kv_heads, bits;
   float floor_value;
 };
-// One CTA per (slice, tile) and alpha, a warp on eight vectors; they leave through shared memory as whole 16-byte pieces.  (One
+// One CTA per (slice, tile) and output, a warp on eight vectors; they leave through shared memory as whole 16-byte pieces.  (One
 // CTA for the four alphas of a batch reads its Keys once, but the latency of four rounds showed: 38 us per batch of
 // 2048 x 2 x 4 vectors.)
 constexpr int kPrepChunkStride = kGridTile * 16 + 16;  // padded: the 16 channel groups a warp writes fall into different banks
 template <int PLANES>
-__global__ void __launch_bounds__(256) alpha_grid_prep_kernel(const GridPrep p) {
+__global__ void __launch_bounds__(256) alpha_grid_prep_kernel(const __grid_constant__ GridPrep p) {
   __shared__ __align__(16) uint8_t s_tile[PLANES][16 * kPrepChunkStride];
   __shared__ float s_scale[kGridTile], s_zero[kGridTile];
   __shared__ __align__(16) float s_inv[kHeadDim];
@@ -277,19 +279,21 @@ __global__ void __launch_bounds__(256) alpha_grid_prep_kernel(const GridPrep p) 
   const int n_tiles = (p.n_tokens + kGridTile - 1) / kGridTile;
   const int tile = (int)(blockIdx.x % (unsigned)n_tiles), slice = (int)(blockIdx.x / (unsigned)n_tiles), n_slices = p.n_seq * p.kv_heads;
   const int t0 = tile * kGridTile, rows = min(kGridTile, p.n_tokens - t0), n4 = grid_n4(p.n_tokens);
-  const bool aligned = (reinterpret_cast<uintptr_t>(p.src) & 7) == 0;
+  const int a = blockIdx.y;
+  const bool is_key = a < p.n_keys;
+  const uint16_t *src = is_key ? p.k : p.v;
+  const bool aligned = (reinterpret_cast<uintptr_t>(src) & 7) == 0;
   float x0[8][4];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const int t = t0 + min(warp + 8 * i, rows - 1);
-    load_bf16x4(p.src + ((size_t)t * n_slices + slice) * kHeadDim + 4 * lane, aligned, x0[i]);
+    load_bf16x4(src + ((size_t)t * n_slices + slice) * kHeadDim + 4 * lane, aligned, x0[i]);
   }
-  if (p.is_key) {
+  if (is_key) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) rotate_token(x0[i], p.table + (size_t)(t0 + min(warp + 8 * i, rows - 1)) * 32, lane);
   }
-  const int a = blockIdx.y;
-  if (p.is_key && p.quantize) {
+  if (is_key && p.quantize) {
     if (tid < kHeadDim)
       s_inv[tid] = __fdiv_rn(1.0f, powf(fmaxf(p.amax[(size_t)(slice % p.kv_heads) * kHeadDim + tid], p.floor_value), p.alphas[a]));
     __syncthreads();
@@ -300,7 +304,7 @@ __global__ void __launch_bounds__(256) alpha_grid_prep_kernel(const GridPrep p) 
     const int row = warp + 8 * i;
     float (&x)[4] = x0[i];
     if (p.quantize) {
-      if (p.is_key) {
+      if (is_key) {
         const float4 il = *reinterpret_cast<const float4 *>(s_inv + 4 * lane);
         x[0] = __fmul_rn(x[0], il.x); x[1] = __fmul_rn(x[1], il.y); x[2] = __fmul_rn(x[2], il.z); x[3] = __fmul_rn(x[3], il.w);
       }
@@ -316,7 +320,7 @@ __global__ void __launch_bounds__(256) alpha_grid_prep_kernel(const GridPrep p) 
     *reinterpret_cast<uint2 *>(&s_tile[0][at]) = hi;
     if constexpr (PLANES == 2) *reinterpret_cast<uint2 *>(&s_tile[1][at]) = lo;
   }
-  if (p.vmax && lane == 0) atomicMax(p.vmax + slice, __float_as_uint(smax));  // scale >= 0: uint order = float order
+  if (!is_key && p.quantize && lane == 0) atomicMax(p.vmax + slice, __float_as_uint(smax));  // scale >= 0: uint order = float order
   __syncthreads();
   uint8_t *dst = p.out[a] + ((size_t)slice * p.n_tokens + t0) * (size_t)(256 * PLANES);
 #pragma unroll
@@ -333,7 +337,10 @@ __global__ void __launch_bounds__(256) alpha_grid_prep_kernel(const GridPrep p) 
 
 // ---- causal self-attention of the passes ------------------------------------------------------------------------
 // Grid: (sequences x query heads, alphas of the batch, query blocks from the longest to the shortest); a CTA takes 256
-// queries, two tiles of 128, against their Keys in tiles of 64.  Both contractions run on tcgen05.mma (fp16 in, fp32
+// queries, two tiles of 128, against their Keys in tiles of 64.  With at most 128 tokens (one tile) the two tiles are two query heads of
+// one KV head instead, and the grid has a CTA per pair: a CTA of a short sequence is a chain of 10 us, whatever its second half does
+// (64 tokens x 64 sequences x 8 heads,
+// four alphas: 196 us a call, 264 with a CTA per head, two more launches, three more clears and one more copy to the host). Both contractions run on tcgen05.mma (fp16 in, fp32
 // accumulators in tensor memory): S[query, key] = Q K^T with both operands in shared memory, O[query, channel] += P V with P
 // in tensor memory, where it overwrites the scores it came from.  Warps:
 //   0-3, 4-7   one warpgroup per query tile, thread = query: builds the tile's Q operand (rotated, equalized, scaled by a power of
@@ -360,6 +367,7 @@ constexpr int kGridTmemS = 0, kGridTmemO = 256;    // scores / weights [query ti
 constexpr int kGridUnitLog2 = 6;                   // weights stay below 2^(6 + 8): fp16 with room
 constexpr float kGridMaxAhead = 8.0f;
 
+__host__ __device__ constexpr bool grid_head_pairs(int n_tokens) { return n_tokens <= kGridQTile; }
 struct GridAttn {
   const uint16_t *Q;       // bf16 [n_tokens][n_seq][kv_heads * group][128] before RoPE
   const uint8_t *k[kGridMaxBatch], *v;
@@ -367,7 +375,7 @@ struct GridAttn {
   const unsigned *vmax;    // per slice
   const float *amax;
   const float4 *table;
-  const float *alphas;     // those of this batch
+  float alphas[kGridMaxBatch];  // those of this batch
   float *o_ref;            // the unquantized outputs, [sequence x head][tile of 128 queries][32 groups of 4 channels][rows][4] fp32
   double *loss_sums;       // those of this batch
   unsigned *error_word;
@@ -406,16 +414,20 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ GridShared sh;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int q_heads = p.kv_heads * p.group;
-  const int seq = (int)blockIdx.x / q_heads, q_head = (int)blockIdx.x - seq * q_heads, kv_head = q_head / p.group;
-  const int slice = seq * p.kv_heads + kv_head, batch = blockIdx.y;
+  const int q_heads = p.kv_heads * p.group, batch = blockIdx.y;
+  const bool pairs = grid_head_pairs(p.n_tokens);
+  const int per_kv = pairs ? (p.group + 1) / 2 : p.group;  // CTAs of a KV head
+  const int slice = (int)blockIdx.x / per_kv, in_slice = (int)blockIdx.x - slice * per_kv;
+  const int seq = slice / p.kv_heads, kv_head = slice - seq * p.kv_heads;
+  const int head0 = kv_head * p.group + (pairs ? 2 * in_slice : in_slice);  // query head of the first tile
   const int q_block = ((int)gridDim.z - 1 - (int)blockIdx.z) * kGridQueries;  // long rows first
   const int n = p.n_tokens, n4 = grid_n4(n);
   int nt[2];  // key tiles of the two query tiles
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
-    const int first = q_block + q * kGridQTile;
-    nt[q] = first < n ? (min(n, first + kGridQTile) - 1) / kGridTile + 1 : 0;
+    const int first = pairs ? 0 : q_block + q * kGridQTile;
+    const bool any = pairs ? 2 * in_slice + q < p.group : first < n;
+    nt[q] = any ? (min(n, first + kGridQTile) - 1) / kGridTile + 1 : 0;
   }
   const int n_kt = max(nt[0], nt[1]);
   const bool ragged = n_kt * kGridTile > n;  // the last tile is the slice's short one
@@ -573,7 +585,7 @@ __global__ void __launch_bounds__(kGridThreads, 1) alpha_grid_attn_kernel(const 
   } else if (nt[warp >> 2] > 0) {
     // ---- a query tile ----
     const int q = warp >> 2, row = tid & 127;
-    const int first_q = q_block + q * kGridQTile;
+    const int first_q = pairs ? 0 : q_block + q * kGridQTile, q_head = head0 + (pairs ? q : 0);
     const int qi = min(first_q + row, n - 1);  // a dead row repeats the last query; its output is dropped
     const bool alive = first_q + row < n;
     const uint32_t t_lane = (uint32_t)((warp & 3) * 32) << 16;

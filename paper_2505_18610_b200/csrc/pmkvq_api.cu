@@ -817,13 +817,11 @@ pmkvq_status pmkvq_set_attention_ctas(pmkvq_cache *k, int32_t n_ctas) {
   return PMKVQ_OK;
 }
 
-// |K_rot| maxima into d_amax_bits (zeroed here).  Enough CTAs to fill the GPU several times over, each with at least
+// |K_rot| maxima into d_amax_bits (zero before the call).  Enough CTAs to fill the GPU several times over, each with at least
 // a thousand vectors behind its table of angles.  2048 tokens x 128 sequences x 8 heads, 537 MB: 98 us = 5.5 TB/s
 // (0.85 of the measured copy rate); with a 2-byte load and two shared-memory atomics per element it was 518 us.
 static cudaError_t launch_absmax(const uint16_t *K, unsigned *d_amax_bits, int n_tokens, int n_seq, int kv_heads, double pos_scale,
                                  double theta, cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(d_amax_bits, 0, (size_t)kv_heads * kHeadDim * sizeof(unsigned), st);
-  if (e != cudaSuccess) return e;
   RopeFreqs freqs;
   for (int i = 0; i < 64; ++i) freqs.f[i] = std::pow(theta, -2.0 * i / (double)kHeadDim);
   int tokens = kAbsmaxTokens;
@@ -848,6 +846,7 @@ pmkvq_status pmkvq_calibrate_lambda(const void *d_K, int32_t n_tokens, int32_t n
   if ((int64_t)n_seq * kv_heads > (1 << 20)) return PMKVQ_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int n = kv_heads * kHeadDim;
+  if (cudaMemsetAsync(d_lambda, 0, (size_t)n * sizeof(float), st) != cudaSuccess) return PMKVQ_ERR_CUDA;
   if (launch_absmax(static_cast<const uint16_t *>(d_K), reinterpret_cast<unsigned *>(d_lambda), n_tokens, n_seq, kv_heads, pos_scale, theta,
                     st) != cudaSuccess)
     return PMKVQ_ERR_CUDA;
@@ -858,23 +857,27 @@ pmkvq_status pmkvq_calibrate_lambda(const void *d_K, int32_t n_tokens, int32_t n
 
 static size_t grid_ws_round(size_t b) { return (b + 255) / 256 * 256; }
 
-// Workspace of the alpha grid search: abs-max, rotation table, loss sums, alphas, the error word, three regions of 4 bytes
-// per Key element and the unquantized operator's output.  The unquantized pass keeps its Keys in region 0 and its Values
-// in region 1 (two fp16 planes each).  The quantized passes keep Values in region 2 and scales, zero-points and the slices'
-// largest Value scales in the upper half of region 1; their Keys take region 0 (16 bit), or, as one plane per alpha (codes
-// up to 8 bit), both halves of region 0, the upper half of region 2 and the lower half of region 1.
+// Workspace of the alpha grid search: what starts as zero (abs-max, the slices' largest Value scales, and what the host reads back:
+// loss sums and the error word), rotation table, three regions of 4 bytes per Key element and the unquantized operator's
+// output.  The unquantized pass keeps its Keys in region 0 and its Values in region 1 (two fp16 planes each).  The quantized
+// passes keep Values in region 2 and scales and zero-points in the upper half of region 1; their Keys take region 0 (16 bit),
+// or, as one plane per alpha (codes up to 8 bit), both halves of region 0, the upper half of region 2 and the lower half of region 1.
+struct GridResult {
+  double loss[kMaxAlphas];
+  unsigned error;
+};
 struct GridWorkspace {
-  size_t amax, table, loss, alphas, error, region[3], o_ref, total;
+  size_t amax, vmax, result, zero_bytes, table, region[3], o_ref, total;
 };
 static GridWorkspace grid_workspace(int64_t n_tokens, int64_t n_seq, int64_t kv_heads, int64_t group) {
   GridWorkspace w;
   size_t off = 0;
   const size_t kv = (size_t)(n_tokens * n_seq * kv_heads) * kHeadDim * sizeof(float);
   w.amax = off; off += grid_ws_round((size_t)kv_heads * kHeadDim * sizeof(float));
+  w.vmax = off; off += grid_ws_round((size_t)(n_seq * kv_heads) * sizeof(unsigned));
+  w.result = off; off += grid_ws_round(sizeof(GridResult));
+  w.zero_bytes = off;
   w.table = off; off += grid_ws_round((size_t)n_tokens * 64 * sizeof(float2));
-  w.loss = off; off += grid_ws_round(kMaxAlphas * sizeof(double));
-  w.alphas = off; off += grid_ws_round(kMaxAlphas * sizeof(float));
-  w.error = off; off += 256;
   for (int r = 0; r < 3; ++r) { w.region[r] = off; off += grid_ws_round(kv); }
   w.o_ref = off; off += grid_ws_round(kv * (size_t)group);
   w.total = off;
@@ -904,32 +907,29 @@ pmkvq_status pmkvq_alpha_grid_search(const void *d_K, const void *d_Q, const voi
   uint8_t *ws = static_cast<uint8_t *>(d_workspace);
   float *d_amax = reinterpret_cast<float *>(ws + w.amax);
   float *d_table = reinterpret_cast<float *>(ws + w.table);
-  double *d_loss = reinterpret_cast<double *>(ws + w.loss);
-  float *d_alphas = reinterpret_cast<float *>(ws + w.alphas);
-  unsigned *d_error = reinterpret_cast<unsigned *>(ws + w.error);
+  unsigned *d_vmax = reinterpret_cast<unsigned *>(ws + w.vmax);
+  GridResult *d_result = reinterpret_cast<GridResult *>(ws + w.result);
   float *d_o_ref = reinterpret_cast<float *>(ws + w.o_ref);
-  if (cudaMemsetAsync(d_loss, 0, kMaxAlphas * sizeof(double), st) != cudaSuccess ||
-      cudaMemsetAsync(d_error, 0, sizeof(unsigned), st) != cudaSuccess ||
-      cudaMemcpyAsync(d_alphas, h_alphas, (size_t)n_alphas * sizeof(float), cudaMemcpyHostToDevice, st) != cudaSuccess)
-    return PMKVQ_ERR_CUDA;
+  if (cudaMemsetAsync(ws, 0, w.zero_bytes, st) != cudaSuccess) return PMKVQ_ERR_CUDA;
   const uint16_t *K = static_cast<const uint16_t *>(d_K), *Q = static_cast<const uint16_t *>(d_Q),
                  *V = static_cast<const uint16_t *>(d_V);
   if (launch_absmax(K, reinterpret_cast<unsigned *>(d_amax), n_tokens, n_seq, kv_heads, pos_scale, theta, st) != cudaSuccess)
     return PMKVQ_ERR_CUDA;
-  rope_table_kernel<<<(unsigned)((n_tokens * 64 + 255) / 256), 256, 0, st>>>(d_table, n_tokens, pos_scale, theta);
+  uint64_t launches = 0;
+  if (launch(launches, rope_table_kernel, dim3((unsigned)((n_tokens * 64 + 255) / 256)), 256, 0, st, d_table, n_tokens, pos_scale, theta) != cudaSuccess)
+    return PMKVQ_ERR_CUDA;
   const size_t slices = (size_t)n_seq * kv_heads, half = (size_t)n_tokens * slices * 256;  // half a region: one fp16 plane of all vectors
   const size_t meta_bytes = slices * (size_t)grid_n4(n_tokens) * sizeof(float);
   const int n_tiles = (n_tokens + kGridTile - 1) / kGridTile;
   const int planes = bits <= 8 ? 1 : 2, per_batch = planes == 1 ? kGridMaxBatch : 1;
   uint8_t *meta = ws + w.region[1] + half;
   auto meta_array = [&](int i) { return reinterpret_cast<float *>(meta + (size_t)i * meta_bytes); };
-  unsigned *d_vmax = reinterpret_cast<unsigned *>(meta + (2 * kGridMaxBatch + 2) * meta_bytes);
 
   GridPrep prep{};
   prep.amax = d_amax; prep.table = reinterpret_cast<const float4 *>(d_table); prep.n_tokens = n_tokens; prep.n_seq = n_seq; prep.kv_heads = kv_heads;
-  prep.bits = bits; prep.floor_value = floor_value;
+  prep.k = K; prep.v = V; prep.bits = bits; prep.floor_value = floor_value;
   GridAttn attn{};
-  attn.Q = Q; attn.amax = d_amax; attn.table = prep.table; attn.o_ref = d_o_ref; attn.error_word = d_error;
+  attn.Q = Q; attn.amax = d_amax; attn.table = prep.table; attn.o_ref = d_o_ref; attn.error_word = &d_result->error;
   attn.n_tokens = n_tokens; attn.n_seq = n_seq; attn.kv_heads = kv_heads; attn.group = group; attn.floor_value = floor_value;
   auto run_prep = [&](int pl, int n_out) {
     const dim3 grid((unsigned)(slices * (size_t)n_tiles), (unsigned)n_out);
@@ -938,23 +938,19 @@ pmkvq_status pmkvq_alpha_grid_search(const void *d_K, const void *d_Q, const voi
   };
   auto run_attn = [&](auto kernel, int n_pass) {
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGridSmemBytes) != cudaSuccess) return;
-    const dim3 grid((unsigned)(n_seq * kv_heads * group), (unsigned)n_pass, (unsigned)((n_tokens + kGridQueries - 1) / kGridQueries));
+    const int per_kv = grid_head_pairs(n_tokens) ? (group + 1) / 2 : group;
+    const dim3 grid((unsigned)(n_seq * kv_heads * per_kv), (unsigned)n_pass, (unsigned)((n_tokens + kGridQueries - 1) / kGridQueries));
     kernel<<<grid, kGridThreads, kGridSmemBytes, st>>>(attn);
   };
   // the unquantized operator
-  prep.src = K; prep.is_key = 1; prep.out[0] = ws + w.region[0];
-  run_prep(2, 1);
-  prep.src = V; prep.is_key = 0; prep.out[0] = ws + w.region[1];
-  run_prep(2, 1);
-  attn.k[0] = ws + w.region[0]; attn.v = ws + w.region[1];
+  prep.n_keys = 1; prep.out[0] = ws + w.region[0]; prep.out[1] = ws + w.region[1];
+  run_prep(2, 2);
+  attn.k[0] = prep.out[0]; attn.v = prep.out[1];
   run_attn(alpha_grid_attn_kernel<2, false>, 1);
-  // Eq. 9 at each alpha: the Values once, the Keys of up to four alphas at a time
-  if (cudaMemsetAsync(d_vmax, 0, slices * sizeof(unsigned), st) != cudaSuccess) return PMKVQ_ERR_CUDA;
+  // Eq. 9 at each alpha: the Keys of up to four alphas at a time, with the first of them the Values
   prep.quantize = 1;
-  prep.out[0] = ws + w.region[2]; prep.scale[0] = meta_array(0); prep.zero[0] = meta_array(1); prep.vmax = d_vmax;
-  run_prep(planes, 1);
-  attn.v = prep.out[0]; attn.v_scale = prep.scale[0]; attn.v_zero = prep.zero[0]; attn.vmax = d_vmax;
-  prep.src = K; prep.is_key = 1; prep.vmax = nullptr;
+  prep.vmax = d_vmax;
+  attn.v = ws + w.region[2]; attn.v_scale = meta_array(0); attn.v_zero = meta_array(1); attn.vmax = d_vmax;
   uint8_t *const buffers[kGridMaxBatch] = {ws + w.region[0], ws + w.region[0] + half, ws + w.region[2] + half, ws + w.region[1]};
   for (int i = 0; i < kGridMaxBatch; ++i) {
     attn.k[i] = prep.out[i] = buffers[i];
@@ -962,25 +958,26 @@ pmkvq_status pmkvq_alpha_grid_search(const void *d_K, const void *d_Q, const voi
     attn.k_zero[i] = prep.zero[i] = meta_array(3 + 2 * i);
   }
   for (int first = 0; first < n_alphas; first += per_batch) {
-    const int count = std::min(per_batch, n_alphas - first);
-    prep.alphas = attn.alphas = d_alphas + first;
-    attn.loss_sums = d_loss + first;
-    run_prep(planes, count);
+    const int count = std::min(per_batch, n_alphas - first), values = first == 0 ? 1 : 0;
+    for (int i = 0; i < count; ++i) prep.alphas[i] = attn.alphas[i] = h_alphas[first + i];
+    attn.loss_sums = d_result->loss + first;
+    prep.n_keys = count;
+    if (values) {
+      prep.out[count] = ws + w.region[2]; prep.scale[count] = meta_array(0); prep.zero[count] = meta_array(1);
+    }
+    run_prep(planes, count + values);
     if (planes == 1) run_attn(alpha_grid_attn_kernel<1, true>, count);
     else run_attn(alpha_grid_attn_kernel<2, true>, count);
   }
   if (cudaGetLastError() != cudaSuccess) return PMKVQ_ERR_CUDA;
-  unsigned error = 0;
-  if (cudaMemcpyAsync(&error, d_error, sizeof(error), cudaMemcpyDeviceToHost, st) != cudaSuccess) return PMKVQ_ERR_CUDA;
-  double sums[kMaxAlphas];
-  if (cudaMemcpyAsync(sums, d_loss, (size_t)n_alphas * sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-      cudaStreamSynchronize(st) != cudaSuccess)
+  GridResult result;
+  if (cudaMemcpyAsync(&result, d_result, sizeof(result), cudaMemcpyDeviceToHost, st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
     return PMKVQ_ERR_CUDA;
-  if (error) return PMKVQ_ERR_DEVICE_WAIT;
+  if (result.error) return PMKVQ_ERR_DEVICE_WAIT;
   const double count = (double)n_tokens * n_seq * kv_heads * group * kHeadDim;
   int best = 0;
   for (int i = 0; i < n_alphas; ++i) {
-    h_losses[i] = sums[i] / count;
+    h_losses[i] = result.loss[i] / count;
     if (h_losses[i] < h_losses[best]) best = i;  // the first one on ties
   }
   if (h_best) *h_best = best;

@@ -32,6 +32,19 @@ def test_losses_match_the_oracle_at_tile_edges(n_tokens, n_seq, kv_heads, group,
     assert np.allclose(got, want, rtol=2e-2 if bits == 8 else 2e-3, atol=0)
 
 
+@pytest.mark.parametrize("group", [1, 2, 3, 5])
+@pytest.mark.parametrize("n_tokens,n_seq,kv_heads,bits", [(1, 2, 1, 2), (17, 2, 3, 4), (64, 1, 2, 2), (127, 1, 1, 8), (128, 2, 2, 2), (129, 1, 2, 4)])
+def test_pairs_of_heads_of_a_short_sequence(n_tokens, n_seq, kv_heads, group, bits):
+    """Up to 128 tokens a CTA takes two query heads of a KV head, the last one of an odd group alone."""
+    from paper_2505_18610_b200 import binding as B
+    k, q, v = _tensors(n_tokens, n_seq, kv_heads, group, n_tokens)
+    q *= torch.arange(1, kv_heads * group + 1).view(-1, 1) / (kv_heads * group)      # no two heads alike
+    alphas = [0.0, 0.3, 0.5, 0.8, 1.0]
+    want = O.attention_reconstruction_losses(k.float().numpy(), q.float().numpy(), v.float().numpy(), group, bits, alphas)
+    _, got = B.alpha_grid_search(k.cuda(), q.cuda(), v.cuda(), bits, alphas=alphas)
+    assert np.allclose(got, want, rtol=2e-2 if bits == 8 else 2e-3, atol=0)           # as above
+
+
 @pytest.mark.parametrize("n_tokens", [65, 300])
 def test_sixteen_bit_codes_lose_next_to_nothing(n_tokens):
     from paper_2505_18610_b200 import binding as B
