@@ -55,6 +55,20 @@ def test_sixteen_bit_codes_lose_next_to_nothing(n_tokens):
     assert np.all(l16 >= 0) and np.all(l16 < l8 / 100.0)
 
 
+@pytest.mark.parametrize("v_scale", [1.0, 2.0 ** 9])
+@pytest.mark.parametrize("n_tokens,n_seq,kv_heads,group", [(2, 1, 1, 1), (63, 2, 1, 2), (64, 1, 2, 2), (65, 2, 2, 2), (128, 1, 2, 1),
+                                                           (129, 1, 1, 3), (256, 1, 1, 2), (300, 2, 2, 2)])
+def test_sixteen_bit_losses_match_the_oracle_at_tile_edges(n_tokens, n_seq, kv_heads, group, v_scale):
+    """The two-plane form.  Both outputs are good to 2^-20 of Values of unit size (root mean square), so the root of the loss is, by
+    the triangle inequality; without a second plane a Key is good to 2^-12 and the root of the loss is off by 2^-13 or more."""
+    from paper_2505_18610_b200 import binding as B
+    k, q, v = _tensors(n_tokens, n_seq, kv_heads, group, 5, v_scale)
+    alphas = [0.0, 0.3, 0.5, 1.0]
+    want = O.attention_reconstruction_losses(k.float().numpy(), q.float().numpy(), v.float().numpy(), group, 16, alphas)
+    _, got = B.alpha_grid_search(k.cuda(), q.cuda(), v.cuda(), 16, alphas=alphas)
+    assert np.all(np.abs(np.sqrt(got) - np.sqrt(want)) <= 2.0 ** -20 * v_scale)
+
+
 @pytest.mark.parametrize("offset", [1, 2, 4])
 @pytest.mark.parametrize("bits", [4, 16])
 def test_tensors_at_any_bf16_address(offset, bits):
