@@ -14,18 +14,17 @@
 // last partial of a slice (atomic ticket, nobody waits) merges the slice and writes the output.
 //
 // A segment's fixed part is a chain of latencies, and a short context is nothing else: which block and slice
-// (the host says which block a CTA starts in, divisions are 32-bit or double products), query, fragments, ...,
-// warp merge, publish, combine.  Written as few dependent steps as possible it costs about 5 us of the 10.5 us a
-// one-block launch over a 4K context takes (15.6 us before, with 64-bit divisions, a fence in every thread,
-// bank conflicts in the merge and one memory round trip per pass of the combine).
+// (the host says which block a CTA starts in, divisions are 32-bit or products with a reciprocal), query, fragments, ...,
+// warp merge, publish, combine.  Written as few dependent steps as possible; a one-block launch over one slice of 4K tokens at
+// 4 bit is little else and takes 8.2 us behind its like in a graph (15.6 us with 64-bit divisions, a fence in every thread, bank
+// conflicts in the merge and one memory round trip per pass of the combine).
 //
-// Two contraction paths share this decomposition.  The 4- and 2-bit body, which holds most bytes of a
-// cache in its steady state, runs on tcgen05.mma with its code operands in tensor memory
-// (kernels_attn_tc.cuh).  INT16 tiles (sink, window) and an 8- or 16-bit body run on warp-level
-// mma.sync.m16n8k16 (f16 inputs, f32 accumulate) with register operands, the body tiles staged through a
-// per-warp cp.async ring in shared memory (a tile is one contiguous run of bytes); in both paths packed
-// codes become MMA operands with one logic operation per pair of codes - a code field left in place
-// inside an fp16 bit pattern below bit 11 is the exact value code * 2^(pos-24) (fp16 subnormals and the
+// Two contraction paths share this decomposition.  The default one, and on both the INT16 tiles (sink, window) and an 8- or
+// 16-bit body, is warp-level mma.sync.m16n8k16 (f16 inputs, f32 accumulate) with register operands, the body tiles staged
+// through a per-warp cp.async ring in shared memory (a tile is one contiguous run of bytes; 16 bit reads global memory).  A cache
+// created for the other path has its 4- and 2-bit body on tcgen05.mma with the code operands in tensor memory
+// (kernels_attn_tc.cuh).  In both, packed codes become MMA operands with one logic operation per pair of codes - a code field
+// left in place inside an fp16 bit pattern below bit 11 is the exact value code * 2^(pos-24) (fp16 subnormals and the
 // first binade are linear in the bit pattern).
 //   scores:  S[h, t]  = sum_i Q''[h, i] * c_K[t, i]      A = Q'' (rows 0-7: fp16 "hi" part of the 8 heads,
 //                                                        rows 8-15: the "lo" remainder), B = K codes
@@ -92,10 +91,7 @@ __device__ __forceinline__ void mma_f16(float (&c)[4], uint32_t a0, uint32_t a1,
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-__device__ __forceinline__ void cp_async16(uint32_t smem_addr, const void *gptr) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr), "l"(gptr) : "memory");
-}
-// the same at byte offset OFF of both addresses (an immediate: no address arithmetic per copy)
+// 16 bytes, past L1, at byte offset OFF of both addresses (an immediate: no address arithmetic per copy)
 template <int OFF>
 __device__ __forceinline__ void cp_async16_at(uint32_t smem_addr, const void *gptr) {
   asm volatile("cp.async.cg.shared.global [%0 + %2], [%1 + %2], 16;\n" ::"r"(smem_addr), "l"(gptr), "n"(OFF) : "memory");
@@ -1177,8 +1173,9 @@ static_assert(kMaxFusedLayers <= 256 && sizeof(FusedParams) <= 4096, "block numb
 // 130 560 tiles at 2 / 4 / 8 / 16 bit, i.e. 50 / 55 / 89 / 174) make mixed launches slower: 20 blocks at 2 and 8 at 4 bit
 // 2965 -> 2982 us for two steps, 8 and 4 bit mixed 756 -> 764 us for four.
 __host__ __device__ constexpr int tile_weight(int bits) { return bits == 16 ? 152 : bits == 8 ? 80 : bits == 4 ? 53 : 50; }
-// Fixed cost of one more segment (set-up, warp merge, publish, its share of the slice combine), in
-// body tiles of each width: about 12 us at the measured per-SM tile rates.
+// Fixed cost of one more segment (set-up, warp merge, publish, its share of the slice combine), in body tiles of each
+// width.  Measured (a third segment of 249 body and 9 INT16 tiles per CTA, less the tiles' own time): 7.7 / 7.8 / 8.0 / 11.7 us at
+// 2 / 4 / 8 / 16 bit, i.e. 169 / 156 / 91 / 70 tiles.
 __host__ __device__ constexpr int segment_cost_tiles(int bits) { return bits == 16 ? 48 : bits == 8 ? 96 : bits == 4 ? 176 : 160; }
 __host__ __device__ constexpr int int16_units(int bits) { return (tile_bytes(16) + tile_bytes(bits) - 1) / tile_bytes(bits); }
 __device__ __forceinline__ unsigned long long inv_tile_weight(int bits) {

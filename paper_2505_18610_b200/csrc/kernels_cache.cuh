@@ -865,7 +865,9 @@ __device__ __forceinline__ void evict_tile_one(int is_value, int slice, int grou
 // body, new rows of it to the window ring, or rows of it that leave the window (a group may be several items); a warp takes
 // half (K or V) of an item of one slice.  Only sink tokens go one by one.  The one hazard is the ring: new window tokens may
 // land in slots of tokens that leave it.  The warp that writes a slot then moves its old contents out first, and the
-// leaving rows' own item leaves them out.
+// leaving rows' own item leaves them out.  Both sides tell which old token meets which new one from the group alone, and a group's
+// rows may lie on both sides of a multiple of the ring's length behind n_old: that comes out right because the ring holds at least 16
+// tokens more than window + evict_chunk - 1 (pmkvq_cache plan), so no token that far back is still in it.
 // (Before, the window and the ragged ends went token by token, 16 times the warps, in three to four launches: 16.8 us per block
 // for a 2537-token prompt, 35 us for a chunk of 2048 tokens x 32 slices.)
 // What bounds it: a single wave is one chain of about 1000 instructions per warp, hence the split in parts and the 72
@@ -932,8 +934,8 @@ __global__ void __launch_bounds__(128, 7) append_bulk_kernel(const uint16_t *__r
 // One decode step's cache update in a single launch: the tokens that leave the window (warps
 // [0, 2 n_evict n_slices)) and the one new token (the rest).  Only valid when no evicted token
 // shares its ring slot with the new token (single-token appends: the ring is larger than window +
-// evict_chunk) and the new token does not enter a body tile that an evicted token enters too (the host
-// sends the one configuration where that happens, window = 0 with evict_chunk > 1, through two launches).
+// evict_chunk) and the new token does not enter a body tile that an evicted token enters too (the host sends the one
+// configuration where that happens, window = 0 with evict_chunk > 1, the way of a run of tokens).
 __global__ void __launch_bounds__(128) append_decode_kernel(const uint16_t *__restrict__ K,
                                                             const uint16_t *__restrict__ V,
                                                             const float *__restrict__ inv_lambda, unsigned *vmax_bits,

@@ -221,11 +221,16 @@ cudaError_t attention_setup_path(pmkvq_cache *k, int sms) {
   return e;
 }
 
+cudaError_t sm_count(int &sms) {  // of the current device
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  return e == cudaSuccess ? cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) : e;
+}
+
 // Dynamic shared memory opt-in and the size of one wave of resident CTAs, per body width.
 cudaError_t attention_setup(pmkvq_cache *k) {
-  int dev = 0, sms = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  int sms = 0;
+  cudaError_t e = sm_count(sms);
   k->sms = sms;
   if (e == cudaSuccess) e = k->rows ? attention_setup_path<true>(k, sms) : attention_setup_path<false>(k, sms);
   return e;
@@ -415,7 +420,7 @@ pmkvq_status pmkvq_append(pmkvq_cache *k, int32_t layer, const void *d_K, const 
   unsigned *vmax = reinterpret_cast<unsigned *>(k->arena + k->off_vmax) + (size_t)layer * k->n_slices;
   const int n_evict = std::max(0, ev_last - ev_first);
   // With window = 0 and chunked eviction the new token enters the body together with the chunk's other
-  // tokens, possibly in one tile: they then go through separate launches (see append_decode_kernel).
+  // tokens, possibly in one tile, which append_decode_kernel does not allow: such a token goes the way of a run.
   const bool shares_tile = k->window == 0 && k->evict_chunk > 1;
   const uint16_t *K = static_cast<const uint16_t *>(d_K), *V = static_cast<const uint16_t *>(d_V);
   cudaError_t e = cudaSuccess;
@@ -630,7 +635,7 @@ pmkvq_status pmkvq_decode_step(pmkvq_cache *k, const void *d_K, const void *d_V,
     if (s != PMKVQ_OK) return s;
   }
   if (k->layers > kMaxStepLayers || (k->window == 0 && k->evict_chunk > 1)) {
-    // too many blocks for one argument block, or appends that need two launches per block: block by block
+    // too many blocks for one argument block, or a new token that shares a tile with the ones it evicts: block by block
     for (int layer = 0; layer < k->layers; ++layer) {
       pmkvq_status s = pmkvq_append(k, layer, static_cast<const uint8_t *>(d_K) + layer * kv_stride,
                                     static_cast<const uint8_t *>(d_V) + layer * kv_stride, 1, stream);
@@ -818,19 +823,22 @@ pmkvq_status pmkvq_set_attention_ctas(pmkvq_cache *k, int32_t n_ctas) {
 }
 
 // |K_rot| maxima into d_amax_bits (zero before the call).  Enough CTAs to fill the GPU several times over, each with at least
-// a thousand vectors behind its table of angles.  2048 tokens x 128 sequences x 8 heads, 537 MB: 98 us = 5.5 TB/s
-// (0.85 of the measured copy rate); with a 2-byte load and two shared-memory atomics per element it was 518 us.
+// a thousand vectors behind its table of angles.  2048 tokens x 128 sequences x 8 heads, 537 MB: a call (clear, this launch, the
+// power) takes 105 us = 5.1 TB/s, 0.78 of the measured copy rate; with a 2-byte load and two shared-memory atomics per element 525 us.
 static cudaError_t launch_absmax(const uint16_t *K, unsigned *d_amax_bits, int n_tokens, int n_seq, int kv_heads, double pos_scale,
                                  double theta, cudaStream_t st) {
+  int sms = 0;
+  const cudaError_t e = sm_count(sms);
+  if (e != cudaSuccess) return e;
   RopeFreqs freqs;
   for (int i = 0; i < 64; ++i) freqs.f[i] = std::pow(theta, -2.0 * i / (double)kHeadDim);
   int tokens = kAbsmaxTokens;
-  while (tokens < kAbsmaxMaxTokens && n_tokens > tokens * 148 * 8 && (long long)n_seq * kv_heads < 256) tokens += kAbsmaxTokens;
+  while (tokens < kAbsmaxMaxTokens && n_tokens > tokens * sms * 8 && (long long)n_seq * kv_heads < 256) tokens += kAbsmaxTokens;
   const int tc = (n_tokens + tokens - 1) / tokens;
   // split the sequences while that leaves a CTA 1024 vectors
   auto parts = [&](int seqs) { return (n_seq + seqs - 1) / seqs; };
   int seqs = n_seq;
-  while (seqs > 1 && (long long)tokens * ((seqs + 1) / 2) * kv_heads >= 1024 && (long long)tc * parts(seqs) < 148 * 16 &&
+  while (seqs > 1 && (long long)tokens * ((seqs + 1) / 2) * kv_heads >= 1024 && (long long)tc * parts(seqs) < sms * 16 &&
          parts((seqs + 1) / 2) <= 65535)
     seqs = (seqs + 1) / 2;
   uint64_t launches = 0;
