@@ -325,6 +325,11 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   asm("max.f32 %0, %1, %2, %3;\n" : "=f"(r) : "f"(a), "f"(b), "f"(c));
   return r;
 }
+__device__ __forceinline__ float min_or_nan(float a, float b) {  // fminf would pass over a NaN (the scale of infinities only, or of NaNs only)
+  float r;
+  asm("min.NaN.f32 %0, %1, %2;\n" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
 template <int BYTES>
 __device__ __forceinline__ void copy_async(uint32_t to, const void *from) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(to), "l"(from), "n"(BYTES) : "memory");
@@ -376,8 +381,7 @@ __device__ __forceinline__ TokenScale two_tokens(float2 mn, float2 mx) {
   TokenScale t;
   token_scale(mn.x, mx.x, t.nmn.x, t.s.x, t.ns.x, t.y.x, t.yl.x);
   token_scale(mn.y, mx.y, t.nmn.y, t.s.y, t.ns.y, t.y.y, t.yl.y);
-  // each on its own: the minimum and the maximum of the two would pass over a NaN (infinities only, NaNs only)
-  t.plain = t.s.x >= 0x1p-60f && t.s.x <= 0x1p60f && t.s.y >= 0x1p-60f && t.s.y <= 0x1p60f;
+  t.plain = min_or_nan(t.s.x, t.s.y) >= 0x1p-60f && fmaxf(t.s.x, t.s.y) <= 0x1p60f;
   return t;
 }
 // the codes of both values, one in each half of the result
