@@ -553,7 +553,7 @@ __device__ __forceinline__ QueryLoad load_query(const AttnParams &p, int b, int 
       q.raw.x = __ldcg(src) | ((uint32_t)__ldcg(src + 1) << 16);
       q.raw.y = __ldcg(src + 2) | ((uint32_t)__ldcg(src + 3) << 16);
     }
-    q.lam = __ldcg(reinterpret_cast<const float4 *>(p.lambda + hkv * kHeadDim + 4 * lane));
+    q.lam = *reinterpret_cast<const float4 *>(p.lambda + hkv * kHeadDim + 4 * lane);  // (as it was when the cache was made)
   }
   return q;
 }
