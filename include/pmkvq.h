@@ -89,7 +89,7 @@ void pmkvq_cache_destroy(pmkvq_cache *cache);
 /* Quantize-on-append (Eq. 1-2 at 16 bit; Keys multiplied by Lambda^-1 first, Eq. 9) of n_new
  * tokens, then window eviction: tokens leaving the INT16 window are shifted (Eq. 3, repeatedly)
  * to the block's current width.
- *   d_K_bf16, d_V_bf16: DEVICE bf16 [n_new][batch][kv_heads][128], read only.
+ *   d_K_bf16, d_V_bf16: DEVICE bf16 [n_new][batch][kv_heads][128], read only, on an 8-byte boundary (INVALID_ARG otherwise).
  * Returns BUDGET_FULL (state unchanged) if the block must be reduced first and auto_reduce is 0,
  * INVALID_ARG for n_new < 1 (an empty append is refused, nothing is launched), CAPACITY beyond max_tokens. */
 pmkvq_status pmkvq_append(pmkvq_cache *cache, int32_t layer, const void *d_K_bf16, const void *d_V_bf16,
