@@ -29,6 +29,7 @@
 //   scores:  S[h, t]  = sum_i Q''[h, i] * c_K[t, i]      A = Q'' (rows 0-7: fp16 "hi" part of the 8 heads,
 //                                                        rows 8-15: the "lo" remainder), B = K codes
 //   output:  O^T[i,h] = sum_t c_V[t, i] * w[t, h]        A = V codes, B = w = p * S_V (one fp16)
+// (With up to four query heads the 2- and 4-bit steps have the tokens on M and the heads' hi and lo parts as columns: process_tiles4.)
 // The per-token scale and zero-point never touch the codes: q.k = S_K (q.c) + Z_K sum(q) and
 // sum_t p_t v_t = sum_t (p_t S_V,t) c_t + sum_t p_t Z_V,t.
 //
@@ -39,6 +40,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <cstdint>
+#include <type_traits>
 
 #include "kernels_cache.cuh"
 #include "layout.cuh"
@@ -436,6 +438,135 @@ __device__ __forceinline__ void process_tiles(const uint8_t *tile0, uint32_t mas
   softmax_pv_phase<BITS, NT, MASKED>(tile0, mask, st, dot2, mu, sumq, inv_sigma_e, lane);
 }
 
+// ---- 2- and 4-bit steps of slices with at most four query heads -------------------------------------------------------
+// The other form's score MMAs have the heads' hi and lo rows on M and would be half empty.  Here the tokens are on M and the eight
+// columns are hi and lo of four heads: 8 score MMAs per tile instead of 16, no duplicated work on idle heads (a lane has two tokens
+// of one head per tile), and the weights' hi and lo parts fill the columns of the output MMAs, so the weight has 22 bits and the sums take
+// the probabilities as they are.  The lo part is scaled up by 2^11, so that weights that are subnormal as fp16 keep their bits too.
+// Instead of the other form, four heads (us per block of 64 slices x 32K tokens, four blocks in a launch): 2 bit 49.1 -> 41.9, 4 bit, close to what
+// memory gives, 51.3 -> 49.8 and at the clock that the power cap leaves 16 blocks x 64 slices x 20K tokens 611 -> 569 us a step.
+constexpr float kWeightLoScale = 2048.0f;
+struct WarpState4 {
+  float m;          // reference of head tig
+  float2 l, zs;     // sums over this lane's tokens, two partial sums each
+  float acc[8][4];  // O^T: columns 2 tig (weights' hi parts) and 2 tig + 1 (lo parts) of head tig
+};
+
+__device__ __forceinline__ uint32_t transpose_8x8(uint32_t x) {  // of 16-bit elements: lane 4 g + tig holds elements 2 tig, 2 tig + 1 of row g
+  uint32_t y;
+  asm("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
+  return y;
+}
+
+// A whole step.  s_q4: B fragments of the queries, entry (k-step s, lane) = head g / 2, part g mod 2 (0 hi, 1 lo), at channels as in q_fragment.
+// `mask` (NT == 1 only) as in softmax_phase; sumq4 over mu.
+template <int BITS, int NT, bool MASKED>
+__device__ __forceinline__ void process_tiles4(const uint8_t *tile0, uint32_t mask, WarpState4 &st, const uint2 *s_q4, float mu, float sumq,
+                                               float inv_sigma_e, int lane) {
+  using F = Fmt<BITS>;
+  constexpr int TB = tile_bytes(BITS);
+  const int g = lane >> 2;
+  // ---- scores: S = K Q''^T ----
+  float sacc[NT][4];
+  {
+    uint32_t kw[NT][2 * BITS];
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+      sacc[nt][0] = sacc[nt][1] = sacc[nt][2] = sacc[nt][3] = 0.f;
+#pragma unroll
+      for (int q = 0; q < BITS / 2; ++q) {
+        const uint4 a = *reinterpret_cast<const uint4 *>(tile0 + nt * TB + lane * 16 + q * 512);
+        kw[nt][4 * q] = a.x; kw[nt][4 * q + 1] = a.y; kw[nt][4 * q + 2] = a.z; kw[nt][4 * q + 3] = a.w;
+      }
+    }
+#pragma unroll
+    for (int w = 0; w < BITS; ++w) {
+      uint2 qf[F::N / 2];
+#pragma unroll
+      for (int jj = 0; jj < F::N / 2; ++jj) qf[jj] = s_q4[32 * ((w * F::N) / 2 + jj) + lane];
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt) {
+        uint32_t e0[F::N], e1[F::N];  // tokens g, g + 8
+        F::extract(kw[nt][w], e0);
+        F::extract(kw[nt][BITS + w], e1);
+#pragma unroll
+        for (int jj = 0; jj < F::N / 2; ++jj) mma_f16(sacc[nt], e0[2 * jj], e1[2 * jj], e0[2 * jj + 1], e1[2 * jj + 1], qf[jj].x, qf[jj].y);
+      }
+    }
+  }
+  // ---- softmax: tokens g and g + 8 of each tile, head tig ----
+  float2 sc[NT], s_e[NT], zv[NT];
+  float mx = -INFINITY;
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt) {
+    const float *rec = reinterpret_cast<const float *>(tile0 + nt * TB + meta_offset(BITS)) + (g >> 1) * 16 + (g & 1);
+    const float2 dot = make_float2(sacc[nt][0] + sacc[nt][1], sacc[nt][2] + sacc[nt][3]);
+    sc[nt] = __ffma2_rn(make_float2(rec[0], rec[2]), dot, __fmul2_rn(make_float2(rec[4], rec[6]), make_float2(sumq, sumq)));
+    s_e[nt] = make_float2(fmaxf(rec[8] * inv_sigma_e, 0x1p-10f), fmaxf(rec[10] * inv_sigma_e, 0x1p-10f));  // (the floor: see softmax_phase)
+    zv[nt] = make_float2(rec[12], rec[14]);
+    if constexpr (MASKED) {
+      if (!((mask >> g) & 1u)) { sc[nt].x = -INFINITY; s_e[nt].x = 1.f; zv[nt].x = 0.f; }
+      if (!((mask >> (g + 8)) & 1u)) { sc[nt].y = -INFINITY; s_e[nt].y = 1.f; zv[nt].y = 0.f; }
+    }
+    mx = max3(mx, sc[nt].x, sc[nt].y);
+  }
+  mx *= mu;
+  if (__any_sync(0xffffffffu, mx > st.m + kMaxAhead)) {
+#pragma unroll
+    for (int o = 4; o <= 16; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    const float m_new = fmaxf(st.m, mx), f = ex2(st.m - m_new);
+    st.m = m_new;
+    st.l = __fmul2_rn(st.l, make_float2(f, f));
+    st.zs = __fmul2_rn(st.zs, make_float2(f, f));
+#pragma unroll
+    for (int mt = 0; mt < 8; ++mt) {
+      st.acc[mt][0] *= f; st.acc[mt][1] *= f; st.acc[mt][2] *= f; st.acc[mt][3] *= f;
+    }
+  }
+  uint32_t pb[2 * NT];
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt) {
+    const float2 arg = __ffma2_rn(sc[nt], make_float2(mu, mu), make_float2(-st.m, -st.m));
+    const float2 p = make_float2(ex2(arg.x), ex2(arg.y));
+    st.l = __fadd2_rn(st.l, p);
+    st.zs = __ffma2_rn(p, zv[nt], st.zs);
+    const float2 w = __fmul2_rn(p, s_e[nt]);
+    const uint32_t hi = pack_half2(w.x, w.y);
+    const float2 back = __half22float2(*reinterpret_cast<const __half2 *>(&hi));
+    const float2 rest = __fmul2_rn(__fadd2_rn(w, make_float2(-back.x, -back.y)), make_float2(kWeightLoScale, kWeightLoScale));
+    const uint32_t lo = pack_half2(rest.x, rest.y);
+    pb[2 * nt] = transpose_8x8(__byte_perm(hi, lo, 0x5410));      // (hi, lo) of token g -> tokens 2 tig, 2 tig + 1 of column g
+    pb[2 * nt + 1] = transpose_8x8(__byte_perm(hi, lo, 0x7632));  // of token g + 8
+  }
+  pv_phase<BITS, NT>(tile0, st.acc, pb, lane);
+}
+
+// To the general form: accumulator columns 2 tig, 2 tig + 1 are heads, the sums of head g lie in its quad.
+__device__ __forceinline__ void to_general(const WarpState4 &a, WarpState &st, int lane) {
+  const int g = lane >> 2, tig = lane & 3, src0 = (lane & ~3) | (2 * tig & 3);
+  const bool some = tig < 2;
+#pragma unroll
+  for (int mt = 0; mt < 8; ++mt) {
+#pragma unroll
+    for (int rr = 0; rr < 2; ++rr) {
+      const float o = fmaf(a.acc[mt][2 * rr + 1], 1.0f / kWeightLoScale, a.acc[mt][2 * rr]);
+      const float o0 = __shfl_sync(0xffffffffu, o, src0), o1 = __shfl_sync(0xffffffffu, o, src0 + 1);
+      st.acc[mt][2 * rr] = some ? o0 : 0.f;
+      st.acc[mt][2 * rr + 1] = some ? o1 : 0.f;
+    }
+  }
+  float l = a.l.x + a.l.y, zs = a.zs.x + a.zs.y;
+#pragma unroll
+  for (int o = 4; o <= 16; o <<= 1) {
+    l += __shfl_xor_sync(0xffffffffu, l, o);
+    zs += __shfl_xor_sync(0xffffffffu, zs, o);
+  }
+  const float m_g = __shfl_sync(0xffffffffu, a.m, g & 3), l_g = __shfl_sync(0xffffffffu, l, g & 3), z_g = __shfl_sync(0xffffffffu, zs, g & 3);
+  st.m = g < 4 ? m_g : kNegBig;
+  st.l = make_float2(g < 4 && tig == 0 ? l_g : 0.f, 0.f);
+  st.zs = make_float2(g < 4 && tig == 0 ? z_g : 0.f, 0.f);
+}
+
 // ---- where the partials of a slice live ------------------------------------------------------
 // Slice s covers units [s U, (s+1) U); the segment of CTA c in it publishes partial number (c - cta_origin) + s.
 // A unit belongs to the CTA whose piece holds the unit's first fine unit (per_cta counts fine units).  Fine units
@@ -527,6 +658,17 @@ __device__ __forceinline__ void fill_q_fragments(uint4 *s_frag, const float (*s_
   if (i >= 0 && i < 256) {
     const int l = i & 31, g = l >> 2;
     s_frag[i] = q_fragment<BITS>(s_q, (int)s_stat[g], g, l & 3, i >> 5);
+  }
+}
+
+// The same fragments as process_tiles4 reads them, by the threads first_thread .. first_thread + 255.
+template <int BITS>
+__device__ __forceinline__ void fill_q_fragments4(uint2 *s_q4, const float (*s_q)[kHeadDim], const float *s_stat, int first_thread) {
+  const int i = (int)threadIdx.x - first_thread;
+  if (i >= 0 && i < 256) {
+    const int l = i & 31, h = l >> 3;
+    const uint4 f = q_fragment<BITS>(s_q, (int)s_stat[h], h, l & 3, i >> 5);
+    s_q4[i] = (l >> 2) & 1 ? make_uint2(f.y, f.w) : make_uint2(f.x, f.z);
   }
 }
 
@@ -807,7 +949,7 @@ __device__ __forceinline__ void segment_ranges(const AttnParams &p, int u_lo, in
 //   8 and 16 bit, bound by memory: INT16 tiles first, then body steps, both from counters, which keep the SM's share of the
 //     memory busy however the warps drift apart (dealt out as above: 2 % slower).
 // `ring` is the CTA's dynamic shared memory: the per-warp cp.async stages while tiles stream, then the warps' outputs.
-template <int BITS>
+template <int BITS, bool HEADS4>
 __device__ __forceinline__ void run_segment(const AttnParams &p, int slice, int u_lo, int u_hi,
                                             float (*s_q)[kHeadDim], float *s_stat, int *s_ctr, uint4 *s_frag,
                                             uint8_t *ring) {
@@ -883,7 +1025,8 @@ __device__ __forceinline__ void run_segment(const AttnParams &p, int slice, int 
   const int e_g = (int)s_stat[g];
   const float sumq = s_stat[8 + g];
   fill_q_fragments<16>(s_frag, s_q, s_stat);  // half of the threads each
-  if constexpr (BITS != 16) fill_q_fragments<BITS>(s_frag + 256, s_q, s_stat, 256);
+  if constexpr (HEADS4) fill_q_fragments4<BITS>(reinterpret_cast<uint2 *>(s_frag + 256), s_q, s_stat, 256);
+  else if constexpr (BITS != 16) fill_q_fragments<BITS>(s_frag + 256, s_q, s_stat, 256);
   __syncthreads();
 
   WarpState st;
@@ -930,6 +1073,28 @@ __device__ __forceinline__ void run_segment(const AttnParams &p, int slice, int 
         else process_tiles<BITS, 1, false>(src, 0xFFFFu, st, qa, mu, sumq, inv_sigma_e, lane);
       }
     } else {
+      WarpState4 st4;
+      float mu4 = 0.f, sumq4 = 0.f;
+      if constexpr (HEADS4) {
+        const int e4 = (int)s_stat[lane & 3];
+        mu4 = exp2i(24 - F::EQ + e4);
+        sumq4 = s_stat[8 + (lane & 3)] * exp2i(-e4) * exp2i(F::EQ - 24);
+        st4.m = kNegBig; st4.l = st4.zs = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int mt = 0; mt < 8; ++mt) st4.acc[mt][0] = st4.acc[mt][1] = st4.acc[mt][2] = st4.acc[mt][3] = 0.f;
+      }
+      // NT_ tiles of a step from the stage
+      auto step = [&](auto nt_, auto masked, const uint8_t *tile, uint32_t mask) {
+        constexpr int N = decltype(nt_)::value;
+        constexpr bool M = decltype(masked)::value;
+        if constexpr (HEADS4) {
+          process_tiles4<BITS, N, M>(tile, mask, st4, reinterpret_cast<const uint2 *>(s_frag + 256), mu4, sumq4, inv_sigma_e, lane);
+        } else {
+          process_tiles<BITS, N, M>(tile, mask, st, qa, mu, sumq, inv_sigma_e, lane);
+        }
+      };
+      const std::integral_constant<int, 1> one;
+      const std::integral_constant<int, NT> whole;
       for (int slot = 0; u < u_end; slot ^= 1) {
         int next;
         if constexpr (kDealt) {
@@ -945,19 +1110,20 @@ __device__ __forceinline__ void run_segment(const AttnParams &p, int slice, int 
         __syncwarp();
         const uint8_t *tile = my_ring + slot * SB;
         if (fast(u)) {
-          process_tiles<BITS, NT, false>(tile, 0xFFFFu, st, qa, mu, sumq, inv_sigma_e, lane);
+          step(whole, std::false_type(), tile, 0xFFFFu);
         } else {
 #pragma unroll 1
           for (int k = 0; k < NT; ++k) {
             const int tk = first_tile(u) + 8 * k;
             if (!live(tk)) continue;
-            if (tk == tail_tile) process_tiles<BITS, 1, true>(tile + k * TB, tail_mask, st, qa, mu, sumq, inv_sigma_e, lane);
-            else process_tiles<BITS, 1, false>(tile + k * TB, 0xFFFFu, st, qa, mu, sumq, inv_sigma_e, lane);
+            if (tk == tail_tile) step(one, std::true_type(), tile + k * TB, tail_mask);
+            else step(one, std::false_type(), tile + k * TB, 0xFFFFu);
           }
         }
         __syncwarp();
         u = next;
       }
+      if constexpr (HEADS4) to_general(st4, st, lane);
     }
   }
   if constexpr (F::SLOTS > 0) cp_async_wait<0>();
@@ -1105,7 +1271,11 @@ __device__ __forceinline__ void tc_teardown(TcCtx &tc) {
 // block: 25.0 -> 24.8 us per append and attention; 28 blocks x 4 slices x 3K tokens 42.7 -> 42.3 us per step.  At 4 and 2 bit the 16
 // registers are worth more (128 slices x 64K tokens at 2 bit, append and attention: 196 us, 203 with 112).
 constexpr int attn_registers(int bits) { return bits >= 8 ? 112 : 128; }
-template <int BODY_BITS, bool ROWS>
+// HEADS4 (both kernels): slices of at most four query heads, their 2- and 4-bit tiles in the form for these.  A segment in that form ends with
+// its state brought to the general one, half a microsecond more, so a launch takes it only if its CTAs have enough tiles
+// (heads4_pays); otherwise a 4K context at 4 bit, 32 tiles per CTA, went from 45.4 to 47.2 us for four steps.
+constexpr int kHeads4Tiles = 512;
+template <int BODY_BITS, bool ROWS, bool HEADS4>
 __global__ void __maxnreg__(attn_registers(BODY_BITS)) decode_attn_splitk_kernel(const AttnParams p, unsigned *error_word) {
   __shared__ __align__(16) float s_q[kMaxGroup][kHeadDim];
   __shared__ __align__(16) float s_stat[16 + 2 * kParts * kMaxGroup];  // head stats, per-partial (m, l)
@@ -1126,7 +1296,7 @@ __global__ void __maxnreg__(attn_registers(BODY_BITS)) decode_attn_splitk_kernel
     const int lo = max(u_begin - base, 0), hi = min(u_end - base, p.units_slice);
     if (hi > p.units_lead) {
       if constexpr (tensor_path) run_segment_tc<BODY_BITS>(p, slice, lo, hi, s_q, s_stat, s_ctr, s_frag, tc);
-      else run_segment<BODY_BITS>(p, slice, lo, hi, s_q, s_stat, s_ctr, s_frag, ring);
+      else run_segment<BODY_BITS, HEADS4>(p, slice, lo, hi, s_q, s_stat, s_ctr, s_frag, ring);
     }
   }
   if constexpr (tensor_path) tc_teardown(tc);
@@ -1213,7 +1383,7 @@ __device__ __forceinline__ void fused_layer_params(const FusedParams &fp, int l,
   p.qk_scale = fp.qk_scale;
 }
 
-template <bool ROWS>
+template <bool ROWS, bool HEADS4>
 __global__ void __maxnreg__(112) decode_attn_fused_kernel(const __grid_constant__ FusedParams fp) {
   __shared__ __align__(16) float s_q[kMaxGroup][kHeadDim];
   __shared__ __align__(16) float s_stat[16 + 2 * kParts * kMaxGroup];
@@ -1241,15 +1411,15 @@ __global__ void __maxnreg__(112) decode_attn_fused_kernel(const __grid_constant_
       const int lo = max(u_begin - base, 0), hi = min(u_end - base, p.units_slice);
       if (hi <= p.units_lead) continue;
       switch (p.cur_bits) {
-        case 16: run_segment<16>(p, slice, lo, hi, s_q, s_stat, s_ctr, s_frag, ring); break;
-        case 8: run_segment<8>(p, slice, lo, hi, s_q, s_stat, s_ctr, s_frag, ring); break;
+        case 16: run_segment<16, false>(p, slice, lo, hi, s_q, s_stat, s_ctr, s_frag, ring); break;
+        case 8: run_segment<8, false>(p, slice, lo, hi, s_q, s_stat, s_ctr, s_frag, ring); break;
         case 4:
           if constexpr (tensor_path) run_segment_tc<4>(p, slice, lo, hi, s_q, s_stat, s_ctr, s_frag, tc);
-          else run_segment<4>(p, slice, lo, hi, s_q, s_stat, s_ctr, s_frag, ring);
+          else run_segment<4, HEADS4>(p, slice, lo, hi, s_q, s_stat, s_ctr, s_frag, ring);
           break;
         default:
           if constexpr (tensor_path) run_segment_tc<2>(p, slice, lo, hi, s_q, s_stat, s_ctr, s_frag, tc);
-          else run_segment<2>(p, slice, lo, hi, s_q, s_stat, s_ctr, s_frag, ring);
+          else run_segment<2, HEADS4>(p, slice, lo, hi, s_q, s_stat, s_ctr, s_frag, ring);
           break;
       }
     }

@@ -194,12 +194,14 @@ cudaError_t launch_reduce(const LayerGeom &g, int n_slices, int n_tiles, cudaStr
 
 template <int BITS, bool ROWS>
 cudaError_t attention_setup_one(int &resident, int sms) {
-  cudaError_t e = cudaFuncSetAttribute(decode_attn_splitk_kernel<BITS, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       attn_smem_bytes<BITS, ROWS>());
+  constexpr int smem = attn_smem_bytes<BITS, ROWS>();
+  cudaError_t e = cudaFuncSetAttribute(decode_attn_splitk_kernel<BITS, ROWS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if constexpr (BITS <= 4 && !ROWS) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_attn_splitk_kernel<BITS, ROWS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  }
   int per_sm = 0;
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, decode_attn_splitk_kernel<BITS, ROWS>, kAttnThreads,
-                                                      attn_smem_bytes<BITS, ROWS>());
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, decode_attn_splitk_kernel<BITS, ROWS, false>, kAttnThreads, smem);
   resident = std::min(kMaxCtas, std::max(1, per_sm) * sms);
   return e;
 }
@@ -210,13 +212,14 @@ cudaError_t attention_setup_path(pmkvq_cache *k, int sms) {
   if (e == cudaSuccess) e = attention_setup_one<8, ROWS>(k->resident_ctas[1], sms);
   if (e == cudaSuccess) e = attention_setup_one<4, ROWS>(k->resident_ctas[2], sms);
   if (e == cudaSuccess) e = attention_setup_one<2, ROWS>(k->resident_ctas[3], sms);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(decode_attn_fused_kernel<ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             attn_fused_smem_bytes<ROWS>());
+  constexpr int smem = attn_fused_smem_bytes<ROWS>();
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_attn_fused_kernel<ROWS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if constexpr (!ROWS) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_attn_fused_kernel<ROWS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  }
   int per_sm = 0;
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, decode_attn_fused_kernel<ROWS>, kAttnThreads,
-                                                      attn_fused_smem_bytes<ROWS>());
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, decode_attn_fused_kernel<ROWS, false>, kAttnThreads, smem);
   k->resident_fused = std::min(kMaxCtas, std::max(1, per_sm) * sms);
   return e;
 }
@@ -510,11 +513,18 @@ static pmkvq_status attn_params(pmkvq_cache *k, int32_t layer, const void *d_Q, 
   return PMKVQ_OK;
 }
 
+// `tiles`: tiles of work a CTA has
+static bool heads4_pays(const pmkvq_cache *k, long long tiles) { return k->group <= 4 && !k->rows && tiles >= kHeads4Tiles; }
+
 template <int BITS>
 static cudaError_t attn_launch_width(pmkvq_cache *k, const AttnParams &p, unsigned n_ctas, cudaStream_t st, unsigned *error_word) {
   if (p.geom.rows)
-    return launch(k->launches, decode_attn_splitk_kernel<BITS, true>, n_ctas, kAttnThreads, attn_smem_bytes<BITS, true>(), st, p, error_word);
-  return launch(k->launches, decode_attn_splitk_kernel<BITS, false>, n_ctas, kAttnThreads, attn_smem_bytes<BITS, false>(), st, p, error_word);
+    return launch(k->launches, decode_attn_splitk_kernel<BITS, true, false>, n_ctas, kAttnThreads, attn_smem_bytes<BITS, true>(), st, p, error_word);
+  if constexpr (BITS <= 4) {
+    if (heads4_pays(k, p.per_cta))
+      return launch(k->launches, decode_attn_splitk_kernel<BITS, false, true>, n_ctas, kAttnThreads, attn_smem_bytes<BITS, false>(), st, p, error_word);
+  }
+  return launch(k->launches, decode_attn_splitk_kernel<BITS, false, false>, n_ctas, kAttnThreads, attn_smem_bytes<BITS, false>(), st, p, error_word);
 }
 
 static cudaError_t attn_launch(pmkvq_cache *k, const AttnParams &p, unsigned n_ctas, cudaStream_t st) {
@@ -587,9 +597,10 @@ static pmkvq_status attention_all_blocks(pmkvq_cache *k, const void *d_Q, float 
     while (fp.start[l0 + 1] <= (long long)c * fp.per_cta) ++l0;
     fp.first_layer[c] = (unsigned char)l0;
   }
-  const cudaError_t e =
-      k->rows ? launch(k->launches, decode_attn_fused_kernel<true>, n_ctas, kAttnThreads, attn_fused_smem_bytes<true>(), st, fp)
-              : launch(k->launches, decode_attn_fused_kernel<false>, n_ctas, kAttnThreads, attn_fused_smem_bytes<false>(), st, fp);
+  auto run = [&](auto kernel, int smem) { return launch(k->launches, kernel, n_ctas, kAttnThreads, smem, st, fp); };
+  const cudaError_t e = k->rows ? run(decode_attn_fused_kernel<true, false>, attn_fused_smem_bytes<true>())
+                        : heads4_pays(k, fp.per_cta / tile_weight(2)) ? run(decode_attn_fused_kernel<false, true>, attn_fused_smem_bytes<false>())
+                                                                      : run(decode_attn_fused_kernel<false, false>, attn_fused_smem_bytes<false>());
   return e == cudaSuccess ? PMKVQ_OK : PMKVQ_ERR_CUDA;
 }
 

@@ -1,0 +1,48 @@
+"""The form of the 2- and 4-bit decode attention for at most four query heads per KV head, against the fp64 oracle at the
+stated tolerance: group sizes, ragged body ends, one or several pieces per launch.  A launch takes that form if its CTAs have
+512 tiles of work or more, which one CTA has here."""
+import numpy as np
+import pytest
+import torch
+
+from tests.helpers import Mirror, make_inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("bits", [2, 4])
+@pytest.mark.parametrize("group,context,ctas", [(1, 2577, 1), (2, 2600, 1), (3, 3001, 1), (4, 2592, 1), (4, 6007, 2), (2, 9000, 2)])
+def test_four_heads_form_against_oracle(bits, group, context, ctas):
+    kvh, batch = 2, 1
+    m = Mirror(1, group * kvh, kvh, batch, context, [bits], window=32)
+    m.cache.restore_layer_state(0, 0, bits)
+    m.oracles[0].p.cur_bits = bits
+    k, v = make_inputs(31, 0, context, batch, kvh)
+    m.append(0, k, v)
+    m.cache.set_attention_ctas(ctas)
+    q = torch.randn(batch, group * kvh, 128, generator=torch.Generator().manual_seed(7)).bfloat16()
+    m.check_attention(0, q)
+    alone, all_blocks = m.cache.decode_attention(0, q.cuda()), m.cache.decode_attention_all(q[None].cuda())[0]
+    # (two partitions of one sum: the bound of the split-invariance test)
+    assert float((alone - all_blocks).abs().max()) <= 1e-3
+    # a smaller piece per CTA takes the general form: the same attention
+    m.cache.set_attention_ctas(64)
+    assert float((alone - m.cache.decode_attention(0, q.cuda())).abs().max()) <= 1e-3
+
+
+@pytest.mark.parametrize("bits", [2, 4])
+def test_four_heads_form_beside_the_exact_result(bits):
+    """No further from the exact result than the general form, whose weights are one fp16 each."""
+    kvh, group, context = 1, 4, 9000
+    m = Mirror(1, group, kvh, 1, context, [bits], window=32)
+    m.cache.restore_layer_state(0, 0, bits)
+    m.oracles[0].p.cur_bits = bits
+    k, v = make_inputs(32, 0, context, 1, kvh)
+    m.append(0, k, v)
+    q = torch.randn(1, group, 128, generator=torch.Generator().manual_seed(8)).bfloat16()
+    ref = m.oracles[0].decode_attention(q.float().numpy().reshape(kvh, group, 128)).reshape(group, 128)
+    err = []
+    for ctas in (1, 64):
+        m.cache.set_attention_ctas(ctas)
+        err.append(np.linalg.norm(m.cache.decode_attention(0, q.cuda()).cpu().numpy().reshape(group, 128) - ref))
+    assert err[0] <= err[1], err
