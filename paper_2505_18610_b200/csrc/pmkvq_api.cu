@@ -193,11 +193,11 @@ cudaError_t launch_reduce(const LayerGeom &g, int n_slices, int n_tiles, cudaStr
 }
 
 template <int BITS, bool ROWS>
-cudaError_t attention_setup_one(int &resident, int sms) {
+cudaError_t attention_setup_one(int &resident, int sms, bool heads4) {
   constexpr int smem = attn_smem_bytes<BITS, ROWS>();
   cudaError_t e = cudaFuncSetAttribute(decode_attn_splitk_kernel<BITS, ROWS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if constexpr (BITS <= 4 && !ROWS) {
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_attn_splitk_kernel<BITS, ROWS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess && heads4) e = cudaFuncSetAttribute(decode_attn_splitk_kernel<BITS, ROWS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   }
   int per_sm = 0;
   if (e == cudaSuccess)
@@ -208,14 +208,15 @@ cudaError_t attention_setup_one(int &resident, int sms) {
 
 template <bool ROWS>
 cudaError_t attention_setup_path(pmkvq_cache *k, int sms) {
-  cudaError_t e = attention_setup_one<16, ROWS>(k->resident_ctas[0], sms);
-  if (e == cudaSuccess) e = attention_setup_one<8, ROWS>(k->resident_ctas[1], sms);
-  if (e == cudaSuccess) e = attention_setup_one<4, ROWS>(k->resident_ctas[2], sms);
-  if (e == cudaSuccess) e = attention_setup_one<2, ROWS>(k->resident_ctas[3], sms);
+  const bool heads4 = k->group <= 4;  // else those kernels need not be loaded
+  cudaError_t e = attention_setup_one<16, ROWS>(k->resident_ctas[0], sms, heads4);
+  if (e == cudaSuccess) e = attention_setup_one<8, ROWS>(k->resident_ctas[1], sms, heads4);
+  if (e == cudaSuccess) e = attention_setup_one<4, ROWS>(k->resident_ctas[2], sms, heads4);
+  if (e == cudaSuccess) e = attention_setup_one<2, ROWS>(k->resident_ctas[3], sms, heads4);
   constexpr int smem = attn_fused_smem_bytes<ROWS>();
   if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_attn_fused_kernel<ROWS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if constexpr (!ROWS) {
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_attn_fused_kernel<ROWS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess && heads4) e = cudaFuncSetAttribute(decode_attn_fused_kernel<ROWS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   }
   int per_sm = 0;
   if (e == cudaSuccess)
